@@ -613,8 +613,296 @@ __global__ void __launch_bounds__(256, 2) screen_kernel(const ScreenArgs a) {
     pdl_trigger();
 }
 
-// Diagnostic evaluation of Eq. dual_bound_eq: one warp per (sequence, query head, block).
-__global__ void __launch_bounds__(128) score_dual_kernel(
+// ------------------------------------------------------------------ bounds on the tensor cores (eta_score_dual)
+//
+// A warp bounds a tile of TILE = 32 consecutive block records of one (sequence, KV head) row for all G query heads of
+// the group.  Both sums of Score_dual are small dense contractions over head_dim: <q, mu> runs in fp16, sum q^2 sigma^2
+// in tf32 with both factors split into two parts that hold them exactly.  The query side (A fragments) is prepared once
+// per CTA in shared memory; the records (B fragments) go from global memory straight into the registers of the lanes
+// that feed them to the MMAs.
+
+constexpr int TILE = 32;             // four 8-column MMA tiles
+constexpr int BND_WARPS = 4;
+
+// D(16x8, fp32) += A(16x8, tf32, row) * B(8x8, tf32, col)
+__device__ __forceinline__ void mma_tf32_1688(float (&c)[4], float a0, float a1, float a2, float a3, float b0, float b1) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(__float_as_uint(a0)), "r"(__float_as_uint(a1)), "r"(__float_as_uint(a2)), "r"(__float_as_uint(a3)),
+                   "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)));
+}
+// the leading 11 significant bits of x: what a tf32 operand holds, so that x = tf32_hi(x) + (x - tf32_hi(x)) exactly and
+// the rest of a 22-bit product fits tf32 too
+__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
+
+// The query side of a row's bounds, in the order the MMAs want it.  Lane (hd = lane / 4, t = lane % 4) feeds row hd (and
+// hd + 8) of A; in k-group j (32 coordinates) it holds coordinates 8 (4 j + t) .. + 7, the ones its 16-byte piece of a
+// record covers on the B side (a dot product does not care about the order of k).
+template <int D, int G>
+struct QTab {
+    static constexpr int J = D / 32;
+    static constexpr int NLO = (G == 8) ? 1 : 0;      // eight heads fill rows 0-7 of A: the second parts go to rows 8-15
+    uint4 f16[J][32];                                 // scaled q as fp16
+    float4 sq[J][32][2];                              // q^2: rows 0-3 leading parts of heads 0-3, rows 4-7 the rest (G <= 4);
+                                                      //      rows 0-7 leading parts (G = 8)
+    float4 sq_lo[NLO ? J : 1][NLO ? 32 : 1][2];       // G = 8: the rest
+    uint4 raw[G * D / 8];                             // the queries as they are (bf16)
+    float n2[J][8];                                   // partial squared norms
+    float norm[8];                                    // ||q_h||
+};
+
+// The power of two that puts a norm in [2^13, 2^14) is 2^qtab_shift.  fp16 holds neither the large nor the tiny end of
+// bf16's range, so a head's query is scaled by it (every coordinate then fits, and one below fp16's normal range is below
+// 2^-27 of the norm) and the sums are scaled back: both exact.  A norm that overflows fp32 gives NaN bounds (the block is
+// admitted), one that underflows to zero a zero sum.
+__device__ __forceinline__ int qtab_shift(float qn) { return min(max(140 - ((__float_as_int(qn) >> 23) & 0xff), -120), 120); }
+__device__ __forceinline__ float qtab_scale(float qn) {
+    const int ef = (__float_as_int(qn) >> 23) & 0xff;
+    return ef == 255 ? __int_as_float(0x7fc00000) : (ef == 0 ? 0.f : __int_as_float((127 + qtab_shift(qn)) << 23));
+}
+__device__ __forceinline__ float qtab_unscale(float qn) {
+    return ((__float_as_int(qn) >> 23) & 0xff) == 0 ? 0.f : __int_as_float((127 - qtab_shift(qn)) << 23);
+}
+
+// Every thread of the CTA calls this with the row's G queries; the first D threads (J warps) work.
+template <int D, int G>
+__device__ __forceinline__ void build_qtab(QTab<D, G>& tab, const __nv_bfloat16* __restrict__ q, int tid) {
+    constexpr int J = D / 32;
+    const bool mine = tid < D;
+    const int j = tid >> 5, hd = (tid & 31) >> 2, t = tid & 3;
+    const int head = hd & (G == 8 ? 7 : 3);           // rows 4-7 hold the second parts of heads 0-3
+    float x[8];
+    if (mine) {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (head < G) v = __ldg(reinterpret_cast<const uint4*>(q + head * D + 8 * (4 * j + t)));
+        if (hd < G) tab.raw[hd * (D / 8) + 4 * j + t] = v;
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        float n2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { x[2 * k] = bf16_lo(w[k]); x[2 * k + 1] = bf16_hi(w[k]); }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) n2 = fmaf(x[k], x[k], n2);
+        n2 += __shfl_xor_sync(0xffffffffu, n2, 1);
+        n2 += __shfl_xor_sync(0xffffffffu, n2, 2);
+        if (t == 0) tab.n2[j][hd] = n2;
+    }
+    __syncthreads();
+    if (mine) {
+        float n2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < J; ++k) n2 += tab.n2[k][hd];
+        const float qn = sqrtf(n2), sc = qtab_scale(qn);
+        uint32_t h[4];
+        float sq[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float a = x[2 * k] * sc, b = x[2 * k + 1] * sc;
+            const __half2 hh = __floats2half2_rn(a, b);
+            h[k] = (hd < G) ? *reinterpret_cast<const uint32_t*>(&hh) : 0u;
+            sq[2 * k] = a * a; sq[2 * k + 1] = b * b;       // exact: q has 8 significant bits
+        }
+        tab.f16[j][tid & 31] = make_uint4(h[0], h[1], h[2], h[3]);
+        const bool second = (G < 8) && hd >= 4;
+        float hi[8], lo[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { hi[k] = tf32_hi(sq[k]); lo[k] = sq[k] - hi[k]; }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float4 a = make_float4(hi[4 * u], hi[4 * u + 1], hi[4 * u + 2], hi[4 * u + 3]);
+            const float4 b = make_float4(lo[4 * u], lo[4 * u + 1], lo[4 * u + 2], lo[4 * u + 3]);
+            tab.sq[j][tid & 31][u] = second ? b : a;
+            if (G == 8) tab.sq_lo[j][tid & 31][u] = b;
+        }
+        if (j == 0 && t == 0 && hd < G) tab.norm[hd] = qn;
+    }
+    __syncthreads();
+}
+
+// One piece (eight coordinates) of a record's sigma as stored
+template <bool PACKED> struct SigmaPiece { uint4 v; };
+template <> struct SigmaPiece<true> { uint2 v; };
+template <int D, bool PACKED>
+__device__ __forceinline__ void load_sigma(SigmaPiece<PACKED>& s, const unsigned char* rec, int piece) {
+    if constexpr (PACKED) s.v = __ldcg(reinterpret_cast<const uint2*>(rec + 2 * D + piece * 8));
+    else s.v = __ldcg(reinterpret_cast<const uint4*>(rec + 2 * D + piece * 16));
+}
+template <bool PACKED>
+__device__ __forceinline__ void sigma_f32(const SigmaPiece<PACKED>& s, float (&out)[8]) {
+    if constexpr (PACKED) {
+        e4m3x8_to_f32(s.v, out);
+    } else {
+        const uint32_t w[4] = {s.v.x, s.v.y, s.v.z, s.v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[k]));
+            out[2 * k] = f.x; out[2 * k + 1] = f.y;
+        }
+    }
+}
+
+// Bounds of the n_rec (1 .. TILE) records that start at rec0, for all heads of the group, by one warp: sb[record][head].
+// mn: the lane's record's largest key norm.  sigma^2 has at most 22 significant bits (sigma is fp16) and q^2 sixteen: each
+// is the sum of two tf32 values, every product of parts is exact and the accumulation is fp32, so the variance term is
+// as good as one computed on the fp32 pipe, without a shuffle tree and with a quarter of the fp32 instructions.  A lane's
+// loads of the next k-group are issued as soon as a tile's registers are free.
+template <int D, int G, bool PACKED>
+__device__ __forceinline__ void bound_tile(const QTab<D, G>& tab, const unsigned char* __restrict__ rec0, int n_rec, float mn,
+                                           float z, float scale, float* __restrict__ sb) {
+    constexpr int J = D / 32, NT = TILE / 8, REC = PACKED ? 3 * D : 4 * D;
+    const int lane = threadIdx.x & 31, n8 = lane >> 2, t = lane & 3;
+    uint4 mu[NT];
+    SigmaPiece<PACKED> sg[NT];
+    const unsigned char* rp[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        rp[nt] = rec0 + (int64_t)min(nt * 8 + n8, n_rec - 1) * REC;
+        mu[nt] = __ldcg(reinterpret_cast<const uint4*>(rp[nt] + t * 16));
+        load_sigma<D, PACKED>(sg[nt], rp[nt], t);
+    }
+    float dot[NT][4], var[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) { dot[nt][c] = 0.f; var[nt][c] = 0.f; }
+#pragma unroll 1
+    for (int j = 0; j < J; ++j) {
+        const uint4 qa = tab.f16[j][lane];
+        const float4 sa = tab.sq[j][lane][0], sb4 = tab.sq[j][lane][1];
+        float4 la = make_float4(0.f, 0.f, 0.f, 0.f), lb = la;
+        if constexpr (G == 8) { la = tab.sq_lo[j][lane][0]; lb = tab.sq_lo[j][lane][1]; }
+        const int next = 4 * (j + 1) + t;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            mma_f16_16816(dot[nt], qa.x, 0u, qa.y, 0u, mu[nt].x, mu[nt].y);
+            mma_f16_16816(dot[nt], qa.z, 0u, qa.w, 0u, mu[nt].z, mu[nt].w);
+            if (j + 1 < J) mu[nt] = __ldcg(reinterpret_cast<const uint4*>(rp[nt] + next * 16));
+            float s[8], hi[8];
+            sigma_f32<PACKED>(sg[nt], s);
+            if (j + 1 < J) load_sigma<D, PACKED>(sg[nt], rp[nt], next);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) { s[k] *= s[k]; hi[k] = tf32_hi(s[k]); s[k] -= hi[k]; }
+            mma_tf32_1688(var[nt], sa.x, la.x, sa.y, la.y, hi[0], hi[1]);
+            mma_tf32_1688(var[nt], sa.x, la.x, sa.y, la.y, s[0], s[1]);
+            mma_tf32_1688(var[nt], sa.z, la.z, sa.w, la.w, hi[2], hi[3]);
+            mma_tf32_1688(var[nt], sa.z, la.z, sa.w, la.w, s[2], s[3]);
+            mma_tf32_1688(var[nt], sb4.x, lb.x, sb4.y, lb.y, hi[4], hi[5]);
+            mma_tf32_1688(var[nt], sb4.x, lb.x, sb4.y, lb.y, s[4], s[5]);
+            mma_tf32_1688(var[nt], sb4.z, lb.z, sb4.w, lb.w, hi[6], hi[7]);
+            mma_tf32_1688(var[nt], sb4.z, lb.z, sb4.w, lb.w, s[6], s[7]);
+        }
+    }
+    // lane (head n8, t) holds records 8 nt + 2 t and + 1
+    const float qn = tab.norm[n8 < G ? n8 : 0], un = qtab_unscale(qn);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float v2 = var[nt][c] + (G == 8 ? var[nt][c + 2] : __shfl_xor_sync(0xffffffffu, var[nt][c], 16));
+            const int rec = nt * 8 + 2 * t + c;
+            const float m = __shfl_sync(0xffffffffu, mn, rec);
+            if (n8 < G) sb[rec * G + n8] = scale * min_keep_nan((dot[nt][c] + z * sqrtf(v2)) * un, qn * m);
+        }
+    __syncwarp();
+}
+
+// Bound of one record by one warp in plain fp32, for all heads of the group (queries in shared memory).
+template <int D, int G, bool PACKED>
+__device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const unsigned char* __restrict__ src,
+                                          float mn, float z, float scale, float* __restrict__ sb) {
+    constexpr int LPR = D / 8;
+    const int lane = threadIdx.x & 31, cl = lane % LPR;
+    const uint4 m4 = __ldcg(reinterpret_cast<const uint4*>(src + cl * 16));
+    SigmaPiece<PACKED> sp;
+    load_sigma<D, PACKED>(sp, src, cl);
+    const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
+    float mu[8], s2[8];
+    sigma_f32<PACKED>(sp, s2);
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+        const float2 mf = __half22float2(*reinterpret_cast<const __half2*>(&mw[kk]));
+        mu[2 * kk] = mf.x; mu[2 * kk + 1] = mf.y;
+    }
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) s2[kk] *= s2[kk];
+#pragma unroll 1
+    for (int gq = 0; gq < G; ++gq) {
+        const uint4 qv = qw[gq * LPR + cl];
+        const uint32_t qq[4] = {qv.x, qv.y, qv.z, qv.w};
+        float dot = 0.f, var = 0.f, n2 = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+            const float x = (kk & 1) ? bf16_hi(qq[kk >> 1]) : bf16_lo(qq[kk >> 1]);
+            n2 = fmaf(x, x, n2);
+            dot = fmaf(x, mu[kk], dot);
+            var = fmaf(x * x, s2[kk], var);
+        }
+#pragma unroll
+        for (int sh = 1; sh < LPR; sh <<= 1) {
+            n2 += __shfl_xor_sync(0xffffffffu, n2, sh);
+            dot += __shfl_xor_sync(0xffffffffu, dot, sh);
+            var += __shfl_xor_sync(0xffffffffu, var, sh);
+        }
+        if (lane == 0) sb[gq] = scale * min_keep_nan(dot + z * sqrtf(var), sqrtf(n2) * mn);
+    }
+    __syncwarp();
+}
+
+// A tile's bounds including the records the tensor-core path cannot do: an infinite sigma has no exact split and a
+// query's norm may overflow, both of which show as a NaN bound, computed again in fp32.
+template <int D, int G, bool PACKED>
+__device__ __forceinline__ void bound_tile_checked(const QTab<D, G>& tab, const unsigned char* __restrict__ rec0, int n_rec,
+                                                   float mn, float z, float scale, float* __restrict__ sb) {
+    constexpr int REC = PACKED ? 3 * D : 4 * D;
+    bound_tile<D, G, PACKED>(tab, rec0, n_rec, mn, z, scale, sb);
+    const int lane = threadIdx.x & 31;
+    bool bad = false;
+#pragma unroll
+    for (int g = 0; g < G; ++g) bad = bad || (lane < n_rec && sb[lane * G + g] != sb[lane * G + g]);
+    unsigned todo = __ballot_sync(0xffffffffu, bad);
+    while (todo) {
+        const int rec = __ffs(todo) - 1;
+        todo &= todo - 1;
+        bound_one<D, G, PACKED>(tab.raw, rec0 + (int64_t)rec * REC, __shfl_sync(0xffffffffu, mn, rec), z, scale, sb + rec * G);
+    }
+}
+
+// Eq. dual_bound_eq for every block.  Bound by HBM (33.8 MB of records in, 8.4 MB of bounds out at 65536 blocks, d = 128,
+// G = 4: 6.4 us at the copy rate); a record is read once for all heads of its group, by 16-byte loads.  12.3 us there,
+// against 108 us with a warp per (head, block) that read every record G times in 2-byte pieces and reduced three sums
+// over 32 lanes for each.  A CTA takes `per` passes of BND_WARPS tiles of a row, which share one query table.
+template <int D, int G, bool PACKED>
+__global__ void __launch_bounds__(32 * BND_WARPS, 4) score_dual_kernel(
+    const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ musig, const float* __restrict__ mnorm,
+    const int32_t* __restrict__ seq_lens, int Hq, int Hkv, int b, int t_cap, int nb_cap, int per, int chunks, float z,
+    float scale, float* __restrict__ bound) {
+    constexpr int REC_BYTES = PACKED ? 3 * D : 4 * D;
+    constexpr int PASS = BND_WARPS * TILE;
+    __shared__ QTab<D, G> tab;
+    __shared__ float s_bound[BND_WARPS][TILE * G];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* const sb = s_bound[warp];
+    const int r = blockIdx.x / chunks, i = r / Hkv, hk = r % Hkv;
+    int T = __ldg(seq_lens + i);
+    T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
+    const int NB = min(T / b, nb_cap);
+    const int first = (blockIdx.x % chunks) * per * PASS;
+    if (first >= NB) return;
+    build_qtab<D, G>(tab, q + ((int64_t)i * Hq + hk * G) * D, tid);
+    for (int j0 = first + warp * TILE; j0 < min(NB, first + per * PASS); j0 += PASS) {
+        const int n_rec = min(TILE, NB - j0);
+        const int64_t rec = (int64_t)r * nb_cap + j0;
+        const float mn = lane < n_rec ? __ldg(mnorm + rec + lane) : 0.f;
+        bound_tile_checked<D, G, PACKED>(tab, musig + rec * REC_BYTES, n_rec, mn, z, scale, sb);
+        if (lane < n_rec) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) bound[((int64_t)i * Hq + hk * G + g) * nb_cap + j0 + lane] = sb[lane * G + g];
+        }
+        __syncwarp();
+    }
+}
+
+// The same for arrays that 16-byte loads cannot read (a caller's odd offset): one warp per (sequence, query head, block).
+__global__ void __launch_bounds__(128) score_dual_unaligned_kernel(
     const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ musig, const float* __restrict__ mnorm,
     const int32_t* __restrict__ seq_lens, int B, int Hq, int Hkv, int d, int b, int t_cap, int nb_cap, float z,
     float scale, int packed, float* __restrict__ bound) {
@@ -707,6 +995,18 @@ int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_ctas, cudaS
     return ETA_ERR_UNSUPPORTED;
 }
 
+template <int D, int G, bool PACKED>
+static int launch_score_t(const eta_cache_desc* desc, const __nv_bfloat16* q, const unsigned char* musig, const float* mnorm,
+                          const int32_t* seq_lens, float z, float scale, float* bound, cudaStream_t s) {
+    // four passes per CTA share one query table, one pass where four would leave SMs with fewer than four CTAs
+    const int rows = desc->batch * desc->n_kv_heads, passes = (desc->nb_cap + BND_WARPS * TILE - 1) / (BND_WARPS * TILE);
+    const int per = (int64_t)rows * passes >= 4 * 4 * 148 ? 4 : 1, chunks = (passes + per - 1) / per;
+    score_dual_kernel<D, G, PACKED><<<(unsigned)(rows * chunks), 32 * BND_WARPS, 0, s>>>(
+        q, musig, mnorm, seq_lens, desc->n_q_heads, desc->n_kv_heads, desc->block_size, desc->t_cap, desc->nb_cap, per, chunks,
+        z, scale, bound);
+    return check_launch("eta_score_dual");
+}
+
 }  // namespace eta
 
 extern "C" int eta_score_dual(const eta_cache_desc* desc, const eta_params* params, const void* q,
@@ -716,10 +1016,23 @@ extern "C" int eta_score_dual(const eta_cache_desc* desc, const eta_params* para
     if (rc != ETA_OK) return rc;
     if (!params || !q || !seq_lens || !musig || !mnorm || !bound) return ETA_ERR_INVALID_ARG;
     const float scale = params->scale > 0.f ? params->scale : 1.0f / sqrtf((float)desc->head_dim);
-    const int64_t warps = (int64_t)desc->batch * desc->n_q_heads * desc->nb_cap;
-    eta::score_dual_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __nv_bfloat16*>(q), static_cast<const unsigned char*>(musig), mnorm, seq_lens, desc->batch,
-        desc->n_q_heads, desc->n_kv_heads, desc->head_dim, desc->block_size, desc->t_cap, desc->nb_cap, params->z,
-        scale, (params->flags & ETA_FLAG_PACKED_SIGMA) ? 1 : 0, bound);
-    return eta::check_launch("eta_score_dual");
+    const bool packed = (params->flags & ETA_FLAG_PACKED_SIGMA) != 0;
+    auto qp = static_cast<const __nv_bfloat16*>(q);
+    auto mp = static_cast<const unsigned char*>(musig);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(musig)) & 15) {
+        const int64_t warps = (int64_t)desc->batch * desc->n_q_heads * desc->nb_cap;
+        eta::score_dual_unaligned_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
+            qp, mp, mnorm, seq_lens, desc->batch, desc->n_q_heads, desc->n_kv_heads, desc->head_dim, desc->block_size,
+            desc->t_cap, desc->nb_cap, params->z, scale, packed ? 1 : 0, bound);
+        return eta::check_launch("eta_score_dual");
+    }
+    const int D = desc->head_dim, G = desc->n_q_heads / desc->n_kv_heads;
+#define ETA_CASE(DD, GG) if (D == DD && G == GG) return packed \
+        ? eta::launch_score_t<DD, GG, true>(desc, qp, mp, mnorm, seq_lens, params->z, scale, bound, st) \
+        : eta::launch_score_t<DD, GG, false>(desc, qp, mp, mnorm, seq_lens, params->z, scale, bound, st);
+    ETA_CASE(128, 1) ETA_CASE(128, 2) ETA_CASE(128, 4) ETA_CASE(128, 8)
+    ETA_CASE(64, 1) ETA_CASE(64, 2) ETA_CASE(64, 4) ETA_CASE(64, 8)
+#undef ETA_CASE
+    return ETA_ERR_UNSUPPORTED;
 }
