@@ -94,3 +94,26 @@ def test_calibration_argument_checks():
     args = lambda d, bins: (2, 128, 8, 2, d, one, one, f, 5.0, 0.0, bins, -8.0, 8.0, f, f, one, n.value, None)
     assert lib.eta_calibrate_head_const(*args(96, 256)) == -2          # head_dim
     assert lib.eta_calibrate_head_const(*args(128, 8192)) == -2        # too many bins
+
+
+@pytest.mark.parametrize("T,d,n_bins,lim", [(65, 128, 100, 7.0), (2049, 64, 2, 0.01), (1500, 128, 33, 0.5)])
+def test_calibration_with_few_bins_and_ragged_tiles(T, d, n_bins, lim):
+    """Scores pile up in the end bins (the 32-bit halves of a bin's weight wrap many times) and the last tile is ragged.
+    The total weight is known exactly: row t adds t round(2^40 / t).  The bins differ from the oracle's by the scores
+    within 2e-6 of one of the n_bins - 1 edges: at density <= 0.4 / sigma_S of the scores (sigma_S = 1.5), n_bins - 1
+    edges, both sides of an edge, both bins: <= 8 * 2e-6 * 0.4 / 1.5 per edge, plus one score of a row of weight 1/T."""
+    eb = _eb()
+    dev = torch.device("cuda:0")
+    Q, K, tau = _split(500 + T, 1, 2, 1, T, d, qscale=1.5)
+    tau[0, 0, :5], tau[0, 1, -3:] = float("inf"), float("-inf")      # gates that are exactly 0 and 1
+    ref = orc.calibrate(bits(Q), bits(K), tau.numpy(), beta=5.0, n_bins=n_bins, s_min=-lim, s_max=lim)
+    hc, dbar = torch.empty(2, device=dev), torch.empty(2, device=dev)
+    ws = eb.eta_calibrate_head_const(Q.to(dev), K.to(dev), tau.to(dev), hc, dbar, beta=5.0, n_bins=n_bins, s_min=-lim, s_max=lim)
+    torch.cuda.synchronize()
+    H = ws[:2 * n_bins * 8].view(torch.int64).cpu().numpy().reshape(2, n_bins)
+    assert [int(h.sum()) for h in H] == [sum(t * ((2 ** 40 + t // 2) // t) for t in range(1, T + 1))] * 2
+    Hn = H / H.sum(axis=1, keepdims=True).astype(np.float64)
+    assert np.abs(Hn - ref["hist"]).sum(axis=1).max() <= (n_bins - 1) * (8 * 2e-6 * 0.4 / 1.5) + 4.0 / T / T
+    np.testing.assert_allclose(dbar.cpu().numpy(), ref["dbar"], rtol=0, atol=1e-6)
+    for h in range(2):
+        assert abs(orc.calibration_density(ref["hist"][h], -lim, lim, 5.0, float(hc[h])) - ref["dbar"][h]) <= 5e-6
