@@ -88,8 +88,8 @@ struct ScreenArgs {
     int lwb, rescue_window;
     uint32_t flags;
     int Hq, Hkv, b, b_shift, t_cap, nb_cap, nseg, rows;
-    int n_early, per_early, per_late;     // item split over the CTAs: the first n_early share per_early items evenly, the rest take per_late each
-    FastDiv div_nseg, div_hkv;
+    int passes, group;                    // passes of a row; passes whose bounds are kept before their admission is decided
+    FastDiv div_chunks, div_hkv;          // div_chunks: CTAs per row
     int32_t* seg_count;
     int32_t* seg_list;
     RescueRec* seg_resc;
@@ -98,7 +98,7 @@ struct ScreenArgs {
     uint32_t* status;
     unsigned long long* timeline;
 };
-int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_ctas, cudaStream_t s);
+int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_sm, cudaStream_t s);
 
 // Launch with programmatic dependent launch allowed: the grid may start while its predecessor in the stream is
 // still draining, and must call pdl_wait() before touching anything the predecessor wrote.

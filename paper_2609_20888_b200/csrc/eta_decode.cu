@@ -1180,7 +1180,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     sa.Hq = desc->n_q_heads; sa.Hkv = desc->n_kv_heads; sa.b = b; sa.t_cap = desc->t_cap; sa.nb_cap = desc->nb_cap;
     sa.nseg = L.nseg; sa.rows = L.rows;
     sa.b_shift = (b == 32) ? 5 : (b == 64 ? 6 : 7);
-    sa.div_nseg = FastDiv(L.nseg); sa.div_hkv = FastDiv(desc->n_kv_heads);
+    sa.div_hkv = FastDiv(desc->n_kv_heads);
     sa.seg_count = reinterpret_cast<int32_t*>(ws + L.seg_count);
     sa.seg_list = reinterpret_cast<int32_t*>(ws + L.seg_list);
     sa.seg_resc = reinterpret_cast<RescueRec*>(ws + L.seg_resc);
@@ -1189,7 +1189,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     sa.timeline = debug_timeline();
     sa.status = status_dev;
     profile_mark(2, s);
-    rc = launch_screen(sa, L.rows, D, G, 2 * n_sm, s);
+    rc = launch_screen(sa, L.rows, D, G, n_sm, s);
     profile_mark(3, s);
     if (rc != ETA_OK) return rc;
 
