@@ -124,11 +124,10 @@ WsLayout ws_layout(const eta_cache_desc* d) {
     int G = d->n_q_heads / d->n_kv_heads;
     L.rows = d->batch * d->n_kv_heads;
     L.nseg = (d->nb_cap + SEG - 1) / SEG;
-    L.entries = L.rows * (L.nseg + 2);
+    L.gpr = (L.nseg + GRANULE - 1) / GRANULE;
     size_t off = 0;
-    L.seg_count = off;  off = align_up(off + sizeof(int32_t) * (size_t)L.rows * L.nseg, 256);
+    L.seg_cnt = off;    off = align_up(off + (size_t)L.rows * L.gpr * GRANULE, 256);
     L.seg_list = off;   off = align_up(off + sizeof(int32_t) * (size_t)L.rows * L.nseg * LSTRIDE, 256);
-    L.seg_resc = off;   off = align_up(off + sizeof(RescueRec) * (size_t)L.rows * L.nseg * G, 256);
     L.row_span = off;   off = align_up(off + sizeof(int2) * (size_t)L.rows, 256);
     L.tau_eff = off;    off = align_up(off + sizeof(float) * (size_t)d->batch * d->n_q_heads, 256);
     size_t slots = ((size_t)MAX_CTAS + L.rows) * DECODE_GROUPS;

@@ -32,6 +32,7 @@ void profile_mark(int k, cudaStream_t s);
 // LSTRIDE slots (SEG plus room for one rescued block per query head).
 constexpr int SEG = 64;
 constexpr int LSTRIDE = SEG + 8;
+constexpr int GRANULE = 16;           // segments whose survivor counts are read with one 16-byte load
 constexpr int MAX_CTAS = 256;        // upper bound on streaming CTAs (sizes the scratch; a B200 has 148 SMs)
 constexpr int MAX_ROWS = 1024;        // rows (batch * n_kv_heads) whose unit prefix a streaming CTA keeps in shared memory
 constexpr int DECODE_GROUPS = 3;     // consumer groups per streaming CTA, each with its own partial per piece
@@ -40,10 +41,9 @@ constexpr int DECODE_GROUPS = 3;     // consumer groups per streaming CTA, each 
 struct WsLayout {
     int rows;        // batch * n_kv_heads
     int nseg;        // segments per row
-    int entries;     // rows * (nseg + 2): per row its segments, a rescue pseudo-entry and a tail pseudo-entry
-    size_t seg_count;   // int32 [rows * nseg]
+    int gpr;         // granules per row: groups of GRANULE segments, the last one padded
+    size_t seg_cnt;     // uint8 [rows * gpr * GRANULE]: survivors of each segment (zero in the padding)
     size_t seg_list;    // int32 [rows * nseg * LSTRIDE]: block index | head bits << 24
-    size_t seg_resc;    // {int cnt; float maxb; int arg; int pad} [rows * nseg * G]
     size_t row_span;    // int2 [rows]: first streaming CTA that holds units of the row, number of such CTAs (written by the streaming kernel)
     size_t tau_eff;     // float [batch * n_q_heads]
     size_t part_ml;     // float2 [(MAX_CTAS + rows) * DECODE_GROUPS * G]
@@ -51,8 +51,6 @@ struct WsLayout {
     size_t total;
 };
 WsLayout ws_layout(const eta_cache_desc* d);
-
-struct RescueRec { int cnt; float maxb; int arg; int pad; };
 
 // Division by a run-time constant as multiply-high + shift (exact for 0 <= n < 2^31): integer division costs
 // dozens of instructions, and the single-warp set-up code of the kernels divides by the same few numbers.
@@ -88,11 +86,13 @@ struct ScreenArgs {
     int lwb, rescue_window;
     uint32_t flags;
     int Hq, Hkv, b, b_shift, t_cap, nb_cap, nseg, rows;
-    int passes, group;                    // passes of a row; passes whose bounds are kept before their admission is decided
-    FastDiv div_chunks, div_hkv;          // div_chunks: CTAs per row
-    int32_t* seg_count;
+    int passes, head;                     // passes of a row; of them the row's first CTA takes `head`, the others share the rest
+    int group;                            // passes whose bounds are kept before their admission is decided
+    int nbuf;                             // tiles a warp keeps in flight
+    FastDiv div_chunks, div_rest, div_hkv;          // CTAs per row, those but the first
+    uint8_t* seg_cnt;
+    int gpr;
     int32_t* seg_list;
-    RescueRec* seg_resc;
     float* tau_eff;
     uint8_t* sel_mask;
     uint32_t* status;

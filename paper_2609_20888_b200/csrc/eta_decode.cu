@@ -5,8 +5,9 @@
 //
 // decode_kernel is persistent, one CTA per SM.  Work is the flattened sequence
 // of "units": for each (sequence, KV head) row its surviving blocks (the
-// screening kernel's per-segment lists), then its rescued blocks, then its tail.
-// Every CTA lays that sequence out for itself from the per-segment counts and
+// screening kernel's per-segment lists), then its tail.
+// Every CTA finds its place in that sequence from the per-segment counts (one
+// warp, one round trip to memory for up to 4096 segments, no CTA barrier) and
 // takes an equal, contiguous share of its COST (units, plus a fixed charge for
 // every row boundary inside the share: stream-K), so the load is balanced
 // whatever the per-head survivor counts are; a share may cross rows, and a row
@@ -39,20 +40,21 @@ struct DecodeArgs {
     const int32_t* seq_lens;
     const float* tau_eff;
     const int32_t* seg_list;
-    const int32_t* seg_count;
-    const RescueRec* seg_resc;
-    uint8_t* sel_mask;
+    const uint8_t* seg_cnt;
     int32_t* stats;
     int2* row_span;      // [rows] first streaming CTA that holds units of the row, number of such CTAs
     float2* part_ml;
     float* part_o;
     uint32_t* status;
     float beta, scale;
-    int Hq, Hkv, G, b, t_cap, nb_cap, nseg, entries, rows, rescue_window;
+    int Hq, Hkv, G, b, t_cap, nb_cap, nseg, rows;
+    int gpr, n_gran;     // granules (16 segments) of a row, of all rows
+    int lane_gran;       // granules a lane takes of a chunk: 8, fewer where all of them are less than a chunk
+    int n_chunks, super; // chunks of 32 lanes x 8 granules; chunks whose sums share an entry in shared memory
     int ungate_last;     // the newest token of every sequence keeps its raw logit (ETA_FLAG_UNGATE_LAST)
     const int32_t* block_table;   // paged cache: [batch, table_stride] page of every block of tokens; null: contiguous
     int table_stride;
-    FastDiv div_nseg, div_epr, div_hkv, div_g;
+    FastDiv div_gpr, div_hkv, div_grid;
     unsigned long long* timeline;
 };
 
@@ -60,10 +62,14 @@ constexpr uint32_t UF_END = 1u;
 constexpr int WARPS_PER_GROUP = 4;     // the four warps of a group each take a quarter of a tile's tokens
 // Tiles a row boundary inside a CTA's range is worth (flush of the partials, query reload, a pipeline that runs dry
 // while a group flushes).  Measured: 3 left the CTAs with several pieces last by 8 us on the mixed-length
-// configuration (128 rows); 6, 8, 10 and 14 are within noise of each other on every configuration.
-constexpr int PIECE_COST = 8;
-constexpr int RESC_ROWS = 8;           // rows (from the CTA's first) whose rescue decisions stay in shared memory
-constexpr int PW = 256;                // entries of the unit prefix the producer keeps in shared memory
+// configuration (128 rows); 6, 8, 10 and 14 are within noise of each other on every configuration.  Where that would
+// leave SMs without work (a CTA needs more cost units than a row's padding) a boundary counts as one tile: a problem of
+// 50 blocks then runs on 24 CTAs of two tiles instead of 6 of ten.
+constexpr int PIECE_COST = 8, PIECE_COST_SMALL = 1;
+constexpr int LGRAN = 8;               // granules per lane of a chunk
+constexpr int CHUNK = 32 * LGRAN;      // granules of a chunk: what a warp reads in one round trip
+constexpr int MAX_SUPER = 512;         // sums over `super` chunks each, kept in shared memory when there is more than one chunk
+constexpr int SPAN_ROWS = 64;          // rows a CTA publishes at a time
 
 __device__ __forceinline__ uint32_t u4_get(const uint4& v, int i) {
     return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
@@ -78,60 +84,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 
-// Top-1 rescue of query head g of row r (Algorithm 3, rescue phase): if none of the first
-// Wr = min(rescue_window, NB) blocks was admitted for the head, the first block with the largest bound among them
-// is.  Combines the per-segment statistics the screening kernel left.  -> rescued block index, or -1.
-__device__ __forceinline__ int rescue_of(const RescueRec* __restrict__ seg_resc, int r, int g, int G, int nseg,
-                                          int Wr) {
-    if (Wr <= 0) return -1;
-    const int nsw = (Wr + SEG - 1) / SEG;
-    int cnt = 0, arg = -1;
-    float best = -INFINITY;
-    for (int s0 = 0; s0 < nsw; s0 += 4) {
-        int4 raw[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)          // four segments' statistics in flight at once
-            raw[k] = (s0 + k < nsw) ? __ldg(reinterpret_cast<const int4*>(seg_resc + ((int64_t)r * nseg + s0 + k) * G + g))
-                                    : make_int4(0, 0, -1, 0);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            cnt += raw[k].x;
-            const float mb = __int_as_float(raw[k].y);
-            if (raw[k].z >= 0 && mb > best) { best = mb; arg = raw[k].z; }   // ascending segments: ties keep the lowest index
-        }
-    }
-    if (cnt != 0) return -1;
-    return arg < 0 ? 0 : arg;
-}
-
-// The rescued blocks of a row as fetch units: heads that rescue the same block share one unit.
-// -> number of units; unit k is block uj[k] with head bits um[k].
-__device__ __forceinline__ int rescue_units(const RescueRec* __restrict__ seg_resc, int r, int G, int nseg, int Wr,
-                                            int (&uj)[8], int (&um)[8]) {
-    int n = 0;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        uj[g] = -1; um[g] = 0;
-    }
-#pragma unroll
-    for (int g = 0; g < 8; ++g) {
-        if (g < G) {
-            const int j = rescue_of(seg_resc, r, g, G, nseg, Wr);
-            if (j >= 0) {
-                bool merged = false;
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (k < n && uj[k] == j) { um[k] |= 1 << g; merged = true; }
-                if (!merged) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        if (k == n) { uj[k] = j; um[k] = 1 << g; }
-                    ++n;
-                }
-            }
-        }
-    }
-    return n;
+// sum of the 16 survivor counts of a granule
+__device__ __forceinline__ int granule_sum(const uint4& v) {
+    return (int)__dp4a(v.x, 0x01010101u, __dp4a(v.y, 0x01010101u, __dp4a(v.z, 0x01010101u, __dp4a(v.w, 0x01010101u, 0u))));
 }
 
 template <int D, int TS, int NSTAGE, int NGROUPS>
@@ -139,14 +94,14 @@ struct DecodeSmem {
     static constexpr int HALVES = D / 64;
     static constexpr int TILE_BYTES = TS * 128;                 // one 64-column half tile
     static constexpr int STAGE_BYTES = 2 * HALVES * TILE_BYTES; // K halves then V halves
-    static constexpr int BAR_OFF = NSTAGE * STAGE_BYTES;        // full[NSTAGE], empty[NSTAGE], flush[NGROUPS]
-    static constexpr int DESC_OFF = BAR_OFF + 8 * (2 * NSTAGE + NGROUPS + (NGROUPS & 1));
-    static constexpr int WIN_OFF = DESC_OFF + 16 * NSTAGE;      // int32 pwin[PW + 1] (+3 pad): window of the unit prefix
-    static constexpr int ROW_OFF = WIN_OFF + 4 * (PW + 4);      // int32 rowbase[MAX_ROWS + 1]: unit prefix over rows
-    static constexpr int INFO_OFF = ROW_OFF + 4 * (MAX_ROWS + 4);   // uint8 per row: rescue units | tail flag << 7
-    static constexpr int NZP_OFF = INFO_OFF + MAX_ROWS;         // uint16 per row: rows with at least one unit before the row
-    static constexpr int RESC_OFF = NZP_OFF + 2 * MAX_ROWS;     // int32 [RESC_ROWS][8]: rescued block per head, first rows
-    static constexpr int ML_OFF = RESC_OFF + 4 * 8 * RESC_ROWS; // float m[NGROUPS][4][8], l[NGROUPS][4][8]
+    static constexpr int BAR_OFF = NSTAGE * STAGE_BYTES;        // full[NSTAGE], empty[NSTAGE], flush[NGROUPS], layout
+    static constexpr int DESC_OFF = (BAR_OFF + 8 * (2 * NSTAGE + NGROUPS + 1) + 15) / 16 * 16;
+    static constexpr int WIN_OFF = DESC_OFF + 16 * NSTAGE;      // uint4 [32]: the producer's window of granules
+    static constexpr int GRAN_OFF = WIN_OFF + 16 * 32;          // uint4 [CHUNK]: all granules (one chunk), else int2 [MAX_SUPER]: sums
+    static constexpr int SPAN_OFF = GRAN_OFF + 16 * CHUNK;      // int2 [SPAN_ROWS + 1] (+ pad): units and live rows before a row
+    static constexpr int INFO_OFF = SPAN_OFF + 8 * (SPAN_ROWS + 2);     // uint8 per row: bit 0 has tokens, bit 1 has a tail
+    static constexpr int ML_OFF = INFO_OFF + MAX_ROWS;          // float m[NGROUPS][4][8], l[NGROUPS][4][8]
+    static_assert(16 * CHUNK >= 8 * MAX_SUPER, "sums of the super-chunks share the granules' place");
     static constexpr int MO_OFF = ML_OFF + 4 * 2 * NGROUPS * WARPS_PER_GROUP * 8;
     static size_t bytes(int G) { return 1024 + MO_OFF + sizeof(float) * NGROUPS * WARPS_PER_GROUP * G * D; }
 };
@@ -170,12 +125,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::BAR_OFF);
     uint64_t* empty = full + NSTAGE;
     uint64_t* flushbar = empty + NSTAGE;
+    uint64_t* laybar = flushbar + NGROUPS;
     int4* desc = reinterpret_cast<int4*>(smem + L::DESC_OFF);
-    int32_t* pwin = reinterpret_cast<int32_t*>(smem + L::WIN_OFF);
-    int32_t* rowbase = reinterpret_cast<int32_t*>(smem + L::ROW_OFF);
     uint8_t* rowinfo = smem + L::INFO_OFF;
-    uint16_t* nzp = reinterpret_cast<uint16_t*>(smem + L::NZP_OFF);
-    int32_t* resc_tab = reinterpret_cast<int32_t*>(smem + L::RESC_OFF);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long* const tl = ETA_TL(a.timeline ? a.timeline + (size_t)(TL_DECODE + blockIdx.x) * 8 : nullptr);
@@ -192,256 +144,346 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         s_fill_started = 0;
         for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], WARPS_PER_GROUP); }
         for (int k = 0; k < NGROUPS; ++k) mbar_init(&flushbar[k], 32 * WARPS_PER_GROUP);
+        mbar_init(laybar, 1);
         fence_barrier_init();
         prefetch_tmap(&tmK);
         prefetch_tmap(&tmV);
     }
-    // scratch for the layout, in the (still unused) stage memory
+    // what is known before the predecessor kernel is through: which rows have tokens and which a tail (a caller input)
     constexpr int NWARPS = WARPS_PER_GROUP * NGROUPS + 1;
     constexpr int NTHREADS = 32 * NWARPS;
-    int* resc_j = reinterpret_cast<int*>(smem);                // [rows][8] rescued block per head, -1: none
-    int* s_len = resc_j + 8 * MAX_ROWS;                        // [rows] clamped sequence length
-    int* rowcnt = s_len + MAX_ROWS;                            // [rows] surviving blocks of the row
-    // [rows][nseg + 2] units per entry of the flattened sequence: a row's segments (surviving blocks), then its rescue
-    // units, then its tail (0 or 1): what the producer's first prefix window is summed from, one byte load per entry
-    uint8_t* cnt8 = reinterpret_cast<uint8_t*>(rowcnt + MAX_ROWS);
-    const bool counts_in_smem = (size_t)a.entries + 10 * 4 * MAX_ROWS <= (size_t)NSTAGE * L::STAGE_BYTES;
-    // sequence lengths are a caller input: they can be read while the previous kernel is still running
+    __shared__ int s_row0;                // row of the CTA's first unit; -1: no work
     for (int rr = tid; rr < a.rows; rr += NTHREADS) {
-        const int T = __ldg(a.seq_lens + a.div_hkv.div(rr));
-        s_len[rr] = T < 0 ? 0 : (T > a.t_cap ? a.t_cap : T);
-        rowcnt[rr] = 0;
+        int T = __ldg(a.seq_lens + a.div_hkv.div(rr));
+        T = T < 0 ? 0 : (T > a.t_cap ? a.t_cap : T);
+        rowinfo[rr] = (uint8_t)((T > 0 ? 1 : 0) | ((T & (a.b - 1)) ? 2 : 0));
     }
     __syncthreads();
-    pdl_wait();          // the screening kernel's lists, counts and window statistics are complete from here on
+
+    // ---- layout.  The flattened sequence of units is cut up by granules, 16 segments of a row each (the last one of a row
+    // also holds its tail unit).  Lane l of a warp takes the consecutive granules l lane_gran .. of a chunk; a scan over the
+    // lanes gives each its first unit.  A row that starts inside a CTA's share costs that CTA a flush of its partials and
+    // a query reload, worth `pc` tiles: row r spans the cost interval [units before + pc * live rows before, + pc (if it
+    // has units) + its units).  Every live row has at least one unit (a tail, or what top-1 rescue leaves).
+    uint32_t headm = 0, tailm = 0;        // bit m: the lane's granule m of the chunk is the first of a live row / ends a row with a tail
+    auto lane_flags = [&](int ch) {
+        headm = tailm = 0;
+#pragma unroll 1
+        for (int m = 0; m < a.lane_gran; ++m) {
+            const int q = ch * CHUNK + lane * a.lane_gran + m;
+            if (q >= a.n_gran) break;
+            int r, pos;
+            a.div_gpr.divmod(q, r, pos);
+            const int info = rowinfo[r];
+            headm |= (uint32_t)(pos == 0 && (info & 1)) << m;
+            tailm |= (uint32_t)(pos == a.gpr - 1 && (info & 2)) << m;
+        }
+    };
+    int us[LGRAN];                        // units of the lane's granules
+    int lane_u = 0, lane_z = 0;           // units / live rows in the lane's granules
+    const uint4* const gran = reinterpret_cast<const uint4*>(a.seg_cnt);
+    uint4* const gran_s = reinterpret_cast<uint4*>(smem + L::GRAN_OFF);
+    int2* const super_s = reinterpret_cast<int2*>(smem + L::GRAN_OFF);
+    auto load_chunk = [&](int ch, bool keep) {
+        uint4 v[LGRAN];
+#pragma unroll
+        for (int m = 0; m < LGRAN; ++m) {
+            const int q = ch * CHUNK + lane * a.lane_gran + m;
+            v[m] = make_uint4(0, 0, 0, 0);
+            if (m < a.lane_gran && q < a.n_gran) v[m] = __ldcg(gran + q);
+        }
+        lane_u = 0;
+#pragma unroll
+        for (int m = 0; m < LGRAN; ++m) {
+            us[m] = 0;
+            if (m < a.lane_gran) {
+                us[m] = granule_sum(v[m]) + (int)((tailm >> m) & 1);
+                lane_u += us[m];
+                if (keep) gran_s[lane * a.lane_gran + m] = v[m];
+            }
+        }
+        lane_z = __popc(headm);
+    };
+    int pre_u = 0, pre_z = 0, tot_u = 0, tot_z = 0;       // before the lane within the chunk; of the chunk
+    auto scan_chunk = [&]() {
+        uint32_t x = (uint32_t)lane_u | ((uint32_t)lane_z << 20);          // a chunk: < 2^19 units, <= 256 rows
+#pragma unroll
+        for (int sft = 1; sft < 32; sft <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, x, sft);
+            if (lane >= sft) x += o;
+        }
+        const uint32_t t = __shfl_sync(0xffffffffu, x, 31);
+        tot_u = (int)(t & 0xfffffu); tot_z = (int)(t >> 20);
+        pre_u = (int)(x & 0xfffffu) - lane_u; pre_z = (int)(x >> 20) - lane_z;
+    };
+    const bool one_chunk = a.n_chunks == 1;
+    const bool lays_out = warp == PRODUCER_WARP || warp == 0;              // the producer, and the warp that publishes
+    if (one_chunk && lays_out) lane_flags(0);
+    pdl_wait();          // the screening kernel's lists and counts are complete from here on
     if (tl && tid == 0) tl[7] = globaltimer_ns();
     const unsigned long long clk0 = ETA_TL(reinterpret_cast<unsigned long long*>(1)) ? (unsigned long long)clock64() : 0ull;
 
-    // ---- every CTA lays out the flattened unit sequence for itself: per row the surviving blocks of its
-    // segments, then its rescued blocks, then its tail; a scan over the rows gives each row's first unit.
-    // The code below runs once per CTA on a cold instruction cache, where every instruction costs tens of cycles:
-    // it is written as small loops rather than unrolled, and with as few dependent round trips to L2 as the data
-    // allow (one for the counts and window statistics, later one for the first list words).
-    __shared__ int s_lay[5];      // rows with units; the CTA's unit range; CTAs that share the units; row of the first unit
-    {
-        // All loads of the layout are independent and issued together, before any of them is consumed: per thread
-        // eight segment counts and, for the thread's (row, head) pair, the window statistics of up to four segments
-        // of the rescue window.
-        const int n_cnt = a.rows * a.nseg, n_rh = a.rows * a.G;
-        auto resc_load = [&](int p, int s0, int4 (&raw)[4], int& Wr) {
-            int rr, g;
-            a.div_g.divmod(p, rr, g);
-            Wr = (p < n_rh) ? min(a.rescue_window, min(s_len[min(rr, a.rows - 1)] / a.b, a.nb_cap)) : 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                raw[k] = ((s0 + k) * SEG < Wr)
-                    ? __ldg(reinterpret_cast<const int4*>(a.seg_resc + ((int64_t)rr * a.nseg + s0 + k) * a.G + g))
-                    : make_int4(0, 0, -1, 0);
-        };
-        // combines window statistics in ascending segment order: the admitted counts add up, the largest bound
-        // wins, the first block among equal bounds
-        auto resc_fold = [&](const int4 (&raw)[4], int& cnt, float& best, int& arg) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                cnt += raw[k].x;
-                const float mb = __int_as_float(raw[k].y);
-                if (raw[k].z >= 0 && mb > best) { best = mb; arg = raw[k].z; }
+    const int n_super = (a.n_chunks + a.super - 1) / a.super;
+    if (!one_chunk) {
+        for (int sc = warp; sc < n_super; sc += NWARPS) {
+            int su = 0, sz = 0;
+            for (int ch = sc * a.super; ch < min(a.n_chunks, (sc + 1) * a.super); ++ch) {
+                lane_flags(ch);
+                load_chunk(ch, false);
+                su += lane_u; sz += lane_z;
             }
-        };
-        auto count_consume = [&](int e, int c) {
-            if (e < n_cnt) {
-                const int rr = a.div_nseg.div(e);
-                if (counts_in_smem) cnt8[e + 2 * rr] = (uint8_t)c;       // entry rr (nseg + 2) + segment
-                if (c) atomicAdd(&rowcnt[rr], c);
-            }
-        };
-        int4 raw[4];
-        int Wr;
-        resc_load(tid, 0, raw, Wr);
-        int cv[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int e = tid + k * NTHREADS;
-            cv[k] = (e < n_cnt) ? __ldg(a.seg_count + e) : 0;
+            su = __reduce_add_sync(0xffffffffu, su);
+            sz = __reduce_add_sync(0xffffffffu, sz);
+            if (lane == 0) super_s[sc] = make_int2(su, sz);
         }
+        __syncthreads();
+    }
+    int U = 0, Z = 0;
+    if (lays_out) {
+        if (one_chunk) {
+            load_chunk(0, warp == PRODUCER_WARP);
+            scan_chunk();
+            U = tot_u; Z = tot_z;
+        } else {
+            for (int sc = lane; sc < n_super; sc += 32) { U += super_s[sc].x; Z += super_s[sc].y; }
+            U = __reduce_add_sync(0xffffffffu, U);
+            Z = __reduce_add_sync(0xffffffffu, Z);
+        }
+    }
+    // More cost units per CTA than a row's padding (fewer CTAs take part in a tiny problem): then no CTA's range lies
+    // inside a padding; the CTAs that meet a row are exactly those between two ends that follow from the row's cost
+    // interval in closed form (the merge kernel finds its candidates that way).
+    const uint32_t grid = gridDim.x;
+    const int pc = (uint32_t)U + (uint32_t)(PIECE_COST * Z) >= (PIECE_COST + 1) * grid ? PIECE_COST : PIECE_COST_SMALL;
+    const uint32_t C = (uint32_t)U + (uint32_t)pc * (uint32_t)Z;
+    const uint32_t P = min(grid, max(1u, C / (PIECE_COST_SMALL + 1)));
+    if (warp == 0) {
+        // ---- for the merge kernel and the caller, shared out over the CTAs (all of them find the same layout): the
+        // streaming CTAs that hold units of each row, and the number of blocks fetched per row.  CTA c has the cost
+        // interval [floor(c C / P), floor((c + 1) C / P)), row rr the interval [cs, ce) whose first pc units are
+        // padding, and c holds units of the row exactly when its interval starts before ce and ends after the padding.
+        int2* const span = reinterpret_cast<int2*>(smem + L::SPAN_OFF);
+        const int r_end = (int)(((int64_t)(blockIdx.x + 1) * a.rows) / grid);
+        for (int r_lo = (int)(((int64_t)blockIdx.x * a.rows) / grid); r_lo < r_end; r_lo += SPAN_ROWS) {
+            const int r_hi = min(r_end, r_lo + SPAN_ROWS);
+            if (lane == 0) span[r_hi - r_lo] = make_int2(U, Z);            // for the last row of all
+            __syncwarp();
+            auto store_rows = [&](int ch, int bu, int bz) {
+                int u = bu + pre_u, z = bz + pre_z;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) count_consume(tid + k * NTHREADS, cv[k]);
-        for (int e0 = tid + 8 * NTHREADS; e0 < n_cnt; e0 += NTHREADS) count_consume(e0, __ldg(a.seg_count + e0));
-        // Top-1 rescue of head g of row rr (Algorithm 3, rescue phase): if none of the first
-        // Wr = min(rescue_window, NB) blocks was admitted for the head, the first block with the largest bound among
-        // them is.  The G heads of a row sit in consecutive lanes of one warp: a head whose block an earlier head of
-        // the row rescued too shares that head's fetch unit.
-        for (int p0 = 0; p0 < n_rh; p0 += NTHREADS) {
-            const int p = p0 + tid;
-            if (p0 > 0) resc_load(p, 0, raw, Wr);
-            int cnt = 0, arg = -1;
-            float best = -INFINITY;
-            resc_fold(raw, cnt, best, arg);
-            for (int s0 = 4; s0 * SEG < Wr; s0 += 4) {      // windows of more than four segments
-                resc_load(p, s0, raw, Wr);
-                resc_fold(raw, cnt, best, arg);
-            }
-            const int rj = (p < n_rh && Wr > 0 && cnt == 0) ? (arg < 0 ? 0 : arg) : -1;
-            int rr, g;
-            a.div_g.divmod(p, rr, g);
-            bool dup = false;
-            for (int o = 1; o < a.G; ++o) {
-                const int jo = __shfl_up_sync(0xffffffffu, rj, o);
-                dup = dup || (o <= g && jo == rj);
-            }
-            const unsigned uniq = __ballot_sync(0xffffffffu, rj >= 0 && !dup);
-            if (p < n_rh) {
-                resc_j[rr * 8 + g] = rj;
-                if (g == 0) {
-                    const int n_resc = __popc((uniq >> (lane & 31)) & ((1u << a.G) - 1u));
-                    const int tailf = (s_len[rr] & (a.b - 1)) ? 1 : 0;
-                    rowinfo[rr] = (uint8_t)(n_resc | (tailf << 7));
-                    if (counts_in_smem) {
-                        cnt8[rr * (a.nseg + 2) + a.nseg] = (uint8_t)n_resc;
-                        cnt8[rr * (a.nseg + 2) + a.nseg + 1] = (uint8_t)tailf;
+                for (int m = 0; m < LGRAN; ++m) {
+                    const int q = ch * CHUNK + lane * a.lane_gran + m;
+                    if (m < a.lane_gran && q < a.n_gran) {
+                        int r, pos;
+                        a.div_gpr.divmod(q, r, pos);
+                        if (pos == 0 && r >= r_lo && r <= r_hi) span[r - r_lo] = make_int2(u, z);
+                        u += us[m]; z += (int)((headm >> m) & 1);
                     }
                 }
-            }
-        }
-    }
-    if (tl2 && tid == 0) tl2[0] = (unsigned long long)clock64() - clk0;
-    __syncthreads();
-    // Publishing for the merge kernel and the caller is shared out over the CTAs (all of them hold the same layout):
-    // CTA c takes the rows c, c + gridDim.x, ...  Here the rescued heads' admission bits and the number of blocks
-    // fetched per row; the rows' spans of CTAs follow once the split is known.
-    if (warp >= 1) {
-        for (int rr = blockIdx.x + (tid - 32) * gridDim.x; rr < a.rows; rr += (NTHREADS - 32) * gridDim.x) {
-            int extra = 0;
-            for (int g = 0; g < a.G; ++g) {
-                const int j = resc_j[rr * 8 + g];
-                if (j < 0) continue;
-                uint8_t* mp = a.sel_mask + (int64_t)rr * a.nb_cap + j;
-                const unsigned w = *mp;
-                bool dup = false;
-                for (int g2 = 0; g2 < g; ++g2) dup = dup || (resc_j[rr * 8 + g2] == j);
-                if (w == 0 && !dup) ++extra;      // a block no head had admitted: one more block fetched
-                *mp = (uint8_t)(w | (1u << g));
-            }
-            if (a.stats) a.stats[rr] = rowcnt[rr] + extra;
-        }
-    }
-    // Equal shares of COST, not of units: a row that starts inside a CTA's range costs that CTA a flush of its
-    // partials and a query reload, worth about PIECE_COST tiles.  Row rr spans the cost interval
-    // [rowbase[rr] + PIECE_COST * nzp[rr], +PIECE_COST (if it has units) + its units).  The first warp scans the
-    // rows, two of its lanes find the CTA's two range ends; everybody else picks them up after the barrier.
-    if (warp == 0) {
-        int carry_u = 0, carry_z = 0;
-        int my_units = 0, my_base = 0, my_nzp = 0;          // of row `lane` (used when there are at most 32 rows)
-        for (int r0 = 0; r0 < a.rows; r0 += 32) {
-            const int rr = r0 + lane;
-            int units = 0;
-            if (rr < a.rows) {
-                const int info = rowinfo[rr];
-                units = rowcnt[rr] + (info & 0x7f) + (info >> 7);      // surviving blocks, rescued blocks, tail
-            }
-            const int nzf = units > 0 ? 1 : 0;
-            int iu = units, iz = nzf;
-#pragma unroll
-            for (int sft = 1; sft < 32; sft <<= 1) {
-                const int ou = __shfl_up_sync(0xffffffffu, iu, sft);
-                const int oz = __shfl_up_sync(0xffffffffu, iz, sft);
-                if (lane >= sft) { iu += ou; iz += oz; }
-            }
-            my_units = units; my_base = carry_u + iu - units; my_nzp = carry_z + iz - nzf;
-            if (rr < a.rows) { rowbase[rr] = my_base; nzp[rr] = (uint16_t)my_nzp; }
-            carry_u += __shfl_sync(0xffffffffu, iu, 31);
-            carry_z += __shfl_sync(0xffffffffu, iz, 31);
-        }
-        if (lane == 0) { rowbase[a.rows] = carry_u; s_lay[0] = carry_z; }
-        __syncwarp();
-        const int nz_rows = carry_z, U = carry_u;
-        // More cost units per CTA than a row's padding (fewer CTAs take part in a tiny problem): then no CTA's
-        // range lies inside a padding; the CTAs that meet a row are exactly those between two ends that follow
-        // from the row's cost interval in closed form (the merge kernel finds its candidates that way).
-        const uint32_t C = (uint32_t)U + (uint32_t)PIECE_COST * (uint32_t)nz_rows;
-        const uint32_t P = min((uint32_t)gridDim.x, max(1u, C / (uint32_t)(PIECE_COST + 1)));
-        const uint32_t cq = C / P, cr = C - cq * P;
-        // cost position x -> unit: the last row rr in [0, rows] whose cost interval starts at or before x holds it
-        // (rows start in ascending order of cost).  Up to 32 rows: every lane compares its own row, a ballot counts;
-        // more rows: a binary search over the prefix arrays.
-        auto cost_to_unit = [&](uint32_t c) {
-            if (c >= P) return U;
-            const uint32_t x = c * cq + (c * cr) / P;        // floor(c C / P) without a 64-bit division: c cr < 2^16
-            int lo, lo_units, lo_base, lo_nzp;
-            if (a.rows <= 32) {
-                const bool le = lane < a.rows && (uint32_t)my_base + (uint32_t)PIECE_COST * (uint32_t)my_nzp <= x;
-                lo = __popc(__ballot_sync(0xffffffffu, le)) - 1;        // x >= 0 = the first row's start: lo >= 0
-                if (C <= x) return U;                                   // (cannot happen for c < P; the sentinel row)
-                lo_units = __shfl_sync(0xffffffffu, my_units, lo);
-                lo_base = __shfl_sync(0xffffffffu, my_base, lo);
-                lo_nzp = __shfl_sync(0xffffffffu, my_nzp, lo);
+            };
+            if (one_chunk) {
+                store_rows(0, 0, 0);
             } else {
-                int l2 = 0, h2 = a.rows;
-                while (l2 < h2) {
-                    const int mid = (l2 + h2 + 1) >> 1;
-                    const uint32_t nzb = (mid < a.rows) ? nzp[mid] : (uint32_t)nz_rows;
-                    if ((uint32_t)rowbase[mid] + (uint32_t)PIECE_COST * nzb <= x) l2 = mid; else h2 = mid - 1;
+                const int ch0 = (r_lo * a.gpr) / CHUNK, ch1 = min(a.n_chunks - 1, (r_hi * a.gpr) / CHUNK);
+                int bu = 0, bz = 0, ch = 0;
+                for (; ch + a.super <= ch0; ch += a.super) { bu += super_s[ch / a.super].x; bz += super_s[ch / a.super].y; }
+                for (; ch <= ch1; ++ch) {
+                    lane_flags(ch);
+                    load_chunk(ch, false);
+                    scan_chunk();
+                    if (ch >= ch0) store_rows(ch, bu, bz);
+                    bu += tot_u; bz += tot_z;
                 }
-                if (l2 >= a.rows) return U;
-                lo = l2; lo_base = rowbase[lo]; lo_units = rowbase[lo + 1] - lo_base; lo_nzp = nzp[lo];
             }
-            int off = (int)(x - ((uint32_t)lo_base + (uint32_t)PIECE_COST * (uint32_t)lo_nzp)) - (lo_units > 0 ? PIECE_COST : 0);
-            off = off < 0 ? 0 : (off > lo_units ? lo_units : off);
-            return lo_base + off;
-        };
-        const int unit0 = cost_to_unit(blockIdx.x), unit1 = cost_to_unit(blockIdx.x + 1);
-        // row holding the CTA's first unit: the last row that starts at or before it
-        int r_first;
-        if (a.rows <= 32) {
-            r_first = max(0, __popc(__ballot_sync(0xffffffffu, lane < a.rows && my_base <= unit0)) - 1);
-        } else {
-            int l2 = 0, h2 = a.rows - 1;
-            while (l2 < h2) {
-                const int mid = (l2 + h2 + 1) >> 1;
-                if (rowbase[mid] <= unit0) l2 = mid; else h2 = mid - 1;
+            __syncwarp();
+            for (int k = lane; k < r_hi - r_lo; k += 32) {
+                const int rr = r_lo + k, units = span[k + 1].x - span[k].x;
+                int c_lo = 0, n_span = 0;
+                if (units > 0) {
+                    const int64_t cs = (int64_t)span[k].x + (int64_t)pc * span[k].y, ce = cs + pc + units;
+                    const int c_hi = (int)((ce * P - 1) / C);
+                    c_lo = (int)(((cs + pc + 1) * P + C - 1) / C) - 1;
+                    n_span = c_hi - c_lo + 1;
+                }
+                a.row_span[rr] = make_int2(c_lo, n_span);
+                if (a.stats) a.stats[rr] = units - ((rowinfo[rr] >> 1) & 1);
             }
-            r_first = l2;
-        }
-        if (lane == 0) { s_lay[1] = unit0; s_lay[2] = unit1; s_lay[3] = (int)P; s_lay[4] = r_first; }
-        if (tl2 && tid == 0) tl2[3] = (unsigned long long)clock64() - clk0;
-    }
-    __syncthreads();
-    if (tl2 && tid == 0) tl2[4] = (unsigned long long)clock64() - clk0;
-    const int U = rowbase[a.rows];
-    const int u0 = s_lay[1], u1 = s_lay[2];
-    const int row0 = s_lay[4];
-    if (warp == 1) {
-        // For the merge kernel: the streaming CTAs that hold units of each row.  CTA c has the cost interval
-        // [floor(c C / P), floor((c + 1) C / P)), row rr the interval [cs, ce) whose first PIECE_COST units are
-        // padding, and c holds units of the row exactly when its interval starts before ce and ends after the
-        // padding.
-        const int64_t C = (int64_t)U + (int64_t)PIECE_COST * s_lay[0];
-        const int64_t P = s_lay[3];
-        for (int rr = blockIdx.x + lane * gridDim.x; rr < a.rows; rr += 32 * gridDim.x) {
-            const int units = rowbase[rr + 1] - rowbase[rr];
-            int c_lo = 0, n_span = 0;
-            if (units > 0) {
-                const int64_t cs = (int64_t)rowbase[rr] + (int64_t)PIECE_COST * nzp[rr], ce = cs + PIECE_COST + units;
-                const int c_hi = (int)((ce * P - 1) / C);
-                c_lo = (int)(((cs + PIECE_COST + 1) * P + C - 1) / C) - 1;
-                n_span = c_hi - c_lo + 1;
-            }
-            a.row_span[rr] = make_int2(c_lo, n_span);
+            __syncwarp();
         }
     }
     if (tl && tid == 0) tl[1] = globaltimer_ns();
-    if (u0 >= u1) return;
 
     if (warp == PRODUCER_WARP) {
         // ------------------------------------------------------------ producer
-        // The CTA's units [u0, u1) are located through a shared-memory window of the unit prefix (PW entries from
-        // entry e_base on): each lane finds the entry of one unit by binary search in the window and fetches that
-        // unit's list word, so a batch of up to 32 units costs one round trip to L2, and the next batch is fetched
-        // while the current one is being issued.
-        const int EPR = a.nseg + 2;        // per row: its segments, then the rescue entry, then the tail entry
-        const int E = a.entries;
-        int e_base = row0 * EPR;
-        int base_units = rowbase[row0];    // units before entry e_base
+        // the CTA's share of the cost, [x0, x1), and the units it stands for
+        uint32_t x0 = C, x1 = C;
+        if (blockIdx.x < P) {
+            if (P == grid) {
+                const uint32_t cq = (uint32_t)a.div_grid.div((int)C), cr = C - cq * grid;        // floor(c C / P): c cr < 2^16
+                x0 = blockIdx.x * cq + (uint32_t)a.div_grid.div((int)(blockIdx.x * cr));
+                x1 = (blockIdx.x + 1) * cq + (uint32_t)a.div_grid.div((int)((blockIdx.x + 1) * cr));
+            } else {
+                const uint32_t cq = C / P, cr = C - cq * P;
+                x0 = blockIdx.x * cq + blockIdx.x * cr / P;
+                x1 = (blockIdx.x + 1) * cq + (blockIdx.x + 1) * cr / P;
+            }
+        }
+        // cost position x < C -> unit, a granule at or before the one that holds it, units before that granule.  A position in a
+        // row's padding stands for the row's first unit.
+        auto locate = [&](uint32_t x, int& unit, int& gq, int& gu) {
+            int bu = 0, bz = 0, ch = 0;
+            if (!one_chunk) {
+                for (int sc = 0; sc + 1 < n_super; ++sc) {
+                    const int2 t = super_s[sc];
+                    if (x < (uint32_t)(bu + t.x) + (uint32_t)pc * (uint32_t)(bz + t.y)) break;
+                    bu += t.x; bz += t.y; ch += a.super;
+                }
+                while (true) {
+                    lane_flags(ch);
+                    load_chunk(ch, false);
+                    scan_chunk();
+                    if (ch + 1 >= a.n_chunks || x < (uint32_t)(bu + tot_u) + (uint32_t)pc * (uint32_t)(bz + tot_z)) break;
+                    bu += tot_u; bz += tot_z; ++ch;
+                }
+            }
+            int u = bu + pre_u, fu = 0, fq = 0, fgu = 0;
+            uint32_t c = (uint32_t)u + (uint32_t)pc * (uint32_t)(bz + pre_z);
+            const int src = 31 - __clz(__ballot_sync(0xffffffffu, c <= x));      // the last lane that starts at or before x
+            bool found = false;
+#pragma unroll
+            for (int m = 0; m < LGRAN; ++m) {
+                if (m < a.lane_gran) {
+                    const uint32_t pad = ((headm >> m) & 1) ? (uint32_t)pc : 0u;
+                    if (!found && x < c + pad + (uint32_t)us[m]) {
+                        found = true;
+                        fu = u + (x > c + pad ? (int)(x - c - pad) : 0);
+                        fq = ch * CHUNK + lane * a.lane_gran + m; fgu = u;
+                    }
+                    c += pad + (uint32_t)us[m]; u += us[m];
+                }
+            }
+            unit = __shfl_sync(0xffffffffu, fu, src);
+            gq = __shfl_sync(0xffffffffu, fq, src);
+            gu = __shfl_sync(0xffffffffu, fgu, src);
+        };
+        int u0 = U, u1 = U, wq = 0, wu = 0;          // the CTA's units; the window's first granule, units before it
+        if (x0 < C) {
+            int nq, nu;
+            if (x1 < C) locate(x1, u1, nq, nu);
+            locate(x0, u0, wq, wu);
+        }
+        if (tl2 && lane == 0) tl2[3] = (unsigned long long)clock64() - clk0;
+        // Window: granule wq + l in lane l, its counts in shared memory, the units before it in pre_w.
+        uint4* const win = reinterpret_cast<uint4*>(smem + L::WIN_OFF);
+        int pre_w = 0, wend = 0;
+        bool first_window = one_chunk;
+        auto load_window = [&]() {
+            __syncwarp();
+            const int q = wq + lane;
+            uint4 v = make_uint4(0, 0, 0, 0);
+            int tail = 0;
+            if (q < a.n_gran) {
+                v = first_window ? gran_s[q] : __ldcg(gran + q);
+                int r, pos;
+                a.div_gpr.divmod(q, r, pos);
+                tail = (pos == a.gpr - 1) ? (rowinfo[r] >> 1) & 1 : 0;
+            }
+            win[lane] = v;
+            const int n = granule_sum(v) + tail;
+            int incl = n;
+#pragma unroll
+            for (int sft = 1; sft < 32; sft <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, sft);
+                if (lane >= sft) incl += o;
+            }
+            pre_w = wu + incl - n;
+            wend = wu + __shfl_sync(0xffffffffu, incl, 31);
+            __syncwarp();
+        };
+        auto search = [&](int uu) {          // the last lane whose granule starts at or before unit uu
+            int lo = 0;
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1) {
+                const int v = __shfl_sync(0xffffffffu, pre_w, lo + step);
+                if (v <= uu) lo += step;
+            }
+            return lo;
+        };
+        // make the window hold the granule of unit ub; -> number of units of the batch starting at ub
+        auto batch_size = [&](int ub) {
+            while (true) {
+                const int want = min(32, u1 - ub);
+                if (wq + 32 >= a.n_gran || wend >= ub + want) return want;
+                if (wend <= ub) { wq += 32; wu = wend; load_window(); continue; }
+                const int k0 = search(ub);
+                if (k0 == 0) return min(want, wend - ub);
+                wu = __shfl_sync(0xffffffffu, pre_w, k0);
+                wq += k0;
+                load_window();
+            }
+        };
+        // per-lane description of unit ub + lane (row < 0: no such unit in this batch)
+        auto fetch = [&](int ub, int nb, int& row, int& ent, int& nrows, int& page) {
+            const int uu = ub + min(lane, nb - 1);
+            const int k = search(uu);
+            int off = uu - __shfl_sync(0xffffffffu, pre_w, k);
+            row = -1; ent = 0; nrows = 0; page = 0;
+            if (lane < nb) {
+                const uint4 v = win[k];
+                int r, pos;
+                a.div_gpr.divmod(wq + k, r, pos);
+                // the segment whose units include number `off` of the granule: first the word, then the byte
+                const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+                int sg = 0;
+                uint32_t w = 0;
+                bool in = false;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int n = (int)__dp4a(w4[j], 0x01010101u, 0u);
+                    if (!in) {
+                        if (off < n) { in = true; w = w4[j]; sg = 4 * j; } else off -= n;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const int n = (int)(w & 0xffu);
+                    if (in && off >= n) { off -= n; w >>= 8; ++sg; } else if (in) { w = 0x7fu; }
+                }
+                row = r;
+                int T = 0;
+                if (!in || a.ungate_last) {
+                    T = __ldg(a.seq_lens + a.div_hkv.div(r));
+                    T = T < 0 ? 0 : (T > a.t_cap ? a.t_cap : T);
+                }
+                if (!in) {
+                    const int NB = min(T / a.b, a.nb_cap);
+                    ent = NB | (0xff << 24);           // the tail: every head attends it
+                    nrows = T - NB * a.b;
+                    if (a.ungate_last) nrows |= 0x10000;      // its last token is the sequence's newest
+                } else {
+                    ent = __ldcg(a.seg_list + ((int64_t)r * a.nseg + pos * GRANULE + sg) * LSTRIDE + off);
+                    nrows = a.b;
+                    if (a.ungate_last && ((ent & 0xffffff) + 1) * a.b == T) nrows |= 0x10000;   // the block the newest token closes
+                }
+                // paged cache: the page that holds the unit's block of tokens (one more dependent load per batch,
+                // hidden like the list fetch behind the tiles already on their way)
+                if (a.block_table)
+                    page = __ldg(a.block_table + (int64_t)a.div_hkv.div(r) * a.table_stride + (ent & 0xffffff));
+            }
+        };
+        if (u0 >= u1) {
+            if (lane == 0) { s_row0 = -1; mbar_arrive(laybar); }
+            return;
+        }
+        load_window();
+        first_window = false;
+        int u = u0;
+        int nb = batch_size(u);
+        if (tl2 && lane == 0) tl2[6] = (unsigned long long)clock64() - clk0;
+        int c_row, c_ent, c_nrows, c_page;
+        fetch(u, nb, c_row, c_ent, c_nrows, c_page);
+        if (lane == 0) { s_row0 = c_row; mbar_arrive(laybar); }
+        if (tl2 && lane == 0) tl2[7] = (unsigned long long)clock64() - clk0 + (c_ent & 0);
         uint32_t fill = 0;
         int piece = -1, prev_row = -1;
         uint32_t piece_f0 = 0;
@@ -458,147 +500,6 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             }
         };
 
-        // units of entry e: survivors of a segment, rescue units of the row, or the row's tail
-        bool first_window = counts_in_smem;     // the counts of the layout phase are still in the stage memory
-        auto entry_count = [&](int e) {
-            if (first_window) return (e < E) ? (int)cnt8[e] : 0;
-            int r, sg;
-            a.div_epr.divmod(min(e, E - 1), r, sg);
-            const bool is_seg = sg < a.nseg;
-            int v = 0;
-            if (e < E && is_seg) v = __ldg(a.seg_count + r * a.nseg + sg);
-            const int info = rowinfo[r];
-            return (e >= E) ? 0 : (is_seg ? v : (sg == a.nseg ? (info & 0x7f) : (info >> 7)));
-        };
-        // pwin[k] = units before entry e_base + k, k = 0 .. PW: lane l counts the PW / 32 consecutive entries from
-        // e_base + l PW / 32 on, one warp scan over the lanes' totals gives each lane its first prefix
-        auto load_window = [&]() {
-            __syncwarp();
-            constexpr int EPL = PW / 32;
-            int cw[EPL];
-#pragma unroll
-            for (int m = 0; m < EPL; ++m) cw[m] = entry_count(e_base + EPL * lane + m);   // all loads in flight
-            int tot = 0;
-#pragma unroll
-            for (int m = 0; m < EPL; ++m) tot += cw[m];
-            int incl = tot;
-#pragma unroll
-            for (int sft = 1; sft < 32; sft <<= 1) {
-                const int o = __shfl_up_sync(0xffffffffu, incl, sft);
-                if (lane >= sft) incl += o;
-            }
-            int run = base_units + incl - tot;
-#pragma unroll
-            for (int m = 0; m < EPL; ++m) { pwin[EPL * lane + m] = run; run += cw[m]; }
-            if (lane == 31) pwin[PW] = run;
-            __syncwarp();
-        };
-        auto search = [&](int uu) {          // largest k in [0, PW) with pwin[k] <= uu
-            int lo = 0, hi = PW - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (pwin[mid] <= uu) lo = mid; else hi = mid - 1;
-            }
-            return lo;
-        };
-        // make the window hold the entry of unit ub; -> number of units of the batch starting at ub
-        auto batch_size = [&](int ub) {
-            while (true) {
-                const bool reaches_end = (e_base + PW >= E);
-                const int wend = pwin[PW];
-                const int want = min(32, u1 - ub);
-                if (reaches_end || wend >= ub + want) return want;
-                if (wend <= ub) { e_base += PW; base_units = wend; load_window(); continue; }
-                const int k0 = search(ub);
-                if (k0 == 0) return min(want, wend - ub);
-                base_units = pwin[k0];
-                e_base += k0;
-                load_window();
-            }
-        };
-        // per-lane description of unit ub + lane (row < 0: no such unit in this batch)
-        auto fetch = [&](int ub, int nb, int& row, int& ent, int& nrows, int& page) {
-            row = -1; ent = 0; nrows = 0; page = 0;
-            if (lane < nb) {
-                const int uu = ub + lane;
-                const int k = search(uu);
-                const int e = e_base + k;
-                int r, sg;
-                a.div_epr.divmod(e, r, sg);
-                row = r;
-                if (sg >= a.nseg) {
-                    int T = __ldg(a.seq_lens + a.div_hkv.div(r));
-                    T = T < 0 ? 0 : (T > a.t_cap ? a.t_cap : T);
-                    const int NB = min(T / a.b, a.nb_cap);
-                    if (sg == a.nseg) {
-                        // a rescued block, attended by the rescued head(s) only
-                        int uj[8], um[8];
-                        if (r - row0 < RESC_ROWS) {
-                            // same merge of equal blocks as rescue_units, from the table kept in shared memory
-                            int n = 0;
-#pragma unroll
-                            for (int g8 = 0; g8 < 8; ++g8) { uj[g8] = -1; um[g8] = 0; }
-#pragma unroll
-                            for (int g8 = 0; g8 < 8; ++g8) {
-                                const int j8 = resc_tab[(r - row0) * 8 + g8];
-                                if (j8 >= 0) {
-                                    bool merged = false;
-#pragma unroll
-                                    for (int q8 = 0; q8 < 8; ++q8)
-                                        if (q8 < n && uj[q8] == j8) { um[q8] |= 1 << g8; merged = true; }
-                                    if (!merged) {
-#pragma unroll
-                                        for (int q8 = 0; q8 < 8; ++q8)
-                                            if (q8 == n) { uj[q8] = j8; um[q8] = 1 << g8; }
-                                        ++n;
-                                    }
-                                }
-                            }
-                        } else {
-                            rescue_units(a.seg_resc, r, a.G, a.nseg, min(a.rescue_window, NB), uj, um);
-                        }
-                        const int idx = uu - pwin[k];
-                        int j = 0, m = 0;
-#pragma unroll
-                        for (int q8 = 0; q8 < 8; ++q8)
-                            if (q8 == idx) { j = uj[q8]; m = um[q8]; }
-                        ent = j | (m << 24);
-                        nrows = a.b;
-                    } else {
-                        ent = NB | (0xff << 24);           // the tail: every head attends it
-                        nrows = T - NB * a.b;
-                        if (a.ungate_last) nrows |= 0x10000;      // its last token is the sequence's newest
-                    }
-                } else {
-                    ent = __ldg(a.seg_list + ((int64_t)r * a.nseg + sg) * LSTRIDE + (uu - pwin[k]));
-                    nrows = a.b;
-                    if (a.ungate_last) {
-                        int T = __ldg(a.seq_lens + a.div_hkv.div(r));
-                        T = T < 0 ? 0 : (T > a.t_cap ? a.t_cap : T);
-                        if (((ent & 0xffffff) + 1) * a.b == T) nrows |= 0x10000;   // the block the newest token closes
-                    }
-                }
-                // paged cache: the page that holds the unit's block of tokens (one more dependent load per batch,
-                // hidden like the list fetch behind the tiles already on their way)
-                if (a.block_table)
-                    page = __ldg(a.block_table + (int64_t)a.div_hkv.div(r) * a.table_stride + (ent & 0xffffff));
-            }
-        };
-
-        // the rescue decisions of the first rows of this CTA's range outlive the layout scratch
-        for (int t = lane; t < 8 * RESC_ROWS; t += 32) {
-            const int rr = row0 + t / 8;
-            resc_tab[t] = (rr < a.rows && (t & 7) < a.G) ? resc_j[rr * 8 + (t & 7)] : -1;
-        }
-        if (tl2 && lane == 0) tl2[5] = (unsigned long long)clock64() - clk0;
-        load_window();
-        first_window = false;       // from the first copy on, the stage memory belongs to the tiles
-        int u = u0;
-        int nb = batch_size(u);
-        if (tl2 && lane == 0) tl2[6] = (unsigned long long)clock64() - clk0;
-        int c_row, c_ent, c_nrows, c_page;
-        fetch(u, nb, c_row, c_ent, c_nrows, c_page);
-        if (tl2 && lane == 0) tl2[7] = (unsigned long long)clock64() - clk0 + (c_ent & 0);
         while (u < u1 && ok) {
             // the next batch is fetched once the first tiles of this batch are on their way, so that its loads
             // are in flight while the rest of this batch is issued
@@ -733,7 +634,12 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         te = head ? __ldg(a.tau_eff + (int64_t)i * a.Hq + hk * a.G + g) : 0.f;
         q_row = r;
     };
-    load_q(row0);       // the row of the CTA's first unit: fetched while the producer sets up
+    if (!mbar_wait(laybar, 0)) {
+        if (lane == 0 && a.status) atomicOr(a.status, ETA_DEV_TIMEOUT);
+        return;
+    }
+    if (s_row0 < 0) return;
+    load_q(s_row0);       // the row of the CTA's first unit: fetched while its first tiles are on their way
 
     for (uint32_t fill = group;; fill += NGROUPS) {
         const int stage = fill % NSTAGE;
@@ -1181,9 +1087,9 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     sa.nseg = L.nseg; sa.rows = L.rows;
     sa.b_shift = (b == 32) ? 5 : (b == 64 ? 6 : 7);
     sa.div_hkv = FastDiv(desc->n_kv_heads);
-    sa.seg_count = reinterpret_cast<int32_t*>(ws + L.seg_count);
+    sa.seg_cnt = ws + L.seg_cnt;
+    sa.gpr = L.gpr;
     sa.seg_list = reinterpret_cast<int32_t*>(ws + L.seg_list);
-    sa.seg_resc = reinterpret_cast<RescueRec*>(ws + L.seg_resc);
     sa.tau_eff = reinterpret_cast<float*>(ws + L.tau_eff);
     sa.sel_mask = sel_mask;
     sa.timeline = debug_timeline();
@@ -1202,30 +1108,32 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
 
     DecodeArgs da;
     da.q = sa.q; da.seq_lens = seq_lens; da.tau_eff = sa.tau_eff; da.seg_list = sa.seg_list;
-    da.seg_count = sa.seg_count; da.seg_resc = sa.seg_resc; da.sel_mask = sel_mask; da.stats = stats;
+    da.seg_cnt = sa.seg_cnt; da.stats = stats;
     da.row_span = reinterpret_cast<int2*>(ws + L.row_span);
     da.part_ml = reinterpret_cast<float2*>(ws + L.part_ml);
     da.part_o = reinterpret_cast<float*>(ws + L.part_o);
     da.status = status_dev;
     da.beta = params->beta; da.scale = scale;
     da.Hq = desc->n_q_heads; da.Hkv = desc->n_kv_heads; da.G = G; da.b = b; da.t_cap = desc->t_cap;
-    da.nseg = L.nseg; da.entries = L.entries; da.rows = L.rows; da.nb_cap = desc->nb_cap;
-    da.rescue_window = params->rescue_window;
+    da.nseg = L.nseg; da.rows = L.rows; da.nb_cap = desc->nb_cap;
+    da.gpr = L.gpr; da.n_gran = L.rows * L.gpr;
+    da.n_chunks = (da.n_gran + CHUNK - 1) / CHUNK;
+    da.super = (da.n_chunks + MAX_SUPER - 1) / MAX_SUPER;
+    da.lane_gran = da.n_chunks == 1 ? (da.n_gran + 31) / 32 : LGRAN;
     da.ungate_last = (!dense && (params->flags & ETA_FLAG_UNGATE_LAST)) ? 1 : 0;
     da.block_table = pages ? pages->block_table : nullptr;
     da.table_stride = pages ? pages->table_stride : 0;
-    da.div_nseg = FastDiv(L.nseg); da.div_epr = FastDiv(L.nseg + 2); da.div_hkv = FastDiv(desc->n_kv_heads);
-    da.div_g = FastDiv(G);
+    da.div_gpr = FastDiv(L.gpr); da.div_hkv = FastDiv(desc->n_kv_heads); da.div_grid = FastDiv(n_ctas);
     da.timeline = debug_timeline();
     if (D == 128 && TS == 64) {
         rc = (G == 8) ? launch_decode_t<128, 64, 5, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s)
                       : launch_decode_t<128, 64, 6, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else if (D == 128 && TS == 32) {
-        rc = launch_decode_t<128, 32, 8, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<128, 32, 9, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else if (D == 64 && TS == 64) {
-        rc = launch_decode_t<64, 64, 8, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<64, 64, 12, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else {
-        rc = launch_decode_t<64, 32, 8, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<64, 32, 18, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     }
     if (rc != ETA_OK) return rc;
     profile_mark(4, s);

@@ -13,13 +13,12 @@
 // screen_kernel: a CTA of four warps takes a run of passes (four tiles each) of a
 // row.  Phase 1 (bounds; needs neither thresholds nor the newest summary)
 // never waits for a predecessor kernel; phase 2 (admission, pinning, mask,
-// ballot + popc compaction, rescue-window statistics) takes a warp per segment
-// of SEG records after the dependency wait.  Nothing returns to the host.
+// ballot + popc compaction) takes a warp per segment of SEG records after the
+// dependency wait.  Nothing returns to the host.
 //
-// Top-1 rescue needs the whole rescue window of a head, which may span several
-// segments: this kernel only leaves per-segment window statistics (admitted
-// count, largest bound and its index per head); the streaming kernel combines
-// them when it lays out its work.
+// Top-1 rescue needs the whole rescue window of a head: the first CTA of a row
+// takes at least the passes the window spans, and decides rescue before it
+// writes its lists.
 #include "eta_common.cuh"
 #include "eta_timeline.h"
 
@@ -168,17 +167,19 @@ __device__ __forceinline__ void sigma_f32(const SigmaPiece<PACKED>& s, float (&o
 // `lane`.  sigma^2 has at most 22 significant bits (sigma is fp16) and q^2 sixteen: each is the sum of two tf32 values, every
 // product of parts is exact and the accumulation is fp32, so the variance term is as good as one computed on the fp32
 // pipe, without a shuffle tree and with a quarter of the fp32 instructions.
+// -> whether some lane saw a NaN among the bounds of the first n records.  Two accumulators for the variance term: a tile
+// is a chain of dependent MMAs, and its latency is what a CTA of one or two tiles per warp takes (unrolling k gained nothing).
 template <int D, int G, bool PACKED>
-__device__ __forceinline__ void bound_tile(const QTab<D, G>& tab, uint32_t recs, float mn, float z, float scale,
+__device__ __forceinline__ bool bound_tile(const QTab<D, G>& tab, uint32_t recs, int n, float mn, float z, float scale,
                                            float* __restrict__ sb) {
     constexpr int J = D / 32, NT = TileOf<D>::NT, REC = PACKED ? 3 * D : 4 * D;
     const int lane = threadIdx.x & 31, n8 = lane >> 2, t = lane & 3;
     const uint32_t rp = recs + n8 * REC;
-    float dot[NT][4], var[NT][4];
+    float dot[NT][4], vhi[NT][4], vlo[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { dot[nt][c] = 0.f; var[nt][c] = 0.f; }
+        for (int c = 0; c < 4; ++c) { dot[nt][c] = 0.f; vhi[nt][c] = 0.f; vlo[nt][c] = 0.f; }
 #pragma unroll 1
     for (int j = 0; j < J; ++j) {
         const uint4 qa = tab.f16[j][lane];
@@ -200,36 +201,42 @@ __device__ __forceinline__ void bound_tile(const QTab<D, G>& tab, uint32_t recs,
             sigma_f32<PACKED>(sg[nt], s);
 #pragma unroll
             for (int k = 0; k < 8; ++k) { s[k] *= s[k]; hi[k] = tf32_hi(s[k]); s[k] -= hi[k]; }
-            mma_tf32_1688(var[nt], sa.x, la.x, sa.y, la.y, hi[0], hi[1]);
-            mma_tf32_1688(var[nt], sa.x, la.x, sa.y, la.y, s[0], s[1]);
-            mma_tf32_1688(var[nt], sa.z, la.z, sa.w, la.w, hi[2], hi[3]);
-            mma_tf32_1688(var[nt], sa.z, la.z, sa.w, la.w, s[2], s[3]);
-            mma_tf32_1688(var[nt], sb4.x, lb.x, sb4.y, lb.y, hi[4], hi[5]);
-            mma_tf32_1688(var[nt], sb4.x, lb.x, sb4.y, lb.y, s[4], s[5]);
-            mma_tf32_1688(var[nt], sb4.z, lb.z, sb4.w, lb.w, hi[6], hi[7]);
-            mma_tf32_1688(var[nt], sb4.z, lb.z, sb4.w, lb.w, s[6], s[7]);
+            mma_tf32_1688(vhi[nt], sa.x, la.x, sa.y, la.y, hi[0], hi[1]);
+            mma_tf32_1688(vlo[nt], sa.x, la.x, sa.y, la.y, s[0], s[1]);
+            mma_tf32_1688(vhi[nt], sa.z, la.z, sa.w, la.w, hi[2], hi[3]);
+            mma_tf32_1688(vlo[nt], sa.z, la.z, sa.w, la.w, s[2], s[3]);
+            mma_tf32_1688(vhi[nt], sb4.x, lb.x, sb4.y, lb.y, hi[4], hi[5]);
+            mma_tf32_1688(vlo[nt], sb4.x, lb.x, sb4.y, lb.y, s[4], s[5]);
+            mma_tf32_1688(vhi[nt], sb4.z, lb.z, sb4.w, lb.w, hi[6], hi[7]);
+            mma_tf32_1688(vlo[nt], sb4.z, lb.z, sb4.w, lb.w, s[6], s[7]);
         }
     }
     // lane (head n8, t) holds records 8 nt + 2 t and + 1
     const float qn = tab.norm[n8 < G ? n8 : 0], un = qtab_unscale(qn);
+    bool bad = false;
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            const float v2 = var[nt][c] + (G == 8 ? var[nt][c + 2] : __shfl_xor_sync(0xffffffffu, var[nt][c], 16));
+            const float v = vhi[nt][c] + vlo[nt][c];
+            const float v2 = v + (G == 8 ? vhi[nt][c + 2] + vlo[nt][c + 2] : __shfl_xor_sync(0xffffffffu, v, 16));
             const int rec = nt * 8 + 2 * t + c;
             const float m = __shfl_sync(0xffffffffu, mn, rec);
-            if (n8 < G) sb[rec * G + n8] = scale * min_keep_nan((dot[nt][c] + z * sqrtf(v2)) * un, qn * m);
+            const float bound = scale * min_keep_nan((dot[nt][c] + z * sqrtf(v2)) * un, qn * m);
+            if (n8 < G) sb[rec * G + n8] = bound;
+            bad = bad || (n8 < G && rec < n && bound != bound);
         }
     __syncwarp();
+    return __any_sync(0xffffffffu, bad);
 }
 
-// Bound of one record by one warp in plain fp32, for all heads of the group (queries in shared memory).
+// Bound of one record by one warp in plain fp32, for all heads of the group (queries in shared memory): 32 / (D / 8) heads
+// side by side.
 template <int D, int G, bool PACKED>
 __device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const unsigned char* __restrict__ src,
                                           float mn, float z, float scale, float* __restrict__ sb) {
-    constexpr int LPR = D / 8;
-    const int lane = threadIdx.x & 31, cl = lane % LPR;
+    constexpr int LPR = D / 8, HP = 32 / LPR;
+    const int lane = threadIdx.x & 31, cl = lane % LPR, sub = lane / LPR;
     const uint4 m4 = __ldcg(reinterpret_cast<const uint4*>(src + cl * 16));
     SigmaPiece<PACKED> sp;
     load_sigma<D, PACKED>(sp, src, cl);
@@ -244,8 +251,9 @@ __device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const un
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk) s2[kk] *= s2[kk];
 #pragma unroll 1
-    for (int gq = 0; gq < G; ++gq) {
-        const uint4 qv = qw[gq * LPR + cl];
+    for (int g0 = 0; g0 < G; g0 += HP) {
+        const int gq = g0 + sub;
+        const uint4 qv = qw[min(gq, G - 1) * LPR + cl];
         const uint32_t qq[4] = {qv.x, qv.y, qv.z, qv.w};
         float dot = 0.f, var = 0.f, n2 = 0.f;
 #pragma unroll
@@ -261,74 +269,78 @@ __device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const un
             dot += __shfl_xor_sync(0xffffffffu, dot, sh);
             var += __shfl_xor_sync(0xffffffffu, var, sh);
         }
-        if (lane == 0) sb[gq] = scale * min_keep_nan(dot + z * sqrtf(var), sqrtf(n2) * mn);
+        if (cl == 0 && gq < G) sb[gq] = scale * min_keep_nan(dot + z * sqrtf(var), sqrtf(n2) * mn);
     }
     __syncwarp();
 }
 
-// A warp's stream of tiles: one bulk copy in flight, into the warp's own shared memory.
+// A warp's stream of tiles: one or two bulk copies in flight, into the warp's own shared memory.
 template <int D, int G, bool PACKED>
 struct TileStream {
     static constexpr int REC = PACKED ? 3 * D : 4 * D;
     using T = TileOf<D>;
-    unsigned char* buf;
-    uint64_t* bar;
+    unsigned char* bufs;               // nbuf tiles
+    uint64_t* bars;                    // two barriers
     const unsigned char* rec_row;      // records and largest norms of the row
     const float* mn_row;
-    int NB, n, j0;                     // full blocks of the row; records and first record of the tile in flight
-    uint32_t parity;
+    int NB, nbuf;                      // full blocks of the row
+    int in, out;                       // tiles issued and consumed so far
+    uint32_t parity;                   // bit k: of buffer k
     bool alive;                        // false once a wait ran out: nothing is issued any more
-    float mn;
 
-    // starts the copy of the tile at record j (the previous one has been read by the whole warp)
+    // starts the copy of the tile at record j (the buffer's previous tile has been read by the whole warp)
     __device__ __forceinline__ void issue(int j) {
-        const int lane = threadIdx.x & 31;
-        j0 = j;
-        n = max(0, min(T::RECS, NB - j));
-        if (n > 0 && alive) {
-            if (lane == 0) {
-                mbar_arrive_expect_tx(bar, n * REC);
-                tma_load_1d(buf, rec_row + (int64_t)j * REC, n * REC, bar);
-            }
-            mn = lane < n ? __ldcg(mn_row + j + lane) : 0.f;
+        const int k = nbuf == 2 ? (in & 1) : 0, n = min(T::RECS, NB - j);
+        ++in;
+        if (n > 0 && alive && (threadIdx.x & 31) == 0) {
+            mbar_arrive_expect_tx(bars + k, n * REC);
+            tma_load_1d(bufs + k * T::BYTES, rec_row + (int64_t)j * REC, n * REC, bars + k);
         }
     }
-    // Bounds of the tile in flight into sb[record][head]; false when the copy did not arrive.  A wait that runs out admits
-    // the tile's blocks (NaN bounds: the safe direction).  What the tensor-core path cannot do shows as a NaN bound too (an
-    // infinite sigma has no exact split, a query's norm may overflow) and is computed again in fp32.
-    __device__ __forceinline__ bool bounds(const QTab<D, G>& tab, float z, float scale, float* __restrict__ sb) {
-        const int lane = threadIdx.x & 31;
+    // Bounds of the oldest tile in flight, whose first record is j, into sb[record][head]; false when the copy did not arrive.
+    // A wait that runs out admits the tile's blocks (NaN bounds: the safe direction).  What the tensor-core path cannot do
+    // shows as a NaN bound too (an infinite sigma has no exact split, a query's norm may overflow) and is computed again in
+    // fp32.
+    __device__ __forceinline__ bool bounds(const QTab<D, G>& tab, int j, float z, float scale, float* __restrict__ sb) {
+        const int lane = threadIdx.x & 31, k = nbuf == 2 ? (out & 1) : 0, n = min(T::RECS, NB - j);
+        ++out;
         if (n <= 0) return true;
+        const float mn = lane < n ? __ldcg(mn_row + j + lane) : 0.f;
         const bool was_alive = alive;
-        if (alive) alive = __all_sync(0xffffffffu, mbar_wait(bar, parity));
+        if (alive) alive = __all_sync(0xffffffffu, mbar_wait(bars + k, (parity >> k) & 1));
         if (!alive) {
-            for (int k = lane; k < n * G; k += 32) sb[k] = __int_as_float(0x7fc00000);
-            if (was_alive) mbar_wait(bar, parity);      // bounded: time for the copy to land before the CTA's memory is released
+            for (int e = lane; e < n * G; e += 32) sb[e] = __int_as_float(0x7fc00000);
+            if (was_alive) {                           // bounded: time for the copies to land before the CTA's memory is released
+                mbar_wait(bars + k, (parity >> k) & 1);
+                if (in > out) mbar_wait(bars + (k ^ 1), (parity >> (k ^ 1)) & 1);
+            }
             __syncwarp();
             return false;
         }
-        parity ^= 1;
-        bound_tile<D, G, PACKED>(tab, smem_u32(buf), mn, z, scale, sb);
-        bool bad = false;
+        parity ^= 1u << k;
+        if (bound_tile<D, G, PACKED>(tab, smem_u32(bufs + k * T::BYTES), n, mn, z, scale, sb)) {
+            bool bad = false;
 #pragma unroll
-        for (int g = 0; g < G; ++g) bad = bad || (lane < n && sb[lane * G + g] != sb[lane * G + g]);
-        unsigned todo = __ballot_sync(0xffffffffu, bad);
-        while (todo) {
-            const int rec = __ffs(todo) - 1;
-            todo &= todo - 1;
-            bound_one<D, G, PACKED>(tab.raw, rec_row + (int64_t)(j0 + rec) * REC, __shfl_sync(0xffffffffu, mn, rec), z, scale, sb + rec * G);
+            for (int g = 0; g < G; ++g) bad = bad || (lane < n && sb[lane * G + g] != sb[lane * G + g]);
+            unsigned todo = __ballot_sync(0xffffffffu, bad);
+            while (todo) {
+                const int rec = __ffs(todo) - 1;
+                todo &= todo - 1;
+                bound_one<D, G, PACKED>(tab.raw, rec_row + (int64_t)(j + rec) * REC, __shfl_sync(0xffffffffu, mn, rec), z, scale, sb + rec * G);
+            }
         }
         return true;
     }
 };
 
-// Shared memory of both kernels: the warps' tiles, the query table, a barrier per warp, bounds of `recs` records
+// Shared memory of both kernels: the query table, two barriers per warp, the warps' tiles, bounds of `recs` records
 template <int D, int G>
 struct ScreenSmem {
-    static constexpr int TAB_OFF = SCR_WARPS * TileOf<D>::BYTES;
-    static constexpr int BAR_OFF = TAB_OFF + (int)((sizeof(QTab<D, G>) + 15) / 16 * 16);
-    static constexpr int BOUND_OFF = BAR_OFF + 8 * SCR_WARPS;
-    static size_t bytes(int recs) { return BOUND_OFF + sizeof(float) * (size_t)recs * G + 112; }   // + slack for a 128-byte base
+    static constexpr int BAR_OFF = (int)((sizeof(QTab<D, G>) + 15) / 16 * 16);
+    static constexpr int TILE_OFF = (BAR_OFF + 16 * SCR_WARPS + 127) / 128 * 128;
+    static size_t bytes(int recs, int nbuf) {            // + slack for a 128-byte base
+        return TILE_OFF + (size_t)nbuf * SCR_WARPS * TileOf<D>::BYTES + sizeof(float) * (size_t)recs * G + 112;
+    }
 };
 // CTAs per SM the screening grid is sized for.  A fifth would fit an empty SM, but the append and predictor CTAs are still
 // on some of them: with 5 the last CTAs only start when the first have had their thresholds (65536 blocks at d = 128: 71.7
@@ -348,9 +360,10 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
     constexpr int REC_BYTES = PACKED ? 3 * D : 4 * D;
     extern __shared__ unsigned char scr_raw[];
     unsigned char* sm = scr_raw + ((128u - (smem_u32(scr_raw) & 127u)) & 127u);
-    QTab<D, G>& tab = *reinterpret_cast<QTab<D, G>*>(sm + L::TAB_OFF);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
-    float* const sbound_all = reinterpret_cast<float*>(sm + L::BOUND_OFF);      // [record of the group][G]
+    QTab<D, G>& tab = *reinterpret_cast<QTab<D, G>*>(sm);
+    float* const sbound_all = reinterpret_cast<float*>(sm + L::TILE_OFF + a.nbuf * SCR_WARPS * TL::BYTES);      // [record of the group][G]
+    __shared__ uint32_t s_bkey[G];                      // per head: largest bound of the rescue window (as an ordered integer)
+    __shared__ int s_best[G];                           // and the first block that attains it
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool dense = (a.flags & ETA_FLAG_DENSE) != 0;
@@ -362,22 +375,53 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
     a.div_chunks.divmod(blockIdx.x, r, c);
     a.div_hkv.divmod(r, i, hk);
     const int Traw = __ldg(a.seq_lens + i);
-    const int p_first = a.div_chunks.div(c * a.passes), p_last = a.div_chunks.div((c + 1) * a.passes);
+    const int rest = a.passes - a.head;
+    const int p_first = c == 0 ? 0 : a.head + a.div_rest.div((c - 1) * rest);
+    const int p_last = c == 0 ? a.head : a.head + a.div_rest.div(c * rest);
     const int T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
     const int NB = min(T >> a.b_shift, a.nb_cap);
     const unsigned char* const rec_row = reinterpret_cast<const unsigned char*>(a.musig) + (int64_t)r * a.nb_cap * REC_BYTES;
     const float* const mn_row = a.mnorm + (int64_t)r * a.nb_cap;
 
-    if (lane == 0) { mbar_init(&bars[warp], 1); fence_barrier_init(); }
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF) + 2 * warp;
+    if (lane == 0) { mbar_init(&bars[0], 1); mbar_init(&bars[1], 1); fence_barrier_init(); }
+    if (tid < G) { s_bkey[tid] = 0u; s_best[tid] = 0; }
     __syncwarp();
-    TileStream<D, G, PACKED> ts{sm + warp * TL::BYTES, &bars[warp], rec_row, mn_row, dense ? 0 : NB, 0, 0, 0u, true, 0.f};
-    ts.issue(p_first * TL::PASS + warp * TL::RECS);
+    TileStream<D, G, PACKED> ts{sm + L::TILE_OFF + warp * a.nbuf * TL::BYTES, bars, rec_row, mn_row, dense ? 0 : NB, a.nbuf, 0, 0, 0u, true};
+    for (int p = p_first; p < min(p_last, p_first + a.nbuf); ++p) ts.issue(p * TL::PASS + warp * TL::RECS);
     if (!dense) build_qtab<D, G>(tab, a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
 
     // an ungated newest token must be attended: when it closes a full block, that block counts as pinned
     const int lwb = ((a.flags & ETA_FLAG_UNGATE_LAST) && T > 0 && (T & (a.b - 1)) == 0 && a.lwb < 1) ? 1 : a.lwb;
+    const int Wr = min(a.rescue_window, NB);
     float te_l = -INFINITY;               // lane gq < G: effective threshold of head gq
+    // Top-1 rescue (Algorithm 3): a head that admits none of the first Wr blocks attends the first one with the largest
+    // bound among them.  It admits none exactly when that bound is below its threshold and no block of the window is pinned
+    // (a NaN bound admits), so the row's first CTA looks for the largest bounds ahead of the wait for the thresholds, a warp
+    // per head, with bounds compared as order-preserving integers.
+    const bool rescues = c == 0 && !dense && Wr > 0 && !(lwb > 0 && NB - lwb < Wr);
+    const bool stale = !dense && NB > 0 && (T & (a.b - 1)) == 0;      // the newest block's record may not have been final yet
+    auto window_max = [&](int p0, int p1) {
+        const int n_win = min(Wr, p1 * TL::PASS) - p0 * TL::PASS;
+        for (int gq = warp; gq < G; gq += SCR_WARPS) {
+            uint32_t key = 0;                     // 0: no record of the window in this lane
+            int arg = 0x7fffffff;
+            for (int rec = lane; rec < n_win; rec += 32) {                  // ascending: a lane keeps the first of equal bounds
+                const float bd = sbound_all[rec * G + gq] + 0.f;            // (-0 counts as +0)
+                const uint32_t u = __float_as_uint(bd);
+                uint32_t k2 = (u & 0x80000000u) ? ~u : (u | 0x80000000u);    // ascending with the value
+                if (bd != bd) k2 = 0xffffffffu;
+                if (k2 > key) { key = k2; arg = rec; }
+            }
+            const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+            const int amin = __reduce_min_sync(0xffffffffu, key == kmax ? arg : 0x7fffffff);
+            if (lane == 0 && kmax > s_bkey[gq]) { s_bkey[gq] = kmax; s_best[gq] = p0 * TL::PASS + amin; }
+        }
+        __syncthreads();
+    };
     bool waited = false;
+    unsigned missing = 0;                 // heads to rescue, known with the first group of passes where that holds the window
+    const bool whole_window = Wr <= min(p_last, a.group) * TL::PASS;
     for (int p0 = p_first; p0 < p_last; p0 += a.group) {
         const int p1 = min(p_last, p0 + a.group);
         // -------------------------------------------------------- phase 1: bounds of a group of passes
@@ -387,42 +431,46 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
         // row that may be stale (the newest block of a just-completed length) gets a bound there like any other, and
         // the warp that handles its segment in phase 2, after the wait, computes that bound again.
         for (int p = p0; p < p1; ++p) {
-            const bool ok = ts.bounds(tab, a.z, a.scale, sbound_all + ((p - p0) * TL::PASS + warp * TL::RECS) * G);
+            const bool ok = ts.bounds(tab, p * TL::PASS + warp * TL::RECS, a.z, a.scale, sbound_all + ((p - p0) * TL::PASS + warp * TL::RECS) * G);
             if (!ok && lane == 0 && a.status) atomicOr(a.status, ETA_DEV_TIMEOUT);
-            if (p + 1 < p_last) ts.issue((p + 1) * TL::PASS + warp * TL::RECS);
+            if (p + a.nbuf < p_last) ts.issue((p + a.nbuf) * TL::PASS + warp * TL::RECS);
             if (tl && tid == 0 && p == p_first) tl[1] = globaltimer_ns();
         }
         __syncthreads();
+        const bool stale_in = stale && NB - 1 >= p0 * TL::PASS && NB - 1 < p1 * TL::PASS;
+        if (rescues && p0 * TL::PASS < Wr && !stale_in) window_max(p0, p1);
         if (tl && tid == 0 && !waited) tl[2] = globaltimer_ns();
         // -------------------------------------------------------- phase 2: a warp per segment
+        const int seg_0 = p0 * (TL::PASS / SEG), s_end = min(a.nseg, p1 * (TL::PASS / SEG));
         if (!waited) {
             pdl_wait();                   // the thresholds (and the newest summaries) are final now
-            waited = true;
             if (tl && tid == 0) tl[3] = globaltimer_ns();
             if (!dense && lane < G) {
                 const int h = hk * G + lane;
                 te_l = (a.tau ? __ldcg(a.tau + (int64_t)i * a.Hq + h) : __ldg(a.head_const + h)) - a.a;
             }
-            if (c == 0 && warp == 0) {
-                if (lane < G) a.tau_eff[(int64_t)i * a.Hq + hk * G + lane] = te_l;
-                if (lane == 0 && a.status) {
-                    if (Traw > a.t_cap) atomicOr(a.status, ETA_DEV_LEN_CLAMPED);
-                    if (Traw <= 0) atomicOr(a.status, ETA_DEV_EMPTY_ROW);
-                }
+        }
+        // the newest block's bound again, while the thresholds are on their way
+        if (stale_in) {
+            if (((NB - 1) / SEG - seg_0) % SCR_WARPS == warp)
+                bound_one<D, G, PACKED>(tab.raw, rec_row + (int64_t)(NB - 1) * REC_BYTES, __ldcg(mn_row + NB - 1), a.z, a.scale,
+                                        sbound_all + (NB - 1 - p0 * TL::PASS) * G);
+        }
+        if (!waited && c == 0 && warp == 0) {
+            if (lane < G) a.tau_eff[(int64_t)i * a.Hq + hk * G + lane] = te_l;
+            if (lane == 0 && a.status) {
+                if (Traw > a.t_cap) atomicOr(a.status, ETA_DEV_LEN_CLAMPED);
+                if (Traw <= 0) atomicOr(a.status, ETA_DEV_EMPTY_ROW);
             }
         }
+        waited = true;
         float te_g[G];
 #pragma unroll
         for (int gq = 0; gq < G; ++gq) te_g[gq] = __shfl_sync(0xffffffffu, te_l, gq);
-        const int s_end = min(a.nseg, p1 * (TL::PASS / SEG));
-        for (int seg = p0 * (TL::PASS / SEG) + warp; seg < s_end; seg += SCR_WARPS) {
-            const int j0 = seg * SEG, n_rec = max(0, min(SEG, NB - j0));
-            float (*sbound)[G] = reinterpret_cast<float (*)[G]>(sbound_all + (j0 - p0 * TL::PASS) * G);
-            if (!dense && n_rec > 0 && (T & (a.b - 1)) == 0 && j0 + n_rec == NB)
-                bound_one<D, G, PACKED>(tab.raw, rec_row + (int64_t)(NB - 1) * REC_BYTES, __ldcg(mn_row + NB - 1), a.z, a.scale,
-                                        sbound[NB - 1 - j0]);
-            // admission bits of records lane and lane + 32
-            unsigned m[SEG / 32];
+        // admission bits of records lane and lane + 32 of a segment
+        auto admit = [&](int seg, unsigned (&m)[SEG / 32]) {
+            const int j0 = seg * SEG, n_rec = min(SEG, NB - j0);
+            const float (*sbound)[G] = reinterpret_cast<const float (*)[G]>(sbound_all + (j0 - p0 * TL::PASS) * G);
 #pragma unroll
             for (int half = 0; half < SEG / 32; ++half) {
                 const int rec = half * 32 + lane;
@@ -433,64 +481,70 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
                     for (int gq = 0; gq < G; ++gq)
                         if (dense || pinned || !(sbound[rec][gq] < te_g[gq])) m[half] |= 1u << gq;
                 }
-                // user-visible bits; entries of this segment that are not full blocks read as "not attended"
-                if (j0 + rec < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j0 + rec] = (uint8_t)m[half];
             }
-            // segment-local compaction of the union (ballot + popc prefix), ascending block order
-            {
-                int carry = 0;
-                int32_t* list = a.seg_list + ((int64_t)r * a.nseg + seg) * LSTRIDE;
+        };
+        if (rescues && p0 * TL::PASS < Wr) {
+            if (stale_in) { __syncthreads(); window_max(p0, p1); }
+            if (p1 * TL::PASS >= Wr) {
 #pragma unroll
-                for (int half = 0; half < SEG / 32; ++half) {
-                    const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
-                    if (m[half]) list[carry + __popc(nz & ((1u << lane) - 1u))] = (j0 + half * 32 + lane) | (int)(m[half] << 24);
-                    carry += __popc(nz);
-                }
-                if (lane == 0) a.seg_count[r * a.nseg + seg] = carry;
-            }
-            // rescue statistics of the part of the rescue window inside this segment, per query head: how many of its
-            // blocks the head admits, the largest bound and the first block that attains it.  Bounds are compared as
-            // order-preserving integers (one hardware max-reduction and one ballot per head instead of a shuffle tree).
-            const int Wr = min(a.rescue_window, NB);
-            if (j0 < Wr && n_rec > 0) {
-                const int nwin = min(n_rec, Wr - j0);
-#pragma unroll 1
                 for (int gq = 0; gq < G; ++gq) {
-                    uint32_t key = 0;                 // 0: no record of the window in this lane
-                    int arg = 0x7fffffff;
-#pragma unroll
-                    for (int half = 0; half < SEG / 32; ++half) {
-                        const int rec = half * 32 + lane;
-                        if (rec < nwin) {
-                            const float bd = (dense ? 0.f : sbound[rec][gq]) + 0.f;        // (-0 counts as +0)
-                            const uint32_t u = __float_as_uint(bd);
-                            uint32_t k2 = (u & 0x80000000u) ? ~u : (u | 0x80000000u);           // ascending with the value
-                            if (bd != bd) k2 = 1;                                               // a NaN bound never wins
-                            if (k2 > key) { key = k2; arg = rec; }                              // ties keep the lower index
-                        }
-                    }
-                    const int cnt = __popc(__ballot_sync(0xffffffffu, (m[0] >> gq) & 1 && lane < nwin)) +
-                                    __popc(__ballot_sync(0xffffffffu, (m[1] >> gq) & 1 && lane + 32 < nwin));
-                    const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
-                    // among the lanes that hold the maximum the lowest record index wins: a lane's own candidate is its
-                    // lower record unless the higher one is strictly larger, so compare the candidates' indices
-                    const int amin = __reduce_min_sync(0xffffffffu, key == kmax ? arg : 0x7fffffff);
-                    if (lane == 0) {
-                        RescueRec rr;
-                        float best = -INFINITY;
-                        if (kmax > 1) {
-                            const uint32_t u = (kmax & 0x80000000u) ? (kmax & 0x7fffffffu) : ~kmax;
-                            best = __uint_as_float(u);
-                        }
-                        rr.cnt = cnt; rr.maxb = best;
-                        rr.arg = (kmax <= 1 || amin == 0x7fffffff) ? -1 : (j0 + amin);
-                        rr.pad = 0;
-                        a.seg_resc[((int64_t)r * a.nseg + seg) * G + gq] = rr;
-                    }
+                    const uint32_t k = s_bkey[gq];
+                    const float top = __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);      // (0xffffffff: a NaN)
+                    if (top < te_g[gq]) missing |= 1u << gq;
                 }
             }
         }
+        for (int seg = seg_0 + warp; seg < s_end; seg += SCR_WARPS) {
+            const int j0 = seg * SEG;
+            unsigned m[SEG / 32];
+            admit(seg, m);
+            if (whole_window) {
+                for (unsigned left = missing; left; left &= left - 1) {
+                    const int gq = __ffs(left) - 1, rec = s_best[gq] - j0;
+                    if (rec == lane) m[0] |= 1u << gq;
+                    if (rec == lane + 32) m[1] |= 1u << gq;
+                }
+            }
+            // user-visible bits; entries of this segment that are not full blocks read as "not attended"
+#pragma unroll
+            for (int half = 0; half < SEG / 32; ++half)
+                if (j0 + half * 32 + lane < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j0 + half * 32 + lane] = (uint8_t)m[half];
+            // segment-local compaction of the union (ballot + popc prefix), ascending block order
+            int carry = 0;
+            int32_t* list = a.seg_list + ((int64_t)r * a.nseg + seg) * LSTRIDE;
+#pragma unroll
+            for (int half = 0; half < SEG / 32; ++half) {
+                const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
+                if (m[half]) list[carry + __popc(nz & ((1u << lane) - 1u))] = (j0 + half * 32 + lane) | (int)(m[half] << 24);
+                carry += __popc(nz);
+            }
+            if (lane == 0) a.seg_cnt[((int64_t)r * a.gpr) * GRANULE + seg] = (uint8_t)carry;
+        }
         if (p1 < p_last) __syncthreads();          // the bounds of this group have been read: the next may overwrite them
+    }
+    // counts past the row's last segment
+    if (p_last == a.passes)
+        for (int seg = a.nseg + tid; seg < a.gpr * GRANULE; seg += 32 * SCR_WARPS) a.seg_cnt[((int64_t)r * a.gpr) * GRANULE + seg] = 0;
+    // A rescue window of several groups of passes: the rescued blocks join lists that are already written.  A block another
+    // head fetches anyway gets the head's bit, any other goes to the end of its segment's list.
+    if (missing && !whole_window) {
+        __syncthreads();                  // lists, counts and mask of this CTA are written
+        for (unsigned left = warp == 0 ? missing : 0u; left; left &= left - 1) {
+            const int gq = __ffs(left) - 1, j = s_best[gq], seg = j / SEG;
+            volatile uint8_t* mp = a.sel_mask + (int64_t)r * a.nb_cap + j;
+            volatile uint8_t* np = a.seg_cnt + ((int64_t)r * a.gpr) * GRANULE + seg;
+            volatile int32_t* list = a.seg_list + ((int64_t)r * a.nseg + seg) * LSTRIDE;
+            const unsigned w = *mp, n = *np;
+            __syncwarp();                 // every lane has read them
+            if (w == 0) {
+                if (lane == 0) { list[n] = j | (1 << (24 + gq)); *np = (uint8_t)(n + 1); }
+            } else {
+                for (unsigned k = lane; k < n; k += 32)
+                    if ((list[k] & 0xffffff) == j) list[k] = list[k] | (1 << (24 + gq));
+            }
+            if (lane == 0) *mp = (uint8_t)(w | (1u << gq));
+            __syncwarp();
+        }
     }
     if (tl && tid == 0) tl[5] = globaltimer_ns();
     pdl_trigger();
@@ -509,26 +563,26 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     using TL = TileOf<D>;
     extern __shared__ unsigned char scr_raw[];
     unsigned char* sm = scr_raw + ((128u - (smem_u32(scr_raw) & 127u)) & 127u);
-    QTab<D, G>& tab = *reinterpret_cast<QTab<D, G>*>(sm + L::TAB_OFF);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
+    QTab<D, G>& tab = *reinterpret_cast<QTab<D, G>*>(sm);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float* const sb = reinterpret_cast<float*>(sm + L::BOUND_OFF) + warp * TL::RECS * G;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF) + 2 * warp;
+    float* const sb = reinterpret_cast<float*>(sm + L::TILE_OFF + SCR_WARPS * TL::BYTES) + warp * TL::RECS * G;
     const int r = blockIdx.x / chunks, i = r / Hkv, hk = r % Hkv;
     int T = __ldg(seq_lens + i);
     T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
     const int NB = min(T / b, nb_cap);
     const int first = (blockIdx.x % chunks) * per * TL::PASS;
     if (first >= NB) return;
-    if (lane == 0) { mbar_init(&bars[warp], 1); fence_barrier_init(); }
+    if (lane == 0) { mbar_init(&bars[0], 1); mbar_init(&bars[1], 1); fence_barrier_init(); }
     __syncwarp();
-    TileStream<D, G, PACKED> ts{sm + warp * TL::BYTES, &bars[warp], musig + (int64_t)r * nb_cap * TileStream<D, G, PACKED>::REC,
-                                mnorm + (int64_t)r * nb_cap, NB, 0, 0, 0u, true, 0.f};
+    TileStream<D, G, PACKED> ts{sm + L::TILE_OFF + warp * TL::BYTES, bars, musig + (int64_t)r * nb_cap * TileStream<D, G, PACKED>::REC,
+                                mnorm + (int64_t)r * nb_cap, NB, 1, 0, 0, 0u, true};
     const int last = min(NB, first + per * TL::PASS);
     ts.issue(first + warp * TL::RECS);
     build_qtab<D, G>(tab, q + ((int64_t)i * Hq + hk * G) * D, tid);
     for (int j0 = first + warp * TL::RECS; j0 < last; j0 += TL::PASS) {
-        const int n = ts.n;
-        ts.bounds(tab, z, scale, sb);
+        const int n = min(TL::RECS, NB - j0);
+        ts.bounds(tab, j0, z, scale, sb);
         if (j0 + TL::PASS < last) ts.issue(j0 + TL::PASS);
         if (lane < n) {
 #pragma unroll
@@ -592,11 +646,20 @@ static int launch_screen_t(const ScreenArgs& a, int rows, int n_sm, cudaStream_t
     constexpr int SPP = TileOf<D>::PASS / SEG;
     ScreenArgs b2 = a;
     b2.passes = (a.nseg + SPP - 1) / SPP;
-    const int chunks = ctas_per_row(rows, b2.passes, SCR_SLOTS * n_sm), per = (b2.passes + chunks - 1) / chunks;
+    int chunks = ctas_per_row(rows, b2.passes, SCR_SLOTS * n_sm);
+    const int window = a.rescue_window < a.nb_cap ? a.rescue_window : a.nb_cap;
+    const int even = (b2.passes + chunks - 1) / chunks, need = (window + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
+    b2.head = even > need ? even : need;
+    if (b2.head >= b2.passes) { b2.head = b2.passes; chunks = 1; }
+    if (chunks - 1 > b2.passes - b2.head) chunks = 1 + b2.passes - b2.head;
     b2.div_chunks = FastDiv(chunks);
-    b2.group = per < SCR_GROUP ? per : SCR_GROUP;        // passes whose bounds wait in shared memory for the thresholds
+    b2.div_rest = FastDiv(chunks > 1 ? chunks - 1 : 1);
+    b2.group = b2.head < SCR_GROUP ? b2.head : SCR_GROUP;      // passes whose bounds wait in shared memory for the thresholds
+    // A second buffer per warp (three CTAs per SM) where all CTAs are still resident at once: a CTA of two passes, such as
+    // the one that holds the rescue window, then has both on their way from the start.
+    b2.nbuf = (b2.head > 1 && rows * chunks <= 3 * n_sm) ? 2 : 1;
     return launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)(rows * chunks)), dim3(32 * SCR_WARPS),
-                      ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS), s, b2);
+                      ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, b2);
 }
 
 int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_sm, cudaStream_t s) {
@@ -618,7 +681,7 @@ static int launch_score_t(const eta_cache_desc* desc, const __nv_bfloat16* q, co
     if (e != cudaSuccess) { set_cuda_error(e, "device query"); return ETA_ERR_CUDA; }
     const int rows = desc->batch * desc->n_kv_heads, passes = (desc->nb_cap + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
     const int want = ctas_per_row(rows, passes, 5 * n_sm), per = (passes + want - 1) / want, chunks = (passes + per - 1) / per;
-    const size_t smem = ScreenSmem<D, G>::bytes(TileOf<D>::PASS);
+    const size_t smem = ScreenSmem<D, G>::bytes(TileOf<D>::PASS, 1);
     const int rc = configure_kernel(reinterpret_cast<const void*>(score_dual_kernel<D, G, PACKED>), smem);
     if (rc != ETA_OK) return rc;
     score_dual_kernel<D, G, PACKED><<<(unsigned)(rows * chunks), 32 * SCR_WARPS, smem, s>>>(

@@ -11,11 +11,11 @@
 namespace eta {
 constexpr int TL_DECODE = 0;
 constexpr int TL_DECODE2 = 256;       // second row of stamps of the streaming kernel (set-up phases)
-constexpr int TL_SCREEN = 512, TL_SCREEN_N = 296;
-constexpr int TL_MERGE = 808, TL_MERGE_N = 128;
-constexpr int TL_PREDICT = 936, TL_PREDICT_N = 32;
-constexpr int TL_APPEND = 968, TL_APPEND_N = 48;
-constexpr int TL_SLOTS = 1024;
+constexpr int TL_SCREEN = 512, TL_SCREEN_N = 740;
+constexpr int TL_MERGE = 1252, TL_MERGE_N = 128;
+constexpr int TL_PREDICT = 1380, TL_PREDICT_N = 32;
+constexpr int TL_APPEND = 1412, TL_APPEND_N = 48;
+constexpr int TL_SLOTS = 1460;
 }  // namespace eta
 
 #ifdef ETA_TIMELINE
