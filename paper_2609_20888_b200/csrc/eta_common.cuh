@@ -86,10 +86,14 @@ struct ScreenArgs {
     int lwb, rescue_window;
     uint32_t flags;
     int Hq, Hkv, b, b_shift, t_cap, nb_cap, nseg, rows;
-    int passes, head;                     // passes of a row; of them the row's first CTA takes `head`, the others share the rest
+    // split of the rows' passes over the CTAs (see launch_screen)
+    int batch, passes, need;              // sequences; passes of a row at full capacity, those the rescue window spans
+    int by_length;                        // the kernel splits by the sequences' lengths; else by capacity, with the next two
+    int tp, ctas_row, ctas_all;           // passes per CTA, CTAs per row, all CTAs
+    int slots;                            // CTAs the GPU holds at once
     int group;                            // passes whose bounds are kept before their admission is decided
     int nbuf;                             // tiles a warp keeps in flight
-    FastDiv div_chunks, div_rest, div_hkv;          // CTAs per row, those but the first
+    FastDiv div_ctas, div_slots, div_hkv;
     uint8_t* seg_cnt;
     int gpr;
     int32_t* seg_list;

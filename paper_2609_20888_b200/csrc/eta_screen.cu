@@ -348,6 +348,15 @@ struct ScreenSmem {
 constexpr int SCR_SLOTS = 4;
 constexpr int SCR_GROUP = 4;         // most passes whose bounds wait in shared memory for the thresholds
 
+// Zeroes n bytes with the threads of a CTA: 16 at a time between the ends
+__device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
+    if (n <= 0) return;
+    const int lead = min(n, (int)(-reinterpret_cast<uintptr_t>(p) & 15)), body = (n - lead) >> 4, rest = (n - lead) & 15;
+    if (tid < lead) p[tid] = 0;
+    for (int k = tid; k < body; k += 32 * SCR_WARPS) reinterpret_cast<uint4*>(p + lead)[k] = make_uint4(0, 0, 0, 0);
+    if (tid < rest) p[lead + 16 * body + tid] = 0;
+}
+
 // What bounds it: HBM for the records (33.8 MB for 65536 blocks at d = 128, 5.2 us at the copy rate) once enough of them are
 // requested; small CTAs, because the hardware then fills whatever the predecessor kernels leave of each SM, and all of them
 // resident at once, because none can finish before the thresholds are there.  A step of 65536 blocks at d = 128, G = 4 takes
@@ -370,14 +379,56 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
     unsigned long long* const tl = ETA_TL((a.timeline && blockIdx.x < TL_SCREEN_N) ? a.timeline + (size_t)(TL_SCREEN + blockIdx.x) * 8 : nullptr);
     if (tl && tid == 0) tl[0] = globaltimer_ns();
 
-    // the CTA's passes of its row: an even share
-    int r, c, i, hk;
-    a.div_chunks.divmod(blockIdx.x, r, c);
-    a.div_hkv.divmod(r, i, hk);
-    const int Traw = __ldg(a.seq_lens + i);
-    const int rest = a.passes - a.head;
-    const int p_first = c == 0 ? 0 : a.head + a.div_rest.div((c - 1) * rest);
-    const int p_last = c == 0 ? a.head : a.head + a.div_rest.div(c * rest);
+    // The CTA's row and its passes [p_first, p_last) of it.  A row's first CTA takes `head` passes (its rescue window at
+    // least), each further one `tp`.
+    int i, hk, c, n_ctas = a.ctas_row, P = a.passes, tp = a.tp, Traw;    // P: passes of the row; n_ctas: CTAs of the row, c: this one
+    bool by_capacity = true;
+    if (a.by_length) {
+        // Rows of one launch may differ in length, and the slowest CTA sets the kernel's end: every warp looks at the lengths (a
+        // sequence per lane) and, unless all rows fill their capacity, works out the smallest tp with which all CTAs fit
+        // the slots, and which of them it is.
+        const bool seq = lane < a.batch;
+        const int Tl = seq ? __ldg(a.seq_lens + lane) : 0;
+        const int nb = min(max(min(Tl, a.t_cap), 0) >> a.b_shift, a.nb_cap);
+        const int Pl = seq ? max(1, (nb + TL::PASS - 1) / TL::PASS) : 0;
+        if (!__all_sync(0xffffffffu, !seq || Pl == a.passes)) {
+            by_capacity = false;
+            const int total = __reduce_add_sync(0xffffffffu, Pl) * a.Hkv;
+            tp = a.div_slots.div(total + a.slots - 1);
+            int k, incl;
+            while (true) {
+                // 1 + ceil((Pl - head) / tp), by a reciprocal: exact, the numbers are small
+                const int over = max(0, Pl - max(tp, a.need)) + tp - 1;
+                k = seq ? 1 + (int)(__fdividef((float)over + 0.5f, (float)tp)) : 0;
+                incl = k * a.Hkv;
+#pragma unroll
+                for (int sft = 1; sft < 32; sft <<= 1) {
+                    const int o = __shfl_up_sync(0xffffffffu, incl, sft);
+                    if (lane >= sft) incl += o;
+                }
+                if (tp >= a.passes || __shfl_sync(0xffffffffu, incl, 31) <= a.slots) break;
+                tp += max(1, tp >> 3);
+            }
+            const unsigned before = __ballot_sync(0xffffffffu, incl <= (int)blockIdx.x);
+            if (before == 0xffffffffu) return;                // more CTAs than these lengths need
+            i = __popc(before);
+            n_ctas = __shfl_sync(0xffffffffu, k, i);
+            P = __shfl_sync(0xffffffffu, Pl, i);
+            Traw = __shfl_sync(0xffffffffu, Tl, i);
+            const int rem = (int)blockIdx.x - (__shfl_sync(0xffffffffu, incl, i) - n_ctas * a.Hkv);
+            hk = (int)__fdividef((float)rem + 0.5f, (float)n_ctas);
+            c = rem - hk * n_ctas;
+        }
+    }
+    if (by_capacity) {
+        if ((int)blockIdx.x >= a.ctas_all) return;
+        int rr;
+        a.div_ctas.divmod(blockIdx.x, rr, c);
+        a.div_hkv.divmod(rr, i, hk);
+        Traw = __ldg(a.seq_lens + i);
+    }
+    const int r = i * a.Hkv + hk, head = max(tp, a.need);
+    const int p_first = c == 0 ? 0 : head + (c - 1) * tp, p_last = min(P, head + c * tp);
     const int T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
     const int NB = min(T >> a.b_shift, a.nb_cap);
     const unsigned char* const rec_row = reinterpret_cast<const unsigned char*>(a.musig) + (int64_t)r * a.nb_cap * REC_BYTES;
@@ -522,9 +573,12 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
         }
         if (p1 < p_last) __syncthreads();          // the bounds of this group have been read: the next may overwrite them
     }
-    // counts past the row's last segment
-    if (p_last == a.passes)
-        for (int seg = a.nseg + tid; seg < a.gpr * GRANULE; seg += 32 * SCR_WARPS) a.seg_cnt[((int64_t)r * a.gpr) * GRANULE + seg] = 0;
+    // what the row's passes do not reach: no survivors, nothing attended
+    if (c == n_ctas - 1) {
+        const int seg_n = min(a.nseg, P * (TL::PASS / SEG)), rec_n = min(a.nb_cap, P * TL::PASS);
+        zero_bytes(a.seg_cnt + (int64_t)r * a.gpr * GRANULE + seg_n, a.gpr * GRANULE - seg_n, tid);
+        zero_bytes(a.sel_mask + (int64_t)r * a.nb_cap + rec_n, a.nb_cap - rec_n, tid);
+    }
     // A rescue window of several groups of passes: the rescued blocks join lists that are already written.  A block another
     // head fetches anyway gets the head's bit, any other goes to the end of its segment's list.
     if (missing && !whole_window) {
@@ -635,30 +689,32 @@ __global__ void __launch_bounds__(128) score_dual_unaligned_kernel(
 
 // ------------------------------------------------------------------ launchers (host)
 
-// CTAs per row: an even share of the slots the GPU has, at most one pass each
-static int ctas_per_row(int rows, int passes, int slots) {
-    const int c = slots / rows;
-    return c < 1 ? 1 : (c < passes ? c : passes);
-}
-
 template <int D, int G, bool PACKED>
 static int launch_screen_t(const ScreenArgs& a, int rows, int n_sm, cudaStream_t s) {
     constexpr int SPP = TileOf<D>::PASS / SEG;
     ScreenArgs b2 = a;
     b2.passes = (a.nseg + SPP - 1) / SPP;
-    int chunks = ctas_per_row(rows, b2.passes, SCR_SLOTS * n_sm);
+    b2.batch = rows / a.Hkv;
+    b2.slots = SCR_SLOTS * n_sm;
     const int window = a.rescue_window < a.nb_cap ? a.rescue_window : a.nb_cap;
-    const int even = (b2.passes + chunks - 1) / chunks, need = (window + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
-    b2.head = even > need ? even : need;
-    if (b2.head >= b2.passes) { b2.head = b2.passes; chunks = 1; }
-    if (chunks - 1 > b2.passes - b2.head) chunks = 1 + b2.passes - b2.head;
-    b2.div_chunks = FastDiv(chunks);
-    b2.div_rest = FastDiv(chunks > 1 ? chunks - 1 : 1);
-    b2.group = b2.head < SCR_GROUP ? b2.head : SCR_GROUP;      // passes whose bounds wait in shared memory for the thresholds
+    b2.need = (window + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
+    // the split at full length: what rows of any length stay below, and what is used where there are too many to look at
+    const int64_t all = (int64_t)rows * b2.passes;
+    b2.tp = (int)((all + b2.slots - 1) / b2.slots);
+    const int head = b2.tp > b2.need ? b2.tp : b2.need;
+    b2.ctas_row = b2.passes <= head ? 1 : 1 + (b2.passes - head + b2.tp - 1) / b2.tp;
+    b2.div_ctas = FastDiv(b2.ctas_row);
+    b2.ctas_all = rows * b2.ctas_row;
+    // by length where a warp can look at all sequences and there are enough passes for the split to matter
+    b2.by_length = b2.batch > 1 && b2.batch <= 32 && all > b2.slots && rows <= b2.slots;
+    b2.div_slots = FastDiv(b2.slots);
+    const int grid = b2.by_length && b2.ctas_all < b2.slots ? b2.slots : b2.ctas_all;
+    b2.group = head < b2.passes ? head : b2.passes;      // passes whose bounds wait in shared memory for the thresholds
+    if (b2.group > SCR_GROUP) b2.group = SCR_GROUP;
     // A second buffer per warp (three CTAs per SM) where all CTAs are still resident at once: a CTA of two passes, such as
     // the one that holds the rescue window, then has both on their way from the start.
-    b2.nbuf = (b2.head > 1 && rows * chunks <= 3 * n_sm) ? 2 : 1;
-    return launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)(rows * chunks)), dim3(32 * SCR_WARPS),
+    b2.nbuf = (b2.group > 1 && all <= 3 * n_sm) ? 2 : 1;
+    return launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)grid), dim3(32 * SCR_WARPS),
                       ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, b2);
 }
 
@@ -680,7 +736,8 @@ static int launch_score_t(const eta_cache_desc* desc, const __nv_bfloat16* q, co
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) { set_cuda_error(e, "device query"); return ETA_ERR_CUDA; }
     const int rows = desc->batch * desc->n_kv_heads, passes = (desc->nb_cap + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
-    const int want = ctas_per_row(rows, passes, 5 * n_sm), per = (passes + want - 1) / want, chunks = (passes + per - 1) / per;
+    const int64_t all = (int64_t)rows * passes;
+    const int per = (int)((all + 5 * n_sm - 1) / (5 * n_sm)), chunks = (passes + per - 1) / per;      // about five CTAs per SM
     const size_t smem = ScreenSmem<D, G>::bytes(TileOf<D>::PASS, 1);
     const int rc = configure_kernel(reinterpret_cast<const void*>(score_dual_kernel<D, G, PACKED>), smem);
     if (rc != ETA_OK) return rc;
