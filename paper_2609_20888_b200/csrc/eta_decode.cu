@@ -103,7 +103,9 @@ struct DecodeSmem {
     static constexpr int ML_OFF = INFO_OFF + MAX_ROWS;          // float m[NGROUPS][4][8], l[NGROUPS][4][8]
     static_assert(16 * CHUNK >= 8 * MAX_SUPER, "sums of the super-chunks share the granules' place");
     static constexpr int MO_OFF = ML_OFF + 4 * 2 * NGROUPS * WARPS_PER_GROUP * 8;
-    static size_t bytes(int G) { return 1024 + MO_OFF + sizeof(float) * NGROUPS * WARPS_PER_GROUP * G * D; }
+    // heads whose accumulators a flush parks at a time: eight heads of 128 columns would cost the ring a stage
+    static constexpr int FLUSH_HEADS = 512 / D;
+    static size_t bytes(int G) { return 1024 + MO_OFF + sizeof(float) * NGROUPS * WARPS_PER_GROUP * (G < FLUSH_HEADS ? G : FLUSH_HEADS) * D; }
 };
 
 // The streaming kernel.  Warp roles: NGROUPS consumer groups of four warps, then one producer warp.  Group k
@@ -133,15 +135,10 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     unsigned long long* const tl = ETA_TL(a.timeline ? a.timeline + (size_t)(TL_DECODE + blockIdx.x) * 8 : nullptr);
     unsigned long long* const tl2 = ETA_TL(a.timeline ? a.timeline + (size_t)(TL_DECODE2 + blockIdx.x) * 8 : nullptr);
     if (tl && tid == 0) tl[0] = globaltimer_ns();
-    // When NSTAGE is not a multiple of NGROUPS a stage serves different groups in successive rounds, and a parity
-    // wait only tells the current phase of a barrier from the one before it: a group that runs ahead could ask for
-    // round k of a stage while round k - 1 (another group's) has not completed and be told "done".  In those
-    // configurations the producer publishes the number of fills it has started (each only after the stage's
-    // previous round was consumed) and a consumer looks at its barrier only once its fill is among them.
-    constexpr bool SHARED_STAGES = (NSTAGE % NGROUPS) != 0;
-    __shared__ int s_fill_started;
+    // A stage serves the same group in every round: a parity wait only tells the current phase of a barrier from the one
+    // before it, and a group that ran ahead on a stage of another group could be told "done" too early.
+    static_assert(NSTAGE % NGROUPS == 0, "stages must be a multiple of the consumer groups");
     if (tid == 0) {
-        s_fill_started = 0;
         for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], WARPS_PER_GROUP); }
         for (int k = 0; k < NGROUPS; ++k) mbar_init(&flushbar[k], 32 * WARPS_PER_GROUP);
         mbar_init(laybar, 1);
@@ -373,6 +370,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             locate(x0, u0, wq, wu);
         }
         if (tl2 && lane == 0) tl2[3] = (unsigned long long)clock64() - clk0;
+        const int tpu = a.b > TS ? a.b / TS : 1;          // tiles of a full unit
         // Window: granule wq + l in lane l, its counts in shared memory, the units before it in pre_w.
         uint4* const win = reinterpret_cast<uint4*>(smem + L::WIN_OFF);
         int pre_w = 0, wend = 0;
@@ -412,7 +410,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         // make the window hold the granule of unit ub; -> number of units of the batch starting at ub
         auto batch_size = [&](int ub) {
             while (true) {
-                const int want = min(32, u1 - ub);
+                const int want = min(32 / tpu, u1 - ub);
                 if (wq + 32 >= a.n_gran || wend >= ub + want) return want;
                 if (wend <= ub) { wq += 32; wu = wend; load_window(); continue; }
                 const int k0 = search(ub);
@@ -422,13 +420,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 load_window();
             }
         };
-        // per-lane description of unit ub + lane (row < 0: no such unit in this batch)
+        // per-lane description of unit ub + lane / tpu (row < 0: no such unit in this batch)
         auto fetch = [&](int ub, int nb, int& row, int& ent, int& nrows, int& page) {
-            const int uu = ub + min(lane, nb - 1);
+            const int uu = ub + min(lane / tpu, nb - 1);
             const int k = search(uu);
             int off = uu - __shfl_sync(0xffffffffu, pre_w, k);
             row = -1; ent = 0; nrows = 0; page = 0;
-            if (lane < nb) {
+            if (lane / tpu < nb) {
                 const uint4 v = win[k];
                 int r, pos;
                 a.div_gpr.divmod(wq + k, r, pos);
@@ -484,79 +482,104 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         fetch(u, nb, c_row, c_ent, c_nrows, c_page);
         if (lane == 0) { s_row0 = c_row; mbar_arrive(laybar); }
         if (tl2 && lane == 0) tl2[7] = (unsigned long long)clock64() - clk0 + (c_ent & 0);
+        // A lane per tile: lane TPU j + sub is part `sub` of the batch's unit j.  Lanes whose stage is free issue their copies
+        // together, so a tile costs the warp a fraction of a pass through this loop; with one tile per pass (its
+        // description broadcast by shuffles) the producer took 550 ns a tile, which held every tile of less than 32 KB (64
+        // columns or 32 tokens) below half of the copy rate.
+        const int usub = lane % tpu;
         uint32_t fill = 0;
         int piece = -1, prev_row = -1;
         uint32_t piece_f0 = 0;
         bool ok = true;
 
         // groups that receive no tile of a piece never write its partial: mark those slots "absent" for the merge
-        auto close_piece = [&]() {
+        auto close_piece = [&](uint32_t end) {
             if (prev_row < 0) return;
-            const uint32_t n = fill - piece_f0;
+            const uint32_t n = end - piece_f0;
             for (uint32_t k = n; k < (uint32_t)NGROUPS; ++k) {
                 const int grp = (int)((piece_f0 + k) % NGROUPS);
                 const int64_t slot = ((int64_t)blockIdx.x + prev_row) * NGROUPS + grp;
                 if (lane < a.G) a.part_ml[slot * a.G + lane] = make_float2(-INFINITY, 0.f);
             }
         };
-
         while (u < u1 && ok) {
-            // the next batch is fetched once the first tiles of this batch are on their way, so that its loads
-            // are in flight while the rest of this batch is issued
             const int un = u + nb;
-            int nbn = 0, n_row = -1, n_ent = 0, n_nrows = 0, n_page = 0;
-            const int k_prefetch = min(nb, NSTAGE) - 1;
-            for (int k = 0; k < nb && ok; ++k) {
-                const int r = __shfl_sync(0xffffffffu, c_row, k);
-                const int ent = __shfl_sync(0xffffffffu, c_ent, k);
-                const int nrows_raw = __shfl_sync(0xffffffffu, c_nrows, k);
-                const int page = __shfl_sync(0xffffffffu, c_page, k);
-                const int nrows = nrows_raw & 0xffff;
-                const bool holds_newest = (nrows_raw >> 16) != 0;
-                const int j = ent & 0xffffff;
-                const int hmask = (ent >> 24) & 0xff;
-                int i, hk;
-                a.div_hkv.divmod(r, i, hk);
-                if (r != prev_row) {                               // a new (CTA, row) piece starts here
-                    close_piece();
-                    ++piece; prev_row = r; piece_f0 = fill;
-                }
-                for (int sub = 0; sub * TS < nrows && ok; ++sub) {
-                    const int nvalid = min(TS, nrows - sub * TS);
-                    const int stage = fill % NSTAGE;
-                    const uint32_t round = fill / NSTAGE;
-                    if (lane == 0) {
-                        if (tl2 && fill == 0) tl2[1] = (unsigned long long)clock64() - clk0;
-                        if (!mbar_wait(&empty[stage], (round & 1) ^ 1)) {
-                            ok = false;
-                        } else {
-                            if (SHARED_STAGES) st_volatile(&s_fill_started, (int)fill + 1);
-                            // bits 8..15: row of the tile whose token stays ungated, 0xff: none
-                            const int urow = (holds_newest && (sub + 1) * TS >= nrows) ? nvalid - 1 : 0xff;
-                            desc[stage] = make_int4(r, piece << 1, hmask | (urow << 8), nvalid);
-                            unsigned char* st = smem + stage * L::STAGE_BYTES;
-                            mbar_arrive_expect_tx(&full[stage], L::STAGE_BYTES);
-                            // one copy per tile: 64 columns x TS tokens x HALVES half tiles, each half swizzled.  The
-                            // outermost coordinate is the sequence (contiguous cache: token offset in the sequence) or
-                            // the page (paged cache: token offset in the page)
-                            const int y = a.block_table ? sub * TS : j * a.b + sub * TS;
-                            const int w4 = a.block_table ? page : i;
-                            tma_load_5d(st, &tmK, 0, y, 0, hk, w4, &full[stage]);
-                            tma_load_5d(st + HALVES * L::TILE_BYTES, &tmV, 0, y, 0, hk, w4, &full[stage]);
-                        }
-                    }
-                    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-                    ++fill;
-                }
-                if (k == k_prefetch && un < u1) {
-                    nbn = batch_size(un);
-                    fetch(un, nbn, n_row, n_ent, n_nrows, n_page);
-                }
+            const int nrows = c_nrows & 0xffff;
+            const bool valid = c_row >= 0 && usub * TS < nrows;
+            const unsigned vmask = __ballot_sync(0xffffffffu, valid);
+            const uint32_t my_fill = fill + (uint32_t)__popc(vmask & ((1u << lane) - 1u));
+            // pieces: a new one starts where the row changes
+            const int left = __shfl_up_sync(0xffffffffu, c_row, 1);
+            unsigned starts = __ballot_sync(0xffffffffu, c_row >= 0 && c_row != (lane == 0 ? prev_row : left));
+            const int my_piece = piece + __popc(starts & (0xffffffffu >> (31 - lane)));
+            piece += __popc(starts);
+            for (; starts; starts &= starts - 1) {
+                const int sl = __ffs(starts) - 1;
+                const uint32_t f = __shfl_sync(0xffffffffu, my_fill, sl);
+                close_piece(f);
+                prev_row = __shfl_sync(0xffffffffu, c_row, sl);
+                piece_f0 = f;
             }
+            const int stage = (int)(my_fill % NSTAGE);
+            const uint32_t parity = ((my_fill / NSTAGE) & 1) ^ 1;
+            bool done = !valid;
+            int my_i, my_hk;
+            a.div_hkv.divmod(max(c_row, 0), my_i, my_hk);
+            // The outermost coordinate is the sequence (contiguous cache: token offset in the sequence) or the page (paged
+            // cache: token offset in the page)
+            const int my_y = a.block_table ? usub * TS : (c_ent & 0xffffff) * a.b + usub * TS;
+            const int my_w = a.block_table ? c_page : my_i;
+            unsigned char* const my_smem = smem + stage * L::STAGE_BYTES;
+            const int nvalid = min(TS, nrows - usub * TS);
+            // bits 8..15: row of the tile whose token stays ungated, 0xff: none
+            const int urow = ((c_nrows >> 16) != 0 && (usub + 1) * TS >= nrows) ? nvalid - 1 : 0xff;
+            const int4 my_desc = make_int4(c_row, my_piece << 1, ((c_ent >> 24) & 0xff) | (urow << 8), nvalid);
+            // One pass: lanes whose stage is free issue.  A lane looks at its stage's barrier only when the tile that used the
+            // stage before it is on its way (parity tells two rounds apart, not three), that is, within NSTAGE tiles of
+            // the first one that is not.
+            auto issue_pass = [&]() {
+                const unsigned open = __ballot_sync(0xffffffffu, !done);
+                const int first = __ffs(open) - 1;
+                const uint32_t f_first = __shfl_sync(0xffffffffu, my_fill, first < 0 ? 0 : first);
+                const bool ready = !done && my_fill < f_first + NSTAGE && mbar_test(&empty[stage], parity);
+                if (ready) {
+                    done = true;
+                    desc[stage] = my_desc;
+                    mbar_arrive_expect_tx(&full[stage], L::STAGE_BYTES);
+                }
+                // one copy per tensor: 64 columns x TS tokens x HALVES half tiles, each half swizzled.  Tile after tile, so that
+                // the first is complete as early as can be.
+                for (unsigned rm = __ballot_sync(0xffffffffu, ready); rm; rm &= rm - 1) {
+                    if (lane == __ffs(rm) - 1) {
+                        tma_load_5d(my_smem, &tmK, 0, my_y, 0, my_hk, my_w, &full[stage]);
+                        tma_load_5d(my_smem + HALVES * L::TILE_BYTES, &tmV, 0, my_y, 0, my_hk, my_w, &full[stage]);
+                    }
+                }
+                return __any_sync(0xffffffffu, !done) != 0;
+            };
+            if (tl2 && lane == 0 && fill == 0) tl2[1] = (unsigned long long)clock64() - clk0;
+            bool more = issue_pass();
+            // the next batch is fetched once what fits of this one is on its way
+            int nbn = 0, n_row = -1, n_ent = 0, n_nrows = 0, n_page = 0;
+            if (un < u1) {
+                nbn = batch_size(un);
+                fetch(un, nbn, n_row, n_ent, n_nrows, n_page);
+            }
+            for (uint32_t it = 0; more; ++it) {
+                more = issue_pass();
+                if (it >= WAIT_LIMIT) { ok = false; break; }
+                if (more && it >= 2) __nanosleep(20);
+            }
+            if (!ok) {                    // give up: time for this batch's copies to land (those before it are waited for below)
+                if (valid && done) mbar_wait(&full[stage], parity ^ 1);
+                __syncwarp();
+                break;
+            }
+            fill += (uint32_t)__popc(vmask);
             u = un;
             nb = nbn; c_row = n_row; c_ent = n_ent; c_nrows = n_nrows; c_page = n_page;
         }
-        close_piece();
+        close_piece(fill);
         pdl_trigger();       // everything is issued: the merge kernel may start to set up
         // one end marker per group (no data): the next NGROUPS fills reach every group exactly once
         for (int k = 0; k < NGROUPS && ok; ++k) {
@@ -565,7 +588,6 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 if (!mbar_wait(&empty[stage], ((fill / NSTAGE) & 1) ^ 1)) {
                     ok = false;
                 } else {
-                    if (SHARED_STAGES) st_volatile(&s_fill_started, (int)fill + 1);
                     desc[stage] = make_int4(0, (int)UF_END, 0, 0);
                     mbar_arrive(&full[stage]);
                 }
@@ -588,7 +610,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const int group = warp / WARPS_PER_GROUP, wq = warp % WARPS_PER_GROUP;
     float* sm_m = reinterpret_cast<float*>(smem + L::ML_OFF) + group * 2 * WARPS_PER_GROUP * 8;
     float* sm_l = sm_m + WARPS_PER_GROUP * 8;
-    float* sm_o = reinterpret_cast<float*>(smem + L::MO_OFF) + group * WARPS_PER_GROUP * a.G * D;
+    const int fheads = min(a.G, L::FLUSH_HEADS);       // heads per round of a flush
+    float* sm_o = reinterpret_cast<float*>(smem + L::MO_OFF) + group * WARPS_PER_GROUP * fheads * D;
     const int gtid = tid - group * 32 * WARPS_PER_GROUP;    // thread index inside the group
     const int g = lane >> 2, t = lane & 3;
     const int rb = wq * WT;                            // first token row of this warp inside a tile
@@ -643,14 +666,6 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
 
     for (uint32_t fill = group;; fill += NGROUPS) {
         const int stage = fill % NSTAGE;
-        if (SHARED_STAGES) {
-            bool started = false;
-            for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-                if ((uint32_t)ld_volatile(&s_fill_started) > fill) { started = true; break; }
-                __nanosleep(40);
-            }
-            if (!started) { ok = false; break; }
-        }
         if (!mbar_wait(&full[stage], (fill / NSTAGE) & 1)) { ok = false; break; }
         const int4 ds = desc[stage];
         const bool end = (ds.y & (int)UF_END) != 0;
@@ -669,45 +684,49 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             float lsum = l_run + __shfl_xor_sync(0xffffffffu, l_run, 1);
             lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
             if (t == 0) { sm_m[wq * 8 + g] = m_run; sm_l[wq * 8 + g] = lsum; }
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int mt = 0; mt < 4; ++mt) {
-                    const int dcol = 64 * hf + 8 * vchunk + 2 * mt;
-                    if (2 * t < a.G)
-                        *reinterpret_cast<float2*>(sm_o + ((wq * a.G + 2 * t) * D + dcol)) = make_float2(o[hf][mt][0], o[hf][mt][2]);
-                    if (2 * t + 1 < a.G)
-                        *reinterpret_cast<float2*>(sm_o + ((wq * a.G + 2 * t + 1) * D + dcol)) = make_float2(o[hf][mt][1], o[hf][mt][3]);
-                }
-#ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
-            // test build only: one warp of the first CTA never arrives, so that the group's bounded wait runs out and
-            // the give-up path (status flag, orderly exit of the whole CTA) executes
-            if (!(blockIdx.x == 0 && group == 0 && wq == 1))
-#endif
-            mbar_arrive(&flushbar[group]);
-            if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
-            flush_phase ^= 1;
             const int64_t slot = ((int64_t)blockIdx.x + row) * NGROUPS + group;
-            for (int idx = gtid; idx < a.G * D; idx += 32 * WARPS_PER_GROUP) {
-                const int hh = idx / D, dd = idx % D;
-                float M = -INFINITY;
+            for (int h0 = 0; h0 < a.G && ok; h0 += fheads) {
+                const int ha = 2 * t - h0, hb = ha + 1;         // this lane's two heads within the round
 #pragma unroll
-                for (int w = 0; w < WARPS_PER_GROUP; ++w) M = fmaxf(M, sm_m[w * 8 + hh]);
-                float acc = 0.f, lacc = 0.f;
-                if (M != -INFINITY) {
+                for (int hf = 0; hf < HALVES; ++hf)
 #pragma unroll
-                    for (int w = 0; w < WARPS_PER_GROUP; ++w) {
-                        const float sc = exp2f((sm_m[w * 8 + hh] - M) * LOG2E);
-                        acc = fmaf(sm_o[(w * a.G + hh) * D + dd], sc, acc);
-                        lacc = fmaf(sm_l[w * 8 + hh], sc, lacc);
+                    for (int mt = 0; mt < 4; ++mt) {
+                        const int dcol = 64 * hf + 8 * vchunk + 2 * mt;
+                        if (ha >= 0 && ha < fheads)
+                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + ha) * D + dcol)) = make_float2(o[hf][mt][0], o[hf][mt][2]);
+                        if (hb >= 0 && hb < fheads)
+                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + hb) * D + dcol)) = make_float2(o[hf][mt][1], o[hf][mt][3]);
                     }
+#ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
+                // test build only: one warp of the first CTA never arrives, so that the group's bounded wait runs out and
+                // the give-up path (status flag, orderly exit of the whole CTA) executes
+                if (!(blockIdx.x == 0 && group == 0 && wq == 1))
+#endif
+                mbar_arrive(&flushbar[group]);
+                if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
+                flush_phase ^= 1;
+                for (int idx = gtid; idx < fheads * D; idx += 32 * WARPS_PER_GROUP) {
+                    const int hr = idx / D, dd = idx % D, hh = h0 + hr;
+                    float M = -INFINITY;
+#pragma unroll
+                    for (int w = 0; w < WARPS_PER_GROUP; ++w) M = fmaxf(M, sm_m[w * 8 + hh]);
+                    float acc = 0.f, lacc = 0.f;
+                    if (M != -INFINITY) {
+#pragma unroll
+                        for (int w = 0; w < WARPS_PER_GROUP; ++w) {
+                            const float sc = exp2f((sm_m[w * 8 + hh] - M) * LOG2E);
+                            acc = fmaf(sm_o[(w * fheads + hr) * D + dd], sc, acc);
+                            lacc = fmaf(sm_l[w * 8 + hh], sc, lacc);
+                        }
+                    }
+                    a.part_o[(slot * a.G + hh) * D + dd] = acc;
+                    if (dd == 0) a.part_ml[slot * a.G + hh] = make_float2(M, lacc);
                 }
-                a.part_o[(slot * a.G + hh) * D + dd] = acc;
-                if (dd == 0) a.part_ml[slot * a.G + hh] = make_float2(M, lacc);
+                mbar_arrive(&flushbar[group]);
+                if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
+                flush_phase ^= 1;
             }
-            mbar_arrive(&flushbar[group]);
-            if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
-            flush_phase ^= 1;
+            if (!ok) break;
         }
         if (end) {
             if (tl && warp == 0 && lane == 0) tl[5] = globaltimer_ns();
@@ -1126,14 +1145,13 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     da.div_gpr = FastDiv(L.gpr); da.div_hkv = FastDiv(desc->n_kv_heads); da.div_grid = FastDiv(n_ctas);
     da.timeline = debug_timeline();
     if (D == 128 && TS == 64) {
-        rc = (G == 8) ? launch_decode_t<128, 64, 5, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s)
-                      : launch_decode_t<128, 64, 6, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<128, 64, 6, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else if (D == 128 && TS == 32) {
-        rc = launch_decode_t<128, 32, 9, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<128, 32, 12, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else if (D == 64 && TS == 64) {
         rc = launch_decode_t<64, 64, 12, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     } else {
-        rc = launch_decode_t<64, 32, 18, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
+        rc = launch_decode_t<64, 32, 24, DECODE_GROUPS>(tmK, tmV, da, n_ctas, s);
     }
     if (rc != ETA_OK) return rc;
     profile_mark(4, s);
