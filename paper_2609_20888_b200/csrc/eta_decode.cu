@@ -705,22 +705,25 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 mbar_arrive(&flushbar[group]);
                 if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
                 flush_phase ^= 1;
-                for (int idx = gtid; idx < fheads * D; idx += 32 * WARPS_PER_GROUP) {
-                    const int hr = idx / D, dd = idx % D, hh = h0 + hr;
-                    float M = -INFINITY;
+                for (int idx = gtid; idx < fheads * D / 4; idx += 32 * WARPS_PER_GROUP) {
+                    const int hr = idx / (D / 4), dq = idx % (D / 4), hh = h0 + hr;
+                    float mw[WARPS_PER_GROUP], M = -INFINITY;
 #pragma unroll
-                    for (int w = 0; w < WARPS_PER_GROUP; ++w) M = fmaxf(M, sm_m[w * 8 + hh]);
-                    float acc = 0.f, lacc = 0.f;
+                    for (int w = 0; w < WARPS_PER_GROUP; ++w) { mw[w] = sm_m[w * 8 + hh]; M = fmaxf(M, mw[w]); }
+                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float lacc = 0.f;
                     if (M != -INFINITY) {
 #pragma unroll
                         for (int w = 0; w < WARPS_PER_GROUP; ++w) {
-                            const float sc = exp2f((sm_m[w * 8 + hh] - M) * LOG2E);
-                            acc = fmaf(sm_o[(w * fheads + hr) * D + dd], sc, acc);
+                            const float sc = exp2f((mw[w] - M) * LOG2E);
+                            const float4 x = *reinterpret_cast<const float4*>(sm_o + (w * fheads + hr) * D + 4 * dq);
+                            acc.x = fmaf(x.x, sc, acc.x); acc.y = fmaf(x.y, sc, acc.y);
+                            acc.z = fmaf(x.z, sc, acc.z); acc.w = fmaf(x.w, sc, acc.w);
                             lacc = fmaf(sm_l[w * 8 + hh], sc, lacc);
                         }
                     }
-                    a.part_o[(slot * a.G + hh) * D + dd] = acc;
-                    if (dd == 0) a.part_ml[slot * a.G + hh] = make_float2(M, lacc);
+                    *reinterpret_cast<float4*>(a.part_o + (slot * a.G + hh) * D + 4 * dq) = acc;
+                    if (dq == 0) a.part_ml[slot * a.G + hh] = make_float2(M, lacc);
                 }
                 mbar_arrive(&flushbar[group]);
                 if (!mbar_wait(&flushbar[group], flush_phase)) { ok = false; break; }
@@ -896,18 +899,22 @@ constexpr int MERGE_WARPS = 8;
 // that a small batch still fills the GPU (with one sequence and four KV heads there are only 16 (row, head) pairs,
 // each with up to 3 x 148 partials to fold).  The candidate parts are the (streaming CTA, consumer group) pairs of
 // the streaming CTAs that hold units of the row, which the streaming kernel lists per row; a part marked absent
-// weighs nothing.  Warp w takes a contiguous share of the candidates, 32 a round: lane k reads the statistics of
-// candidate k while O rows are already on their way (a row slice is DW / 4 lanes wide, so a warp instruction
-// fetches 128 / DW candidates' slices, eight instructions in flight), the warp takes the largest m of its share,
-// weighs and adds the rows; lanes that hold the same coordinates, then the eight warps, are combined in a fixed
-// order:  o = sum_k O_k e^{m_k - m*} / sum_k l_k e^{m_k - m*},  m* = max_k m_k.
+// weighs nothing.  Warp w takes a contiguous share of the candidates, MB warp instructions' worth a round (a row slice is
+// DW / 4 lanes wide, so an instruction fetches 128 / DW candidates' slices): statistics and rows of a round are on their
+// way together, and every lane weighs its own candidates, so a share of one round - the usual case - needs no exchange
+// before the warps meet.  Lanes that hold the same coordinates, then the eight warps, are combined in a fixed order:
+// o = sum_k O_k e^{m_k - m*} / sum_k l_k e^{m_k - m*},  m* = max_k m_k.
+//
+// Bound by latency: the chain wait - span - parts - output.  The span is read ahead of the wait as well (the streaming
+// CTAs wrote it some 30 us earlier) and the parts it names are requested with the span itself, which is then checked.
 template <int D, int DS>
 __global__ void __launch_bounds__(32 * MERGE_WARPS) merge_kernel(const MergeArgs a) {
     constexpr int DW = D / DS;             // coordinates of this CTA's slice
     constexpr int LPC = DW / 4;            // lanes per candidate row slice (a float4 each)
     constexpr int CPW = 32 / LPC;          // candidates per warp instruction
+    constexpr int MB = 4;                  // candidates per lane and round
     static_assert(DW >= 4 && LPC <= 32 && LPC * CPW == 32, "slice must be 4 .. 128 coordinates");
-    __shared__ float s_acc[MERGE_WARPS][DW];
+    __shared__ __align__(16) float s_acc[MERGE_WARPS][DW];
     __shared__ float s_l[MERGE_WARPS];
     __shared__ float s_m[MERGE_WARPS];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -917,75 +924,74 @@ __global__ void __launch_bounds__(32 * MERGE_WARPS) merge_kernel(const MergeArgs
     unsigned long long* const tl = ETA_TL((a.timeline && blockIdx.x < TL_MERGE_N) ? a.timeline + (size_t)(TL_MERGE + blockIdx.x) * 8 : nullptr);
     if (tl && tid == 0) tl[0] = globaltimer_ns();
     pdl_trigger();
+    // what the span will most likely be; clamped, so that whatever is read here names slots of the scratch
+    int2 guess = __ldcg(a.row_span + r);
+    guess.x = min(max(guess.x, 0), MAX_CTAS - 1);
+    guess.y = min(max(guess.y, 0), MAX_CTAS - guess.x);
     pdl_wait();          // every partial of the streaming kernel is in memory from here on
     if (tl && tid == 0) tl[1] = globaltimer_ns();
-    const int2 span = a.row_span[r];
-    const int c_lo = span.x, n_cand = span.y * a.ngroups;
-    if (tl && tid == 0) tl[2] = globaltimer_ns() + (n_cand & 0);
-    auto slot_of = [&](int k) { return ((int64_t)(c_lo + k / a.ngroups) + r) * a.ngroups + k % a.ngroups; };
     const int sub = lane / LPC, dl = lane % LPC;        // candidate within a warp instruction, float4 within the slice
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    float m_w = -INFINITY, l_w = 0.f;        // this warp's running maximum and weighted l
-    const int per = (n_cand + MERGE_WARPS - 1) / MERGE_WARPS;
-    const int k_begin = warp * per, k_end = min(n_cand, k_begin + per);
-    for (int k0 = k_begin; k0 < k_end; k0 += 32) {
-        const int k = k0 + lane;
-        const int nk = min(32, k_end - k0);
-        float m_k = -INFINITY, l_k = 0.f;
-        if (k < k_end) {
-            const float2 ml = a.part_ml[slot_of(k) * a.G + gq];
-            m_k = ml.x; l_k = ml.y;
-        }
-        // the first O rows of the round do not wait for the statistics
-        float4 xv[8];
-        auto load_rows = [&](int j0) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float m_w = -INFINITY, l_w = 0.f;                   // this lane's running maximum and weighted l
+    const int2 span = __ldcg(a.row_span + r);
+    auto fold_span = [&](const int2& sp, bool check) {
+        const int n_cand = sp.y * a.ngroups;
+        const int per = (n_cand + MERGE_WARPS - 1) / MERGE_WARPS;
+        const int k_begin = warp * per, k_end = min(n_cand, k_begin + per);
+        for (int k0 = k_begin + sub; k0 < k_end; k0 += MB * CPW) {
+            float2 ml[MB];
+            float4 x[MB];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = j0 + u * CPW + sub;
-                xv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (j < nk)
-                    xv[u] = __ldg(reinterpret_cast<const float4*>(a.part_o + (slot_of(k0 + j) * a.G + gq) * D + dpart * DW) + dl);
+            for (int u = 0; u < MB; ++u) {
+                const int k = k0 + u * CPW;
+                ml[u] = make_float2(-INFINITY, 0.f);
+                x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (k < k_end) {
+                    const int64_t ph = (((int64_t)sp.x + r) * a.ngroups + k) * a.G + gq;
+                    ml[u] = __ldcg(a.part_ml + ph);
+                    x[u] = __ldcg(reinterpret_cast<const float4*>(a.part_o + ph * D + dpart * DW) + dl);
+                }
             }
-        };
-        load_rows(0);
-        float m_round = m_k;
+            if (check && (span.x != sp.x || span.y != sp.y)) return false;       // (the loads above are on their way)
+            float m_new = m_w;
 #pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) m_round = fmaxf(m_round, __shfl_xor_sync(0xffffffffu, m_round, s));
-        const float m_new = fmaxf(m_w, m_round);
-        if (m_new == -INFINITY) continue;        // nothing real in this round (warp-uniform)
-        const float rescale = (m_w == -INFINITY) ? 0.f : __expf(m_w - m_new);
-        const float w = (m_k == -INFINITY) ? 0.f : __expf(m_k - m_new);
+            for (int u = 0; u < MB; ++u) m_new = fmaxf(m_new, ml[u].x);
+            if (m_new == -INFINITY) continue;
+            const float keep = __expf(m_w - m_new);         // m_w = -inf gives 0
+            acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+            l_w *= keep;
+            m_w = m_new;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[v] *= rescale;
-        float lw = l_k * w;
-#pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, s);
-        l_w = l_w * rescale + lw;
-        m_w = m_new;
-        for (int j0 = 0; j0 < nk; j0 += 8 * CPW) {
-            if (j0 > 0) load_rows(j0);
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = j0 + u * CPW + sub;
-                const float wk = __shfl_sync(0xffffffffu, w, min(j, 31));
-                if (j < nk && wk != 0.f) {       // an absent part's row is stale memory: never touch it
-                    acc[0] = fmaf(xv[u].x, wk, acc[0]); acc[1] = fmaf(xv[u].y, wk, acc[1]);
-                    acc[2] = fmaf(xv[u].z, wk, acc[2]); acc[3] = fmaf(xv[u].w, wk, acc[3]);
+            for (int u = 0; u < MB; ++u) {
+                if (ml[u].x != -INFINITY) {                 // an absent part's row is stale memory: never touch it
+                    const float w = __expf(ml[u].x - m_new);
+                    acc.x = fmaf(x[u].x, w, acc.x); acc.y = fmaf(x[u].y, w, acc.y);
+                    acc.z = fmaf(x[u].z, w, acc.z); acc.w = fmaf(x[u].w, w, acc.w);
+                    l_w = fmaf(ml[u].y, w, l_w);
                 }
             }
         }
+        return span.x == sp.x && span.y == sp.y;
+    };
+    if (!fold_span(guess, true)) {
+        acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        m_w = -INFINITY; l_w = 0.f;
+        fold_span(span, false);
     }
     // lanes that hold the same coordinates of different candidates
 #pragma unroll
     for (int o = LPC; o < 32; o <<= 1) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+        const float m_o = __shfl_xor_sync(0xffffffffu, m_w, o), m_new = fmaxf(m_w, m_o);
+        const float keep = m_w == -INFINITY ? 0.f : __expf(m_w - m_new), wo = m_o == -INFINITY ? 0.f : __expf(m_o - m_new);
+        acc.x = acc.x * keep + __shfl_xor_sync(0xffffffffu, acc.x, o) * wo;
+        acc.y = acc.y * keep + __shfl_xor_sync(0xffffffffu, acc.y, o) * wo;
+        acc.z = acc.z * keep + __shfl_xor_sync(0xffffffffu, acc.z, o) * wo;
+        acc.w = acc.w * keep + __shfl_xor_sync(0xffffffffu, acc.w, o) * wo;
+        l_w = l_w * keep + __shfl_xor_sync(0xffffffffu, l_w, o) * wo;
+        m_w = m_new;
     }
-    if (tl && tid == 0) tl[3] = globaltimer_ns() + (__float_as_int(acc[0]) & 0);
-    if (sub == 0) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) s_acc[warp][dl * 4 + v] = acc[v];
-    }
+    if (tl && tid == 0) tl[3] = globaltimer_ns() + (__float_as_int(acc.x) & 0);
+    if (sub == 0) *reinterpret_cast<float4*>(&s_acc[warp][dl * 4]) = acc;
     if (lane == 0) { s_l[warp] = l_w; s_m[warp] = m_w; }
     __syncthreads();
     if (tid < DW) {
