@@ -1,8 +1,11 @@
-"""Thin ctypes binding of the C-ABI library (`include/eta.h`).
+"""Thin binding of the C-ABI library (`include/eta.h`).
 
 Argument marshalling only: torch tensors provide device memory and the current
 CUDA stream; every step of the path runs in the library's kernels.  There is no
-CPU fallback: a missing library or a CPU tensor raises.
+CPU fallback: a missing library or a CPU tensor raises.  The library is loaded
+with ctypes; the calls of a decode step are marshalled by the compiled module
+`_eta_torch` (`csrc/eta_torch.cpp`), because ctypes takes longer over their
+arguments than a small step takes on the GPU.
 """
 from __future__ import annotations
 
@@ -50,13 +53,23 @@ class EtaError(RuntimeError):
 
 
 _lib = None
+_native = None          # the compiled marshalling module
+_STEP_CALLS = ("eta_append_summary", "eta_append_summary_paged", "eta_predict_threshold", "eta_decode", "eta_decode_paged",
+               "eta_decode_static")
 
 
 def load(path: str | None = None) -> ctypes.CDLL:
     """Load the in-tree library; fails loudly when it has not been built.  With a path: another build of the same
     sources (a test variant), loaded beside the product library and not remembered."""
-    global _lib
+    global _lib, _native
     if _lib is None or path is not None:
+        if _native is None:
+            try:
+                from . import _eta_torch
+            except ImportError as e:
+                raise EtaError(f"_eta_torch is missing ({e}): build it with `python -m paper_2609_20888_b200.build`") from e
+            _eta_torch.set_error(EtaError)
+            _native = _eta_torch
         lib_path = path or LIB_PATH
         if not os.path.exists(lib_path):
             raise EtaError(f"{lib_path} is missing: build it with `python -m paper_2609_20888_b200.build` "
@@ -96,6 +109,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
             if name not in ("eta_strerror", "eta_last_cuda_error", "eta_decode_kernel_count",
                             "eta_profile_kernel_name", "eta_static_scratch_bytes"):
                 getattr(lib, name).restype = ctypes.c_int
+        lib.addresses = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _STEP_CALLS}
         if path is not None:
             return lib
         _lib = lib
@@ -116,15 +130,6 @@ def _dev(t: torch.Tensor | None, dtype=None, name="tensor"):
     if dtype is not None and t.dtype != dtype:
         raise EtaError(f"{name} must be {dtype}, got {t.dtype}")
     return ctypes.c_void_p(t.data_ptr())
-
-
-def _dev_or_pinned(t: torch.Tensor, dtype=None, name="tensor"):
-    """Device pointer of a CUDA tensor, or of a page-locked host tensor (addressable by the device as it is)."""
-    if t is not None and not t.is_cuda and t.is_pinned():
-        if dtype is not None and t.dtype != dtype:
-            raise EtaError(f"{name} must be {dtype}, got {t.dtype}")
-        return ctypes.c_void_p(t.data_ptr())
-    return _dev(t, dtype, name)
 
 
 def _dev_musig(t: torch.Tensor):
@@ -208,10 +213,10 @@ def eta_build_block_summaries(desc, K, seq_lens, musig, mnorm, flags: int = 0) -
 
 
 def eta_append_summary(desc, K, seq_lens_after, musig, mnorm, flags: int = 0) -> None:
-    _check(load().eta_append_summary(ctypes.byref(desc), _dev(K, torch.bfloat16, "K"),
-                                     _dev(seq_lens_after, torch.int32, "seq_lens"), _dev_musig(musig),
-                                     _dev(mnorm, torch.float32, "mnorm"), flags, _stream()),
-           "eta_append_summary")
+    lib = _lib or load()
+    rc = _native.append(lib.addresses["eta_append_summary"], desc, None, K, seq_lens_after, musig, mnorm, flags)
+    if rc:
+        _check(rc, "eta_append_summary")
 
 
 def eta_build_block_summaries_paged(desc, pages: PageTable, K_pool, seq_lens, musig, mnorm, flags: int = 0) -> None:
@@ -223,11 +228,10 @@ def eta_build_block_summaries_paged(desc, pages: PageTable, K_pool, seq_lens, mu
 
 
 def eta_append_summary_paged(desc, pages: PageTable, K_pool, seq_lens_after, musig, mnorm, flags: int = 0) -> None:
-    _check(load().eta_append_summary_paged(ctypes.byref(desc), ctypes.byref(pages), _dev(K_pool, torch.bfloat16, "K_pool"),
-                                           _dev(seq_lens_after, torch.int32, "seq_lens"),
-                                           _dev_musig(musig), _dev(mnorm, torch.float32, "mnorm"),
-                                           flags, _stream()),
-           "eta_append_summary_paged")
+    lib = _lib or load()
+    rc = _native.append(lib.addresses["eta_append_summary_paged"], desc, pages, K_pool, seq_lens_after, musig, mnorm, flags)
+    if rc:
+        _check(rc, "eta_append_summary_paged")
 
 
 def eta_stage_query(q_host, q_dev) -> None:
@@ -242,10 +246,10 @@ def eta_stage_query(q_host, q_dev) -> None:
 
 
 def eta_predict_threshold(q, W, bias, tau) -> None:
-    B, Hq, d = q.shape
-    _check(load().eta_predict_threshold(B, Hq, d, _dev(q, torch.bfloat16, "q"), _dev(W, torch.float32, "W"),
-                                        _dev(bias, torch.float32, "bias"), _dev(tau, torch.float32, "tau"), _stream()),
-           "eta_predict_threshold")
+    lib = _lib or load()
+    rc = _native.predict(lib.addresses["eta_predict_threshold"], q, W, bias, tau)
+    if rc:
+        _check(rc, "eta_predict_threshold")
 
 
 def eta_score_dual(desc, params: DecodeParams, q, seq_lens, musig, mnorm, bound) -> None:
@@ -280,45 +284,31 @@ def eta_calibrate_head_const(Q, K, tau, head_const, dbar=None, beta=5.0, scale=0
 
 def eta_decode(desc, params: DecodeParams, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask,
                workspace, stats=None, status=None, lib=None) -> None:
-    p = params.c()
-    _check((lib or load()).eta_decode(ctypes.byref(desc), ctypes.byref(p), _dev(q, torch.bfloat16, "q"),
-                             _dev(K, torch.bfloat16, "K"), _dev(V, torch.bfloat16, "V"),
-                             _dev(seq_lens, torch.int32, "seq_lens"), _dev_musig(musig),
-                             _dev(mnorm, torch.float32, "mnorm"), _dev(tau, torch.float32, "tau"),
-                             _dev(head_const, torch.float32, "head_const"), _dev_or_pinned(out, torch.float32, "out"),
-                             _dev(sel_mask, torch.uint8, "sel_mask"), _dev(stats, torch.int32, "stats"),
-                             _dev(status, torch.int32, "status"), _dev(workspace, torch.uint8, "workspace"),
-                             workspace.numel(), _stream()),
-           "eta_decode")
+    lib = lib or _lib or load()
+    rc = _native.decode(lib.addresses["eta_decode"], desc, None, params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out,
+                        sel_mask, stats, status, workspace)
+    if rc:
+        _check(rc, "eta_decode")
 
 
 def eta_decode_paged(desc, pages: PageTable, params: DecodeParams, q, K_pool, V_pool, seq_lens, musig, mnorm, tau,
                      head_const, out, sel_mask, workspace, stats=None, status=None) -> None:
-    p = params.c()
-    _check(load().eta_decode_paged(ctypes.byref(desc), ctypes.byref(pages), ctypes.byref(p), _dev(q, torch.bfloat16, "q"),
-                                   _dev(K_pool, torch.bfloat16, "K_pool"), _dev(V_pool, torch.bfloat16, "V_pool"),
-                                   _dev(seq_lens, torch.int32, "seq_lens"), _dev_musig(musig),
-                                   _dev(mnorm, torch.float32, "mnorm"), _dev(tau, torch.float32, "tau"),
-                                   _dev(head_const, torch.float32, "head_const"), _dev_or_pinned(out, torch.float32, "out"),
-                                   _dev(sel_mask, torch.uint8, "sel_mask"), _dev(stats, torch.int32, "stats"),
-                                   _dev(status, torch.int32, "status"), _dev(workspace, torch.uint8, "workspace"),
-                                   workspace.numel(), _stream()),
-           "eta_decode_paged")
+    lib = _lib or load()
+    rc = _native.decode(lib.addresses["eta_decode_paged"], desc, pages, params, q, K_pool, V_pool, seq_lens, musig, mnorm, tau,
+                        head_const, out, sel_mask, stats, status, workspace)
+    if rc:
+        _check(rc, "eta_decode_paged")
 
 
 def eta_decode_static(desc, params: DecodeParams, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask,
                       stats=None, status=None) -> None:
     """eta_decode without a workspace argument, for callers that have no device memory to give: the scratch is
     an 8 MiB array built into the library (see include/eta.h for its limit and sharing rules)."""
-    p = params.c()
-    _check(load().eta_decode_static(ctypes.byref(desc), ctypes.byref(p), _dev(q, torch.bfloat16, "q"),
-                                    _dev(K, torch.bfloat16, "K"), _dev(V, torch.bfloat16, "V"),
-                                    _dev(seq_lens, torch.int32, "seq_lens"), _dev_musig(musig),
-                                    _dev(mnorm, torch.float32, "mnorm"), _dev(tau, torch.float32, "tau"),
-                                    _dev(head_const, torch.float32, "head_const"), _dev_or_pinned(out, torch.float32, "out"),
-                                    _dev(sel_mask, torch.uint8, "sel_mask"), _dev(stats, torch.int32, "stats"),
-                                    _dev(status, torch.int32, "status"), _stream()),
-           "eta_decode_static")
+    lib = _lib or load()
+    rc = _native.decode(lib.addresses["eta_decode_static"], desc, None, params, q, K, V, seq_lens, musig, mnorm, tau, head_const,
+                        out, sel_mask, stats, status, False)
+    if rc:
+        _check(rc, "eta_decode_static")
 
 
 def eta_static_scratch_bytes() -> int:

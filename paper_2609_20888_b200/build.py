@@ -31,6 +31,8 @@ def needs_build(lib: str = LIB) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False, lib: str = LIB, extra_flags: tuple = ()) -> str:
+    if lib == LIB:
+        build_torch_module(force)
     if not force and not needs_build(lib):
         return lib
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -42,6 +44,30 @@ def build(force: bool = False, verbose: bool = False, lib: str = LIB, extra_flag
         cmd.insert(2, "-v")
     subprocess.run(cmd, check=True)
     return lib
+
+
+# The marshalling of a decode step's calls for torch: a Python module of its own, compiled by the host compiler.
+TORCH_MODULE = os.path.join(HERE, "_eta_torch.so")
+TORCH_SOURCE = os.path.join(CSRC, "eta_torch.cpp")
+
+
+def build_torch_module(force: bool = False) -> str:
+    deps = [TORCH_SOURCE, HEADER]
+    if not force and os.path.exists(TORCH_MODULE) and all(os.path.getmtime(p) <= os.path.getmtime(TORCH_MODULE) for p in deps):
+        return TORCH_MODULE
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-o", TORCH_MODULE, TORCH_SOURCE,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for inc in (os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]):
+        cmd += ["-isystem", inc]
+    cmd += ["-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    subprocess.run(cmd, check=True)
+    return TORCH_MODULE
 
 
 def build_giveup_variant(force: bool = False) -> str:

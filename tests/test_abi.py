@@ -97,3 +97,27 @@ def test_binding_refuses_cpu_tensors(lib):
     mn = torch.zeros((1, 2, 2), dtype=torch.float32)
     with pytest.raises(eb.EtaError):
         eb.eta_build_block_summaries(d, K, torch.zeros(1, dtype=torch.int32), ms, mn)
+
+
+def test_step_calls_check_their_tensors():
+    """The compiled marshalling refuses what the binding refuses: host tensors, other types, things that are no tensors."""
+    import pytest
+    import torch
+
+    from paper_2609_20888_b200 import binding as eb
+    eb.load()
+    K = torch.zeros((1, 1, 64, 64), dtype=torch.bfloat16)
+    f, i = torch.zeros(4), torch.zeros(1, dtype=torch.int32)
+    desc = eb.cache_desc(K, K, 1, 64)
+    with pytest.raises(eb.EtaError, match="K must be a CUDA tensor"):
+        eb.eta_append_summary(desc, K, i, f, f)
+    with pytest.raises(TypeError):
+        eb.eta_append_summary(desc, 17, i, f, f)
+    with pytest.raises(TypeError):
+        eb.eta_append_summary(i.numpy(), K, i, f, f)
+    with pytest.raises(eb.EtaError, match="q must be a CUDA tensor"):
+        eb.eta_predict_threshold(torch.zeros((1, 1, 64), dtype=torch.bfloat16), f, f, f)
+    with pytest.raises(RuntimeError):          # invalid argument; without a GPU, no stream to call it on
+        eb.eta_decode(desc, eb.DecodeParams(), None, None, None, None, None, None, None, None, None, None, None)
+    with pytest.raises(AttributeError):
+        eb.eta_decode(desc, object(), None, None, None, None, None, None, None, None, None, None, None)
