@@ -258,7 +258,7 @@ __device__ __forceinline__ double2 block_sum2_fixed(double a, double b, double2*
 
 // A serial chain of evaluations of g, each n_bins double-precision sigmoids: what counts is how many there are.  The root
 // is found by Newton steps inside a bracket, with a halving wherever a step would leave the bracket or shrink too slowly:
-// about eight evaluations to double precision where plain halving took eighty (with the launch: 177 -> c. 30 us).
+// about eight evaluations to double precision where plain halving took eighty (177 -> 55 us; a first approximation in fp32 ahead of them gained nothing).
 __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
     const unsigned long long* __restrict__ hist, const double* __restrict__ dpart, int Hq, int n_seq, int n_ttiles,
     int T, int n_bins, double s_min, double s_max, double beta, int iters, float* __restrict__ head_const,

@@ -3,6 +3,7 @@
 // the kernels use (mbarrier, bulk / tensor TMA copies, warp MMA).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -93,6 +94,10 @@ struct ScreenArgs {
     int slots;                            // CTAs the GPU holds at once
     int group;                            // passes whose bounds are kept before their admission is decided
     int nbuf;                             // tiles a warp keeps in flight
+    // survivors whose K and V start on their way into the L2
+    int prefetch, tiles, tile_tokens;     // blocks per segment at most; copies per block and tensor, tokens of a copy
+    const int32_t* block_table;           // paged cache (null: contiguous)
+    int table_stride;
     FastDiv div_ctas, div_slots, div_hkv;
     uint8_t* seg_cnt;
     int gpr;
@@ -102,7 +107,7 @@ struct ScreenArgs {
     uint32_t* status;
     unsigned long long* timeline;
 };
-int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_sm, cudaStream_t s);
+int launch_screen(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int G, int n_sm, cudaStream_t s);
 
 // Launch with programmatic dependent launch allowed: the grid may start while its predecessor in the stream is
 // still draining, and must call pdl_wait() before touching anything the predecessor wrote.
@@ -233,9 +238,20 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const void* tmap, int x, 
 // 5-D tiled copy (this CTA's shared memory only): used with the head_dim split into 64-column halves as an extra dimension, so one
 // instruction brings both swizzled half tiles of a K or V tile.
 __device__ __forceinline__ void tma_load_5d(void* dst, const void* tmap, int c0, int c1, int c2, int c3, int c4,
-                                            uint64_t* bar) {
-    asm volatile("cp.async.bulk.tensor.5d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tmap), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
+                                            uint64_t* bar, uint64_t l2_policy) {
+    asm volatile("cp.async.bulk.tensor.5d.shared::cta.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+                 ::"r"(smem_u32(dst)), "l"(tmap), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(l2_policy) : "memory");
+}
+__device__ __forceinline__ uint64_t l2_policy(bool evict_first) {
+    uint64_t p;
+    if (evict_first) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+// the same box into the L2 only
+__device__ __forceinline__ void tma_prefetch_5d(const void* tmap, int c0, int c1, int c2, int c3, int c4) {
+    asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global.tile [%0, {%1, %2, %3, %4, %5}];"
+                 ::"l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");

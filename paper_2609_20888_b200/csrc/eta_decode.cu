@@ -54,6 +54,7 @@ struct DecodeArgs {
     int ungate_last;     // the newest token of every sequence keeps its raw logit (ETA_FLAG_UNGATE_LAST)
     const int32_t* block_table;   // paged cache: [batch, table_stride] page of every block of tokens; null: contiguous
     int table_stride;
+    int read_once;       // K and V leave the L2 first
     FastDiv div_gpr, div_hkv, div_grid;
     unsigned long long* timeline;
 };
@@ -66,6 +67,7 @@ constexpr int WARPS_PER_GROUP = 4;     // the four warps of a group each take a 
 // leave SMs without work (a CTA needs more cost units than a row's padding) a boundary counts as one tile: a problem of
 // 50 blocks then runs on 24 CTAs of two tiles instead of 6 of ten.
 constexpr int PIECE_COST = 8, PIECE_COST_SMALL = 1;
+constexpr int64_t LARGE_CACHE_BYTES = 256ll << 20, PREFETCH_BYTES = 32ll << 20;       // see decode_impl
 constexpr int LGRAN = 8;               // granules per lane of a chunk
 constexpr int CHUNK = 32 * LGRAN;      // granules of a chunk: what a warp reads in one round trip
 constexpr int MAX_SUPER = 512;         // sums over `super` chunks each, kept in shared memory when there is more than one chunk
@@ -487,6 +489,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         // description broadcast by shuffles) the producer took 550 ns a tile, which held every tile of less than 32 KB (64
         // columns or 32 tokens) below half of the copy rate.
         const int usub = lane % tpu;
+        const uint64_t once = l2_policy(a.read_once != 0);
         uint32_t fill = 0;
         int piece = -1, prev_row = -1;
         uint32_t piece_f0 = 0;
@@ -551,8 +554,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 // the first is complete as early as can be.
                 for (unsigned rm = __ballot_sync(0xffffffffu, ready); rm; rm &= rm - 1) {
                     if (lane == __ffs(rm) - 1) {
-                        tma_load_5d(my_smem, &tmK, 0, my_y, 0, my_hk, my_w, &full[stage]);
-                        tma_load_5d(my_smem + HALVES * L::TILE_BYTES, &tmV, 0, my_y, 0, my_hk, my_w, &full[stage]);
+                        tma_load_5d(my_smem, &tmK, 0, my_y, 0, my_hk, my_w, &full[stage], once);
+                        tma_load_5d(my_smem + HALVES * L::TILE_BYTES, &tmV, 0, my_y, 0, my_hk, my_w, &full[stage], once);
                     }
                 }
                 return __any_sync(0xffffffffu, !done) != 0;
@@ -1119,16 +1122,29 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     sa.sel_mask = sel_mask;
     sa.timeline = debug_timeline();
     sa.status = status_dev;
-    profile_mark(2, s);
-    rc = launch_screen(sa, L.rows, D, G, n_sm, s);
-    profile_mark(3, s);
-    if (rc != ETA_OK) return rc;
-
     CUtensorMap tmK, tmV;
     const int n_pages = pages ? pages->n_pages : 0;
     rc = make_tmap(&tmK, K, desc, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t, TS, n_pages);
     if (rc != ETA_OK) return rc;
     rc = make_tmap(&tmV, V, desc, desc->v_stride_b, desc->v_stride_h, desc->v_stride_t, TS, n_pages);
+    if (rc != ETA_OK) return rc;
+
+    sa.tiles = b / TS; sa.tile_tokens = TS;
+    sa.block_table = pages ? pages->block_table : nullptr;
+    sa.table_stride = pages ? pages->table_stride : 0;
+    // A cache well beyond the L2 (126 MB): what a step reads of it will not be there for the next step, so its lines leave
+    // the L2 first, and the screening kernel starts the first survivors of every segment on their way, 32 MB in all (five of
+    // the 8 us the memory would idle before the streaming kernel's first copies).  Batch 4 at 128K: 66.7 -> 60.5 us a step with
+    // the first of the two, 58.4 with both (24, 48 and 80 MB within 1 us of 32); 32K x 8: 58.0 -> 51.2; 512K: 51.2 -> 43.4.
+    // Where the cache fits, or nearly, both cost time: 50K x 1 with 4 KV heads (104 MB) 24.7 -> 27.8, 8K x 7 (30 MB) 24.7 -> 28.8;
+    // between 140 and 330 MB the sign depends on how much survives (51.3 -> 45.0, 33.9 -> 33.2, 30.0 -> 32.4).
+    const int64_t unit_bytes = (int64_t)4 * b * D, segs = (int64_t)L.rows * L.nseg;
+    const bool large = (int64_t)L.rows * desc->nb_cap * unit_bytes > LARGE_CACHE_BYTES;
+    const int64_t share = (PREFETCH_BYTES + segs * unit_bytes - 1) / (segs * unit_bytes);
+    sa.prefetch = !large ? 0 : (int)(share < SEG ? share : SEG);
+    profile_mark(2, s);
+    rc = launch_screen(sa, tmK, tmV, L.rows, D, G, n_sm, s);
+    profile_mark(3, s);
     if (rc != ETA_OK) return rc;
 
     DecodeArgs da;
@@ -1148,6 +1164,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     da.ungate_last = (!dense && (params->flags & ETA_FLAG_UNGATE_LAST)) ? 1 : 0;
     da.block_table = pages ? pages->block_table : nullptr;
     da.table_stride = pages ? pages->table_stride : 0;
+    da.read_once = large ? 1 : 0;
     da.div_gpr = FastDiv(L.gpr); da.div_hkv = FastDiv(desc->n_kv_heads); da.div_grid = FastDiv(n_ctas);
     da.timeline = debug_timeline();
     if (D == 128 && TS == 64) {

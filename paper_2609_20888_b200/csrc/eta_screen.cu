@@ -363,7 +363,8 @@ __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
 // 68.8 us instead of 71.1 (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
 // barrier per segment); 65536 blocks at d = 64, G = 8, where both terms were on that pipe, 116.3 instead of 126.9.
 template <int D, int G, bool PACKED>
-__global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenArgs a) {
+__global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                                    const __grid_constant__ CUtensorMap tmV, const ScreenArgs a) {
     using L = ScreenSmem<D, G>;
     using TL = TileOf<D>;
     constexpr int REC_BYTES = PACKED ? 3 * D : 4 * D;
@@ -570,6 +571,25 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const ScreenA
                 carry += __popc(nz);
             }
             if (lane == 0) a.seg_cnt[((int64_t)r * a.gpr) * GRANULE + seg] = (uint8_t)carry;
+            // The memory is idle from here until the streaming kernel's first copies, some 8 us: the segment's first survivors
+            // start on their way into the L2.
+            if (a.prefetch) {
+                int rank = 0;
+#pragma unroll
+                for (int half = 0; half < SEG / 32; ++half) {
+                    const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
+                    if (m[half] && rank + __popc(nz & ((1u << lane) - 1u)) < a.prefetch) {
+                        const int j = j0 + half * 32 + lane;
+                        const int w4 = a.block_table ? __ldg(a.block_table + (int64_t)i * a.table_stride + j) : i;
+                        for (int k = 0; k < a.tiles; ++k) {
+                            const int y = (a.block_table ? 0 : j * a.b) + k * a.tile_tokens;
+                            tma_prefetch_5d(&tmK, 0, y, 0, hk, w4);
+                            tma_prefetch_5d(&tmV, 0, y, 0, hk, w4);
+                        }
+                    }
+                    rank += __popc(nz);
+                }
+            }
         }
         if (p1 < p_last) __syncthreads();          // the bounds of this group have been read: the next may overwrite them
     }
@@ -690,7 +710,7 @@ __global__ void __launch_bounds__(128) score_dual_unaligned_kernel(
 // ------------------------------------------------------------------ launchers (host)
 
 template <int D, int G, bool PACKED>
-static int launch_screen_t(const ScreenArgs& a, int rows, int n_sm, cudaStream_t s) {
+static int launch_screen_t(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int n_sm, cudaStream_t s) {
     constexpr int SPP = TileOf<D>::PASS / SEG;
     ScreenArgs b2 = a;
     b2.passes = (a.nseg + SPP - 1) / SPP;
@@ -715,13 +735,13 @@ static int launch_screen_t(const ScreenArgs& a, int rows, int n_sm, cudaStream_t
     // the one that holds the rescue window, then has both on their way from the start.
     b2.nbuf = (b2.group > 1 && all <= 3 * n_sm) ? 2 : 1;
     return launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)grid), dim3(32 * SCR_WARPS),
-                      ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, b2);
+                      ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, tmK, tmV, b2);
 }
 
-int launch_screen(const ScreenArgs& a, int rows, int D, int G, int n_sm, cudaStream_t s) {
+int launch_screen(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int G, int n_sm, cudaStream_t s) {
     const bool packed = (a.flags & ETA_FLAG_PACKED_SIGMA) != 0;
-#define ETA_CASE(DD, GG) if (D == DD && G == GG) return packed ? launch_screen_t<DD, GG, true>(a, rows, n_sm, s) \
-                                                                : launch_screen_t<DD, GG, false>(a, rows, n_sm, s);
+#define ETA_CASE(DD, GG) if (D == DD && G == GG) return packed ? launch_screen_t<DD, GG, true>(a, tmK, tmV, rows, n_sm, s) \
+                                                                : launch_screen_t<DD, GG, false>(a, tmK, tmV, rows, n_sm, s);
     ETA_CASE(128, 1) ETA_CASE(128, 2) ETA_CASE(128, 4) ETA_CASE(128, 8)
     ETA_CASE(64, 1) ETA_CASE(64, 2) ETA_CASE(64, 4) ETA_CASE(64, 8)
 #undef ETA_CASE
