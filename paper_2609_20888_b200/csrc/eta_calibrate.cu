@@ -7,8 +7,7 @@
 //
 // calib_hist_kernel: a CTA per (128-query tile, head, sequence).  The scores of a
 // 128 x 64 tile are a small dense contraction and go through the tensor cores
-// (mma.m16n8k16, bf16 in, fp32 out; the whole pass is a few GFLOP, so nothing
-// heavier is warranted); each score is binned into a histogram in shared memory.
+// (tcgen05, bf16 in, fp32 accumulators in tensor memory); each score is binned into a histogram in shared memory.
 // The causal row weight 1/t is added as the integer round(2^40 / t), so the
 // histogram does not depend on the order in which the atomics land; the gates
 // sigmoid(beta (S - tau_t)) are summed per row and reduced in a fixed order.
@@ -20,9 +19,11 @@
 
 namespace eta {
 
-constexpr int CAL_THREADS = 256;      // eight warps: 16 query rows each
-constexpr int CAL_ROWS = CAL_THREADS / 2;       // queries per CTA
+constexpr int CAL_ROWS = 128;         // queries per CTA: the rows of an MMA tile
+constexpr int CAL_WARPS = 8;          // warps that count: a thread has one row and half of a tile's keys
+constexpr int CAL_THREADS = 32 * (CAL_WARPS + 1);       // ... and one that loads tiles and issues MMAs
 constexpr int CAL_KEYS = 64;          // keys per tile
+constexpr int CAL_TMEM = 128;         // columns of tensor memory: up to 64 for the queries, 64 for the scores of a tile
 constexpr int CAL_WSHIFT = 40;        // row weights are integers: round(2^40 / t)
 constexpr int CAL_SPLIT = 16;         // bits of a weight that go to the histogram's low plane
 constexpr int CAL_FLUSH = 512;        // keys after which the planes are emptied
@@ -69,131 +70,125 @@ __device__ __forceinline__ void red_shared(uint32_t addr, uint32_t v) {
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool in) {      // zeroes where !in
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+// ---- 5th-generation tensor core (one CTA): 128 query rows x CAL_KEYS keys, bf16 in, fp32 accumulators in tensor memory
+// Shared-memory operand in the layout the copies leave: rows of 128 bytes, 128-byte swizzle, eight rows (1024 bytes) to a group
+__device__ __forceinline__ uint64_t umma_operand(uint32_t addr) {
+    return (uint64_t)((addr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// fp32 accumulator, bf16 x bf16, both operands with k contiguous, N = CAL_KEYS, M = CAL_ROWS; A in tensor memory
+constexpr uint32_t CAL_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((CAL_KEYS >> 3) << 17) | ((CAL_ROWS >> 4) << 24);
+__device__ __forceinline__ void umma_bf16(uint32_t acc, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(acc), "r"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+}
+// arrives on the barrier when every MMA issued so far has completed
+__device__ __forceinline__ void umma_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tmem_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+// 16 lanes x 32 columns: rows lane / 4 and lane / 4 + 8; v[4 k + 0, 1] are columns 8 k + 2 (lane % 4) + 0, 1 of the first of
+// the two rows, v[4 k + 2, 3] those of the second
+__device__ __forceinline__ void tmem_load_16x32(uint32_t addr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(addr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(r[c]);
 }
 
-// What bounds it: latency and issue of c. 27 instructions per score (two of them atomics; 24 warps per SM at 80 registers,
-// half of the issue slots used, tensor and special-function pipes at 30 %).  A row weight of up to 41 bits is added as two
-// 32-bit numbers to two planes of the histogram, w mod 2^16 and w / 2^16: 32-bit shared atomics without a return value are
-// native, a 64-bit one is a compare-and-swap loop.  Neither plane can wrap before it is emptied into the 64-bit histogram in
-// memory: a row's weights sum to 2^40, so 128 rows put at most 2^31 into the high plane, and CAL_FLUSH = 512 keys of 128
-// rows less than 2^32 into the low one.  16 x 1024 tokens, 32 heads, d = 128, 2048 bins: 470 us, against 1217 us with a
-// 64-bit atomic, a double add and a true division per score.
+// 32 bf16 of this thread's lane (32 lanes per warp) as 16 columns
+__device__ __forceinline__ void tmem_store16(uint32_t addr, const uint4 (&q)[4]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(addr), "r"(q[0].x), "r"(q[0].y), "r"(q[0].z), "r"(q[0].w), "r"(q[1].x), "r"(q[1].y), "r"(q[1].z), "r"(q[1].w),
+          "r"(q[2].x), "r"(q[2].y), "r"(q[2].z), "r"(q[2].w), "r"(q[3].x), "r"(q[3].y), "r"(q[3].z), "r"(q[3].w) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+template <int D>
+struct CalSmem {
+    static constexpr int K_BYTES = CAL_KEYS * D * 2;
+    static constexpr size_t bytes(int n_bins) { return 1024 + 2 * K_BYTES + 8 * (size_t)n_bins; }
+};
+
+// What bounds it: the shared-memory pipe (90 % of its passes), by the two atomics of a score: 3.55 passes each, which is what
+// 32 lanes on random banks take.  A row weight of up to 41 bits is added as two 32-bit numbers to two planes of the histogram,
+// w mod 2^16 and w / 2^16: 32-bit shared atomics without a return value are native, a 64-bit one is a compare-and-swap loop
+// (19 cycles a warp and SM), and one that returns the sum, to pass on carries, is no faster than two that do not.  Neither
+// plane can wrap before it is emptied into the 64-bit histogram in memory: a row's weights sum to 2^40, so 128 rows put at
+// most 2^31 into the high plane, and CAL_FLUSH = 512 keys of 128 rows less than 2^32 into the low one.
+// Everything else is kept off that pipe.  Fragments for mma.sync were 37 of its 102 million passes at 16 x 1024 tokens, 32
+// heads, d = 128 (all of it 435 us): now keys go to the tensor core by bulk copy and descriptor, scores come back through
+// tensor memory, and the queries sit there too (as an operand in shared memory they were read again for every tile: 14
+// million passes, 4.7 are left).  One accumulator of 64 keys: the MMA of a tile runs while the second half of the tile before
+// it is counted.  Two of 32 keys with a barrier each (347 us a calibration, against 313) cost more than they hide, two of 64
+// do not fit the tensor memory of three CTAs beside the queries.  With 2048 bins: 515 -> 333 (queries in shared memory) ->
+// 313 us, of which the histogram 435 -> 290.
 template <int D>
 __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
-    const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K, const float* __restrict__ tau,
+    const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const float* __restrict__ tau,
     int Hq, int Hkv, int T, float c2, float scale, int n_bins, float s_min, float inv_w,
     unsigned long long* __restrict__ hist, double* __restrict__ dpart) {
-    // padded row of the key tile: rows g and g + 1 start 64 bytes apart in the banks, so that the two rows a quarter-warp
-    // touches in one 16-byte load never share a bank
-    constexpr int KS = D + 32;
-    constexpr int NP = D / 32;            // 16-byte pieces of a row per lane
-    extern __shared__ __align__(16) unsigned char cal_raw[];
-    __nv_bfloat16* sK = reinterpret_cast<__nv_bfloat16*>(cal_raw);               // two key tiles
-    uint32_t* lo = reinterpret_cast<uint32_t*>(cal_raw + 2 * CAL_KEYS * KS * 2); // histogram: sums of w mod 2^16
-    uint32_t* hi = lo + n_bins;                                                  // sums of w / 2^16
-    __shared__ double s_red[CAL_THREADS / 32];
+    using L = CalSmem<D>;
+    extern __shared__ unsigned char cal_raw[];
+    unsigned char* sK = cal_raw + ((1024 - (smem_u32(cal_raw) & 1023)) & 1023);       // two key tiles, first of all the queries
+    uint32_t* lo = reinterpret_cast<uint32_t*>(sK + 2 * L::K_BYTES);   // histogram: sums of w mod 2^16
+    uint32_t* hi = lo + n_bins;                                        // sums of w / 2^16
+    __shared__ double s_red[CAL_WARPS];
+    __shared__ __align__(8) uint64_t bar_q, bar_in[2], bar_acc, bar_free;      // queries, keys arrived; scores complete; ... read by all
+    __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, tq = lane & 3;
-    const int ttile = gridDim.x - 1 - blockIdx.x, h = blockIdx.y, x = blockIdx.z;      // the longest tiles start first
-    const int hk = h / (Hq / Hkv);
+    const int h = blockIdx.x, x = blockIdx.y, ttile = gridDim.z - 1 - blockIdx.z;      // the longest tiles start first
     const int t0 = ttile * CAL_ROWS;
-    const __nv_bfloat16* Qh = Q + (((int64_t)x * Hq + h) * T) * D;
-    const __nv_bfloat16* Kh = K + (((int64_t)x * Hkv + hk) * T) * D;
-    const float* tauh = tau + ((int64_t)x * Hq + h) * T;
-    const int s_end = min(T, t0 + CAL_ROWS);          // keys of the CTA's longest row
+    const int n_tiles = (min(T, t0 + CAL_ROWS) + CAL_KEYS - 1) / CAL_KEYS;              // up to the CTA's longest row
 
-    auto fetch = [&](int s0, int buf) {               // key tile -> shared memory; rows past the end read as zero
-        const uint32_t dst = smem_u32(sK + buf * CAL_KEYS * KS);
-#pragma unroll
-        for (int u = 0; u < CAL_KEYS * (D / 8) / CAL_THREADS; ++u) {
-            const int p = tid + u * CAL_THREADS, row = p / (D / 8), piece = p % (D / 8);
-            const bool in = s0 + row < T;
-            cp_async16(dst + (row * KS + piece * 8) * 2, Kh + (int64_t)(in ? s0 + row : 0) * D + piece * 8, in);
+    if (warp == CAL_WARPS) {
+        if (lane == 0) {
+            for (uint64_t* b : {&bar_q, &bar_in[0], &bar_in[1], &bar_acc}) mbar_init(b, 1);
+            mbar_init(&bar_free, CAL_WARPS);
+            fence_barrier_init();
+            mbar_arrive_expect_tx(&bar_q, 2 * L::K_BYTES);
+            tma_load_4d(sK, &tmQ, 0, t0, 0, x * Hq + h, &bar_q);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    fetch(0, 0);
-    for (int b = tid; b < 2 * n_bins; b += CAL_THREADS) lo[b] = 0u;
-
-    // this thread's two query rows and their A fragments: piece m of a lane is the coordinates 8 (4 m + tq) .. + 7, the
-    // same ones its 16-byte load of a key covers (a dot product does not care about the order of k)
-    const int rw = t0 + warp * 16, r0 = rw + g, r1 = r0 + 8;
-    uint4 qa[NP], qb[NP];
-#pragma unroll
-    for (int m = 0; m < NP; ++m) {
-        const int c = 8 * (4 * m + tq);
-        qa[m] = (r0 < T) ? __ldg(reinterpret_cast<const uint4*>(Qh + (int64_t)r0 * D + c)) : make_uint4(0, 0, 0, 0);
-        qb[m] = (r1 < T) ? __ldg(reinterpret_cast<const uint4*>(Qh + (int64_t)r1 * D + c)) : make_uint4(0, 0, 0, 0);
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&s_tmem)), "r"(CAL_TMEM) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    const float tau0 = (r0 < T) ? tauh[r0] : 0.f, tau1 = (r1 < T) ? tauh[r1] : 0.f;
-    // t counts from 1: row index r is decoding step t = r + 1
-    const unsigned long long w0 = (((1ull << CAL_WSHIFT) + (unsigned)(r0 + 1) / 2) / (unsigned)(r0 + 1));
-    const unsigned long long w1 = (((1ull << CAL_WSHIFT) + (unsigned)(r1 + 1) / 2) / (unsigned)(r1 + 1));
-    const uint32_t wl[2] = {(uint32_t)w0 & ((1u << CAL_SPLIT) - 1), (uint32_t)w1 & ((1u << CAL_SPLIT) - 1)};
-    const uint32_t wh[2] = {(uint32_t)(w0 >> CAL_SPLIT), (uint32_t)(w1 >> CAL_SPLIT)};
-    const uint64_t one2 = pack2(1.f, 1.f);
-    // Sums of the two rows' gates (even and odd keys apart) as value + error: Dekker's sum, exact because the value starts
-    // at 1 and never falls below a gate.  Twice fp32's precision on the fp32 pipe; a conversion to double and a double add
-    // per gate would take four times as long.
-    uint64_t gs[2] = {one2, one2}, ge[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
-    const float b_max = (float)n_bins - 0.5f;
-    const uint32_t lo_addr = smem_u32(lo) - (0x4B000000u << 2), hi_off = (uint32_t)n_bins * 4;
-
-    auto add = [&](float y, int row) {
-        // floor(y) sits in the low bits of 2^23 + y rounded down; the exponent bits are folded into lo_addr
-        const float f = __fadd_rd(fminf(fmaxf(y, 0.f), b_max), 8388608.f);
-        const uint32_t addr = lo_addr + (__float_as_uint(f) << 2);
-        red_shared(addr, wl[row]);
-        red_shared(addr + hi_off, wh[row]);
-    };
-    auto tile = [&](int s0, int buf, auto masked) {
-        constexpr bool MASK = decltype(masked)::value;
-        // two 8-key MMA tiles at a time: independent chains for the tensor cores and the arithmetic behind them
-#pragma unroll 1
-        for (int nn = 0; nn < CAL_KEYS / 8; nn += 2) {
-            float acc[2][4];
-            const __nv_bfloat16* krow = sK + (buf * CAL_KEYS + nn * 8 + g) * KS + 8 * tq;
+    for (int b = tid; b < 2 * n_bins; b += CAL_THREADS) lo[b] = 0u;
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
+    const uint32_t tmem = s_tmem, tmem_acc = tmem + CAL_TMEM - CAL_KEYS;
+    double dsum = 0.0;
+    bool ok = true;
+    if (warp < CAL_ROWS / 32) {             // the queries into tensor memory, a row per lane
+        ok = __all_sync(0xffffffffu, mbar_wait(&bar_q, 0));
+        const int row = warp * 32 + lane;
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+        for (int c = 0; c < D / 32; ++c) {
+            uint4 q[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[u][c] = 0.f;
-#pragma unroll
-            for (int m = 0; m < NP; ++m) {
-                const uint4 k0 = *reinterpret_cast<const uint4*>(krow + 32 * m);
-                const uint4 k1 = *reinterpret_cast<const uint4*>(krow + 8 * KS + 32 * m);
-                mma_bf16_16816(acc[0], qa[m].x, qb[m].x, qa[m].y, qb[m].y, k0.x, k0.y);
-                mma_bf16_16816(acc[1], qa[m].x, qb[m].x, qa[m].y, qb[m].y, k1.x, k1.y);
-                mma_bf16_16816(acc[0], qa[m].z, qb[m].z, qa[m].w, qb[m].w, k0.z, k0.w);
-                mma_bf16_16816(acc[1], qa[m].z, qb[m].z, qa[m].w, qb[m].w, k1.z, k1.w);
-            }
-            // acc[u][0], acc[u][1]: row r0, keys col, col + 1; acc[u][2], acc[u][3]: row r1
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int col = s0 + (nn + u) * 8 + 2 * tq;
-#pragma unroll
-                for (int row = 0; row < 2; ++row) {
-                    const int r = row ? r1 : r0;
-                    const float tr = row ? tau1 : tau0;
-                    const uint64_t S = mul2(pack2(acc[u][2 * row], acc[u][2 * row + 1]), pack2(scale, scale));
-                    // the gate 1 / (1 + 2^y), y = -beta log2(e) (S - tau)
-                    const float2 y = unpack2(mul2(sub2p(S, pack2(tr, tr)), pack2(c2, c2)));
-                    float ma = rcp_approx1(1.f + ex2_approx(y.x)), mb = rcp_approx1(1.f + ex2_approx(y.y));
-                    if (MASK) { ma = (r < T && col <= r) ? ma : 0.f; mb = (r < T && col + 1 <= r) ? mb : 0.f; }
-                    const uint64_t m = pack2(ma, mb), sum = add2p(gs[row], m);
-                    ge[row] = add2p(ge[row], sub2p(m, sub2p(sum, gs[row])));
-                    gs[row] = sum;
-                    const float2 bin = unpack2(mul2(sub2p(S, pack2(s_min, s_min)), pack2(inv_w, inv_w)));
-                    if (!MASK || (r < T && col <= r)) add(bin.x, row);
-                    if (!MASK || (r < T && col + 1 <= r)) add(bin.y, row);
-                }
-            }
+            for (int u = 0; u < 4; ++u)
+                q[u] = *reinterpret_cast<const uint4*>(sK + (c / 2) * (CAL_ROWS * 128) + row * 128 + ((((c & 1) * 4 + u) ^ (row & 7)) << 4));
+            tmem_store16(tmem + ((uint32_t)(warp * 32) << 16) + 16 * c, q);
         }
-    };
+        fence_proxy_async();
+        tmem_fence_before();
+    }
+    __syncthreads();
+    tmem_fence_after();
+
+    // by threads that count only, all of them
     auto flush = [&]() {
-        for (int b = tid; b < n_bins; b += CAL_THREADS) {
+        for (int b = tid; b < n_bins; b += 32 * CAL_WARPS) {
             const unsigned long long v = ((unsigned long long)hi[b] << CAL_SPLIT) + lo[b];
             if (v) {
                 atomicAdd(&hist[(int64_t)h * n_bins + b], v);
@@ -201,35 +196,121 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
             }
         }
     };
-    for (int s0 = 0, buf = 0; s0 < s_end; s0 += CAL_KEYS, buf ^= 1) {
-        // one barrier per tile: every thread's copies of this tile have landed, every warp is through with the one before,
-        // whose buffer the next tile's copies may have
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        if (s0 && s0 % CAL_FLUSH == 0) { flush(); __syncthreads(); }
-        if (s0 + CAL_KEYS < s_end) fetch(s0 + CAL_KEYS, buf ^ 1);
-        // a warp whose rows all lie past the tile counts every score; one whose rows end before it none
-        if (s0 + CAL_KEYS - 1 <= rw && rw + 16 <= T) tile(s0, buf, std::false_type{});
-        else if (s0 <= rw + 15 && rw < T) tile(s0, buf, std::true_type{});
-    }
-    __syncthreads();
-    // density contribution of this tile: sum over its rows of (1/t) * (sum of the row's gates), fixed order
-    double dsum = 0.0;
+    auto meet = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(32 * CAL_WARPS) : "memory"); };
+
+    if (warp == CAL_WARPS) {
+        if (lane == 0) {
+            const int hk = x * Hkv + h / (Hq / Hkv);
+            auto load = [&](int i) {
+                mbar_arrive_expect_tx(&bar_in[i & 1], L::K_BYTES);
+                tma_load_4d(sK + (i & 1) * L::K_BYTES, &tmK, 0, i * CAL_KEYS, 0, hk, &bar_in[i & 1]);
+            };
+            load(0);
+            for (int i = 0; i < n_tiles; ++i) {
+                // a wait that runs out: nothing more is issued; what is still on its way gets as long again
+                if (!mbar_wait(&bar_in[i & 1], (i >> 1) & 1)) { mbar_wait(&bar_in[i & 1], (i >> 1) & 1); break; }
+                if (i > 0 && !mbar_wait(&bar_free, (i - 1) & 1)) break;
+                if (i + 1 < n_tiles) load(i + 1);          // the scores of the tile before are complete: its keys have been read
+                tmem_fence_after();
+                const uint32_t keys = smem_u32(sK) + (i & 1) * L::K_BYTES;
 #pragma unroll
-    for (int row = 0; row < 2; ++row) {
-        const float2 v = unpack2(gs[row]), e = unpack2(ge[row]);
-        const int r = row ? r1 : r0;
-        if (r < T) dsum += (((double)v.x - 1.0) + ((double)v.y - 1.0) + ((double)e.x + (double)e.y)) / (double)(r + 1);
-    }
+                for (int k = 0; k < D / 16; ++k)       // 16 columns: 32 bytes along the swizzled row of a 64-column half
+                    umma_bf16(tmem_acc, tmem + 8 * k, umma_operand(keys + (k / 4) * (CAL_KEYS * 128) + (k % 4) * 32),
+                              CAL_IDESC, k > 0);
+                umma_commit(&bar_acc);
+            }
+        }
+        __syncwarp();
+    } else {
+        const int l16 = (warp & 3) * 32 + (warp >> 2) * 16;      // the warp's 16 lanes of tensor memory
+        const int rw = t0 + l16, r0 = rw + (lane >> 2), r1 = r0 + 8;
+        const float* tauh = tau + ((int64_t)x * Hq + h) * T;
+        const float tau0 = (r0 < T) ? tauh[r0] : 0.f, tau1 = (r1 < T) ? tauh[r1] : 0.f;
+        // t counts from 1: row index r is decoding step t = r + 1
+        const unsigned long long w0 = (((1ull << CAL_WSHIFT) + (unsigned)(r0 + 1) / 2) / (unsigned)(r0 + 1));
+        const unsigned long long w1 = (((1ull << CAL_WSHIFT) + (unsigned)(r1 + 1) / 2) / (unsigned)(r1 + 1));
+        const uint32_t wl[2] = {(uint32_t)w0 & ((1u << CAL_SPLIT) - 1), (uint32_t)w1 & ((1u << CAL_SPLIT) - 1)};
+        const uint32_t wh[2] = {(uint32_t)(w0 >> CAL_SPLIT), (uint32_t)(w1 >> CAL_SPLIT)};
+        // Sums of the two rows' gates (even and odd keys apart) as value + error: Dekker's sum, exact because the value
+        // starts at 1 and never falls below a gate.  Twice fp32's precision on the fp32 pipe; a conversion to double and a
+        // double add per gate would take four times as long.
+        const uint64_t one2 = pack2(1.f, 1.f);
+        uint64_t gs[2] = {one2, one2}, ge[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+        const float b_max = (float)n_bins - 0.5f;
+        const uint32_t lo_addr = smem_u32(lo) - (0x4B000000u << 2), hi_off = (uint32_t)n_bins * 4;
+
+        auto add = [&](float y, int row) {
+            // floor(y) sits in the low bits of 2^23 + y rounded down; the exponent bits are folded into lo_addr
+            const float f = __fadd_rd(fminf(fmaxf(y, 0.f), b_max), 8388608.f);
+            const uint32_t addr = lo_addr + (__float_as_uint(f) << 2);
+            red_shared(addr, wl[row]);
+            red_shared(addr + hi_off, wh[row]);
+        };
+        auto count = [&](const float (&acc)[16], int key, auto masked) {
+            constexpr bool MASK = decltype(masked)::value;
 #pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, s);
-    if (lane == 0) s_red[warp] = dsum;
-    flush();
+            for (int u = 0; u < 8; ++u) {
+                const int row = u & 1, r = row ? r1 : r0, col = key + (u / 2) * 8 + 2 * (lane & 3);
+                const float tr = row ? tau1 : tau0;
+                const uint64_t S = mul2(pack2(acc[2 * u], acc[2 * u + 1]), pack2(scale, scale));
+                // the gate 1 / (1 + 2^y), y = -beta log2(e) (S - tau)
+                const float2 y = unpack2(mul2(sub2p(S, pack2(tr, tr)), pack2(c2, c2)));
+                float ma = rcp_approx1(1.f + ex2_approx(y.x)), mb = rcp_approx1(1.f + ex2_approx(y.y));
+                const bool in_a = !MASK || (r < T && col <= r), in_b = !MASK || (r < T && col + 1 <= r);
+                if (MASK) { ma = in_a ? ma : 0.f; mb = in_b ? mb : 0.f; }
+                const uint64_t m = pack2(ma, mb), sum = add2p(gs[row], m);
+                ge[row] = add2p(ge[row], sub2p(m, sub2p(sum, gs[row])));
+                gs[row] = sum;
+                const float2 bin = unpack2(mul2(sub2p(S, pack2(s_min, s_min)), pack2(inv_w, inv_w)));
+                if (in_a) add(bin.x, row);
+                if (in_b) add(bin.y, row);
+            }
+        };
+        for (int i = 0; i < n_tiles; ++i) {
+            if (i && i * CAL_KEYS % CAL_FLUSH == 0) { meet(); flush(); meet(); }
+            ok = ok && mbar_wait(&bar_acc, i & 1);
+            ok = __all_sync(0xffffffffu, ok);
+            tmem_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < CAL_KEYS; c += 32) {
+                const int key = i * CAL_KEYS + c;
+                const bool some = ok && key <= rw + 15 && rw < T;          // a warp whose rows end before the keys counts none
+                float acc[16];
+                if (some) tmem_load_16x32(tmem_acc + ((uint32_t)l16 << 16) + c, acc);
+                if (c + 32 == CAL_KEYS) {          // the next tile's MMA runs while these are counted
+                    tmem_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar_free);
+                }
+                if (!some) continue;
+                if (key + 31 <= rw && rw + 16 <= T) count(acc, key, std::false_type{});      // ... all past them: every score
+                else count(acc, key, std::true_type{});
+            }
+        }
+        meet();
+        flush();
+        // density contribution of this tile: sum over its rows of (1/t) * (sum of the row's gates), fixed order
+#pragma unroll
+        for (int row = 0; row < 2; ++row) {
+            const float2 v = unpack2(gs[row]), e = unpack2(ge[row]);
+            const int r = row ? r1 : r0;
+            if (r < T) dsum += (((double)v.x - 1.0) + ((double)v.y - 1.0) + ((double)e.x + (double)e.y)) / (double)(r + 1);
+        }
+        if (!ok) dsum = __longlong_as_double(0x7ff8000000000000ll);       // a wait ran out: the density becomes NaN
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, s);
+        if (lane == 0) s_red[warp] = dsum;
+    }
+    tmem_fence_before();
     __syncthreads();
+    if (warp == CAL_WARPS) {
+        tmem_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(CAL_TMEM) : "memory");
+    }
     if (tid == 0) {
         double tot = 0.0;
-        for (int w = 0; w < CAL_THREADS / 32; ++w) tot += s_red[w];
-        dpart[((int64_t)x * Hq + h) * gridDim.x + ttile] = tot;
+        for (int w = 0; w < CAL_WARPS; ++w) tot += s_red[w];
+        dpart[((int64_t)x * Hq + h) * gridDim.z + ttile] = tot;
     }
 }
 
@@ -322,6 +403,26 @@ __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
     }
 }
 
+// [heads][T][D] bf16, dense: boxes of `rows` tokens, a 64-column half after the other in shared memory
+static int cal_tmap(CUtensorMap* tm, const void* base, int64_t heads, int T, int D, int rows) {
+    const cuuint64_t dims[4] = {64, (cuuint64_t)T, (cuuint64_t)(D / 64), (cuuint64_t)heads};
+    const cuuint64_t strides[3] = {(cuuint64_t)D * 2, 128, (cuuint64_t)T * D * 2};
+    const cuuint32_t box[4] = {64, (cuuint32_t)rows, (cuuint32_t)(D / 64), 1};
+    return encode_tiles(tm, base, 4, dims, strides, box);
+}
+
+template <int D>
+static int launch_hist(const CUtensorMap& tmQ, const CUtensorMap& tmK, const float* tau, int Hq, int Hkv, int T, int n_seq,
+                       float c2, float scale, int n_bins, float s_min, float inv_w, unsigned long long* hist, double* dpart,
+                       cudaStream_t s) {
+    const int rc = configure_kernel(reinterpret_cast<const void*>(calib_hist_kernel<D>), CalSmem<D>::bytes(4096));
+    if (rc != ETA_OK) return rc;
+    const dim3 grid((unsigned)Hq, (unsigned)n_seq, (unsigned)((T + CAL_ROWS - 1) / CAL_ROWS));
+    calib_hist_kernel<D><<<grid, CAL_THREADS, CalSmem<D>::bytes(n_bins), s>>>(tmQ, tmK, tau, Hq, Hkv, T, c2, scale, n_bins,
+                                                                               s_min, inv_w, hist, dpart);
+    return check_launch("calibration histogram");
+}
+
 static size_t cal_align(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace eta
@@ -368,23 +469,13 @@ int eta_calibrate_head_const(int32_t n_seq, int32_t seq_len, int32_t n_q_heads, 
 
     const float sc = scale > 0.f ? scale : 1.0f / sqrtf((float)head_dim);
     const float inv_w = (float)n_bins / (s_max - s_min);
-    const dim3 grid((unsigned)n_ttiles, (unsigned)n_q_heads, (unsigned)n_seq);
     const float c2 = (float)(-(double)beta * 1.4426950408889634);      // exp(-beta x) = 2^(c2 x)
-    const size_t smem = (size_t)2 * CAL_KEYS * (head_dim + 32) * 2 + sizeof(unsigned long long) * (size_t)n_bins;
-    auto Qp = static_cast<const __nv_bfloat16*>(Q);
-    auto Kp = static_cast<const __nv_bfloat16*>(K);
-    if (head_dim == 128) {
-        rc = configure_kernel(reinterpret_cast<const void*>(calib_hist_kernel<128>), 80 * 1024);
-        if (rc != ETA_OK) return rc;
-        calib_hist_kernel<128><<<grid, CAL_THREADS, smem, s>>>(Qp, Kp, tau, n_q_heads, n_kv_heads, seq_len, c2, sc,
-                                                               n_bins, s_min, inv_w, hist, dpart);
-    } else {
-        rc = configure_kernel(reinterpret_cast<const void*>(calib_hist_kernel<64>), 80 * 1024);
-        if (rc != ETA_OK) return rc;
-        calib_hist_kernel<64><<<grid, CAL_THREADS, smem, s>>>(Qp, Kp, tau, n_q_heads, n_kv_heads, seq_len, c2, sc,
-                                                              n_bins, s_min, inv_w, hist, dpart);
-    }
-    rc = check_launch("calibration histogram");
+    CUtensorMap tmQ, tmK;
+    rc = cal_tmap(&tmQ, Q, (int64_t)n_seq * n_q_heads, seq_len, head_dim, CAL_ROWS);
+    if (rc == ETA_OK) rc = cal_tmap(&tmK, K, (int64_t)n_seq * n_kv_heads, seq_len, head_dim, CAL_KEYS);
+    if (rc != ETA_OK) return rc;
+    rc = (head_dim == 128 ? launch_hist<128> : launch_hist<64>)(tmQ, tmK, tau, n_q_heads, n_kv_heads, seq_len, n_seq, c2, sc,
+                                                               n_bins, s_min, inv_w, hist, dpart, s);
     if (rc != ETA_OK) return rc;
     calib_bisect_kernel<<<n_q_heads, CAL_BISECT_THREADS, sizeof(double) * (size_t)n_bins, s>>>(
         hist, dpart, n_q_heads, n_seq, n_ttiles, seq_len, n_bins, (double)s_min, (double)s_max, (double)beta, 160,

@@ -107,6 +107,8 @@ struct ScreenArgs {
     uint32_t* status;
     unsigned long long* timeline;
 };
+int encode_tiles(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                 const cuuint32_t* box);
 int launch_screen(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int G, int n_sm, cudaStream_t s);
 
 // Launch with programmatic dependent launch allowed: the grid may start while its predecessor in the stream is

@@ -1036,28 +1036,34 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
+// Tensor map of bf16 boxes in the 128-byte swizzle; what lies outside the tensor reads as zero
+int encode_tiles(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                 const cuuint32_t* box) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return ETA_ERR_CUDA;
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult rc = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box,
+                           estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (rc != CUDA_SUCCESS) {
+        set_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
+        return ETA_ERR_CUDA;
+    }
+    return ETA_OK;
+}
+
 // K or V as a 5-D tensor (c within a 64-column half, t, half, hk, i) of bf16; a box is 64 columns x TS tokens x
 // all halves: in shared memory, one 128-byte-swizzled [TS][64] tile per half, back to back.
 // Tensor map of a K or V cache: 64 columns x tokens x column halves x KV heads x sequences, or, for a paged cache
 // (n_pages > 0), ... x tokens of a page x ... x pages, with sb the stride between pages.
 static int make_tmap(CUtensorMap* tm, const void* base, const eta_cache_desc* d, int64_t sb, int64_t sh, int64_t st,
                      int TS, int n_pages) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return ETA_ERR_CUDA;
     const cuuint32_t halves = (cuuint32_t)(d->head_dim / 64);
     cuuint64_t dims[5] = {64, (cuuint64_t)(n_pages > 0 ? d->block_size : d->t_cap), halves, (cuuint64_t)d->n_kv_heads,
                           (cuuint64_t)(n_pages > 0 ? n_pages : d->batch)};
     cuuint64_t strides[4] = {(cuuint64_t)st * 2, 128, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
     cuuint32_t box[5] = {64, (cuuint32_t)TS, halves, 1, 1};
-    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    CUresult rc = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (rc != CUDA_SUCCESS) {
-        set_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
-        return ETA_ERR_CUDA;
-    }
-    return ETA_OK;
+    return encode_tiles(tm, base, 5, dims, strides, box);
 }
 
 template <int D, int TS, int NSTAGE, int NGROUPS>

@@ -117,3 +117,24 @@ def test_calibration_with_few_bins_and_ragged_tiles(T, d, n_bins, lim):
     np.testing.assert_allclose(dbar.cpu().numpy(), ref["dbar"], rtol=0, atol=1e-6)
     for h in range(2):
         assert abs(orc.calibration_density(ref["hist"][h], -lim, lim, 5.0, float(hc[h])) - ref["dbar"][h]) <= 5e-6
+
+
+@pytest.mark.parametrize("T,d", [(32, 128), (127, 64), (128, 128), (129, 128), (192, 64), (577, 128)])
+def test_calibration_at_tile_edges(T, d):
+    """Sequences that end at, just before and just past a tile of queries (128) or keys (64) and, with 577, in the tile after
+    the planes were emptied; two sequences and shared key heads, so that every index of a tile counts.  Bounds as above."""
+    eb = _eb()
+    dev = torch.device("cuda:0")
+    n_bins, lim = 65, 7.0
+    Q, K, tau = _split(900 + T, 2, 4, 2, T, d, qscale=1.5)
+    ref = orc.calibrate(bits(Q), bits(K), tau.numpy(), beta=5.0, n_bins=n_bins, s_min=-lim, s_max=lim)
+    hc, dbar = torch.empty(4, device=dev), torch.empty(4, device=dev)
+    ws = eb.eta_calibrate_head_const(Q.to(dev), K.to(dev), tau.to(dev), hc, dbar, beta=5.0, n_bins=n_bins, s_min=-lim, s_max=lim)
+    torch.cuda.synchronize()
+    H = ws[:4 * n_bins * 8].view(torch.int64).cpu().numpy().reshape(4, n_bins)
+    assert [int(h.sum()) for h in H] == [2 * sum(t * ((2 ** 40 + t // 2) // t) for t in range(1, T + 1))] * 4
+    Hn = H / H.sum(axis=1, keepdims=True).astype(np.float64)
+    assert np.abs(Hn - ref["hist"]).sum(axis=1).max() <= (n_bins - 1) * (8 * 2e-6 * 0.4 / 1.5) + 4.0 / T / T
+    np.testing.assert_allclose(dbar.cpu().numpy(), ref["dbar"], rtol=0, atol=1e-6)
+    for h in range(4):
+        assert abs(orc.calibration_density(ref["hist"][h], -lim, lim, 5.0, float(hc[h])) - ref["dbar"][h]) <= 5e-6
