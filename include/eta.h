@@ -129,7 +129,8 @@ int eta_build_block_summaries(const eta_cache_desc* desc, const void* K, const i
  * for every sequence whose new length is a positive multiple of b, the block
  * that just became full (index seq_lens[i]/b - 1) is summarised exactly as
  * eta_build_block_summaries would; other sequences are untouched.  Stateless and
- * idempotent.
+ * idempotent.  Launched with programmatic dependent launch: the kernel waits for everything
+ * before it in the stream before it reads, and releases its successors only then.
  */
 int eta_append_summary(const eta_cache_desc* desc, const void* K, const int32_t* seq_lens_after,
                        void* musig, float* mnorm, uint32_t flags, void* stream);

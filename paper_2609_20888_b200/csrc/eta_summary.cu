@@ -317,6 +317,10 @@ __global__ void __launch_bounds__(128) append_summary_kernel(
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned long long* const tl = ETA_TL((timeline && r < TL_APPEND_N) ? timeline + (size_t)(TL_APPEND + r) * 8 : nullptr);
     if (tl && tid == 0) tl[0] = globaltimer_ns();
+    // The first kernel of a step: it may be on the SMs while the step before it ends, but reads, and lets its own successors
+    // start, only once all before it is complete, since those read the step's inputs without waiting again.  Steps called one
+    // after the other take 1.4 us less than with an ordinary launch (2K x 1 19.0 -> 17.6, 16K x 1 24.7 -> 23.2).
+    pdl_wait();
     pdl_trigger();       // nothing later in a decode step needs this kernel's output before it has waited for it
     const int i = r / Hkv, hk = r % Hkv;
     const int T = seq_lens[i];
@@ -447,19 +451,12 @@ static int append_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     const int env = ((flags & ETA_BUILD_SIGMA_ENVELOPE) ? 1 : 0) | ((flags & ETA_BUILD_PACKED_SIGMA) ? 2 : 0);
     auto Kp = static_cast<const __nv_bfloat16*>(K);
     auto mp = static_cast<unsigned char*>(musig);
-    rc = eta::configure_kernel(desc->head_dim == 128 ? reinterpret_cast<const void*>(eta::append_summary_kernel<128>)
-                                                     : reinterpret_cast<const void*>(eta::append_summary_kernel<64>), 0);
-    if (rc != ETA_OK) return rc;
     eta::profile_mark(0, s);
-    if (desc->head_dim == 128)
-        eta::append_summary_kernel<128><<<grid, 128, 0, s>>>(Kp, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t,
-            desc->n_kv_heads, desc->block_size, desc->t_cap, desc->nb_cap, rows, seq_lens_after, env, mp, mnorm,
-            table, tstride, eta::debug_timeline());
-    else
-        eta::append_summary_kernel<64><<<grid, 128, 0, s>>>(Kp, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t,
-            desc->n_kv_heads, desc->block_size, desc->t_cap, desc->nb_cap, rows, seq_lens_after, env, mp, mnorm,
-            table, tstride, eta::debug_timeline());
-    return eta::check_launch("eta_append_summary");
+    return eta::launch_pdl("eta_append_summary",
+                           desc->head_dim == 128 ? eta::append_summary_kernel<128> : eta::append_summary_kernel<64>, dim3(grid),
+                           dim3(128), 0, s, Kp, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t, desc->n_kv_heads,
+                           desc->block_size, desc->t_cap, desc->nb_cap, rows, seq_lens_after, env, mp, mnorm, table, tstride,
+                           eta::debug_timeline());
 }
 
 }  // namespace eta
