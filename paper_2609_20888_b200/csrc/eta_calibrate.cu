@@ -128,7 +128,7 @@ struct CalSmem {
 // tensor memory, and the queries sit there too (as an operand in shared memory they were read again for every tile: 14
 // million passes, 4.7 are left).  One accumulator of 64 keys: the MMA of a tile runs while the second half of the tile before
 // it is counted.  Two of 32 keys with a barrier each (347 us a calibration, against 313) cost more than they hide, two of 64
-// do not fit the tensor memory of three CTAs beside the queries.  With 2048 bins: 515 -> 333 (queries in shared memory) ->
+// do not fit the tensor memory of three CTAs beside the queries.  Four CTAs at 56 registers: 321.  With 2048 bins: 515 -> 333 (queries in shared memory) ->
 // 313 us, of which the histogram 435 -> 290.
 template <int D>
 __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
