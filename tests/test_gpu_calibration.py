@@ -138,3 +138,22 @@ def test_calibration_at_tile_edges(T, d):
     np.testing.assert_allclose(dbar.cpu().numpy(), ref["dbar"], rtol=0, atol=1e-6)
     for h in range(4):
         assert abs(orc.calibration_density(ref["hist"][h], -lim, lim, 5.0, float(hc[h])) - ref["dbar"][h]) <= 5e-6
+
+
+@pytest.mark.parametrize("beta,lim", [(5.0, 8.0), (50.0, 8.0), (5.0, 0.5)])
+def test_saturated_densities_give_the_end_of_the_bracket(beta, lim):
+    """A threshold below (above) every score gives a density of exactly 1 (0), which every constant far enough below (above)
+    the scores has too: the halving's answer is the end of its bracket, [s_min - 40 / beta, s_max + 40 / beta].  Two tokens: the
+    sums of their gates, 1 / 1 and 2 / 2, are exact on both sides."""
+    eb = _eb()
+    dev = torch.device("cuda:0")
+    Q, K, tau = _split(31, 8, 4, 2, 2, 64)
+    tau[:, 0], tau[:, 1], tau[:, 2] = float("-inf"), -40.0, float("inf")
+    ref = orc.calibrate(bits(Q), bits(K), tau.numpy(), beta=beta, n_bins=512, s_min=-lim, s_max=lim)
+    assert list(ref["dbar"][:3]) == [1.0, 1.0, 0.0]
+    hc = torch.full((4,), float("nan"), device=dev)
+    eb.eta_calibrate_head_const(Q.to(dev), K.to(dev), tau.to(dev), hc, None, beta=beta, n_bins=512, s_min=-lim, s_max=lim)
+    torch.cuda.synchronize()
+    end = lim + 40.0 / beta
+    np.testing.assert_allclose(ref["head_const"][:3], [-end, -end, end], rtol=1e-12)
+    np.testing.assert_allclose(hc.cpu().numpy()[:3], [-end, -end, end], rtol=2.0 ** -23)
