@@ -195,6 +195,8 @@ int eta_score_dual(const eta_cache_desc* desc, const eta_params* params, const v
  * device pointers.  Scores are computed in fp32 from the bf16 operands; the row
  * weights are accumulated as integers, so the result does not depend on the
  * order of the atomic updates.  head_dim 64 or 128; n_seq * seq_len <= 2^22.
+ * A head whose density is NaN (a NaN threshold, or a bounded wait inside the kernel that
+ * ran out) gets NaN for its constant as well.
  * workspace: eta_calibration_workspace_bytes() bytes, 256-byte aligned, no
  * initialisation needed.  Prefill-side tool: not part of a decode step.
  */

@@ -374,7 +374,11 @@ __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
     const double w = (s_max - s_min) / n_bins;
     double lo = s_min - 40.0 / beta, hi = s_max + 40.0 / beta;
     double c = 0.5 * (lo + hi), dx_old = hi - lo, dx = dx_old;
-    for (int it = 0; it < iters; ++it) {
+    // A NaN density (a NaN among the thresholds or scores, or a wait of the histogram kernel that ran out) has no root: the
+    // constant is NaN too, since the density is an optional output.
+    const bool bad = target != target;
+    if (bad) c = target;
+    for (int it = 0; it < iters && !bad; ++it) {
         double gs = 0.0, ds = 0.0;
         for (int b = tid; b < n_bins; b += CAL_BISECT_THREADS) {
             const double hb = Hn[b];

@@ -157,3 +157,17 @@ def test_saturated_densities_give_the_end_of_the_bracket(beta, lim):
     end = lim + 40.0 / beta
     np.testing.assert_allclose(ref["head_const"][:3], [-end, -end, end], rtol=1e-12)
     np.testing.assert_allclose(hc.cpu().numpy()[:3], [-end, -end, end], rtol=2.0 ** -23)
+
+
+def test_a_nan_density_gives_a_nan_constant():
+    """The density is an optional output: a head without one must not get a constant that looks like any other."""
+    eb = _eb()
+    dev = torch.device("cuda:0")
+    Q, K, tau = _split(8, 2, 4, 2, 200, 64)
+    hc, hc_nan = torch.empty(4, device=dev), torch.empty(4, device=dev)
+    eb.eta_calibrate_head_const(Q.to(dev), K.to(dev), tau.to(dev), hc)
+    tau[1, 2, 150] = float("nan")
+    eb.eta_calibrate_head_const(Q.to(dev), K.to(dev), tau.to(dev), hc_nan)
+    torch.cuda.synchronize()
+    assert torch.isnan(hc_nan).tolist() == [False, False, True, False]
+    assert torch.equal(hc_nan[[0, 1, 3]], hc[[0, 1, 3]])
