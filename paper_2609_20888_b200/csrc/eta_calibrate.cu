@@ -206,6 +206,7 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
                 tma_load_4d(sK + (i & 1) * L::K_BYTES, &tmK, 0, i * CAL_KEYS, 0, hk, &bar_in[i & 1]);
             };
             load(0);
+            int issued = 0;                                // tiles whose MMAs are under way or complete
             for (int i = 0; i < n_tiles; ++i) {
                 // a wait that runs out: nothing more is issued; what is still on its way gets as long again
                 if (!mbar_wait(&bar_in[i & 1], (i >> 1) & 1)) { mbar_wait(&bar_in[i & 1], (i >> 1) & 1); break; }
@@ -218,7 +219,11 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
                     umma_bf16(tmem_acc, tmem + 8 * k, umma_operand(keys + (k / 4) * (CAL_KEYS * 128) + (k % 4) * 32),
                               CAL_IDESC, k > 0);
                 umma_commit(&bar_acc);
+                ++issued;
             }
+            // the counting warps have waited for the last tile already, unless their wait ran out: the MMAs get as long again
+            // before the tensor memory is given back
+            if (issued) mbar_wait(&bar_acc, (issued - 1) & 1);
         }
         __syncwarp();
     } else {
