@@ -214,7 +214,7 @@ def eta_build_block_summaries(desc, K, seq_lens, musig, mnorm, flags: int = 0) -
 
 def eta_append_summary(desc, K, seq_lens_after, musig, mnorm, flags: int = 0) -> None:
     lib = _lib or load()
-    rc = _native.append(lib.addresses["eta_append_summary"], desc, None, K, seq_lens_after, musig, mnorm, flags)
+    rc = _native.append(lib.addresses["eta_append_summary"], desc, K, seq_lens_after, musig, mnorm, flags)
     if rc:
         _check(rc, "eta_append_summary")
 
@@ -229,7 +229,7 @@ def eta_build_block_summaries_paged(desc, pages: PageTable, K_pool, seq_lens, mu
 
 def eta_append_summary_paged(desc, pages: PageTable, K_pool, seq_lens_after, musig, mnorm, flags: int = 0) -> None:
     lib = _lib or load()
-    rc = _native.append(lib.addresses["eta_append_summary_paged"], desc, pages, K_pool, seq_lens_after, musig, mnorm, flags)
+    rc = _native.append_paged(lib.addresses["eta_append_summary_paged"], desc, pages, K_pool, seq_lens_after, musig, mnorm, flags)
     if rc:
         _check(rc, "eta_append_summary_paged")
 
@@ -285,7 +285,7 @@ def eta_calibrate_head_const(Q, K, tau, head_const, dbar=None, beta=5.0, scale=0
 def eta_decode(desc, params: DecodeParams, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask,
                workspace, stats=None, status=None, lib=None) -> None:
     lib = lib or _lib or load()
-    rc = _native.decode(lib.addresses["eta_decode"], desc, None, params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out,
+    rc = _native.decode(lib.addresses["eta_decode"], desc, params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out,
                         sel_mask, stats, status, workspace)
     if rc:
         _check(rc, "eta_decode")
@@ -294,8 +294,8 @@ def eta_decode(desc, params: DecodeParams, q, K, V, seq_lens, musig, mnorm, tau,
 def eta_decode_paged(desc, pages: PageTable, params: DecodeParams, q, K_pool, V_pool, seq_lens, musig, mnorm, tau,
                      head_const, out, sel_mask, workspace, stats=None, status=None) -> None:
     lib = _lib or load()
-    rc = _native.decode(lib.addresses["eta_decode_paged"], desc, pages, params, q, K_pool, V_pool, seq_lens, musig, mnorm, tau,
-                        head_const, out, sel_mask, stats, status, workspace)
+    rc = _native.decode_paged(lib.addresses["eta_decode_paged"], desc, pages, params, q, K_pool, V_pool, seq_lens, musig, mnorm,
+                              tau, head_const, out, sel_mask, stats, status, workspace)
     if rc:
         _check(rc, "eta_decode_paged")
 
@@ -305,8 +305,8 @@ def eta_decode_static(desc, params: DecodeParams, q, K, V, seq_lens, musig, mnor
     """eta_decode without a workspace argument, for callers that have no device memory to give: the scratch is
     an 8 MiB array built into the library (see include/eta.h for its limit and sharing rules)."""
     lib = _lib or load()
-    rc = _native.decode(lib.addresses["eta_decode_static"], desc, None, params, q, K, V, seq_lens, musig, mnorm, tau, head_const,
-                        out, sel_mask, stats, status, False)
+    rc = _native.decode_static(lib.addresses["eta_decode_static"], desc, params, q, K, V, seq_lens, musig, mnorm, tau, head_const,
+                               out, sel_mask, stats, status)
     if rc:
         _check(rc, "eta_decode_static")
 

@@ -66,7 +66,6 @@ struct Struct {
     Py_buffer view = {};
     bool held = false;
     const T* get(PyObject* o) {
-        if (o == Py_None) return nullptr;
         if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return nullptr;
         held = true;
         if ((size_t)view.len != sizeof(T)) {
@@ -111,7 +110,8 @@ void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
 #define PTR(o, type, name) pointer(o, type, #name, (void**)&name)
 
-// (address, desc, pages | None, K, seq_lens, musig, mnorm, flags) -> return code
+// (address, desc, [pages,] K, seq_lens, musig, mnorm, flags) -> return code
+template <bool PAGED>
 PyObject* append(PyObject*, PyObject* const* v, Py_ssize_t n) {
     using Plain = int (*)(const eta_cache_desc*, const void*, const int32_t*, void*, float*, uint32_t, void*);
     using Paged = int (*)(const eta_cache_desc*, const eta_page_table*, const void*, const int32_t*, void*, float*, uint32_t, void*);
@@ -119,19 +119,21 @@ PyObject* append(PyObject*, PyObject* const* v, Py_ssize_t n) {
     Struct<eta_cache_desc> ds;
     Struct<eta_page_table> ps;
     void *K, *seq_lens, *musig, *mnorm;
-    if (!count(n, 8) || !entry(v[0], &fn)) return nullptr;
+    if (!count(n, PAGED ? 8 : 7) || !entry(v[0], &fn)) return nullptr;
     const eta_cache_desc* desc = ds.get(v[1]);
-    const eta_page_table* pages = ps.get(v[2]);
-    if (PyErr_Occurred()) return nullptr;
-    if (!PTR(v[3], at::kBFloat16, K) || !PTR(v[4], at::kInt, seq_lens) || !musig_pointer(v[5], &musig) || !PTR(v[6], at::kFloat, mnorm))
+    if (!desc) return nullptr;
+    const eta_page_table* pages = nullptr;
+    if (PAGED && !(pages = ps.get(v[2]))) return nullptr;
+    v += PAGED ? 3 : 2;
+    if (!PTR(v[0], at::kBFloat16, K) || !PTR(v[1], at::kInt, seq_lens) || !musig_pointer(v[2], &musig) || !PTR(v[3], at::kFloat, mnorm))
         return nullptr;
-    const uint32_t flags = (uint32_t)PyLong_AsUnsignedLongMask(v[7]);
+    const uint32_t flags = (uint32_t)PyLong_AsUnsignedLongMask(v[4]);
     if (PyErr_Occurred()) return nullptr;
     void* const s = stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = v[2] == Py_None ? reinterpret_cast<Plain>(fn)(desc, K, (const int32_t*)seq_lens, musig, (float*)mnorm, flags, s)
-                         : reinterpret_cast<Paged>(fn)(desc, pages, K, (const int32_t*)seq_lens, musig, (float*)mnorm, flags, s);
+    if (PAGED) rc = reinterpret_cast<Paged>(fn)(desc, pages, K, (const int32_t*)seq_lens, musig, (float*)mnorm, flags, s);
+    else rc = reinterpret_cast<Plain>(fn)(desc, K, (const int32_t*)seq_lens, musig, (float*)mnorm, flags, s);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
@@ -156,8 +158,10 @@ PyObject* predict(PyObject*, PyObject* const* v, Py_ssize_t n) {
     return PyLong_FromLong(rc);
 }
 
-// (address, desc, pages | None, params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask, stats, status,
-//  workspace | False: the variant without one) -> return code
+// (address, desc, [pages,] params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask, stats, status
+//  [, workspace]) -> return code
+enum class Decode { PLAIN, PAGED, STATIC };
+template <Decode KIND>
 PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
     using Plain = int (*)(const eta_cache_desc*, const eta_params*, const void*, const void*, const void*, const int32_t*, const void*,
                           const float*, const float*, const float*, float*, uint8_t*, int32_t*, uint32_t*, void*, size_t, void*);
@@ -166,31 +170,33 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
                           uint32_t*, void*, size_t, void*);
     using Static = int (*)(const eta_cache_desc*, const eta_params*, const void*, const void*, const void*, const int32_t*, const void*,
                            const float*, const float*, const float*, float*, uint8_t*, int32_t*, uint32_t*, void*);
+    constexpr bool PAGED = KIND == Decode::PAGED, WS = KIND != Decode::STATIC;
     void* fn;
     Struct<eta_cache_desc> ds;
     Struct<eta_page_table> ps;
     eta_params p;
-    void *q, *K, *V, *seq_lens, *musig, *mnorm, *tau, *head_const, *out, *sel_mask, *stats, *status, *workspace;
-    if (!count(n, 17) || !entry(v[0], &fn)) return nullptr;
+    void *q, *K, *V, *seq_lens, *musig, *mnorm, *tau, *head_const, *out, *sel_mask, *stats, *status, *workspace = nullptr;
+    if (!count(n, 15 + PAGED + WS) || !entry(v[0], &fn)) return nullptr;
     const eta_cache_desc* desc = ds.get(v[1]);
-    const eta_page_table* pages = ps.get(v[2]);
-    if (PyErr_Occurred() || !params_of(v[3], &p)) return nullptr;
-    if (!PTR(v[4], at::kBFloat16, q) || !PTR(v[5], at::kBFloat16, K) || !PTR(v[6], at::kBFloat16, V) || !PTR(v[7], at::kInt, seq_lens) ||
-        !musig_pointer(v[8], &musig) || !PTR(v[9], at::kFloat, mnorm) || !PTR(v[10], at::kFloat, tau) ||
-        !PTR(v[11], at::kFloat, head_const) || !pointer(v[12], at::kFloat, "out", &out, true) || !PTR(v[13], at::kByte, sel_mask) ||
-        !PTR(v[14], at::kInt, stats) || !PTR(v[15], at::kInt, status) ||
-        !pointer(v[16] == Py_False ? Py_None : v[16], at::kByte, "workspace", &workspace))
+    if (!desc) return nullptr;
+    const eta_page_table* pages = nullptr;
+    if (PAGED && !(pages = ps.get(v[2]))) return nullptr;
+    v += PAGED ? 3 : 2;
+    if (!params_of(v[0], &p)) return nullptr;
+    if (!PTR(v[1], at::kBFloat16, q) || !PTR(v[2], at::kBFloat16, K) || !PTR(v[3], at::kBFloat16, V) || !PTR(v[4], at::kInt, seq_lens) ||
+        !musig_pointer(v[5], &musig) || !PTR(v[6], at::kFloat, mnorm) || !PTR(v[7], at::kFloat, tau) ||
+        !PTR(v[8], at::kFloat, head_const) || !pointer(v[9], at::kFloat, "out", &out, true) || !PTR(v[10], at::kByte, sel_mask) ||
+        !PTR(v[11], at::kInt, stats) || !PTR(v[12], at::kInt, status) || (WS && !PTR(v[13], at::kByte, workspace)))
         return nullptr;
-    const bool has_ws = v[16] != Py_False, paged = v[2] != Py_None;
-    const size_t bytes = workspace ? (size_t)THPVariable_Unpack(v[16]).numel() : 0;
+    const size_t bytes = workspace ? (size_t)THPVariable_Unpack(v[13]).numel() : 0;
     void* const s = stream();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    if (paged)
+    if (KIND == Decode::PAGED)
         rc = reinterpret_cast<Paged>(fn)(desc, pages, &p, q, K, V, (const int32_t*)seq_lens, musig, (const float*)mnorm, (const float*)tau,
                                          (const float*)head_const, (float*)out, (uint8_t*)sel_mask, (int32_t*)stats,
                                          (uint32_t*)status, workspace, bytes, s);
-    else if (has_ws)
+    else if (KIND == Decode::PLAIN)
         rc = reinterpret_cast<Plain>(fn)(desc, &p, q, K, V, (const int32_t*)seq_lens, musig, (const float*)mnorm, (const float*)tau,
                                          (const float*)head_const, (float*)out, (uint8_t*)sel_mask, (int32_t*)stats,
                                          (uint32_t*)status, workspace, bytes, s);
@@ -221,9 +227,12 @@ PyObject* guarded(PyObject* self, PyObject* const* v, Py_ssize_t n) {
 }
 
 PyMethodDef methods[] = {
-    {"append", (PyCFunction)(void (*)(void))guarded<append>, METH_FASTCALL, nullptr},
+    {"append", (PyCFunction)(void (*)(void))guarded<append<false>>, METH_FASTCALL, nullptr},
+    {"append_paged", (PyCFunction)(void (*)(void))guarded<append<true>>, METH_FASTCALL, nullptr},
     {"predict", (PyCFunction)(void (*)(void))guarded<predict>, METH_FASTCALL, nullptr},
-    {"decode", (PyCFunction)(void (*)(void))guarded<decode>, METH_FASTCALL, nullptr},
+    {"decode", (PyCFunction)(void (*)(void))guarded<decode<Decode::PLAIN>>, METH_FASTCALL, nullptr},
+    {"decode_paged", (PyCFunction)(void (*)(void))guarded<decode<Decode::PAGED>>, METH_FASTCALL, nullptr},
+    {"decode_static", (PyCFunction)(void (*)(void))guarded<decode<Decode::STATIC>>, METH_FASTCALL, nullptr},
     {"set_error", set_error, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };

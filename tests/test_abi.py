@@ -121,3 +121,21 @@ def test_step_calls_check_their_tensors():
         eb.eta_decode(desc, eb.DecodeParams(), None, None, None, None, None, None, None, None, None, None, None)
     with pytest.raises(AttributeError):
         eb.eta_decode(desc, object(), None, None, None, None, None, None, None, None, None, None, None)
+
+
+def test_the_signature_of_a_step_call_does_not_hang_on_its_arguments():
+    """None for a page table, a descriptor or parameters, and False for a workspace, are refused; none of them selects another
+    signature for the same entry point."""
+    eb.load()
+    d, p, none = _desc(), eb.DecodeParams(), [None] * 10
+    for call in (lambda: eb.eta_append_summary_paged(d, None, None, None, None, None),
+                 lambda: eb.eta_decode_paged(d, None, p, *none, None),
+                 lambda: eb.eta_append_summary(None, None, None, None, None),
+                 lambda: eb.eta_decode(None, p, *none, None),
+                 lambda: eb.eta_decode_static(None, p, *none),
+                 lambda: eb.eta_decode(d, p, *none, False),
+                 lambda: eb.eta_decode_paged(d, eb.PageTable(), p, *none, False)):
+        with pytest.raises(TypeError):
+            call()
+    with pytest.raises(AttributeError):
+        eb.eta_decode(d, None, *none, None)
