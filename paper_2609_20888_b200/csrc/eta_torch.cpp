@@ -16,8 +16,9 @@
 
 namespace {
 
-PyObject* g_error = nullptr;          // EtaError
-
+// classes of the binding: the exception, the ctypes structures
+PyObject* g_error = nullptr;
+PyObject *g_desc = nullptr, *g_pages = nullptr;
 
 bool fail(const char* name, const char* what) {
     PyErr_Format(g_error, "%s must be %s", name, what);
@@ -60,12 +61,17 @@ bool pointer(PyObject* o, at::ScalarType type, const char* name, void** out, boo
 }
 bool musig_pointer(PyObject* o, void** out) { return pointer(o, at::kHalf, "musig", out, false, at::kByte); }
 
-// The bytes of a ctypes structure
+// The bytes of a ctypes structure of the binding's class `cls`
 template <typename T>
 struct Struct {
     Py_buffer view = {};
     bool held = false;
-    const T* get(PyObject* o) {
+    const T* get(PyObject* o, PyObject* cls) {
+        const int is = PyObject_IsInstance(o, cls);
+        if (is <= 0) {
+            if (is == 0) PyErr_Format(PyExc_TypeError, "%R expected, got %s", cls, Py_TYPE(o)->tp_name);
+            return nullptr;
+        }
         if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return nullptr;
         held = true;
         if ((size_t)view.len != sizeof(T)) {
@@ -120,10 +126,10 @@ PyObject* append(PyObject*, PyObject* const* v, Py_ssize_t n) {
     Struct<eta_page_table> ps;
     void *K, *seq_lens, *musig, *mnorm;
     if (!count(n, PAGED ? 8 : 7) || !entry(v[0], &fn)) return nullptr;
-    const eta_cache_desc* desc = ds.get(v[1]);
+    const eta_cache_desc* desc = ds.get(v[1], g_desc);
     if (!desc) return nullptr;
     const eta_page_table* pages = nullptr;
-    if (PAGED && !(pages = ps.get(v[2]))) return nullptr;
+    if (PAGED && !(pages = ps.get(v[2], g_pages))) return nullptr;
     v += PAGED ? 3 : 2;
     if (!PTR(v[0], at::kBFloat16, K) || !PTR(v[1], at::kInt, seq_lens) || !musig_pointer(v[2], &musig) || !PTR(v[3], at::kFloat, mnorm))
         return nullptr;
@@ -177,10 +183,10 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
     eta_params p;
     void *q, *K, *V, *seq_lens, *musig, *mnorm, *tau, *head_const, *out, *sel_mask, *stats, *status, *workspace = nullptr;
     if (!count(n, 15 + PAGED + WS) || !entry(v[0], &fn)) return nullptr;
-    const eta_cache_desc* desc = ds.get(v[1]);
+    const eta_cache_desc* desc = ds.get(v[1], g_desc);
     if (!desc) return nullptr;
     const eta_page_table* pages = nullptr;
-    if (PAGED && !(pages = ps.get(v[2]))) return nullptr;
+    if (PAGED && !(pages = ps.get(v[2], g_pages))) return nullptr;
     v += PAGED ? 3 : 2;
     if (!params_of(v[0], &p)) return nullptr;
     if (!PTR(v[1], at::kBFloat16, q) || !PTR(v[2], at::kBFloat16, K) || !PTR(v[3], at::kBFloat16, V) || !PTR(v[4], at::kInt, seq_lens) ||
@@ -208,10 +214,14 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
     return PyLong_FromLong(rc);
 }
 
-PyObject* set_error(PyObject*, PyObject* cls) {
-    Py_INCREF(cls);
-    Py_XDECREF(g_error);
-    g_error = cls;
+// (EtaError, CacheDesc, PageTable)
+PyObject* set_classes(PyObject*, PyObject* const* v, Py_ssize_t n) {
+    if (!count(n, 3)) return nullptr;
+    PyObject** const to[3] = {&g_error, &g_desc, &g_pages};
+    for (int k = 0; k < 3; ++k) {
+        Py_INCREF(v[k]);
+        Py_XSETREF(*to[k], v[k]);
+    }
     Py_RETURN_NONE;
 }
 
@@ -233,7 +243,7 @@ PyMethodDef methods[] = {
     {"decode", (PyCFunction)(void (*)(void))guarded<decode<Decode::PLAIN>>, METH_FASTCALL, nullptr},
     {"decode_paged", (PyCFunction)(void (*)(void))guarded<decode<Decode::PAGED>>, METH_FASTCALL, nullptr},
     {"decode_static", (PyCFunction)(void (*)(void))guarded<decode<Decode::STATIC>>, METH_FASTCALL, nullptr},
-    {"set_error", set_error, METH_O, nullptr},
+    {"set_classes", (PyCFunction)(void (*)(void))set_classes, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_eta_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

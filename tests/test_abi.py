@@ -139,3 +139,17 @@ def test_the_signature_of_a_step_call_does_not_hang_on_its_arguments():
             call()
     with pytest.raises(AttributeError):
         eb.eta_decode(d, None, *none, None)
+
+
+def test_step_calls_take_no_other_structure_of_the_same_size():
+    eb.load()
+    none = [None] * 4
+    wide = ctypes.create_string_buffer(ctypes.sizeof(eb.CacheDesc))
+    two = (ctypes.c_int64 * 2)()
+    assert ctypes.sizeof(two) == ctypes.sizeof(eb.PageTable)
+    for call in (lambda: eb.eta_append_summary(wide, *none),
+                 lambda: eb.eta_append_summary(bytes(wide), *none),
+                 lambda: eb.eta_append_summary_paged(_desc(), two, *none),
+                 lambda: eb.eta_decode(wide, eb.DecodeParams(), *none, *none, None, None, None)):
+        with pytest.raises(TypeError):
+            call()
