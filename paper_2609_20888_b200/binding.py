@@ -68,7 +68,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
                 from . import _eta_torch
             except ImportError as e:
                 raise EtaError(f"_eta_torch is missing ({e}): build it with `python -m paper_2609_20888_b200.build`") from e
-            _eta_torch.set_classes(EtaError, CacheDesc, PageTable)
+            _eta_torch.set_classes(EtaError, CacheDesc, PageTable, DecodeParams, Params)
             _native = _eta_torch
         lib_path = path or LIB_PATH
         if not os.path.exists(lib_path):

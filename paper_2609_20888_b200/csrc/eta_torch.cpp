@@ -18,7 +18,7 @@ namespace {
 
 // classes of the binding: the exception, the ctypes structures
 PyObject* g_error = nullptr;
-PyObject *g_desc = nullptr, *g_pages = nullptr;
+PyObject *g_desc = nullptr, *g_pages = nullptr, *g_decode_params = nullptr, *g_params = nullptr;
 
 bool fail(const char* name, const char* what) {
     PyErr_Format(g_error, "%s must be %s", name, what);
@@ -90,13 +90,36 @@ bool number(PyObject* o, const char* name, double* out) {
     Py_DECREF(v);
     return !(*out == -1.0 && PyErr_Occurred());
 }
+// what a ctypes integer field makes of a value: any integer (or what has __index__), modulo 2^32; floats are refused
+bool integer(PyObject* o, const char* name, uint32_t* out) {
+    PyObject* v = PyObject_GetAttrString(o, name);
+    if (!v) return false;
+    *out = (uint32_t)PyLong_AsUnsignedLongMask(v);
+    Py_DECREF(v);
+    return !PyErr_Occurred();
+}
+// A DecodeParams is read field by field, with the results its c() would have; anything else goes through its c().
 bool params_of(PyObject* o, eta_params* p) {
-    double z, a, beta, scale, lwb, window, flags;
+    if ((PyObject*)Py_TYPE(o) != g_decode_params) {
+        PyObject* c = PyObject_CallMethod(o, "c", nullptr);
+        if (!c) return false;
+        bool ok;
+        {
+            Struct<eta_params> ps;
+            const eta_params* from = ps.get(c, g_params);
+            ok = from != nullptr;
+            if (ok) *p = *from;
+        }
+        Py_DECREF(c);
+        return ok;
+    }
+    double z, a, beta, scale;
+    uint32_t lwb, window;
     if (!number(o, "z", &z) || !number(o, "a", &a) || !number(o, "beta", &beta) || !number(o, "scale", &scale) ||
-        !number(o, "lwb", &lwb) || !number(o, "rescue_window", &window) || !number(o, "flags", &flags))
+        !integer(o, "lwb", &lwb) || !integer(o, "rescue_window", &window) || !integer(o, "flags", &p->flags))
         return false;
     p->z = (float)z; p->a = (float)a; p->beta = (float)beta; p->scale = (float)scale;
-    p->lwb = (int32_t)lwb; p->rescue_window = (int32_t)window; p->flags = (uint32_t)flags;
+    p->lwb = (int32_t)lwb; p->rescue_window = (int32_t)window;
     return true;
 }
 
@@ -214,11 +237,18 @@ PyObject* decode(PyObject*, PyObject* const* v, Py_ssize_t n) {
     return PyLong_FromLong(rc);
 }
 
-// (EtaError, CacheDesc, PageTable)
+// the eta_params a call would get, as bytes (for the tests)
+PyObject* params(PyObject*, PyObject* const* v, Py_ssize_t n) {
+    eta_params p;
+    if (!count(n, 1) || !params_of(v[0], &p)) return nullptr;
+    return PyBytes_FromStringAndSize(reinterpret_cast<const char*>(&p), sizeof p);
+}
+
+// (EtaError, CacheDesc, PageTable, DecodeParams, Params)
 PyObject* set_classes(PyObject*, PyObject* const* v, Py_ssize_t n) {
-    if (!count(n, 3)) return nullptr;
-    PyObject** const to[3] = {&g_error, &g_desc, &g_pages};
-    for (int k = 0; k < 3; ++k) {
+    if (!count(n, 5)) return nullptr;
+    PyObject** const to[5] = {&g_error, &g_desc, &g_pages, &g_decode_params, &g_params};
+    for (int k = 0; k < 5; ++k) {
         Py_INCREF(v[k]);
         Py_XSETREF(*to[k], v[k]);
     }
@@ -243,6 +273,7 @@ PyMethodDef methods[] = {
     {"decode", (PyCFunction)(void (*)(void))guarded<decode<Decode::PLAIN>>, METH_FASTCALL, nullptr},
     {"decode_paged", (PyCFunction)(void (*)(void))guarded<decode<Decode::PAGED>>, METH_FASTCALL, nullptr},
     {"decode_static", (PyCFunction)(void (*)(void))guarded<decode<Decode::STATIC>>, METH_FASTCALL, nullptr},
+    {"params", (PyCFunction)(void (*)(void))guarded<params>, METH_FASTCALL, nullptr},
     {"set_classes", (PyCFunction)(void (*)(void))set_classes, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };

@@ -153,3 +153,28 @@ def test_step_calls_take_no_other_structure_of_the_same_size():
                  lambda: eb.eta_decode(wide, eb.DecodeParams(), *none, *none, None, None, None)):
         with pytest.raises(TypeError):
             call()
+
+
+def test_step_calls_read_parameters_as_ctypes_does():
+    """The marshalled structure has the bytes of DecodeParams.c(): integers modulo 2^32, no truncated floats, whatever an
+    override of c() returns."""
+    import numpy as np
+    eb.load()
+
+    class Doubled(eb.DecodeParams):
+        def c(self):
+            return eb.Params(2 * self.z, self.a, self.beta, self.scale, self.lwb, self.rescue_window, self.flags)
+
+    native = eb._native
+    for kw in (dict(), dict(z=0.1, a=-2, beta=1e300, scale=np.float32(0.3)), dict(lwb=np.int64(3), rescue_window=64, flags=5),
+               dict(lwb=True, flags=-1), dict(lwb=2 ** 32 + 1, rescue_window=2 ** 31), dict(rescue_window=-(2 ** 40) - 7)):
+        for cls in (eb.DecodeParams, Doubled):
+            assert native.params(cls(**kw)) == bytes(cls(**kw).c()), (cls, kw)
+    for kw in (dict(lwb=2.7), dict(rescue_window=64.0), dict(flags=np.float32(1)), dict(lwb=None), dict(z="1"),
+               dict(rescue_window=float("nan"))):
+        with pytest.raises(TypeError):
+            eb.DecodeParams(**kw).c()
+        with pytest.raises(TypeError):
+            native.params(eb.DecodeParams(**kw))
+        with pytest.raises(TypeError):
+            eb.eta_decode(_desc(), eb.DecodeParams(**kw), *[None] * 10, None)
