@@ -53,9 +53,28 @@ class EtaError(RuntimeError):
 
 
 _lib = None
-_native = None          # the compiled marshalling module
+_native = None          # the compiled marshalling module, or what stands for it where it is missing
 _STEP_CALLS = ("eta_append_summary", "eta_append_summary_paged", "eta_predict_threshold", "eta_decode", "eta_decode_paged",
                "eta_decode_static")
+
+
+class _Missing:
+    """Every call through a module that could not be imported raises the reason."""
+
+    def __init__(self, why: Exception):
+        self._why = why
+
+    def __getattr__(self, name):
+        raise EtaError(f"_eta_torch is missing ({self._why}): build it with `python -m paper_2609_20888_b200.build`") from self._why
+
+
+def _marshalling():
+    try:
+        from . import _eta_torch
+    except ImportError as e:
+        return _Missing(e)
+    _eta_torch.set_classes(EtaError, CacheDesc, PageTable, DecodeParams, Params)
+    return _eta_torch
 
 
 def load(path: str | None = None) -> ctypes.CDLL:
@@ -64,12 +83,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
     global _lib, _native
     if _lib is None or path is not None:
         if _native is None:
-            try:
-                from . import _eta_torch
-            except ImportError as e:
-                raise EtaError(f"_eta_torch is missing ({e}): build it with `python -m paper_2609_20888_b200.build`") from e
-            _eta_torch.set_classes(EtaError, CacheDesc, PageTable, DecodeParams, Params)
-            _native = _eta_torch
+            _native = _marshalling()           # only the calls of a decode step need it
         lib_path = path or LIB_PATH
         if not os.path.exists(lib_path):
             raise EtaError(f"{lib_path} is missing: build it with `python -m paper_2609_20888_b200.build` "

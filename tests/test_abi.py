@@ -178,3 +178,20 @@ def test_step_calls_read_parameters_as_ctypes_does():
             native.params(eb.DecodeParams(**kw))
         with pytest.raises(TypeError):
             eb.eta_decode(_desc(), eb.DecodeParams(**kw), *[None] * 10, None)
+
+
+def test_only_the_step_calls_need_the_compiled_marshalling(monkeypatch):
+    """A missing (or unloadable) _eta_torch is an error of the calls that go through it, loudly; the library and the other entry
+    points work without it."""
+    import sys
+    package = eb.__name__.rsplit(".", 1)[0]
+    monkeypatch.setitem(sys.modules, package + "._eta_torch", None)        # an import of it fails
+    monkeypatch.delattr(package + "._eta_torch", raising=False)
+    monkeypatch.setattr(eb, "_native", None)
+    monkeypatch.setattr(eb, "_lib", None)
+    assert eb.eta_workspace_bytes(_desc()) > 0
+    assert eb.eta_static_scratch_bytes() == 8 << 20
+    with pytest.raises(eb.EtaError, match="_eta_torch is missing"):
+        eb.eta_append_summary(_desc(), None, None, None, None)
+    with pytest.raises(eb.EtaError, match="_eta_torch is missing"):
+        eb.eta_decode(_desc(), eb.DecodeParams(), *[None] * 10, None)
