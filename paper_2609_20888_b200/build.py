@@ -51,9 +51,29 @@ TORCH_MODULE = os.path.join(HERE, "_eta_torch.so")
 TORCH_SOURCE = os.path.join(CSRC, "eta_torch.cpp")
 
 
-def build_torch_module(force: bool = False) -> str:
+# It is linked against torch's C++ interface and the interpreter's: beside it stands what it was built for.
+TORCH_STAMP = os.path.join(HERE, "_eta_torch.built_for")
+
+
+def torch_stamp() -> str:
+    import sysconfig
+
+    import torch
+    return f"torch {torch.__version__} {sysconfig.get_config_var('SOABI')}"
+
+
+def torch_module_is_current() -> bool:
     deps = [TORCH_SOURCE, HEADER]
-    if not force and os.path.exists(TORCH_MODULE) and all(os.path.getmtime(p) <= os.path.getmtime(TORCH_MODULE) for p in deps):
+    if not (os.path.exists(TORCH_MODULE) and os.path.exists(TORCH_STAMP)):
+        return False
+    if any(os.path.getmtime(p) > os.path.getmtime(TORCH_MODULE) for p in deps):
+        return False
+    with open(TORCH_STAMP) as f:
+        return f.read() == torch_stamp()
+
+
+def build_torch_module(force: bool = False) -> str:
+    if not force and torch_module_is_current():
         return TORCH_MODULE
     import sysconfig
 
@@ -67,6 +87,8 @@ def build_torch_module(force: bool = False) -> str:
         cmd += ["-isystem", inc]
     cmd += ["-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
     subprocess.run(cmd, check=True)
+    with open(TORCH_STAMP, "w") as f:
+        f.write(torch_stamp())
     return TORCH_MODULE
 
 

@@ -195,3 +195,12 @@ def test_only_the_step_calls_need_the_compiled_marshalling(monkeypatch):
         eb.eta_append_summary(_desc(), None, None, None, None)
     with pytest.raises(eb.EtaError, match="_eta_torch is missing"):
         eb.eta_decode(_desc(), eb.DecodeParams(), *[None] * 10, None)
+
+
+def test_the_marshalling_is_rebuilt_for_another_torch(monkeypatch):
+    """It links against torch's C++ interface: one that was built for another version is not current, whatever its date."""
+    import torch
+    ebuild.build_torch_module()
+    assert ebuild.torch_module_is_current()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert not ebuild.torch_module_is_current()
