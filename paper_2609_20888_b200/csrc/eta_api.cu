@@ -133,6 +133,7 @@ WsLayout ws_layout(const eta_cache_desc* d) {
     size_t slots = ((size_t)MAX_CTAS + L.rows) * DECODE_GROUPS;
     L.part_ml = off;    off = align_up(off + sizeof(float2) * slots * G, 256);
     L.part_o = off;     off = align_up(off + sizeof(float) * slots * G * d->head_dim, 256);
+    L.resc = L.part_ml;
     L.total = off;
     return L;
 }

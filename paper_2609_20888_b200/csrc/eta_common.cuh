@@ -49,6 +49,7 @@ struct WsLayout {
     size_t tau_eff;     // float [batch * n_q_heads]
     size_t part_ml;     // float2 [(MAX_CTAS + rows) * DECODE_GROUPS * G]
     size_t part_o;      // float [(MAX_CTAS + rows) * DECODE_GROUPS * G * d]
+    size_t resc;        // int2 [rows], int2 [CTAs * G] of the screening stage: in place of the partials, which are written after it
     size_t total;
 };
 WsLayout ws_layout(const eta_cache_desc* d);
@@ -103,9 +104,14 @@ struct ScreenArgs {
     int gpr;
     int32_t* seg_list;
     float* tau_eff;
+    // where the rescue window is longer than a CTA's passes, and rescue_kernel decides (else null): [rows] first CTA and number
+    // of CTAs of a row, then [CTA][G] largest bound (as a key) and its block
+    int2* resc;
     uint8_t* sel_mask;
     uint32_t* status;
+#ifdef ETA_TIMELINE
     unsigned long long* timeline;
+#endif
 };
 int encode_tiles(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                  const cuuint32_t* box);

@@ -1125,8 +1125,12 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     sa.gpr = L.gpr;
     sa.seg_list = reinterpret_cast<int32_t*>(ws + L.seg_list);
     sa.tau_eff = reinterpret_cast<float*>(ws + L.tau_eff);
+    // at most rows + slots CTAs screen (launch_screen): with G entries each a small part of the partials' (MAX_CTAS + rows) * 3 G
+    sa.resc = reinterpret_cast<int2*>(ws + L.resc);
     sa.sel_mask = sel_mask;
+#ifdef ETA_TIMELINE
     sa.timeline = debug_timeline();
+#endif
     sa.status = status_dev;
     CUtensorMap tmK, tmV;
     const int n_pages = pages ? pages->n_pages : 0;

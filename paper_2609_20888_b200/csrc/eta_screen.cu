@@ -18,7 +18,8 @@
 //
 // Top-1 rescue needs the whole rescue window of a head: the first CTA of a row
 // takes at least the passes the window spans, and decides rescue before it
-// writes its lists.
+// writes its lists.  Where that would be more passes than the row's other CTAs
+// take, every CTA leaves its largest bounds and rescue_kernel decides.
 #include "eta_common.cuh"
 #include "eta_timeline.h"
 
@@ -28,6 +29,10 @@ namespace eta {
 __device__ __forceinline__ float min_keep_nan(float g, float s) {
     return (g < s) ? g : ((s < g) ? s : ((g != g) ? g : s));
 }
+
+// Bounds as integers that ascend with them: 0xffffffff stands for a NaN, 0 for no bound at all (and reads as a NaN too: a
+// comparison with it never holds)
+__device__ __forceinline__ float key_bound(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k); }
 
 constexpr int SCR_WARPS = 4;
 
@@ -347,6 +352,7 @@ struct ScreenSmem {
 // us a step, 4: 68.8, 3: 70.5, 2: 72.7; 128 rows at d = 64, G = 8: 118.4, 116.3, 120.4, 123.7).
 constexpr int SCR_SLOTS = 4;
 constexpr int SCR_GROUP = 4;         // most passes whose bounds wait in shared memory for the thresholds
+constexpr int SCR_WINDOW = 2;        // passes of a rescue window that a row's first CTA takes in any case
 
 // Zeroes n bytes with the threads of a CTA: 16 at a time between the ends
 __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
@@ -362,9 +368,12 @@ __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
 // resident at once, because none can finish before the thresholds are there.  A step of 65536 blocks at d = 128, G = 4 takes
 // 68.8 us instead of 71.1 (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
 // barrier per segment); 65536 blocks at d = 64, G = 8, where both terms were on that pipe, 116.3 instead of 126.9.
+// 80 registers at d = 128, 96 at 64: CTAs start beside those of the append and the predictor, and with 88 fewer of them fit
+// there (32K x 8 48.8 -> 49.5 us, 128K x 4 55.5 -> 57.2, graph replay).  The bound of six CTAs holds the instances to 80 that would
+// take more by themselves; the others take 78 to 80 at five and lose by it (512K x 1 43.4 -> 44.4 with the 73 that six give).
 template <int D, int G, bool PACKED>
-__global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_constant__ CUtensorMap tmK,
-                                                                    const __grid_constant__ CUtensorMap tmV, const ScreenArgs a) {
+__global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4 && PACKED)) ? 6 : 5) screen_kernel(
+    const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const ScreenArgs a) {
     using L = ScreenSmem<D, G>;
     using TL = TileOf<D>;
     constexpr int REC_BYTES = PACKED ? 3 * D : 4 * D;
@@ -451,7 +460,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_
     // bound among them.  It admits none exactly when that bound is below its threshold and no block of the window is pinned
     // (a NaN bound admits), so the row's first CTA looks for the largest bounds ahead of the wait for the thresholds, a warp
     // per head, with bounds compared as order-preserving integers.
-    const bool rescues = c == 0 && !dense && Wr > 0 && !(lwb > 0 && NB - lwb < Wr);
+    const bool rescues = (c == 0 || a.resc) && !dense && Wr > 0 && !(lwb > 0 && NB - lwb < Wr);
     const bool stale = !dense && NB > 0 && (T & (a.b - 1)) == 0;      // the newest block's record may not have been final yet
     auto window_max = [&](int p0, int p1) {
         const int n_win = min(Wr, p1 * TL::PASS) - p0 * TL::PASS;
@@ -537,13 +546,10 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_
         };
         if (rescues && p0 * TL::PASS < Wr) {
             if (stale_in) { __syncthreads(); window_max(p0, p1); }
-            if (p1 * TL::PASS >= Wr) {
+            if (!a.resc && p1 * TL::PASS >= Wr) {
 #pragma unroll
-                for (int gq = 0; gq < G; ++gq) {
-                    const uint32_t k = s_bkey[gq];
-                    const float top = __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);      // (0xffffffff: a NaN)
-                    if (top < te_g[gq]) missing |= 1u << gq;
-                }
+                for (int gq = 0; gq < G; ++gq)
+                    if (key_bound(s_bkey[gq]) < te_g[gq]) missing |= 1u << gq;
             }
         }
         for (int seg = seg_0 + warp; seg < s_end; seg += SCR_WARPS) {
@@ -593,6 +599,9 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_
         }
         if (p1 < p_last) __syncthreads();          // the bounds of this group have been read: the next may overwrite them
     }
+    // The successor may set up from here on (it waits for the end of this kernel before it reads anything).  After the stores
+    // below, where warps leave one by one, a small eager step took up to a microsecond longer (2K x 1 17.5 -> 18.8).
+    pdl_trigger();
     // what the row's passes do not reach: no survivors, nothing attended
     if (c == n_ctas - 1) {
         const int seg_n = min(a.nseg, P * (TL::PASS / SEG)), rec_n = min(a.nb_cap, P * TL::PASS);
@@ -620,8 +629,55 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) screen_kernel(const __grid_
             __syncwarp();
         }
     }
+    if (a.resc) {
+        if (tid < G) a.resc[a.rows + (int64_t)blockIdx.x * G + tid] = make_int2((int)s_bkey[tid], s_best[tid]);
+        if (c == 0 && tid == 0) a.resc[r] = make_int2(blockIdx.x, n_ctas);
+    }
     if (tl && tid == 0) tl[5] = globaltimer_ns();
+}
+
+// Top-1 rescue of the rows whose window no single CTA of the screening kernel holds: a CTA per row, a warp per head (latency:
+// two dependent reads, then as many for a head that needs rescue).  The largest of the CTAs' bounds decides; the rescued block
+// joins lists that are already written.  A block another head fetches anyway gets the head's bit, any other goes to the end
+// of its segment's list.
+__global__ void __launch_bounds__(256) rescue_kernel(const int2* __restrict__ span, const int2* __restrict__ best,
+                                                     const float* __restrict__ tau_eff, int G, int nb_cap, int nseg, int gpr,
+                                                     uint8_t* sel_mask, uint8_t* seg_cnt, int32_t* seg_list) {
+    __shared__ int s_block[8];            // rescued block of each head, or -1
+    const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_trigger();
+    pdl_wait();                           // the screening kernel's lists are complete
+    if (warp < G) {
+        const float te = __ldcg(tau_eff + (int64_t)r * G + warp);
+        const int2 sp = __ldcg(span + r);
+        uint32_t key = 0;
+        int arg = 0x7fffffff;
+        for (int c = lane; c < sp.y; c += 32) {            // ascending: a lane keeps the first of equal bounds
+            const int2 e = __ldcg(best + (int64_t)(sp.x + c) * G + warp);
+            if ((uint32_t)e.x > key) { key = (uint32_t)e.x; arg = e.y; }
+        }
+        const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+        const int amin = __reduce_min_sync(0xffffffffu, key == kmax ? arg : 0x7fffffff);
+        if (lane == 0) s_block[warp] = key_bound(kmax) < te ? amin : -1;
+    }
+    __syncthreads();
+    for (int gq = 0; gq < G && warp == 0; ++gq) {
+        const int j = s_block[gq], seg = j / SEG;
+        if (j < 0) continue;
+        volatile uint8_t* mp = sel_mask + (int64_t)r * nb_cap + j;
+        volatile uint8_t* np = seg_cnt + (int64_t)r * gpr * GRANULE + seg;
+        volatile int32_t* list = seg_list + ((int64_t)r * nseg + seg) * LSTRIDE;
+        const unsigned w = *mp, n = *np;
+        __syncwarp();                     // every lane has read them
+        if (w == 0) {
+            if (lane == 0) { list[n] = j | (1 << (24 + gq)); *np = (uint8_t)(n + 1); }
+        } else {
+            for (unsigned k = lane; k < n; k += 32)
+                if ((list[k] & 0xffffff) == j) list[k] = list[k] | (1 << (24 + gq));
+        }
+        if (lane == 0) *mp = (uint8_t)(w | (1u << gq));
+        __syncwarp();
+    }
 }
 
 // Eq. dual_bound_eq for every block, for its own sake: the tiles of the screening kernel, stored instead of compared.
@@ -721,6 +777,13 @@ static int launch_screen_t(const ScreenArgs& a, const CUtensorMap& tmK, const CU
     // the split at full length: what rows of any length stay below, and what is used where there are too many to look at
     const int64_t all = (int64_t)rows * b2.passes;
     b2.tp = (int)((all + b2.slots - 1) / b2.slots);
+    // A window of more passes than a row's other CTAs take would be its first CTA's work alone, one pass after another: a kernel
+    // of its own settles rescue then, for 1 to 3 us a step.  128K x 4 (d = 128, two passes per CTA), windows of 128 blocks 58 us;
+    // 256 63.8 in the first CTA, 60.2 this way; 1024 90.9 and 60.5; all blocks 117.6 and 61.0 (512K x 1: 192 and 38.7; 64K, d = 64,
+    // G = 8: 76.0 and 32.6).
+    const bool late = !(a.flags & ETA_FLAG_DENSE) && b2.need > (b2.tp > SCR_WINDOW ? b2.tp : SCR_WINDOW);
+    if (late) b2.need = 0;
+    else b2.resc = nullptr;
     const int head = b2.tp > b2.need ? b2.tp : b2.need;
     b2.ctas_row = b2.passes <= head ? 1 : 1 + (b2.passes - head + b2.tp - 1) / b2.tp;
     b2.div_ctas = FastDiv(b2.ctas_row);
@@ -734,8 +797,12 @@ static int launch_screen_t(const ScreenArgs& a, const CUtensorMap& tmK, const CU
     // A second buffer per warp (three CTAs per SM) where all CTAs are still resident at once: a CTA of two passes, such as
     // the one that holds the rescue window, then has both on their way from the start.
     b2.nbuf = (b2.group > 1 && all <= 3 * n_sm) ? 2 : 1;
-    return launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)grid), dim3(32 * SCR_WARPS),
-                      ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, tmK, tmV, b2);
+    const int rc = launch_pdl("screen launch", screen_kernel<D, G, PACKED>, dim3((unsigned)grid), dim3(32 * SCR_WARPS),
+                              ScreenSmem<D, G>::bytes(b2.group * TileOf<D>::PASS, b2.nbuf), s, tmK, tmV, b2);
+    if (rc != ETA_OK || !late) return rc;
+    return launch_pdl("rescue launch", rescue_kernel, dim3((unsigned)rows), dim3(256), 0, s, (const int2*)a.resc,
+                      (const int2*)(a.resc + rows), (const float*)a.tau_eff, G, a.nb_cap, a.nseg, a.gpr, a.sel_mask, a.seg_cnt,
+                      a.seg_list);
 }
 
 int launch_screen(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int G, int n_sm, cudaStream_t s) {
