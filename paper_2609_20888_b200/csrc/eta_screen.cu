@@ -722,8 +722,9 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     }
 }
 
-// The same for arrays that 16-byte loads cannot read (a caller's odd offset): one warp per (sequence, query head, block).
-__global__ void __launch_bounds__(128) score_dual_unaligned_kernel(
+// The same with a warp per (sequence, query head, block): for arrays that 16-byte loads cannot read (a caller's odd offset), and
+// for few bounds, where warps fill the GPU and tiles do not (what counts is then the length of one tile's chain of steps).
+__global__ void __launch_bounds__(128) score_dual_warp_kernel(
     const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ musig, const float* __restrict__ mnorm,
     const int32_t* __restrict__ seq_lens, int B, int Hq, int Hkv, int d, int b, int t_cap, int nb_cap, float z,
     float scale, int packed, float* __restrict__ bound) {
@@ -847,9 +848,11 @@ extern "C" int eta_score_dual(const eta_cache_desc* desc, const eta_params* para
     auto qp = static_cast<const __nv_bfloat16*>(q);
     auto mp = static_cast<const unsigned char*>(musig);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(musig)) & 15) {
-        const int64_t warps = (int64_t)desc->batch * desc->n_q_heads * desc->nb_cap;
-        eta::score_dual_unaligned_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
+    // Few bounds (counted by capacity), us with warps / with tiles: 256 2.9 / 4.0, 1024 2.9 / 4.0, 4096 3.7 / 3.9, 8192 5.7 / 3.9, 16384
+    // 8.8 / 4.0 (d = 128; 64 alike, but 4.2 to 5.0 with tiles)
+    const int64_t warps = (int64_t)desc->batch * desc->n_q_heads * desc->nb_cap;
+    if (warps <= 4096 || ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(musig)) & 15)) {
+        eta::score_dual_warp_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(
             qp, mp, mnorm, seq_lens, desc->batch, desc->n_q_heads, desc->n_kv_heads, desc->head_dim, desc->block_size,
             desc->t_cap, desc->nb_cap, params->z, scale, packed ? 1 : 0, bound);
         return eta::check_launch("eta_score_dual");

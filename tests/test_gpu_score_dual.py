@@ -16,18 +16,29 @@ def _e4m3(x):
     return x.to(torch.float8_e4m3fn).view(torch.uint8), x.to(torch.float8_e4m3fn).float()
 
 
-@pytest.mark.parametrize("lens", [(32 * 31, 32 * 33 + 5), (0, 32), (32 * 129, 32 * 640 + 31)])
+LENS = [(32 * 31, 32 * 33 + 5), (0, 32), (32 * 129, 32 * 640 + 31)]
+
+
+@pytest.mark.parametrize("lens", LENS)
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("G", [1, 2, 4, 8])
 @pytest.mark.parametrize("packed", [False, True])
-@pytest.mark.parametrize("offset", [0, 1])
-def test_bounds_match_the_definition(lens, d, G, packed, offset):
+@pytest.mark.parametrize("room", [3, 4097])          # blocks past the longest: few bounds in all, or more than 4096 (tiles)
+def test_bounds_match_the_definition(lens, d, G, packed, room):
+    _check(lens, d, G, packed, 0, room)
+
+
+@pytest.mark.parametrize("lens", LENS)
+@pytest.mark.parametrize("d", [64, 128])
+def test_bounds_of_queries_off_a_16_byte_boundary(lens, d):
+    _check(lens, d, 2, False, 1, 4097)
+
+
+def _check(lens, d, G, packed, offset, room):
     from paper_2609_20888_b200 import binding as eb
-    if offset and (G != 2 or packed):
-        pytest.skip("one shape is enough for the path of unaligned arrays")
     Hkv, b, B = 2, 32, 2
     T = max(max(lens), 1)
-    nb = T // b + 3
+    nb = T // b + room
     g = torch.Generator().manual_seed(d + G + T)
     desc = eb.CacheDesc(B, Hkv * G, Hkv, d, b, T, nb, Hkv * T * d, T * d, d, Hkv * T * d, T * d, d)
     q = torch.randn((B, Hkv * G, d), generator=g).to(torch.bfloat16)
