@@ -289,7 +289,7 @@ template <int D>
 __global__ void __launch_bounds__(128, 8) build_summaries_kernel(
     const __nv_bfloat16* __restrict__ K, int64_t sb, int64_t sh, int64_t st, int Hkv, int b, int t_cap, int nb_cap,
     int nb_max, int rows, const int32_t* __restrict__ seq_lens, int mode, unsigned char* __restrict__ musig,
-    float* __restrict__ mnorm, const int32_t* __restrict__ table, int table_stride, int read_once) {
+    float* __restrict__ mnorm, const int32_t* __restrict__ table, int table_stride, int once_from) {
     const int64_t wid = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (wid >= (int64_t)rows * nb_max) return;
     const int r = (int)(wid / nb_max), j = (int)(wid % nb_max);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(128, 8) build_summaries_kernel(
     const int64_t rec = (int64_t)r * nb_cap + j;
     const bool packed = (mode & 2) != 0;      // mode: bit 0 sub-block envelope, bit 1 packed records
     summarize_block<D>(blk, st, b, (mode & 1) != 0, musig + rec * (packed ? 3 * D : 4 * D), packed, mnorm + rec,
-                       l2_policy(read_once != 0));
+                       l2_policy(__any_sync(0xffffffffu, T >= once_from)));
 }
 
 // The append: one CTA of four warps per (sequence, KV head) row whose newest token completed a block.  A decode step
@@ -437,16 +437,20 @@ static int build_impl(const eta_cache_desc* desc, const eta_page_table* pages, c
     // Keys that do not fit the L2 (126 MB) leave it first, so that they push out neither one another nor the records that are
     // still to be written back: 1.07 GB 190 -> 187 us, 268 MB 95.3 -> 88.6 (b = 128, packed, paged), 55.8 -> 51.4 (d = 64),
     // 53.6 -> 50.8 (token-major).  Keys that fit stay for the steps to come and for a build that reads them again (17 MB: 9.7
-    // us this way, 10.4 with the hint).
-    const int read_once = warps * desc->block_size * desc->head_dim * 2 > (128ll << 20);
+    // us this way, 10.4 with the hint).  What counts is what the sequences hold, not the cache's capacity (4K x 4 in a cache of
+    // 128K x 4: 19.1 with the hint, 18.4 without; 16K x 4, the line itself: 31.6 and 33.2), which a warp takes its own sequence
+    // for: as if all were as long.  (The vote makes the policy uniform; with a policy per lane a build took 12 % longer.)
+    const int64_t tokens = (128ll << 20) / ((int64_t)2 * desc->head_dim * desc->n_kv_heads);
+    const int64_t per_sequence = (tokens + desc->batch - 1) / desc->batch;
+    const int once_from = per_sequence > desc->t_cap ? INT32_MAX : (int)per_sequence;
     if (desc->head_dim == 128)
         eta::build_summaries_kernel<128><<<grid, 128, 0, s>>>(Kp, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t,
             desc->n_kv_heads, desc->block_size, desc->t_cap, desc->nb_cap, nb_max, rows, seq_lens, env, mp, mnorm,
-            table, tstride, read_once);
+            table, tstride, once_from);
     else
         eta::build_summaries_kernel<64><<<grid, 128, 0, s>>>(Kp, desc->k_stride_b, desc->k_stride_h, desc->k_stride_t,
             desc->n_kv_heads, desc->block_size, desc->t_cap, desc->nb_cap, nb_max, rows, seq_lens, env, mp, mnorm,
-            table, tstride, read_once);
+            table, tstride, once_from);
     return eta::check_launch("eta_build_block_summaries");
 }
 
