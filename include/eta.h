@@ -97,7 +97,8 @@ typedef struct eta_params {
  * Bytes of scratch eta_decode needs for this cache shape (independent of the
  * sequence lengths).  The caller allocates it once, 256-byte aligned, and may
  * reuse it across calls on the same stream; it carries no state between calls
- * (every word is written before it is read) and needs no initialisation.
+ * and needs no initialisation: no result depends on its earlier contents (the
+ * merge kernel may read a row's span early, as a hint that it clamps and checks).
  * No device is touched by this function.
  */
 int eta_workspace_bytes(const eta_cache_desc* desc, size_t* out_bytes);
@@ -259,7 +260,7 @@ int eta_decode(const eta_cache_desc* desc, const eta_params* params, const void*
  *     call that finds no memory left returns ETA_ERR_CUDA (eta_last_cuda_error names cudaGetSymbolAddress).
  *     The address is looked up once per device and kept; it does not survive a cudaDeviceReset.
  *   - Sharing: all calls on a device use the same array, and it keeps the previous call's contents.  Nothing in
- *     it has to be cleared by the caller: each call writes every word before reading it.  For the same reason
+ *     it has to be cleared by the caller: no result depends on what an earlier call left.  For the same reason
  *     two calls whose kernels can overlap on the GPU (different streams, no dependency between them) race on
  *     the array and corrupt each other; calls on one stream, or otherwise ordered, are fine.
  */

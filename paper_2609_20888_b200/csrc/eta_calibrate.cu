@@ -2,7 +2,7 @@
 // 1/t-Weighted Histograms", Algorithm "Density-Matched Offline Threshold
 // Calibration"): one pass over a calibration split builds, per query head, the
 // 1/t-weighted histogram of the raw causal scores S_ts = s <q_t, k_s> and the
-// density the dynamic thresholds realise; a bisection on the histogram then
+// density the dynamic thresholds realise; a root search on the histogram then
 // finds the static constant with the same density.
 //
 // calib_hist_kernel: a CTA per (128-query tile, head, sequence).  The scores of a

@@ -1147,7 +1147,10 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     // the 8 us the memory would idle before the streaming kernel's first copies).  Batch 4 at 128K: 66.7 -> 60.5 us a step with
     // the first of the two, 58.4 with both (24, 48 and 80 MB within 1 us of 32); 32K x 8: 58.0 -> 51.2; 512K: 51.2 -> 43.4.
     // Where the cache fits, or nearly, both cost time: 50K x 1 with 4 KV heads (104 MB) 24.7 -> 27.8, 8K x 7 (30 MB) 24.7 -> 28.8;
-    // between 140 and 330 MB the sign depends on how much survives (51.3 -> 45.0, 33.9 -> 33.2, 30.0 -> 32.4).
+    // between 140 and 330 MB the sign depends on how much survives (51.3 -> 45.0, 33.9 -> 33.2, 30.0 -> 32.4): the line lies
+    // where most gain, it is not sharp.  It goes by the capacity, which the host knows; of a cache of 128K x 4 that holds little,
+    // a step takes without and with both, 4K x 4 21.3, 21.4; 16K x 4 26.2, 27.1; 32K x 4 34.9, 32.7.  Lengths added up on the device
+    // win the second and cost 0.5 to 2 us on the large steps, 8 where 183 MB are held in 419 (76.6 against 71.3 with both).
     const int64_t unit_bytes = (int64_t)4 * b * D, segs = (int64_t)L.rows * L.nseg;
     const bool large = (int64_t)L.rows * desc->nb_cap * unit_bytes > LARGE_CACHE_BYTES;
     const int64_t share = (PREFETCH_BYTES + segs * unit_bytes - 1) / (segs * unit_bytes);

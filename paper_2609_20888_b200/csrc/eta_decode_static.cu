@@ -63,9 +63,9 @@ int eta_decode_static(const eta_cache_desc* desc, const eta_params* params, cons
     void* scratch = nullptr;
     rc = eta::static_scratch_ptr(&scratch);
     if (rc != ETA_OK) return rc;
-    // every word of the scratch that a kernel reads is written earlier in the same call (counts, lists and window
-    // statistics by the screening kernel, partial slots by the streaming kernel), so nothing carried over from
-    // the previous call is ever consumed
+    // What a result depends on is written earlier in the same call (counts, lists and largest bounds by the screening
+    // kernel, spans and partial slots by the streaming kernel).  The merge kernel reads a row's span before its wait, when it may
+    // still be the previous call's: it is clamped, and checked after the wait.
     return eta_decode(desc, params, q, K, V, seq_lens, musig, mnorm, tau, head_const, out, sel_mask, stats,
                       status_dev, scratch, eta::STATIC_SCRATCH_BYTES, stream);
 }

@@ -349,7 +349,8 @@ struct ScreenSmem {
 };
 // CTAs per SM the screening grid is sized for.  A fifth would fit an empty SM, but the append and predictor CTAs are still
 // on some of them: with 5 the last CTAs only start when the first have had their thresholds (65536 blocks at d = 128: 71.7
-// us a step, 4: 68.8, 3: 70.5, 2: 72.7; 128 rows at d = 64, G = 8: 118.4, 116.3, 120.4, 123.7).
+// us a step, 4: 68.8, 3: 70.5, 2: 72.7; 128 rows at d = 64, G = 8: 118.4, 116.3, 120.4, 123.7; measured before the streaming
+// kernel's changes that brought these steps to 59 and 90 us).
 constexpr int SCR_SLOTS = 4;
 constexpr int SCR_GROUP = 4;         // most passes whose bounds wait in shared memory for the thresholds
 constexpr int SCR_WINDOW = 2;        // passes of a rescue window that a row's first CTA takes in any case
@@ -365,8 +366,8 @@ __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
 
 // What bounds it: HBM for the records (33.8 MB for 65536 blocks at d = 128, 5.2 us at the copy rate) once enough of them are
 // requested; small CTAs, because the hardware then fills whatever the predecessor kernels leave of each SM, and all of them
-// resident at once, because none can finish before the thresholds are there.  A step of 65536 blocks at d = 128, G = 4 takes
-// 68.8 us instead of 71.1 (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
+// resident at once, because none can finish before the thresholds are there.  A step of 65536 blocks at d = 128, G = 4 took
+// 68.8 us instead of 71.1 with it (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
 // barrier per segment); 65536 blocks at d = 64, G = 8, where both terms were on that pipe, 116.3 instead of 126.9.
 // 80 registers at d = 128, 96 at 64: CTAs start beside those of the append and the predictor, and with 88 fewer of them fit
 // there (32K x 8 48.8 -> 49.5 us, 128K x 4 55.5 -> 57.2, graph replay).  The bound of six CTAs holds the instances to 80 that would

@@ -1,4 +1,4 @@
-"""A capacity beyond the L2 makes the streaming kernel's copies leave the L2 first and the screening kernel start the first
+"""A capacity beyond twice the L2 makes the streaming kernel's copies leave the L2 first and the screening kernel start the first
 survivors of every segment on their way; neither may change a result.  The same sequences are decoded through a cache of just
 their size and through one whose capacity lies past the line (256 MiB of K and V)."""
 import pytest

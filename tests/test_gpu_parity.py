@@ -294,9 +294,8 @@ def test_plus_infinite_threshold_attends_rescue_pins_and_tail_only():
 
 
 def test_rescue_window_longer_than_four_segments_and_many_segment_counts():
-    """Two loops of the streaming kernel's set-up that ordinary shapes do not enter: a rescue window of more than
-    4 x 64 blocks (its statistics are then combined in rounds of four segments), and more segment counts than one
-    pass of the set-up loads (8 per thread x 416 threads = 3328; here 64 rows x 56 segments = 3584)."""
+    """Rescue windows that rescue_kernel settles, on more rows than it has elsewhere, and a full chunk of survivor counts:
+    64 rows x 4 granules of 16 segments are the 256 granules that a warp of the streaming kernel reads in one round trip."""
     _eb()
     d, b, B, Hkv, G = 64, 32, 8, 8, 1
     T = 32 * 64 * 56

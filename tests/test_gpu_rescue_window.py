@@ -79,7 +79,8 @@ def _step(rows, nb, G, tau, d=128, b=32):
 
 
 def test_a_window_of_several_groups_of_passes_in_one_cta():
-    """Rows that are one CTA's work each: it settles a window longer than the bounds it keeps at a time."""
+    """Rows that are one CTA's work each: it settles a window longer than the bounds it keeps at a time.  600 rows of counts are also
+    more than the streaming kernel reads in one round trip."""
     G, nb = 2, 640                                     # ten passes of 64 blocks, four of them at a time
     run, sel, bound = _step(600, nb, G, 1e30)
     run(nb - 1)
