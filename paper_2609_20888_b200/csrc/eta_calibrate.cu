@@ -117,6 +117,15 @@ struct CalSmem {
     static constexpr size_t bytes(int n_bins) { return 1024 + 2 * K_BYTES + 8 * (size_t)n_bins; }
 };
 
+// Clears the histogram (512 KB at 32 heads x 2048 bins: latency).  A kernel of its own, not a memset: the next one is launched
+// while it runs and waits for it only when it adds to the histogram.  313 -> 310 us a calibration of 16 x 1024 tokens, 48.8 -> 48.1
+// of 8 x 700, the same within a run's spread for the smallest.
+__global__ void __launch_bounds__(256) calib_clear_kernel(uint4* __restrict__ p, int n16) {
+    pdl_trigger();
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k < n16) p[k] = make_uint4(0, 0, 0, 0);
+}
+
 // What bounds it: the shared-memory pipe (90 % of its passes), by the two atomics of a score: 3.55 passes each, which is what
 // 32 lanes on random banks take.  A row weight of up to 41 bits is added as two 32-bit numbers to two planes of the histogram,
 // w mod 2^16 and w / 2^16: 32-bit shared atomics without a return value are native, a 64-bit one is a compare-and-swap loop
@@ -188,6 +197,7 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
 
     // by threads that count only, all of them
     auto flush = [&]() {
+        pdl_wait();          // the histogram in memory has been cleared
         for (int b = tid; b < n_bins; b += 32 * CAL_WARPS) {
             const unsigned long long v = ((unsigned long long)hi[b] << CAL_SPLIT) + lo[b];
             if (v) {
@@ -435,9 +445,8 @@ static int launch_hist(const CUtensorMap& tmQ, const CUtensorMap& tmK, const flo
     const int rc = configure_kernel(reinterpret_cast<const void*>(calib_hist_kernel<D>), CalSmem<D>::bytes(4096));
     if (rc != ETA_OK) return rc;
     const dim3 grid((unsigned)Hq, (unsigned)n_seq, (unsigned)((T + CAL_ROWS - 1) / CAL_ROWS));
-    calib_hist_kernel<D><<<grid, CAL_THREADS, CalSmem<D>::bytes(n_bins), s>>>(tmQ, tmK, tau, Hq, Hkv, T, c2, scale, n_bins,
-                                                                               s_min, inv_w, hist, dpart);
-    return check_launch("calibration histogram");
+    return launch_pdl("calibration histogram", calib_hist_kernel<D>, grid, dim3(CAL_THREADS), CalSmem<D>::bytes(n_bins), s, tmQ, tmK,
+                      tau, Hq, Hkv, T, c2, scale, n_bins, s_min, inv_w, hist, dpart);
 }
 
 static size_t cal_align(size_t x) { return (x + 255) / 256 * 256; }
@@ -481,8 +490,7 @@ int eta_calibrate_head_const(int32_t n_seq, int32_t seq_len, int32_t n_q_heads, 
     const size_t hist_bytes = cal_align(sizeof(unsigned long long) * (size_t)n_q_heads * n_bins);
     double* dpart = reinterpret_cast<double*>(ws + hist_bytes);
     double* hc_d = reinterpret_cast<double*>(ws + hist_bytes + cal_align(sizeof(double) * (size_t)n_seq * n_q_heads * n_ttiles));
-    cudaError_t e = cudaMemsetAsync(hist, 0, hist_bytes, s);
-    if (e != cudaSuccess) { set_cuda_error(e, "calibration memset"); return ETA_ERR_CUDA; }
+    const int n16 = (int)(hist_bytes / 16);                            // at most 65535 heads x 4096 bins
 
     const float sc = scale > 0.f ? scale : 1.0f / sqrtf((float)head_dim);
     const float inv_w = (float)n_bins / (s_max - s_min);
@@ -490,6 +498,9 @@ int eta_calibrate_head_const(int32_t n_seq, int32_t seq_len, int32_t n_q_heads, 
     CUtensorMap tmQ, tmK;
     rc = cal_tmap(&tmQ, Q, (int64_t)n_seq * n_q_heads, seq_len, head_dim, CAL_ROWS);
     if (rc == ETA_OK) rc = cal_tmap(&tmK, K, (int64_t)n_seq * n_kv_heads, seq_len, head_dim, CAL_KEYS);
+    if (rc != ETA_OK) return rc;
+    calib_clear_kernel<<<(n16 + 255) / 256, 256, 0, s>>>(reinterpret_cast<uint4*>(hist), n16);
+    rc = check_launch("calibration clear");
     if (rc != ETA_OK) return rc;
     rc = (head_dim == 128 ? launch_hist<128> : launch_hist<64>)(tmQ, tmK, tau, n_q_heads, n_kv_heads, seq_len, n_seq, c2, sc,
                                                                n_bins, s_min, inv_w, hist, dpart, s);
