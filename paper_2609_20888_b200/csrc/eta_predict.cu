@@ -129,8 +129,11 @@ __global__ void __launch_bounds__(PRED_THREADS) predict_threshold_kernel(
 
 // Copy of a step's queries from page-locked host memory to device memory by a kernel: for a few tens of
 // kilobytes a kernel's loads over the interconnect cost less than setting up a copy engine.  The kernel never
-// signals its dependents early, so whatever follows it in the stream starts after the copy is complete.
+// signals its dependents early, so whatever follows it in the stream starts after the copy is complete.  It is launched
+// while the kernel before it ends and waits for it before it reads or writes: an eager step of 16K x 1 with its query and
+// output in host memory 33.2 -> 30.9 us, of 2K x 1 25.7 -> 24.5.
 __global__ void __launch_bounds__(256) stage_query_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n16) {
+    pdl_wait();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n16; k += gridDim.x * blockDim.x) {
         uint4 v;
         asm volatile("ld.global.cv.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(src + k));
@@ -149,11 +152,8 @@ extern "C" int eta_stage_query(int32_t batch, int32_t n_q_heads, int32_t head_di
     const int n16 = (int)(bytes / 16);
     int grid = (n16 + 255) / 256;
     if (grid > 296) grid = 296;
-    const int rc = eta::configure_kernel(reinterpret_cast<const void*>(eta::stage_query_kernel), 0);
-    if (rc != ETA_OK) return rc;
-    eta::stage_query_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const uint4*>(q_host),
-                                                                                 static_cast<uint4*>(q_dev), n16);
-    return eta::check_launch("eta_stage_query");
+    return eta::launch_pdl("eta_stage_query", eta::stage_query_kernel, dim3((unsigned)grid), dim3(256), 0, static_cast<cudaStream_t>(stream),
+                           static_cast<const uint4*>(q_host), static_cast<uint4*>(q_dev), n16);
 }
 
 extern "C" int eta_predict_threshold(int32_t batch, int32_t n_q_heads, int32_t head_dim, const void* q,
