@@ -358,9 +358,9 @@ __device__ __forceinline__ double2 block_sum2_fixed(double a, double b, double2*
 // gap between two clusters of scores), every c of the plateau solves the equation: only halvings are taken there, which end
 // at the plateau's lower end, for a density of 1 at the bracket's.
 __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
-    const unsigned long long* __restrict__ hist, const double* __restrict__ dpart, int Hq, int n_seq, int n_ttiles,
-    int T, int n_bins, double s_min, double s_max, double beta, int iters, float* __restrict__ head_const,
-    float* __restrict__ dbar_out, double* __restrict__ head_const_d) {
+    const unsigned long long* hist, const double* dpart, int Hq, int n_seq, int n_ttiles, int T, int n_bins, double s_min,
+    double s_max, double beta, int iters, float* __restrict__ head_const, float* __restrict__ dbar_out,
+    double* __restrict__ head_const_d) {
     extern __shared__ unsigned char bis_raw[];
     double* Hn = reinterpret_cast<double*>(bis_raw);
     __shared__ double2 scratch[CAL_BISECT_THREADS / 32];
@@ -371,7 +371,11 @@ __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
 
     // total weight (an integer: exact whatever the order), then the normalised histogram
     unsigned long long part = 0;
-    for (int b = tid; b < n_bins; b += CAL_BISECT_THREADS) part += Hh[b];
+    for (int b = tid; b < n_bins; b += CAL_BISECT_THREADS) {
+        const unsigned long long v = __ldcg(Hh + b);
+        Hn[b] = (double)v;
+        part += v;
+    }
 #pragma unroll
     for (int s = 16; s >= 1; s >>= 1) part += __shfl_xor_sync(0xffffffffu, part, s);
     if ((tid & 31) == 0) s_tot[tid >> 5] = part;
@@ -380,12 +384,12 @@ __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
 #pragma unroll
     for (int w = 0; w < CAL_BISECT_THREADS / 32; ++w) part += s_tot[w];
     const double tot = (double)part;
-    for (int b = tid; b < n_bins; b += CAL_BISECT_THREADS) Hn[b] = tot > 0.0 ? (double)Hh[b] / tot : 0.0;
+    for (int b = tid; b < n_bins; b += CAL_BISECT_THREADS) Hn[b] = tot > 0.0 ? Hn[b] / tot : 0.0;
     // target density: partial sums of every (sequence, tile) of this head, in a fixed order
     double d = 0.0;
     for (int k = tid; k < n_seq * n_ttiles; k += CAL_BISECT_THREADS) {
         const int x = k / n_ttiles, tt = k % n_ttiles;
-        d += dpart[((int64_t)x * Hq + h) * n_ttiles + tt];
+        d += __ldcg(dpart + ((int64_t)x * Hq + h) * n_ttiles + tt);
     }
     const double target = block_sum2_fixed(d, 0.0, scratch).x / ((double)n_seq * (double)T);
 

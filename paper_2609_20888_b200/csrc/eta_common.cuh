@@ -176,6 +176,10 @@ inline int launch_pdl(const char* what, void (*kernel)(KArgs...), dim3 grid, dim
 
 // Programmatic dependent launch: let the next kernel of the stream start its prologue now / wait until the
 // previous kernel of the stream has completed and its writes are visible.
+//
+// What that kernel may have written is read behind the wait, with __ldcg or a bulk copy, through a pointer that is not
+// `const T* __restrict__`: such a parameter, like __ldg, promises data that nobody writes while this kernel runs, and this
+// kernel runs while its predecessor still does.  Only what was complete before the launch may be read that way.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -468,7 +468,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 // paged cache: the page that holds the unit's block of tokens (one more dependent load per batch,
                 // hidden like the list fetch behind the tiles already on their way)
                 if (a.block_table)
-                    page = __ldg(a.block_table + (int64_t)a.div_hkv.div(r) * a.table_stride + (ent & 0xffffff));
+                    page = __ldcg(a.block_table + (int64_t)a.div_hkv.div(r) * a.table_stride + (ent & 0xffffff));
             }
         };
         if (u0 >= u1) {
@@ -657,7 +657,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 if (head) v = __ldg(reinterpret_cast<const uint4*>(qp + 64 * hf + 32 * m + 8 * t));
                 qa[hf][m][0] = v.x; qa[hf][m][1] = v.y; qa[hf][m][2] = v.z; qa[hf][m][3] = v.w;
             }
-        te = head ? __ldg(a.tau_eff + (int64_t)i * a.Hq + hk * a.G + g) : 0.f;
+        te = head ? __ldcg(a.tau_eff + (int64_t)i * a.Hq + hk * a.G + g) : 0.f;
         q_row = r;
     };
     if (!mbar_wait(laybar, 0)) {

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(PRED_THREADS) predict_threshold_kernel(
 // signals its dependents early, so whatever follows it in the stream starts after the copy is complete.  It is launched
 // while the kernel before it ends and waits for it before it reads or writes: an eager step of 16K x 1 with its query and
 // output in host memory 33.2 -> 30.9 us, of 2K x 1 25.7 -> 24.5.
-__global__ void __launch_bounds__(256) stage_query_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n16) {
+__global__ void __launch_bounds__(256) stage_query_kernel(const uint4* src, uint4* __restrict__ dst, int n16) {
     pdl_wait();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n16; k += gridDim.x * blockDim.x) {
         uint4 v;

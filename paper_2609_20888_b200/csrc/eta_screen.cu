@@ -88,7 +88,7 @@ __device__ __forceinline__ float qtab_unscale(float qn) {
 
 // Every thread of the CTA calls this with the row's G queries; the first D threads (J warps) work.
 template <int D, int G>
-__device__ __forceinline__ void build_qtab(QTab<D, G>& tab, const __nv_bfloat16* __restrict__ q, int tid) {
+__device__ __forceinline__ void build_qtab(QTab<D, G>& tab, const __nv_bfloat16* q, int tid) {
     constexpr int J = D / 32;
     const bool mine = tid < D;
     const int j = tid >> 5, hd = (tid & 31) >> 2, t = tid & 3;
@@ -96,7 +96,7 @@ __device__ __forceinline__ void build_qtab(QTab<D, G>& tab, const __nv_bfloat16*
     float x[8];
     if (mine) {
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (head < G) v = __ldg(reinterpret_cast<const uint4*>(q + head * D + 8 * (4 * j + t)));
+        if (head < G) v = __ldcg(reinterpret_cast<const uint4*>(q + head * D + 8 * (4 * j + t)));
         if (hd < G) tab.raw[hd * (D / 8) + 4 * j + t] = v;
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
         float n2 = 0.f;
@@ -238,7 +238,7 @@ __device__ __forceinline__ bool bound_tile(const QTab<D, G>& tab, uint32_t recs,
 // Bound of one record by one warp in plain fp32, for all heads of the group (queries in shared memory): 32 / (D / 8) heads
 // side by side.
 template <int D, int G, bool PACKED>
-__device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const unsigned char* __restrict__ src,
+__device__ __forceinline__ void bound_one(const uint4* __restrict__ qw, const unsigned char* src,
                                           float mn, float z, float scale, float* __restrict__ sb) {
     constexpr int LPR = D / 8, HP = 32 / LPR;
     const int lane = threadIdx.x & 31, cl = lane % LPR, sub = lane / LPR;
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4
             if (tl && tid == 0) tl[3] = globaltimer_ns();
             if (!dense && lane < G) {
                 const int h = hk * G + lane;
-                te_l = (a.tau ? __ldcg(a.tau + (int64_t)i * a.Hq + h) : __ldg(a.head_const + h)) - a.a;
+                te_l = (a.tau ? __ldcg(a.tau + (int64_t)i * a.Hq + h) : __ldcg(a.head_const + h)) - a.a;
             }
         }
         // the newest block's bound again, while the thresholds are on their way
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4
                     const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
                     if (m[half] && rank + __popc(nz & ((1u << lane) - 1u)) < a.prefetch) {
                         const int j = j0 + half * 32 + lane;
-                        const int w4 = a.block_table ? __ldg(a.block_table + (int64_t)i * a.table_stride + j) : i;
+                        const int w4 = a.block_table ? __ldcg(a.block_table + (int64_t)i * a.table_stride + j) : i;
                         for (int k = 0; k < a.tiles; ++k) {
                             const int y = (a.block_table ? 0 : j * a.b) + k * a.tile_tokens;
                             tma_prefetch_5d(&tmK, 0, y, 0, hk, w4);
@@ -641,9 +641,8 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4
 // two dependent reads, then as many for a head that needs rescue).  The largest of the CTAs' bounds decides; the rescued block
 // joins lists that are already written.  A block another head fetches anyway gets the head's bit, any other goes to the end
 // of its segment's list.
-__global__ void __launch_bounds__(256) rescue_kernel(const int2* __restrict__ span, const int2* __restrict__ best,
-                                                     const float* __restrict__ tau_eff, int G, int nb_cap, int nseg, int gpr,
-                                                     uint8_t* sel_mask, uint8_t* seg_cnt, int32_t* seg_list) {
+__global__ void __launch_bounds__(256) rescue_kernel(const int2* span, const int2* best, const float* tau_eff, int G, int nb_cap,
+                                                     int nseg, int gpr, uint8_t* sel_mask, uint8_t* seg_cnt, int32_t* seg_list) {
     __shared__ int s_block[8];            // rescued block of each head, or -1
     const int r = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_trigger();
@@ -687,9 +686,8 @@ __global__ void __launch_bounds__(256) rescue_kernel(const int2* __restrict__ sp
 // every record G times in 2-byte pieces and reduced three sums over 32 lanes for each.
 template <int D, int G, bool PACKED>
 __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
-    const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ musig, const float* __restrict__ mnorm,
-    const int32_t* __restrict__ seq_lens, int Hq, int Hkv, int b, int t_cap, int nb_cap, int per, int chunks, float z,
-    float scale, float* __restrict__ bound) {
+    const __nv_bfloat16* q, const unsigned char* musig, const float* mnorm, const int32_t* seq_lens, int Hq, int Hkv, int b,
+    int t_cap, int nb_cap, int per, int chunks, float z, float scale, float* __restrict__ bound) {
     using L = ScreenSmem<D, G>;
     using TL = TileOf<D>;
     extern __shared__ unsigned char scr_raw[];
@@ -703,7 +701,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     // 3.2 -> 2.4 for 64.  (It lets no successor start early: the screening kernel reads its inputs without waiting for them.  The
     // summary build, with CTAs by the ten thousand, is slower this way: 165 -> 210 us for 1.07 GB.)
     pdl_wait();
-    int T = __ldg(seq_lens + i);
+    int T = __ldcg(seq_lens + i);
     T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
     const int NB = min(T / b, nb_cap);
     const int first = (blockIdx.x % chunks) * per * TL::PASS;
@@ -730,9 +728,8 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
 // The same with a warp per (sequence, query head, block): for arrays that 16-byte loads cannot read (a caller's odd offset), and
 // for few bounds, where warps fill the GPU and tiles do not (what counts is then the length of one tile's chain of steps).
 __global__ void __launch_bounds__(128) score_dual_warp_kernel(
-    const __nv_bfloat16* __restrict__ q, const unsigned char* __restrict__ musig, const float* __restrict__ mnorm,
-    const int32_t* __restrict__ seq_lens, int B, int Hq, int Hkv, int d, int b, int t_cap, int nb_cap, float z,
-    float scale, int packed, float* __restrict__ bound) {
+    const __nv_bfloat16* q, const unsigned char* musig, const float* mnorm, const int32_t* seq_lens, int B, int Hq, int Hkv,
+    int d, int b, int t_cap, int nb_cap, float z, float scale, int packed, float* __restrict__ bound) {
     const int64_t wid = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     pdl_wait();
@@ -740,7 +737,7 @@ __global__ void __launch_bounds__(128) score_dual_warp_kernel(
     const int j = (int)(wid % nb_cap);
     const int h = (int)((wid / nb_cap) % Hq);
     const int i = (int)(wid / ((int64_t)nb_cap * Hq));
-    int T = seq_lens[i];
+    int T = __ldcg(seq_lens + i);
     T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
     if (j >= T / b) return;
     const int G = Hq / Hkv;
@@ -748,15 +745,15 @@ __global__ void __launch_bounds__(128) score_dual_warp_kernel(
     const __nv_bfloat16* qv = q + ((int64_t)i * Hq + h) * d;
     float dot = 0.f, var = 0.f, n2 = 0.f;
     for (int c = lane; c < d; c += 32) {
-        const float x = __bfloat162float(qv[c]);
+        const float x = __bfloat162float(__ldcg(qv + c));
         const unsigned char* rp = musig + rec * (packed ? 3 * d : 4 * d);
-        const float m = __half2float(reinterpret_cast<const __half*>(rp)[c]);
+        const float m = __half2float(__ldcg(reinterpret_cast<const __half*>(rp) + c));
         float s;
         if (packed) {
-            const uint32_t h2 = e4m3x2_to_f16x2(rp[2 * d + c]);
+            const uint32_t h2 = e4m3x2_to_f16x2(__ldcg(rp + 2 * d + c));
             s = __half2float(*reinterpret_cast<const __half*>(&h2));
         } else {
-            s = __half2float(reinterpret_cast<const __half*>(rp)[d + c]);
+            s = __half2float(__ldcg(reinterpret_cast<const __half*>(rp) + d + c));
         }
         dot = fmaf(x, m, dot);
         var = fmaf(x * x, s * s, var);
@@ -767,7 +764,7 @@ __global__ void __launch_bounds__(128) score_dual_warp_kernel(
         var += __shfl_xor_sync(0xffffffffu, var, s);
         n2 += __shfl_xor_sync(0xffffffffu, n2, s);
     }
-    if (lane == 0) bound[wid] = scale * min_keep_nan(dot + z * sqrtf(var), sqrtf(n2) * mnorm[rec]);
+    if (lane == 0) bound[wid] = scale * min_keep_nan(dot + z * sqrtf(var), sqrtf(n2) * __ldcg(mnorm + rec));
 }
 
 // ------------------------------------------------------------------ launchers (host)

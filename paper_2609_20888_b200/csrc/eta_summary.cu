@@ -167,8 +167,9 @@ __device__ __forceinline__ void summarize_block_onepass(const __nv_bfloat16* __r
 }
 
 // b is a multiple of 8 * (rows per warp instruction) for every supported block size, so the loops need no guards.
-template <int D, bool envelope>
-__device__ __forceinline__ void summarize_block_t(const __nv_bfloat16* __restrict__ blk, int64_t stride_t, int b,
+// FRESH: the keys may have been written by the kernel before this one, which this one was launched beside (the append).
+template <int D, bool envelope, bool FRESH>
+__device__ __forceinline__ void summarize_block_t(const __nv_bfloat16* blk, int64_t stride_t, int b,
                                                   unsigned char* __restrict__ rec, bool packed, float* __restrict__ mn) {
     constexpr int LPR = D / 8;        // lanes per row
     constexpr int RPP = 32 / LPR;     // rows per pass
@@ -186,7 +187,8 @@ __device__ __forceinline__ void summarize_block_t(const __nv_bfloat16* __restric
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             int t = t0 + u * RPP;
-            v[u] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)t * stride_t));
+            const uint4* p = reinterpret_cast<const uint4*>(base + (int64_t)t * stride_t);
+            v[u] = FRESH ? __ldcg(p) : __ldg(p);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -225,7 +227,8 @@ __device__ __forceinline__ void summarize_block_t(const __nv_bfloat16* __restric
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             int t = t0 + u * RPP;
-            v[u] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)t * stride_t));
+            const uint4* p = reinterpret_cast<const uint4*>(base + (int64_t)t * stride_t);
+            v[u] = FRESH ? __ldcg(p) : __ldg(p);
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -279,7 +282,7 @@ template <int D>
 __device__ __forceinline__ void summarize_block(const __nv_bfloat16* __restrict__ blk, int64_t stride_t, int b,
                                                 bool envelope, unsigned char* __restrict__ rec, bool packed,
                                                 float* __restrict__ mn, uint64_t policy) {
-    if (envelope) summarize_block_t<D, true>(blk, stride_t, b, rec, packed, mn);
+    if (envelope) summarize_block_t<D, true, false>(blk, stride_t, b, rec, packed, mn);
     else summarize_block_onepass<D>(blk, stride_t, b, rec, packed, mn, policy);
 }
 
@@ -314,9 +317,9 @@ __global__ void __launch_bounds__(128, 8) build_summaries_kernel(
 // in the L2) to 1.8 us after the rows are parked, against 1.3 to 3.2 us with one warp for all coordinates.
 template <int D>
 __global__ void __launch_bounds__(128) append_summary_kernel(
-    const __nv_bfloat16* __restrict__ K, int64_t sb, int64_t sh, int64_t st, int Hkv, int b, int t_cap, int nb_cap,
-    int rows, const int32_t* __restrict__ seq_lens, int mode, unsigned char* __restrict__ musig,
-    float* __restrict__ mnorm, const int32_t* __restrict__ table, int table_stride, unsigned long long* timeline) {
+    const __nv_bfloat16* K, int64_t sb, int64_t sh, int64_t st, int Hkv, int b, int t_cap, int nb_cap, int rows,
+    const int32_t* seq_lens, int mode, unsigned char* __restrict__ musig, float* __restrict__ mnorm, const int32_t* table,
+    int table_stride, unsigned long long* timeline) {
     constexpr int LPR = D / 8;            // lanes per row
     constexpr int RPP = 32 / LPR;         // rows per warp instruction
     constexpr int RPC = 128 / LPR;        // rows per CTA instruction
@@ -332,11 +335,11 @@ __global__ void __launch_bounds__(128) append_summary_kernel(
     pdl_wait();
     pdl_trigger();       // nothing later in a decode step needs this kernel's output before it has waited for it
     const int i = r / Hkv, hk = r % Hkv;
-    const int T = seq_lens[i];
+    const int T = __ldcg(seq_lens + i);
     if (T <= 0 || T > t_cap || T % b != 0) return;
     const int j = T / b - 1;
     if (j >= nb_cap) return;
-    const __nv_bfloat16* blk = table ? K + (int64_t)table[(int64_t)i * table_stride + j] * sb + hk * sh
+    const __nv_bfloat16* blk = table ? K + (int64_t)__ldcg(table + (int64_t)i * table_stride + j) * sb + hk * sh
                                      : K + i * sb + hk * sh + (int64_t)j * b * st;
     const int64_t rec = (int64_t)r * nb_cap + j;
     const bool packed = (mode & 2) != 0;      // mode: bit 0 sub-block envelope, bit 1 packed records
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(128) append_summary_kernel(
     if (tl && tid == 0) tl[1] = globaltimer_ns();
     if (mode & 1) {
         // the sub-block envelope keeps its own (two-pass, single-warp) routine
-        if (warp == 0) summarize_block_t<D, true>(blk, st, b, recp, packed, mnorm + rec);
+        if (warp == 0) summarize_block_t<D, true, true>(blk, st, b, recp, packed, mnorm + rec);
         return;
     }
     // ---- all four warps: the whole block in flight at once, parked in shared memory; then the norms of the rows a
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(128) append_summary_kernel(
         uint4 v[MAXL];
 #pragma unroll
         for (int u = 0; u < MAXL; ++u)
-            if (t_first + u * RPC < b) v[u] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)(t_first + u * RPC) * st));
+            if (t_first + u * RPC < b) v[u] = __ldcg(reinterpret_cast<const uint4*>(base + (int64_t)(t_first + u * RPC) * st));
 #pragma unroll
         for (int u = 0; u < MAXL; ++u)
             if (t_first + u * RPC < b) s_rows[(t_first + u * RPC) * LPR + cc] = v[u];
