@@ -120,7 +120,11 @@ __global__ void __launch_bounds__(PRED_THREADS) predict_threshold_kernel(
         float s = 0.f;
 #pragma unroll
         for (int c = 0; c < PRED_CLUSTER; ++c) s += cpart[c * Hq + threadIdx.x];
-        tau[(int64_t)i * Hq + threadIdx.x] = s + bias[threadIdx.x];
+        s += bias[threadIdx.x];
+        // The kernel in front may still be running (a merge releases its successor as it starts), and the thresholds may go where
+        // it writes or reads: an output whose memory has been given back, say.
+        pdl_wait();
+        tau[(int64_t)i * Hq + threadIdx.x] = s;
     }
     if (tl && threadIdx.x == 0) tl[4] = globaltimer_ns();
     if (threadIdx.x == 0) pdl_wait();
@@ -181,8 +185,8 @@ extern "C" int eta_predict_threshold(int32_t batch, int32_t n_q_heads, int32_t h
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     // the predictor reads nothing an earlier kernel of the stream writes, so it may run beside its predecessor
-    // (typically the summary append); it only waits for it before it exits, which keeps "this kernel is complete"
-    // meaning "everything before it is complete" for whoever comes next
+    // (typically the summary append); it waits for it before it stores the thresholds, which also keeps "this kernel is
+    // complete" meaning "everything before it is complete" for whoever comes next
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = eta::pdl_enabled() ? 1 : 0;
     cfg.attrs = attr;

@@ -50,3 +50,51 @@ def test_queued_steps_equal_separate_steps(B, Hq, Hkv, d, b, T, frozen):
 
     for a, c in zip(run(True), run(False)):
         assert torch.equal(a, c)
+
+
+def _aligned(eb, desc, dev):
+    ws = torch.zeros(eb.eta_workspace_bytes(desc) + 256, dtype=torch.uint8, device=dev)
+    return ws[-ws.data_ptr() % 256:]
+
+
+def _both_ways(run):
+    """The results of run(after), bit for bit the same with a synchronisation after every call (after()) and without any."""
+    torch.cuda.synchronize()
+    want = [t.clone() for t in run(torch.cuda.synchronize)]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        got = run(lambda: None)
+        torch.cuda.synchronize()
+        for a, c in zip(want, got):
+            assert torch.equal(a, c)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d", [(1, 8, 2, 64), (16, 32, 8, 128), (64, 16, 4, 64)])
+def test_thresholds_written_where_the_step_before_left_its_output(B, Hq, Hkv, d):
+    """A predictor queued right behind a step, with its thresholds in memory that the step's output has just been in (as an
+    allocator hands it out): what the later call writes is what stays."""
+    from paper_2609_20888_b200 import binding as eb
+    dev, b, T = "cuda:0", 32, 900
+    g = torch.Generator(device=dev).manual_seed(B)
+    randn = lambda *s: torch.randn(s, generator=g, device=dev)
+    K, V, q = randn(B, Hkv, T, d).bfloat16(), randn(B, Hkv, T, d).bfloat16(), randn(B, Hq, d).bfloat16()
+    W, bias = 0.1 * randn(Hq * d, Hq), torch.full((Hq,), 0.8, device=dev)
+    lens = torch.full((B,), T, dtype=torch.int32, device=dev)
+    desc = eb.cache_desc(K, V, Hq, b)
+    ws = _aligned(eb, desc, dev)
+    musig, mnorm = eb.alloc_summaries(desc, dev)
+    eb.eta_build_block_summaries(desc, K, lens, musig, mnorm)
+    sel = torch.zeros(B, Hkv, desc.nb_cap, dtype=torch.uint8, device=dev)
+
+    def run(after):
+        tau = []
+        for _ in range(20):
+            out = torch.zeros(B, Hq, d, device=dev)
+            eb.eta_decode(desc, eb.DecodeParams(), q, K, V, lens, musig, mnorm, None, bias, out, sel, ws)
+            after()
+            tau.append(out.view(-1)[:B * Hq].view(B, Hq))
+            eb.eta_predict_threshold(q, W, bias, tau[-1])
+            after()
+        return [torch.stack(tau)]
+
+    _both_ways(run)
