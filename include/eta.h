@@ -142,8 +142,9 @@ int eta_append_summary(const eta_cache_desc* desc, const void* K, const int32_t*
  * [batch, n_q_heads, head_dim] in page-locked host memory that the device can address (cudaHostAlloc /
  * cudaHostRegister; with unified addressing the host pointer itself); q_dev: the same shape in device memory.
  * Both 16-byte aligned, the size a multiple of 16 bytes (else ETA_ERR_UNSUPPORTED).  Ordered like any kernel on
- * `stream`; the calls that follow on the stream see the complete copy.  The host buffer must stay unchanged until
- * the kernel has run.  In the same way `out` of eta_decode may be page-locked host memory: the merge kernel's
+ * `stream`; the calls that follow on the stream see the complete copy.  Launched with programmatic dependent launch: the
+ * kernel waits for everything before it in the stream before it reads or writes, and releases its successors only as it
+ * ends.  The host buffer must stay unchanged until the kernel has run.  In the same way `out` of eta_decode may be page-locked host memory: the merge kernel's
  * stores then go straight to the host and are visible once the stream has been synchronised.
  */
 int eta_stage_query(int32_t batch, int32_t n_q_heads, int32_t head_dim, const void* q_host, void* q_dev,
@@ -157,12 +158,15 @@ int eta_stage_query(int32_t batch, int32_t n_q_heads, int32_t head_dim, const vo
  * tau fp32 [batch, n_q_heads].  fp32 accumulation in a fixed order.
  * Launch order: the kernel is launched with programmatic dependent launch and reads
  * q, W and bias without waiting for the preceding kernel of the stream (it waits for
- * it only before it exits, so that its completion implies its predecessor's).  The
- * producer of q must therefore be complete when that preceding kernel starts: true
- * for copies, for kernels launched without early dependent release (eta_stage_query
- * and eta_append_summary's inputs among them) and for anything ordered by an event
- * or a synchronisation; a kernel that releases its dependents early and then writes
- * q would hand this call a stale query.
+ * it before it stores tau, so that its completion implies its predecessor's).  Their
+ * producers must therefore be complete before that preceding kernel releases its
+ * dependents.  That holds for copies; for the preceding kernel itself where it does
+ * not release early, since its dependents then start when it is complete
+ * (eta_stage_query, eta_score_dual, eta_calibrate_head_const, kernels launched without
+ * programmatic dependent launch); for everything in front of a kernel that waits
+ * before it releases (eta_append_summary); and for anything ordered by an event or a
+ * synchronisation.  A kernel that releases its dependents early and then writes q
+ * would hand this call a stale query.
  */
 int eta_predict_threshold(int32_t batch, int32_t n_q_heads, int32_t head_dim, const void* q,
                           const float* W, const float* bias, float* tau, void* stream);
@@ -173,7 +177,9 @@ int eta_predict_threshold(int32_t batch, int32_t n_q_heads, int32_t head_dim, co
  * bound fp32 [batch, n_q_heads, nb_cap]; entries of blocks that are not full are
  * left untouched.  Same arithmetic as the screening stage of eta_decode (packed
  * records with ETA_FLAG_PACKED_SIGMA in params->flags); meant for diagnostics
- * and for calibrating frozen constants, not for the hot loop.
+ * and for calibrating frozen constants, not for the hot loop.  Launched with
+ * programmatic dependent launch: the kernel waits for everything before it in the
+ * stream before it reads or writes, and releases its successors only as it ends.
  */
 int eta_score_dual(const eta_cache_desc* desc, const eta_params* params, const void* q,
                    const int32_t* seq_lens, const void* musig, const float* mnorm,
@@ -199,7 +205,10 @@ int eta_score_dual(const eta_cache_desc* desc, const eta_params* params, const v
  * A head whose density is NaN (a NaN threshold, or a bounded wait inside the kernel that
  * ran out) gets NaN for its constant as well.
  * workspace: eta_calibration_workspace_bytes() bytes, 256-byte aligned, no
- * initialisation needed.  Prefill-side tool: not part of a decode step.
+ * initialisation needed.  Its kernels are launched with programmatic dependent launch:
+ * the first waits for everything before it in the stream before it writes or lets
+ * another read, and the last releases its successors only as it ends.  Prefill-side
+ * tool: not part of a decode step.
  */
 int eta_calibration_workspace_bytes(int32_t n_seq, int32_t seq_len, int32_t n_q_heads, int32_t n_bins,
                                     size_t* out_bytes);
@@ -230,9 +239,8 @@ int eta_calibrate_head_const(int32_t n_seq, int32_t seq_len, int32_t n_q_heads, 
  * workspace: eta_workspace_bytes() bytes.
  * Launch order: the kernels are launched with programmatic dependent launch and read q, seq_lens and every
  * summary except the newest block's before they wait for the preceding kernel of the stream.  Producers of those
- * inputs must therefore be complete when that preceding kernel starts: true for copies, for kernels launched
- * without early dependent release (eta_stage_query among them) and for anything ordered by an event or a
- * synchronisation; only a kernel that releases its dependents early and then writes q would break it.
+ * inputs must therefore be complete before that preceding kernel releases its dependents, as described for
+ * eta_predict_threshold; only a kernel that releases its dependents early and then writes q would break it.
  */
 int eta_decode(const eta_cache_desc* desc, const eta_params* params, const void* q,
                const void* K, const void* V, const int32_t* seq_lens,
@@ -324,10 +332,11 @@ int eta_profile_read(float* ms, int n);
 const char* eta_profile_kernel_name(int k);
 
 /*
- * Launch policy (the paper has no counterpart).  By default the kernels of a decode step are launched with
- * programmatic dependent launch: each may start its set-up while its predecessor in the stream drains, and
- * waits for the predecessor's completion before reading anything it wrote.  eta_set_pdl(0) makes every launch
- * wait for the full completion of the previous one instead (for A/B timing and for debugging).  Process-wide.
+ * Launch policy (the paper has no counterpart).  By default every kernel but the summary build's is launched with
+ * programmatic dependent launch (the decode step's, the staged query's, the bounds' and the calibration's): each may
+ * start its set-up while its predecessor in the stream drains, and waits for the predecessor's completion before reading
+ * anything it wrote.  eta_set_pdl(0) makes every launch wait for the full completion of the previous one instead (for A/B
+ * timing and for debugging).  Process-wide.
  */
 int eta_set_pdl(int on);
 

@@ -133,9 +133,10 @@ __global__ void __launch_bounds__(PRED_THREADS) predict_threshold_kernel(
 
 // Copy of a step's queries from page-locked host memory to device memory by a kernel: for a few tens of
 // kilobytes a kernel's loads over the interconnect cost less than setting up a copy engine.  The kernel never
-// signals its dependents early, so whatever follows it in the stream starts after the copy is complete.  It is launched
-// while the kernel before it ends and waits for it before it reads or writes: an eager step of 16K x 1 with its query and
-// output in host memory 33.2 -> 30.9 us, of 2K x 1 25.7 -> 24.5.
+// signals its dependents early, so whatever follows it in the stream starts when it is complete, stores included
+// (griddepcontrol asks a dependent to wait where its prerequisite releases early; a fence here would cost a step 0.5 us).  It is
+// launched while the kernel before it ends and waits for it before it reads or writes: eager steps of 16K x 1 queued one after the
+// other, query and output in host memory, 33.1 -> 31.0 us, of 2K x 1 26.7 -> 24.8; one step by itself takes the same.
 __global__ void __launch_bounds__(256) stage_query_kernel(const uint4* src, uint4* __restrict__ dst, int n16) {
     pdl_wait();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n16; k += gridDim.x * blockDim.x) {
