@@ -118,9 +118,10 @@ struct CalSmem {
 };
 
 // Clears the histogram (512 KB at 32 heads x 2048 bins: latency).  A kernel of its own, not a memset: the next one is launched
-// while it runs and waits for it only when it adds to the histogram.  313 -> 310 us a calibration of 16 x 1024 tokens, 48.8 -> 48.1
-// of 8 x 700, the same within a run's spread for the smallest.  It is itself launched while the kernel before it ends (calls one
-// after the other: 2 x 64 tokens 24.8 -> 18.9, 8 x 128 21.0 -> 17.1, 8 x 700 48.1 -> 42.8).
+// while it runs and waits for it only when it adds to the histogram.  Calibrations of 16 x 1024 tokens (32 / 8 heads, d = 128, 2048
+// bins, as all figures here) 310.2 -> 307.2 us, 8 x 700 103.4 -> 101.6, 2 x 64 21.8 -> 20.2.  It is itself launched while the kernel
+// before it ends, which counts where calibrations are queued one after the other (8 x 700 101.6 -> 99.6, 8 x 128 22.7 -> 20.7, 2 x 64
+// 20.2 -> 18.1) and not for one by itself (22.5 for 2 x 64 either way).
 __global__ void __launch_bounds__(256) calib_clear_kernel(uint4* __restrict__ p, int n16) {
     pdl_wait();          // the next kernel reads the call's inputs at once: all before this one has to be complete first
     pdl_trigger();
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(256) calib_clear_kernel(uint4* __restrict__ p,
 // million passes, 4.7 are left).  One accumulator of 64 keys: the MMA of a tile runs while the second half of the tile before
 // it is counted.  Two of 32 keys with a barrier each (347 us a calibration, against 313) cost more than they hide, two of 64
 // do not fit the tensor memory of three CTAs beside the queries.  Four CTAs at 56 registers: 321.  With 2048 bins: 515 -> 333 (queries in shared memory) ->
-// 313 us, of which the histogram 435 -> 290.
+// 313 us, of which the histogram 435 -> 290; with the launches and the root of today 305.
 template <int D>
 __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
     const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const float* __restrict__ tau,
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
         }
         meet();
         flush();
-        pdl_trigger();       // the root search is launched while the last CTAs end: 27.5 -> 24.8 us a calibration of 2 x 64 tokens, 49.8 -> 48.8 of 8 x 700
+        pdl_trigger();       // the root search is launched while the last CTAs end: a calibration of 2 x 64 tokens 24.3 -> 21.8 us, 8 x 700 105.7 -> 103.4
         // density contribution of this tile: sum over its rows of (1/t) * (sum of the row's gates), fixed order
 #pragma unroll
         for (int row = 0; row < 2; ++row) {
@@ -350,8 +351,8 @@ __device__ __forceinline__ double2 block_sum2_fixed(double a, double b, double2*
 }
 
 // A serial chain of evaluations of g, each n_bins double-precision sigmoids: what counts is how many there are.  The root
-// is found by Newton steps inside a bracket, with a halving wherever a step would leave the bracket or shrink too slowly:
-// about eight evaluations to double precision where plain halving took eighty (177 us with halving alone).  What matters most is
+// is found by Newton steps inside a bracket, with a halving wherever a step would leave the bracket or shrink too slowly: four to
+// seven evaluations for thresholds among the scores (twelve in their tail) where plain halving took eighty (177 us).  What matters most is
 // to stop at the root: a step of less than the rounding of c leaves c at an end of the bracket, and the halving that used to
 // follow started over, on the unluckiest head for eighty evaluations (54 -> 15 us).  1024 threads are 6 us slower than 512.
 // Where g is so flat that its own rounding moves the root by more than float's rounding of c (a density of exactly 1 or 0, a
@@ -417,7 +418,7 @@ __global__ void __launch_bounds__(CAL_BISECT_THREADS) calib_bisect_kernel(
         const double cn = c + f / slope, tol = 1e-15 * (fabs(lo) + fabs(hi) + w);
         // at the root, to rounding: c may now be an end of the bracket, which the step below must not leave by a halving
         // (|g''| <= beta |g'|, so a step of d leaves beta d^2 / 2: below a 2^-52 of 1 / beta here.  Going round once more to see the
-        // step shrink below rounding cost an evaluation or two: 52 -> 50 us a calibration of 8 x 700 tokens, 38.5 -> 35.4 of 2 x 300.)
+        // step shrink below rounding cost an evaluation: a calibration of 8 x 700 tokens 107.8 -> 105.7 us, 2 x 300 33.3 -> 31.2.)
         if (!flat && (fabs(cn - c) <= tol || beta * fabs(cn - c) <= 2e-8)) { c = cn; break; }
         double next;
         if (!flat && cn > lo && cn < hi && 2.0 * fabs(f) <= fabs(dx_old * slope)) {

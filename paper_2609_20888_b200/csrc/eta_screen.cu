@@ -682,8 +682,8 @@ __global__ void __launch_bounds__(256) rescue_kernel(const int2* span, const int
 
 // Eq. dual_bound_eq for every block, for its own sake: the tiles of the screening kernel, stored instead of compared.
 // Bound by HBM (33.8 MB of records in, 8.4 MB of bounds out at 65536 blocks, d = 128, G = 4: 6.4 us at the copy rate); a
-// record is read once for all heads of its group.  10.5 us there, against 108 us with a warp per (head, block) that read
-// every record G times in 2-byte pieces and reduced three sums over 32 lanes for each.
+// record is read once for all heads of its group.  12.2 us there for the kernel alone, against 108 us with a warp per (head,
+// block) that read every record G times in 2-byte pieces and reduced three sums over 32 lanes for each.
 template <int D, int G, bool PACKED>
 __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     const __nv_bfloat16* q, const unsigned char* musig, const float* mnorm, const int32_t* seq_lens, int Hq, int Hkv, int b,
@@ -697,9 +697,11 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF) + 2 * warp;
     float* const sb = reinterpret_cast<float*>(sm + L::TILE_OFF + SCR_WARPS * TL::BYTES) + warp * TL::RECS * G;
     const int r = blockIdx.x / chunks, i = r / Hkv, hk = r % Hkv;
-    // Launched while the kernel before it ends, which it waits for before it reads anything: 12.3 -> 10.5 us a call for 65536 blocks,
-    // 3.2 -> 2.4 for 64.  (It lets no successor start early: the screening kernel reads its inputs without waiting for them.  The
-    // summary build, with CTAs by the ten thousand, is slower this way: 165 -> 210 us for 1.07 GB.)
+    // Launched while the kernel before it ends, which it waits for before it reads anything.  That is worth the gap between two
+    // kernels and no more: calls queued one after the other 12.3 -> 10.0 us each for 65536 blocks (9.9 -> 9.7 as nodes of a graph, 64
+    // bounds 2.3 -> 2.2), a call by itself 14.4 between two events either way.  (It lets no successor start early: the screening kernel
+    // reads its inputs without waiting for them.  The summary build, with CTAs by the ten thousand, is slower this way: 174 -> 218 us
+    // for 1.07 GB, three inputs in turn.)
     pdl_wait();
     int T = __ldcg(seq_lens + i);
     T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
