@@ -167,6 +167,17 @@ def heads_without_near_tie(near, batch, n_q_heads):
     return keep
 
 
+def calibration_scratch(ws, n_seq, n_q_heads, seq_len, n_bins, tile=128):
+    """What a calibration leaves in its scratch (private to the library: this is the one place that knows where): integer
+    histogram [Hq, n_bins], density contributions [n_seq, Hq, tiles of `tile` queries], constants [Hq] in double."""
+    n_tiles, at, parts = -(-seq_len // tile), 0, []
+    for shape, t in (((n_q_heads, n_bins), torch.int64), ((n_seq, n_q_heads, n_tiles), torch.float64), ((n_q_heads,), torch.float64)):
+        n = 8 * int(np.prod(shape))
+        parts.append(ws[at:at + n].view(t).cpu().numpy().reshape(shape))
+        at += (n + 255) // 256 * 256
+    return parts
+
+
 def fp16_ulp_distance(a_bits, b_bits):
     """Distance in units in the last place between fp16 bit patterns (sign-magnitude aware)."""
     def key(x):

@@ -8,6 +8,8 @@ import numpy as np
 import pytest
 import torch
 
+from tests.helpers import calibration_scratch
+
 pytestmark = pytest.mark.gpu
 
 
@@ -34,13 +36,8 @@ def test_root_of_the_density_equation(n_bins, beta, mean):
     hc, dbar = torch.empty(Hq, device=dev), torch.empty(Hq, device=dev)
     ws = eb.eta_calibrate_head_const(Q, K, tau, hc, dbar, beta=beta, n_bins=n_bins, s_min=-lim, s_max=lim)
     torch.cuda.synchronize()
-    up = lambda n: (n + 255) // 256 * 256  # noqa: E731
-    n_tt = (T + 127) // 128
-    at = up(8 * Hq * n_bins)
-    H = ws[:8 * Hq * n_bins].view(torch.int64).cpu().numpy().reshape(Hq, n_bins).astype(np.float64)
-    parts = ws[at:at + 8 * n_seq * Hq * n_tt].view(torch.float64).cpu().numpy().reshape(n_seq, Hq, n_tt)
-    at += up(8 * n_seq * Hq * n_tt)
-    got = ws[at:at + 8 * Hq].view(torch.float64).cpu().numpy()
+    H, parts, got = calibration_scratch(ws, n_seq, Hq, T, n_bins)
+    H = H.astype(np.float64)
     s = -lim + (np.arange(n_bins) + 0.5) * (2 * lim / n_bins)
     for h in range(Hq):
         Hn, target = H[h] / H[h].sum(), parts[:, h].sum() / (n_seq * T)
