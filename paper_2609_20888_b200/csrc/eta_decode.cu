@@ -30,7 +30,7 @@
 // (row, head, slice of head_dim).
 #include <cuda.h>
 
-#include "eta_common.cuh"
+#include "eta_attend.cuh"
 #include "eta_timeline.h"
 
 namespace eta {
@@ -60,7 +60,6 @@ struct DecodeArgs {
 };
 
 constexpr uint32_t UF_END = 1u;
-constexpr int WARPS_PER_GROUP = 4;     // the four warps of a group each take a quarter of a tile's tokens
 // Tiles a row boundary inside a CTA's range is worth (flush of the partials, query reload, a pipeline that runs dry
 // while a group flushes).  Measured: 3 left the CTAs with several pieces last by 8 us on the mixed-length
 // configuration (128 rows); 6, 8, 10 and 14 are within noise of each other on every configuration.  Where that would
@@ -72,19 +71,6 @@ constexpr int LGRAN = 8;               // granules per lane of a chunk
 constexpr int CHUNK = 32 * LGRAN;      // granules of a chunk: what a warp reads in one round trip
 constexpr int MAX_SUPER = 512;         // sums over `super` chunks each, kept in shared memory when there is more than one chunk
 constexpr int SPAN_ROWS = 64;          // rows a CTA publishes at a time
-
-__device__ __forceinline__ uint32_t u4_get(const uint4& v, int i) {
-    return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
-}
-// token row inside an 8-row group that MMA column n reads: bits 0 and 2 of n swapped, so that the two
-// rows a quarter-warp touches in one 16-byte load sit in different halves of the swizzle pattern
-__device__ __forceinline__ int rho(int n) { return (n & 2) | ((n & 1) << 2) | ((n >> 2) & 1); }
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 
 // sum of the 16 survivor counts of a granule
 __device__ __forceinline__ int granule_sum(const uint4& v) {
@@ -119,10 +105,7 @@ __global__ void __launch_bounds__(32 * (WARPS_PER_GROUP * NGROUPS + 1), 1)
 decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const DecodeArgs a) {
     using L = DecodeSmem<D, TS, NSTAGE, NGROUPS>;
     constexpr int HALVES = L::HALVES;
-    constexpr int WT = TS / WARPS_PER_GROUP;    // tokens per consumer warp per tile (8 or 16)
-    constexpr int NT = WT / 8;                  // 8-token MMA column tiles per warp
     constexpr int PRODUCER_WARP = WARPS_PER_GROUP * NGROUPS;
-    static_assert(NT == 1 || NT == 2, "tile must give each warp 8 or 16 tokens");
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -616,30 +599,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const int fheads = min(a.G, L::FLUSH_HEADS);       // heads per round of a flush
     float* sm_o = reinterpret_cast<float*>(smem + L::MO_OFF) + group * WARPS_PER_GROUP * fheads * D;
     const int gtid = tid - group * 32 * WARPS_PER_GROUP;    // thread index inside the group
-    const int g = lane >> 2, t = lane & 3;
-    const int rb = wq * WT;                            // first token row of this warp inside a tile
-    const int r0 = rho(2 * t), r1 = rho(2 * t + 1);    // token rows (within an 8-group) of MMA columns 2t, 2t+1
-    const int vchunk = ((g & 1) << 2) | (g >> 1);      // 16-byte chunk of a V half-row this lane reads
     const float LOG2E = 1.4426950408889634f;
-    const bool head = g < a.G;
-
-    // byte offsets inside a half tile of the 16-byte pieces this lane reads (fixed for the whole kernel)
-    uint32_t koff[NT][2], voff[NT][2];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-        const int krow = rb + nt * 8 + rho(g);
-#pragma unroll
-        for (int m = 0; m < 2; ++m) koff[nt][m] = krow * 128 + (((4 * m + t) ^ (krow & 7)) << 4);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int vrow = rb + nt * 8 + (c ? r1 : r0);
-            voff[nt][c] = vrow * 128 + ((vchunk ^ (vrow & 7)) << 4);
-        }
-    }
-
-    uint32_t qa[HALVES][2][4];
-    float o[HALVES][4][4];
-    float m_run = -INFINITY, l_run = 0.f, te = 0.f;
+    Attend<D, TS> at(lane, wq, a.G);
     int row = -1, piece = -1, q_row = -1;
     uint32_t flush_phase = 0;
     bool ok = true;
@@ -648,16 +609,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     auto load_q = [&](int r) {
         int i, hk;
         a.div_hkv.divmod(r, i, hk);
-        const __nv_bfloat16* qp = a.q + ((int64_t)i * a.Hq + hk * a.G + (head ? g : 0)) * D;
-#pragma unroll
-        for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (head) v = __ldg(reinterpret_cast<const uint4*>(qp + 64 * hf + 32 * m + 8 * t));
-                qa[hf][m][0] = v.x; qa[hf][m][1] = v.y; qa[hf][m][2] = v.z; qa[hf][m][3] = v.w;
-            }
-        te = head ? __ldcg(a.tau_eff + (int64_t)i * a.Hq + hk * a.G + g) : 0.f;
+        const int h = hk * a.G + (at.head ? at.g : 0);
+        at.load_q(a.q + ((int64_t)i * a.Hq + h) * D);
+        at.te = at.head ? __ldcg(a.tau_eff + (int64_t)i * a.Hq + h) : 0.f;
         q_row = r;
     };
     if (!mbar_wait(laybar, 0)) {
@@ -684,21 +638,21 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         if (!end && new_piece != piece && ds.x != q_row) load_q(ds.x);
         if ((end || new_piece != piece) && piece >= 0) {
             // ---- this group's part of a piece is complete: combine its four warps and store (m, l, O) per head
-            float lsum = l_run + __shfl_xor_sync(0xffffffffu, l_run, 1);
+            float lsum = at.l_run + __shfl_xor_sync(0xffffffffu, at.l_run, 1);
             lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
-            if (t == 0) { sm_m[wq * 8 + g] = m_run; sm_l[wq * 8 + g] = lsum; }
+            if (at.t == 0) { sm_m[wq * 8 + at.g] = at.m_run; sm_l[wq * 8 + at.g] = lsum; }
             const int64_t slot = ((int64_t)blockIdx.x + row) * NGROUPS + group;
             for (int h0 = 0; h0 < a.G && ok; h0 += fheads) {
-                const int ha = 2 * t - h0, hb = ha + 1;         // this lane's two heads within the round
+                const int ha = 2 * at.t - h0, hb = ha + 1;         // this lane's two heads within the round
 #pragma unroll
                 for (int hf = 0; hf < HALVES; ++hf)
 #pragma unroll
                     for (int mt = 0; mt < 4; ++mt) {
-                        const int dcol = 64 * hf + 8 * vchunk + 2 * mt;
+                        const int dcol = 64 * hf + 8 * at.vchunk + 2 * mt;
                         if (ha >= 0 && ha < fheads)
-                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + ha) * D + dcol)) = make_float2(o[hf][mt][0], o[hf][mt][2]);
+                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + ha) * D + dcol)) = make_float2(at.o[hf][mt][0], at.o[hf][mt][2]);
                         if (hb >= 0 && hb < fheads)
-                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + hb) * D + dcol)) = make_float2(o[hf][mt][1], o[hf][mt][3]);
+                            *reinterpret_cast<float2*>(sm_o + ((wq * fheads + hb) * D + dcol)) = make_float2(at.o[hf][mt][1], at.o[hf][mt][3]);
                     }
 #ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
                 // test build only: one warp of the first CTA never arrives, so that the group's bounded wait runs out and
@@ -741,147 +695,16 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
 
         const int hmask = ds.z & 0xff, urow = (ds.z >> 8) & 0xff, nvalid = ds.w;
         const uint32_t kbase = smem_u32(smem + stage * L::STAGE_BYTES);
-        const uint32_t vbase = kbase + HALVES * L::TILE_BYTES;
 
         if (new_piece != piece) {
             piece = new_piece;
             row = ds.x;
             if (row != q_row) load_q(row);
-            m_run = -INFINITY;
-            l_run = 0.f;
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int mt = 0; mt < 4; ++mt)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) o[hf][mt][c] = 0.f;
+            at.reset();
         }
 
-        // ---- S = q K^T for this warp's WT tokens: heads on M (rows 8..15 are padding), tokens on N
-        float sacc[NT][4];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) sacc[nt][c] = 0.f;
-        {
-            uint4 kv[HALVES][2][NT];
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) kv[hf][m][nt] = lds128(kbase + hf * L::TILE_BYTES + koff[nt][m]);
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        mma_bf16_16816(sacc[nt], qa[hf][m][0], 0u, qa[hf][m][1], 0u, kv[hf][m][nt].x, kv[hf][m][nt].y);
-                        mma_bf16_16816(sacc[nt], qa[hf][m][2], 0u, qa[hf][m][3], 0u, kv[hf][m][nt].z, kv[hf][m][nt].w);
-                    }
-        }
-        // V pieces are requested now so that their latency hides behind the softmax arithmetic
-        uint4 v[HALVES][2 * NT];
-#pragma unroll
-        for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) v[hf][nt * 2 + c] = lds128(vbase + hf * L::TILE_BYTES + voff[nt][c]);
-
-        // ---- gate, mask, online softmax (lane (g,t) holds head g, tokens r0/r1 of each 8-group)
-        const bool head_on = head && ((hmask >> g) & 1);
-        float sg[NT][2];
-        float bmax = -INFINITY;
-        const bool gate_on = (te != -INFINITY);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int trow = rb + nt * 8 + (c ? r1 : r0);
-                const float S = sacc[nt][c] * a.scale;
-                float gated = S;
-                if (gate_on) {
-                    const float x = (a.beta == 0.f) ? 0.f : a.beta * (S - te);
-                    gated = S * rcp_approx(1.f + exp2f(-x * LOG2E));      // S * sigmoid(x); exp2(+inf) -> rcp -> 0
-                }
-                if (trow == urow) gated = S;          // the query's own token (Eq. mult_attn, s = t)
-                gated = (head_on && trow < nvalid) ? gated : -INFINITY;
-                sg[nt][c] = gated;
-                bmax = fmaxf(bmax, gated);
-            }
-        bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 1));
-        bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 2));
-        const float m_new = fmaxf(m_run, bmax);
-        const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
-        const float alpha = (m_run == m_new) ? 1.f : exp2f((m_run - m_use) * LOG2E);   // m_run = -inf gives 0
-        float p[NT][2], psum = 0.f;
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                p[nt][c] = exp2f((sg[nt][c] - m_use) * LOG2E);   // -inf gives 0
-                psum += p[nt][c];
-            }
-        l_run = l_run * alpha + psum;
-        m_run = m_new;
-
-        // accumulators hold heads 2t, 2t+1 in their columns: fetch those heads' rescale factors
-        if (__any_sync(0xffffffffu, alpha != 1.f)) {
-            const float al0 = __shfl_sync(0xffffffffu, alpha, 8 * t);
-            const float al1 = __shfl_sync(0xffffffffu, alpha, 8 * t + 4);
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int mt = 0; mt < 4; ++mt) {
-                    o[hf][mt][0] *= al0; o[hf][mt][1] *= al1; o[hf][mt][2] *= al0; o[hf][mt][3] *= al1;
-                }
-        }
-
-        // ---- P as the B operand: bf16 high part and bf16 residual
-        uint32_t pb_hi[2] = {0u, 0u}, pb_lo[2] = {0u, 0u};
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            const __nv_bfloat162 hi = __floats2bfloat162_rn(p[nt][0], p[nt][1]);
-            const float2 hf2 = __bfloat1622float2(hi);
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(p[nt][0] - hf2.x, p[nt][1] - hf2.y);
-            pb_hi[nt] = *reinterpret_cast<const uint32_t*>(&hi);
-            pb_lo[nt] = *reinterpret_cast<const uint32_t*>(&lo);
-        }
-
-        // ---- O^T += V^T P : head_dim on M, tokens on K, heads on N
-        if (nvalid < TS) {
-            // rows past the end of the sequence hold whatever the cache holds: keep them out of the product
-#pragma unroll
-            for (int hf = 0; hf < HALVES; ++hf)
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-                        if (rb + nt * 8 + (c ? r1 : r0) >= nvalid) v[hf][nt * 2 + c] = make_uint4(0, 0, 0, 0);
-        }
-        // every shared-memory read of this stage has been issued before this point; the arrive (release) orders
-        // them before the producer's next copy into the stage
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[stage]);
-#pragma unroll
-        for (int hf = 0; hf < HALVES; ++hf) {
-#pragma unroll
-            for (int mt = 0; mt < 4; ++mt) {
-                const uint32_t xa = u4_get(v[hf][0], mt), xb = u4_get(v[hf][1], mt);
-                const uint32_t a0 = __byte_perm(xa, xb, 0x5410), a1 = __byte_perm(xa, xb, 0x7632);
-                uint32_t a2 = 0u, a3 = 0u;
-                if (NT == 2) {
-                    const uint32_t xc = u4_get(v[hf][2 * (NT - 1)], mt), xd = u4_get(v[hf][2 * (NT - 1) + 1], mt);
-                    a2 = __byte_perm(xc, xd, 0x5410);
-                    a3 = __byte_perm(xc, xd, 0x7632);
-                }
-                mma_bf16_16816(o[hf][mt], a0, a1, a2, a3, pb_hi[0], pb_hi[1]);
-                mma_bf16_16816(o[hf][mt], a0, a1, a2, a3, pb_lo[0], pb_lo[1]);
-            }
-        }
-
+        // the arrive (release) orders the warp's reads of the stage before the producer's next copy into it
+        at.tile(kbase, hmask, urow, nvalid, a.scale, a.beta, [&]() { if (lane == 0) mbar_arrive(&empty[stage]); });
     }
     if (!ok && lane == 0 && a.status) atomicOr(a.status, ETA_DEV_TIMEOUT);
 }
