@@ -313,7 +313,8 @@ int eta_decode_paged(const eta_cache_desc* desc, const eta_page_table* pages, co
 size_t eta_static_scratch_bytes(void);
 
 /* Number of kernels one eta_decode call launches (for launch accounting); a rescue window that spans more blocks than one
- * CTA screens (by default more than 128, head_dim 128, or 256, head_dim 64) takes one more. */
+ * CTA screens (by default more than 128, head_dim 128, or 256, head_dim 64) takes one more, and a small problem (by
+ * the capacity of the cache: up to 512 blocks a sequence) only one in all, which leaves the workspace alone. */
 int eta_decode_kernel_count(void);
 
 /*

@@ -103,9 +103,12 @@ int KernelAttrTable::configure(int dev, const void* kernel, size_t dyn_smem, Set
 static KernelAttrTable g_attr_table;
 
 static int cuda_setter(void*, const void* kernel, int attr, size_t value) {
-    const cudaError_t e = (attr == KernelAttrTable::ATTR_CARVEOUT)
+    cudaError_t e = (attr == KernelAttrTable::ATTR_CARVEOUT)
         ? cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)
         : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)value);
+    // (a permission only: clusters of more than eight CTAs, for the kernel that is launched in them)
+    if (e == cudaSuccess && attr == KernelAttrTable::ATTR_CARVEOUT)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) { set_cuda_error(e, "kernel attribute"); return ETA_ERR_CUDA; }
     return 0;
 }

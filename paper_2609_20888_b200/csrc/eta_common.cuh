@@ -139,7 +139,7 @@ int configure_kernel(const void* kernel, size_t dyn_smem);
 
 class KernelAttrTable {
 public:
-    static constexpr int MAX_DEVICES = 64, MAX_KERNELS = 64;
+    static constexpr int MAX_DEVICES = 64, MAX_KERNELS = 128;
     static constexpr size_t DEFAULT_DYN_SMEM = 48 * 1024;
     enum { ATTR_CARVEOUT = 0, ATTR_MAX_DYN_SMEM = 1 };
     typedef int (*Setter)(void* ctx, const void* kernel, int attr, size_t value);

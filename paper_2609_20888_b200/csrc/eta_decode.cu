@@ -31,6 +31,7 @@
 #include <cuda.h>
 
 #include "eta_attend.cuh"
+#include "eta_step.h"
 #include "eta_timeline.h"
 
 namespace eta {
@@ -961,6 +962,28 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     if (rc != ETA_OK) return rc;
     rc = make_tmap(&tmV, V, desc, desc->v_stride_b, desc->v_stride_h, desc->v_stride_t, TS, n_pages);
     if (rc != ETA_OK) return rc;
+
+    int step_ctas = dense ? 0 : step_cluster(L.rows, desc->nb_cap, b, n_sm);
+#ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
+    step_ctas = 0;                      // the test is of the streaming kernel
+#endif
+    if (step_ctas) {
+        StepArgs st;
+        st.q = sa.q; st.musig = sa.musig; st.mnorm = mnorm; st.seq_lens = seq_lens; st.tau = tau; st.head_const = head_const;
+        st.z = params->z; st.a = params->a; st.scale = scale; st.beta = params->beta;
+        st.lwb = params->lwb; st.rescue_window = params->rescue_window; st.flags = params->flags;
+        st.Hq = desc->n_q_heads; st.b_shift = sa.b_shift; st.t_cap = desc->t_cap; st.nb_cap = desc->nb_cap;
+        st.block_table = pages ? pages->block_table : nullptr;
+        st.table_stride = pages ? pages->table_stride : 0;
+        st.div_hkv = sa.div_hkv;
+        st.out = out; st.sel_mask = sel_mask; st.stats = stats; st.status = status_dev;
+        profile_mark(2, s);
+        profile_mark(3, s);
+        rc = launch_step(st, tmK, tmV, L.rows, D, TS, G, step_ctas, s);
+        profile_mark(4, s);
+        profile_mark(5, s);
+        return rc;
+    }
 
     sa.tiles = b / TS; sa.tile_tokens = TS;
     sa.block_table = pages ? pages->block_table : nullptr;

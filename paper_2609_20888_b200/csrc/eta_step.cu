@@ -1,0 +1,378 @@
+// A decode step of a small problem in one kernel: screening, attention over the surviving blocks and the merge (Algorithm 3) by
+// one thread-block cluster per (sequence, KV head) row.
+//
+// The general path takes three kernels, because survivors of all rows are dealt out over the whole GPU.  Where a row has a few
+// hundred blocks its step is latency: the boundaries between the kernels and each one's own set-up.  Here every CTA of a row's
+// cluster bounds a share of the row's blocks while the thresholds are still being predicted and stores the bounds to all of them, so
+// that all know the list of survivors; each attends an equal share of the tiles; and the partial results are merged through the
+// cluster's shared memory.
+#include <cooperative_groups.h>
+
+#include "eta_attend.cuh"
+#include "eta_bounds.cuh"
+#include "eta_step.h"
+
+namespace cg = cooperative_groups;
+
+namespace eta {
+
+constexpr int STEP_WARPS = 12;                          // three groups of four that bound and attend ...
+constexpr int STEP_THREADS = 32 * (STEP_WARPS + 1);     // ... and one that issues the copies
+constexpr int STEP_RING = 196608;                       // bytes of the ring of K and V tiles; first the records' tiles, last the partials
+constexpr int STEP_SEGS = STEP_MAX_BLOCKS / SEG;
+
+template <int D, int TS, int G>
+struct StepSmem {
+    static constexpr int STAGE_BYTES = 4 * D * TS, NSTAGE = STEP_RING / STAGE_BYTES;
+    static_assert(NSTAGE % 3 == 0, "a stage serves the same group in every round");
+    static_assert(STEP_WARPS * TileOf<D>::BYTES <= STEP_RING && STEP_WARPS * G * D * 4 <= STEP_RING, "what shares the ring fits it");
+    static constexpr int BAR_OFF = STEP_RING;           // full[NSTAGE], empty[NSTAGE], two per warp for its records
+    static constexpr int TAB_OFF = (BAR_OFF + 8 * (2 * NSTAGE + 2 * STEP_WARPS) + 15) / 16 * 16;
+    static constexpr int BOUND_OFF = TAB_OFF + (int)((sizeof(QTab<D, G>) + 15) / 16 * 16);
+    static constexpr int LIST_OFF = BOUND_OFF + 4 * STEP_MAX_BLOCKS * G;        // survivors in ascending order, then the tail
+    static constexpr int IN_ML_OFF = TAB_OFF + 4 * G * D + 16 * STEP_MAX_CLUSTER;       // behind the parts: float2 [CTA][G]
+    static_assert(IN_ML_OFF + 8 * G * STEP_MAX_CLUSTER <= LIST_OFF, "the parts take the place of the query table and the bounds");
+    static constexpr int WARP_ML_OFF = LIST_OFF + 4 * (STEP_MAX_BLOCKS + 4);    // float m[STEP_WARPS][8], l[STEP_WARPS][8]
+    static constexpr size_t BYTES = 1024 + WARP_ML_OFF + 8 * STEP_WARPS * 8;
+};
+
+// A barrier of the cluster in two halves; what was stored before the first is there after the second
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// What bounds it: latency, of a chain that starts when the thresholds are there: the newest bound and admission (1 us), the list (0.5),
+// the first tiles (1.5 from the L2, more from memory), a tile every 0.6 us of a CTA, the parts of the warps and of the CTAs (1.5).
+// Bounds of the row in each CTA where they are one round of its warps, else in shares, which the cluster exchanges: 1.2 us slower
+// for 32 blocks, 1.2 faster for 257 and 4 for 511.  Six 32 KB tiles in flight: with three, rows of 256 blocks, half of them
+// attended, took 29.5 us instead of 25.5.  Parts are stored to the CTA that adds them up, not fetched by it: one barrier of the
+// cluster instead of two, 0.6 to 0.8 us.
+template <int D, int TS, int G, bool PACKED>
+__global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                               const __grid_constant__ CUtensorMap tmV, const StepArgs a) {
+    using L = StepSmem<D, TS, G>;
+    using TL = TileOf<D>;
+    constexpr int REC_BYTES = PACKED ? 3 * D : 4 * D;
+    extern __shared__ unsigned char step_raw[];
+    unsigned char* const sm = step_raw + ((1024u - (smem_u32(step_raw) & 1023u)) & 1023u);
+    uint64_t* const full = reinterpret_cast<uint64_t*>(sm + L::BAR_OFF);
+    uint64_t* const empty = full + L::NSTAGE;
+    QTab<D, G>& tab = *reinterpret_cast<QTab<D, G>*>(sm + L::TAB_OFF);
+    float* const sbound = reinterpret_cast<float*>(sm + L::BOUND_OFF);
+    int32_t* const list = reinterpret_cast<int32_t*>(sm + L::LIST_OFF);
+    __shared__ uint32_t s_bkey[G];        // per head: largest bound of the rescue window (as an ordered integer)
+    __shared__ int s_best[G];             // and the first block that attains it
+    __shared__ int s_cnt[STEP_SEGS];
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), n_ranks = (int)cluster.num_blocks();
+    const int r = blockIdx.x / n_ranks;
+    int i, hk;
+    a.div_hkv.divmod(r, i, hk);
+    const int Traw = __ldcg(a.seq_lens + i), T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
+    const int NB = min(T >> a.b_shift, a.nb_cap), b = 1 << a.b_shift;
+    const unsigned char* const rec_row = reinterpret_cast<const unsigned char*>(a.musig) + (int64_t)r * a.nb_cap * REC_BYTES;
+    const float* const mn_row = a.mnorm + (int64_t)r * a.nb_cap;
+
+    // ------------------------------------------------------------ bounds of the row's blocks, a share per CTA: needs neither the
+    // thresholds nor the newest record (see below), so it does not wait for the kernels that make them
+    if (a.shared) cluster_arrive();       // (all CTAs of the cluster run when all have come by here)
+    const int of = a.shared ? n_ranks : 1, mine = a.shared ? rank : 0;
+    if (tid == 0) {
+        for (int s = 0; s < L::NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], WARPS_PER_GROUP); }
+        fence_barrier_init();
+        prefetch_tmap(&tmK);
+        prefetch_tmap(&tmV);
+    }
+    uint64_t* const bars = empty + L::NSTAGE + 2 * warp;
+    TileStream<D, G, PACKED> ts{sm + warp * TL::BYTES, bars, rec_row, mn_row, NB, 1, 0, 0, 0u, true};
+    if (warp < STEP_WARPS) {
+        if (lane == 0) { mbar_init(&bars[0], 1); mbar_init(&bars[1], 1); fence_barrier_init(); }
+        __syncwarp();
+        ts.issue((warp * of + mine) * TL::RECS);
+    }
+    build_qtab<D, G>(tab, a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
+    bool ok = true;
+    const int first = (warp * of + mine) * TL::RECS, stride = STEP_WARPS * of * TL::RECS;
+    if (warp < STEP_WARPS) {
+        for (int j = first; j < NB; j += stride) {
+            ok = ts.bounds(tab, j, a.z, a.scale, sbound + j * G) && ok;
+            if (j + stride < NB) ts.issue(j + stride);
+        }
+    }
+    Attend<D, TS> at(lane, warp % WARPS_PER_GROUP, G);
+    at.load_q(a.q + ((int64_t)i * a.Hq + hk * G + (at.head ? at.g : 0)) * D);
+    if (a.shared) {                       // every CTA gets all of them
+        cluster_wait();
+        if (warp < STEP_WARPS) {
+            for (int j = first; j < NB; j += stride)
+                for (int c = 1; c < n_ranks; ++c) {
+                    float4* const dst = reinterpret_cast<float4*>(cluster.map_shared_rank(sbound + j * G, (rank + c) % n_ranks));
+                    for (int k = lane; k < TL::RECS * G / 4; k += 32) dst[k] = reinterpret_cast<const float4*>(sbound + j * G)[k];
+                }
+        }
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
+
+    // Top-1 rescue: a head that admits none of the first Wr blocks attends the first one with the largest bound among them.  It
+    // admits none exactly when that bound is below its threshold and no block of the window is pinned (a NaN bound admits).
+    // An ungated newest token must be attended: when it closes a full block, that block counts as pinned.
+    const int lwb = ((a.flags & ETA_FLAG_UNGATE_LAST) && T > 0 && (T & (b - 1)) == 0 && a.lwb < 1) ? 1 : a.lwb;
+    const int Wr = min(a.rescue_window, NB);
+    const bool rescues = Wr > 0 && !(lwb > 0 && NB - lwb < Wr);
+    const bool stale = NB > 0 && (T & (b - 1)) == 0;       // the newest block's record may not have been final yet
+    const bool late = stale && NB - 1 < Wr;
+    auto window_max = [&]() {
+        for (int gq = warp; gq < G; gq += STEP_WARPS + 1) {
+            uint32_t key = 0;                     // 0: no record of the window in this lane
+            int arg = 0x7fffffff;
+            for (int rec = lane; rec < Wr; rec += 32) {                     // ascending: a lane keeps the first of equal bounds
+                const uint32_t k2 = bound_key(sbound[rec * G + gq]);
+                if (k2 > key) { key = k2; arg = rec; }
+            }
+            const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
+            const int amin = __reduce_min_sync(0xffffffffu, key == kmax ? arg : 0x7fffffff);
+            if (lane == 0) { s_bkey[gq] = kmax; s_best[gq] = amin; }
+        }
+    };
+    if (rescues && !late) window_max();
+    pdl_wait();                           // the thresholds and the newest summaries are final now
+    pdl_trigger();
+    float te_l = -INFINITY;               // lane gq < G: effective threshold of head gq
+    if (lane < G) te_l = (a.tau ? __ldcg(a.tau + (int64_t)i * a.Hq + hk * G + lane) : __ldcg(a.head_const + hk * G + lane)) - a.a;
+    if (stale) {
+        if (warp == 0)
+            bound_one<D, G, PACKED>(tab.raw, rec_row + (int64_t)(NB - 1) * REC_BYTES, __ldcg(mn_row + NB - 1), a.z, a.scale, sbound + (NB - 1) * G);
+        __syncthreads();
+        if (rescues && late) window_max();
+    }
+    __syncthreads();
+    if (rank == 0 && tid == 0 && a.status) {
+        if (Traw > a.t_cap) atomicOr(a.status, ETA_DEV_LEN_CLAMPED);
+        if (Traw <= 0) atomicOr(a.status, ETA_DEV_EMPTY_ROW);
+    }
+
+    // ------------------------------------------------------------ admission, a warp per segment
+    const int j0 = warp * SEG;
+    unsigned m[SEG / 32] = {};
+    int carry = 0;
+    if (warp < STEP_SEGS && j0 < a.nb_cap) {
+#pragma unroll
+        for (int gq = 0; gq < G; ++gq) {
+            const float te_g = __shfl_sync(0xffffffffu, te_l, gq);
+            const int best = rescues && key_bound(s_bkey[gq]) < te_g ? s_best[gq] : -1;
+#pragma unroll
+            for (int half = 0; half < SEG / 32; ++half) {
+                const int j = j0 + half * 32 + lane;
+                if (j < NB && (j >= NB - lwb || j == best || !(sbound[j * G + gq] < te_g))) m[half] |= 1u << gq;
+            }
+        }
+#pragma unroll
+        for (int half = 0; half < SEG / 32; ++half) {
+            const int j = j0 + half * 32 + lane;
+            if (rank == 0 && j < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j] = (uint8_t)m[half];
+            carry += __popc(__ballot_sync(0xffffffffu, m[half] != 0));
+        }
+    }
+    if (warp < STEP_SEGS && lane == 0) s_cnt[warp] = carry;
+    __syncthreads();
+    int n_blocks = 0, at_list = 0;
+#pragma unroll
+    for (int s = 0; s < STEP_SEGS; ++s) {
+        if (s < warp) at_list += s_cnt[s];
+        n_blocks += s_cnt[s];
+    }
+    if (warp < STEP_SEGS) {
+#pragma unroll
+        for (int half = 0; half < SEG / 32; ++half) {
+            const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
+            if (m[half]) list[at_list + __popc(nz & ((1u << lane) - 1u))] = (j0 + half * 32 + lane) | (int)(m[half] << 24);
+            at_list += __popc(nz);
+        }
+    }
+    const int tail = T - NB * b;
+    if (tid == 0) {
+        list[n_blocks] = NB | (0xff << 24);               // the tail: every head attends it
+        if (rank == 0 && a.stats) a.stats[r] = n_blocks;
+    }
+    at.te = __shfl_sync(0xffffffffu, te_l, at.head ? at.g : 0);
+    __syncthreads();
+    cluster_arrive();                     // this CTA needs its query table and bounds no more: the others' parts go there
+
+    // ------------------------------------------------------------ an equal share of the row's tiles
+    const int tpu_shift = a.b_shift - (TS == 64 ? 6 : 5);               // tiles of a full block: 1, or 2 (128 tokens)
+    const int n_full = n_blocks << tpu_shift, n_tiles = n_full + (tail + TS - 1) / TS;
+    const int f0 = n_tiles * rank / n_ranks, n = n_tiles * (rank + 1) / n_ranks - f0;
+    // tile k of the share: its list entry, part of the block, tokens of it in the sequence
+    auto locate = [&](int k, int& ent, int& sub, int& rows) {
+        const int f = f0 + k;
+        const bool whole = f < n_full;
+        sub = whole ? f & ((1 << tpu_shift) - 1) : f - n_full;
+        ent = list[whole ? f >> tpu_shift : n_blocks];
+        rows = (whole ? b : tail) - sub * TS;
+    };
+    if (warp == STEP_WARPS) {
+        // a lane per stage
+        if (lane < L::NSTAGE) {
+            const uint64_t policy = l2_policy(false);
+            int issued = -1;
+            for (int k = lane, parity = 1; k < n && ok; k += L::NSTAGE, parity ^= 1) {
+                ok = mbar_wait(&empty[lane], parity);
+                if (!ok) break;
+                int ent, sub, rows;
+                locate(k, ent, sub, rows);
+                const int j = ent & 0xffffff;
+                const int w = a.block_table ? __ldcg(a.block_table + (int64_t)i * a.table_stride + j) : i;
+                const int y = (a.block_table ? 0 : j * b) + sub * TS;
+                unsigned char* const dst = sm + lane * L::STAGE_BYTES;
+                mbar_arrive_expect_tx(&full[lane], L::STAGE_BYTES);
+                tma_load_5d(dst, &tmK, 0, y, 0, hk, w, &full[lane], policy);
+                tma_load_5d(dst + L::STAGE_BYTES / 2, &tmV, 0, y, 0, hk, w, &full[lane], policy);
+                issued = k;
+            }
+            if (issued >= 0) ok = mbar_wait(&full[lane], (issued / L::NSTAGE) & 1) && ok;      // whatever the others did: the copies have landed
+        }
+        ok = __all_sync(0xffffffffu, ok);
+    } else {
+        for (int k = warp / WARPS_PER_GROUP; k < n; k += STEP_WARPS / WARPS_PER_GROUP) {
+            const int stage = k % L::NSTAGE;
+            ok = __all_sync(0xffffffffu, ok && mbar_wait(&full[stage], (k / L::NSTAGE) & 1));
+            if (!ok) break;
+            int ent, sub, rows;
+            locate(k, ent, sub, rows);
+            const int nvalid = min(TS, rows), last = T - 1 - ((ent & 0xffffff) * b + sub * TS);      // the newest token's row of the tile
+            const int urow = (a.flags & ETA_FLAG_UNGATE_LAST) && last < TS ? last : 0xff;
+            at.tile(smem_u32(sm + stage * L::STAGE_BYTES), (ent >> 24) & 0xff, urow, nvalid, a.scale, a.beta,
+                    [&]() { if (lane == 0) mbar_arrive(&empty[stage]); });
+        }
+    }
+    if (!ok && lane == 0 && a.status) atomicOr(a.status, ETA_DEV_TIMEOUT);
+    __syncthreads();                      // the ring is free
+
+    // ------------------------------------------------------------ the warps' parts, then the CTAs'
+    float* const warp_m = reinterpret_cast<float*>(sm + L::WARP_ML_OFF), * const warp_l = warp_m + STEP_WARPS * 8;
+    float* const parts = reinterpret_cast<float*>(sm);                  // [warp][head][D]
+    // Each CTA makes a slice of the row's output: it gets every CTA's part of the slice, and their statistics
+    const int per = (G * D / 4 + n_ranks - 1) / n_ranks;
+    float4* const in_o = reinterpret_cast<float4*>(sm + L::TAB_OFF);                 // [CTA][per]
+    float2* const in_ml = reinterpret_cast<float2*>(sm + L::IN_ML_OFF);              // [CTA][G]
+    constexpr float LOG2E = 1.4426950408889634f;
+    if (warp < STEP_WARPS) {
+        float lsum = at.l_run + __shfl_xor_sync(0xffffffffu, at.l_run, 1);
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, 2);
+        if (at.t == 0) { warp_m[warp * 8 + at.g] = at.m_run; warp_l[warp * 8 + at.g] = lsum; }
+#pragma unroll
+        for (int hf = 0; hf < D / 64; ++hf)
+#pragma unroll
+            for (int mt = 0; mt < 4; ++mt) {
+                const int ha = 2 * at.t, dcol = 64 * hf + 8 * at.vchunk + 2 * mt;
+                if (ha < G) *reinterpret_cast<float2*>(parts + (warp * G + ha) * D + dcol) = make_float2(at.o[hf][mt][0], at.o[hf][mt][2]);
+                if (ha + 1 < G) *reinterpret_cast<float2*>(parts + (warp * G + ha + 1) * D + dcol) = make_float2(at.o[hf][mt][1], at.o[hf][mt][3]);
+            }
+    }
+    __syncthreads();
+    cluster_wait();
+    for (int idx = tid; idx < G * D / 4; idx += STEP_THREADS) {
+        const int h = idx / (D / 4), dq = idx % (D / 4);
+        float M = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < STEP_WARPS; ++w) M = fmaxf(M, warp_m[w * 8 + h]);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float lacc = 0.f;
+        if (M != -INFINITY) {
+#pragma unroll
+            for (int w = 0; w < STEP_WARPS; ++w) {
+                const float sc = exp2f((warp_m[w * 8 + h] - M) * LOG2E);
+                const float4 x = *reinterpret_cast<const float4*>(parts + (w * G + h) * D + 4 * dq);
+                acc.x = fmaf(x.x, sc, acc.x); acc.y = fmaf(x.y, sc, acc.y);
+                acc.z = fmaf(x.z, sc, acc.z); acc.w = fmaf(x.w, sc, acc.w);
+                lacc = fmaf(warp_l[w * 8 + h], sc, lacc);
+            }
+        }
+        const int owner = idx / per;
+        *cluster.map_shared_rank(in_o + rank * per + idx - owner * per, owner) = acc;
+        if (dq == 0)
+            for (int c = 0; c < n_ranks; ++c) *cluster.map_shared_rank(in_ml + rank * G + h, c) = make_float2(M, lacc);
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int idx = rank * per + tid;
+    if (tid < per && idx < G * D / 4) {
+        const int h = idx / (D / 4);
+        float M = -INFINITY, l = 0.f;
+        for (int c = 0; c < n_ranks; ++c) M = fmaxf(M, in_ml[c * G + h].x);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (M != -INFINITY) {
+            for (int c = 0; c < n_ranks; ++c) {
+                const float2 p = in_ml[c * G + h];
+                const float4 x = in_o[c * per + tid];
+                const float sc = exp2f((p.x - M) * LOG2E);            // a CTA without tiles: 0
+                acc.x = fmaf(x.x, sc, acc.x); acc.y = fmaf(x.y, sc, acc.y);
+                acc.z = fmaf(x.z, sc, acc.z); acc.w = fmaf(x.w, sc, acc.w);
+                l = fmaf(p.y, sc, l);
+            }
+        }
+        if (l > 0.f) { acc.x /= l; acc.y /= l; acc.z /= l; acc.w /= l; }
+        else acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(a.out + ((int64_t)i * a.Hq + hk * G) * D + 4 * idx) = acc;
+    }
+}
+
+template <int D, int TS, int G, bool PACKED>
+static int launch_step_t(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int n_ranks, cudaStream_t s) {
+    using L = StepSmem<D, TS, G>;
+    a.shared = n_ranks > 1 && a.nb_cap > STEP_WARPS * TileOf<D>::RECS;
+    const int rc = configure_kernel(reinterpret_cast<const void*>(step_kernel<D, TS, G, PACKED>), L::BYTES);
+    if (rc != ETA_OK) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(rows * n_ranks));
+    cfg.blockDim = dim3(STEP_THREADS);
+    cfg.dynamicSmemBytes = L::BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)n_ranks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, step_kernel<D, TS, G, PACKED>, tmK, tmV, a);
+    if (e != cudaSuccess) { set_cuda_error(e, "step launch"); return ETA_ERR_CUDA; }
+    return check_launch("step launch");
+}
+
+// Which problems, by what the host knows: the capacity.  A row's cluster has to do alone what the general path spreads over the GPU,
+// so a step is bound by the fullest row; what it saves is two kernels, 6 to 7 us.  us a step, general and this, half / a tenth of
+// the blocks attended (d = 128, blocks of 64, queued calls): 8 rows of 2K 20.7, 14.2 / 19.8, 13.7; 16K 29.2, 24.2 / 22.7, 17.7; 32K
+// 35.3, 32.5 / 23.7, 20.0; 16 rows of 16K 34.5, 30.5 / 23.2, 18.4; 64 rows of 2K 29.1, 23.2 / 21.6, 16.4; 128 rows of 2K 38.7, 31.2 /
+// 28.1, 21.9.  Beyond the line rows of unequal lengths and survivors lose: 24 rows of up to 32K 46.0, 60.7 / 29.5, 27.4, 64 of up to
+// 16K 50.0, 70.6 / 30.7, 35.4.  One or two rows of more than 128 or 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
+// How many CTAs: clusters that fit the GPU at once, 18 SMs to a group, with some to spare for the predictor's: 16 rows in clusters of
+// 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
+int step_cluster(int rows, int nb_cap, int b, int n_sm) {
+    const int tiles = b > 64 ? 2 * nb_cap : nb_cap;
+    if (nb_cap > STEP_MAX_BLOCKS || (int64_t)rows * tiles > STEP_MAX_TILES || tiles > 128 * rows) return 0;
+    if (rows <= 4 && tiles > 64) return STEP_MAX_CLUSTER;
+    const int group = n_sm / 8;
+    for (int c = 8; c >= 1; --c)
+        if (80 * (group / c) >= rows * (c > 4 ? 11 : 10)) return c;
+    return 0;
+}
+
+int launch_step(const StepArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int TS, int G, int n_ranks, cudaStream_t s) {
+    const bool packed = (a.flags & ETA_FLAG_PACKED_SIGMA) != 0;
+#define ETA_CASE(DD, TT, GG) if (D == DD && TS == TT && G == GG) return packed ? launch_step_t<DD, TT, GG, true>(a, tmK, tmV, rows, n_ranks, s) \
+                                                                               : launch_step_t<DD, TT, GG, false>(a, tmK, tmV, rows, n_ranks, s);
+#define ETA_CASES(GG) ETA_CASE(128, 64, GG) ETA_CASE(128, 32, GG) ETA_CASE(64, 64, GG) ETA_CASE(64, 32, GG)
+    ETA_CASES(1) ETA_CASES(2) ETA_CASES(4) ETA_CASES(8)
+#undef ETA_CASES
+#undef ETA_CASE
+    return ETA_ERR_UNSUPPORTED;
+}
+
+}  // namespace eta
