@@ -6,9 +6,9 @@
 // decode_kernel is persistent, one CTA per SM.  Work is the flattened sequence
 // of "units": for each (sequence, KV head) row its surviving blocks (the
 // screening kernel's per-segment lists), then its tail.
-// Every CTA finds its place in that sequence from the per-segment counts (one
-// warp, one round trip to memory for up to 4096 segments, no CTA barrier) and
-// takes an equal, contiguous share of its COST (units, plus a fixed charge for
+// Every CTA finds its place in that sequence from the per-segment counts (a
+// thread per 16 segments and one round trip to memory for up to 4096 of them)
+// and takes an equal, contiguous share of its COST (units, plus a fixed charge for
 // every row boundary inside the share: stream-K), so the load is balanced
 // whatever the per-head survivor counts are; a share may cross rows, and a row
 // may be split over CTAs; each (CTA, row) piece produces one partial (m, l, O)
@@ -50,7 +50,6 @@ struct DecodeArgs {
     float beta, scale;
     int Hq, Hkv, G, b, t_cap, nb_cap, nseg, rows;
     int gpr, n_gran;     // granules (16 segments) of a row, of all rows
-    int lane_gran;       // granules a lane takes of a chunk: 8, fewer where all of them are less than a chunk
     int n_chunks, super; // chunks of 32 lanes x 8 granules; chunks whose sums share an entry in shared memory
     int ungate_last;     // the newest token of every sequence keeps its raw logit (ETA_FLAG_UNGATE_LAST)
     const int32_t* block_table;   // paged cache: [batch, table_stride] page of every block of tokens; null: contiguous
@@ -87,7 +86,8 @@ struct DecodeSmem {
     static constexpr int DESC_OFF = (BAR_OFF + 8 * (2 * NSTAGE + NGROUPS + 1) + 15) / 16 * 16;
     static constexpr int WIN_OFF = DESC_OFF + 16 * NSTAGE;      // uint4 [32]: the producer's window of granules
     static constexpr int GRAN_OFF = WIN_OFF + 16 * 32;          // uint4 [CHUNK]: all granules (one chunk), else int2 [MAX_SUPER]: sums
-    static constexpr int SPAN_OFF = GRAN_OFF + 16 * CHUNK;      // int2 [SPAN_ROWS + 1] (+ pad): units and live rows before a row
+    static constexpr int BEFORE_OFF = GRAN_OFF + 16 * CHUNK;    // int2 [CHUNK + 1] (+ pad): units and live rows before a granule (one chunk)
+    static constexpr int SPAN_OFF = BEFORE_OFF + 8 * (CHUNK + 2);      // int2 [SPAN_ROWS + 1] (+ pad): units and live rows before a row
     static constexpr int INFO_OFF = SPAN_OFF + 8 * (SPAN_ROWS + 2);     // uint8 per row: bit 0 has tokens, bit 1 has a tail
     static constexpr int ML_OFF = INFO_OFF + MAX_ROWS;          // float m[NGROUPS][4][8], l[NGROUPS][4][8]
     static_assert(16 * CHUNK >= 8 * MAX_SUPER, "sums of the super-chunks share the granules' place");
@@ -144,16 +144,20 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     __syncthreads();
 
     // ---- layout.  The flattened sequence of units is cut up by granules, 16 segments of a row each (the last one of a row
-    // also holds its tail unit).  Lane l of a warp takes the consecutive granules l lane_gran .. of a chunk; a scan over the
-    // lanes gives each its first unit.  A row that starts inside a CTA's share costs that CTA a flush of its partials and
+    // also holds its tail unit).  Up to 256 granules: a thread takes one, a scan over the threads gives it the units before it, and
+    // the two threads whose granules hold the ends of the CTA's share say where it starts and ends.  More: lane l of a warp takes
+    // eight consecutive granules of a chunk.  A row that starts inside a CTA's share costs that CTA a flush of its partials and
     // a query reload, worth `pc` tiles: row r spans the cost interval [units before + pc * live rows before, + pc (if it
     // has units) + its units).  Every live row has at least one unit (a tail, or what top-1 rescue leaves).
+    // Bound by the number of instructions in a row, some four cycles each whatever they are: with one warp, eight granules to a
+    // lane, it was 6300 to 8300 cycles from the wait to the first copy, with a thread per granule 4800 to 5300 (128K x 4 59.9 -> 58.4 us a
+    // step, 32K x 8 50.8 -> 49.4, 512K 43.7 -> 42.7, 64K x 32 89.9 -> 88.3).
     uint32_t headm = 0, tailm = 0;        // bit m: the lane's granule m of the chunk is the first of a live row / ends a row with a tail
     auto lane_flags = [&](int ch) {
         headm = tailm = 0;
 #pragma unroll 1
-        for (int m = 0; m < a.lane_gran; ++m) {
-            const int q = ch * CHUNK + lane * a.lane_gran + m;
+        for (int m = 0; m < LGRAN; ++m) {
+            const int q = ch * CHUNK + lane * LGRAN + m;
             if (q >= a.n_gran) break;
             int r, pos;
             a.div_gpr.divmod(q, r, pos);
@@ -167,23 +171,19 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const uint4* const gran = reinterpret_cast<const uint4*>(a.seg_cnt);
     uint4* const gran_s = reinterpret_cast<uint4*>(smem + L::GRAN_OFF);
     int2* const super_s = reinterpret_cast<int2*>(smem + L::GRAN_OFF);
-    auto load_chunk = [&](int ch, bool keep) {
+    auto load_chunk = [&](int ch) {
         uint4 v[LGRAN];
 #pragma unroll
         for (int m = 0; m < LGRAN; ++m) {
-            const int q = ch * CHUNK + lane * a.lane_gran + m;
+            const int q = ch * CHUNK + lane * LGRAN + m;
             v[m] = make_uint4(0, 0, 0, 0);
-            if (m < a.lane_gran && q < a.n_gran) v[m] = __ldcg(gran + q);
+            if (q < a.n_gran) v[m] = __ldcg(gran + q);
         }
         lane_u = 0;
 #pragma unroll
         for (int m = 0; m < LGRAN; ++m) {
-            us[m] = 0;
-            if (m < a.lane_gran) {
-                us[m] = granule_sum(v[m]) + (int)((tailm >> m) & 1);
-                lane_u += us[m];
-                if (keep) gran_s[lane * a.lane_gran + m] = v[m];
-            }
+            us[m] = granule_sum(v[m]) + (int)((tailm >> m) & 1);
+            lane_u += us[m];
         }
         lane_z = __popc(headm);
     };
@@ -201,7 +201,19 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     };
     const bool one_chunk = a.n_chunks == 1;
     const bool lays_out = warp == PRODUCER_WARP || warp == 0;              // the producer, and the warp that publishes
-    if (one_chunk && lays_out) lane_flags(0);
+    // one chunk: a granule per thread
+    static_assert(NTHREADS > CHUNK, "a thread per granule, and one for the end");
+    int2* const before_s = reinterpret_cast<int2*>(smem + L::BEFORE_OFF);
+    __shared__ uint32_t s_warp[CHUNK / 32];
+    __shared__ int s_unit[2], s_gran;
+    uint32_t my_head = 0, my_tail = 0;
+    if (one_chunk && tid < a.n_gran) {
+        int r, pos;
+        a.div_gpr.divmod(tid, r, pos);
+        const int info = rowinfo[r];
+        my_head = pos == 0 && (info & 1);
+        my_tail = pos == a.gpr - 1 && (info & 2);
+    }
     pdl_wait();          // the screening kernel's lists and counts are complete from here on
     if (tl && tid == 0) tl[7] = globaltimer_ns();
     const unsigned long long clk0 = ETA_TL(reinterpret_cast<unsigned long long*>(1)) ? (unsigned long long)clock64() : 0ull;
@@ -212,7 +224,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             int su = 0, sz = 0;
             for (int ch = sc * a.super; ch < min(a.n_chunks, (sc + 1) * a.super); ++ch) {
                 lane_flags(ch);
-                load_chunk(ch, false);
+                load_chunk(ch);
                 su += lane_u; sz += lane_z;
             }
             su = __reduce_add_sync(0xffffffffu, su);
@@ -222,16 +234,37 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         __syncthreads();
     }
     int U = 0, Z = 0;
-    if (lays_out) {
-        if (one_chunk) {
-            load_chunk(0, warp == PRODUCER_WARP);
-            scan_chunk();
-            U = tot_u; Z = tot_z;
-        } else {
-            for (int sc = lane; sc < n_super; sc += 32) { U += super_s[sc].x; Z += super_s[sc].y; }
-            U = __reduce_add_sync(0xffffffffu, U);
-            Z = __reduce_add_sync(0xffffffffu, Z);
+    uint32_t my_n = 0, my_before = 0;        // one chunk: units (and, from bit 20, live rows) of the thread's granule, before it
+    if (one_chunk) {
+        const int n_warps = (a.n_gran + 31) / 32;
+        uint32_t x = 0;
+        if (warp < n_warps) {
+            if (tid < a.n_gran) {
+                const uint4 v = __ldcg(gran + tid);
+                gran_s[tid] = v;
+                my_n = (uint32_t)granule_sum(v) + my_tail;
+            }
+            x = my_n | (my_head << 20);          // all granules: < 2^19 units, <= 256 rows
+#pragma unroll
+            for (int sft = 1; sft < 32; sft <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, x, sft);
+                if (lane >= sft) x += o;
+            }
+            if (lane == 31) s_warp[warp] = x;
+            my_before = x - (my_n | (my_head << 20));
         }
+        __syncthreads();
+        uint32_t all = 0;
+        for (int w = 0; w < n_warps; ++w) {
+            const uint32_t t = s_warp[w];
+            all += t;
+            if (w < warp) my_before += t;
+        }
+        U = (int)(all & 0xfffffu); Z = (int)(all >> 20);
+    } else if (lays_out) {
+        for (int sc = lane; sc < n_super; sc += 32) { U += super_s[sc].x; Z += super_s[sc].y; }
+        U = __reduce_add_sync(0xffffffffu, U);
+        Z = __reduce_add_sync(0xffffffffu, Z);
     }
     // More cost units per CTA than a row's padding (fewer CTAs take part in a tiny problem): then no CTA's range lies
     // inside a padding; the CTAs that meet a row are exactly those between two ends that follow from the row's cost
@@ -240,6 +273,32 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
     const int pc = (uint32_t)U + (uint32_t)(PIECE_COST * Z) >= (PIECE_COST + 1) * grid ? PIECE_COST : PIECE_COST_SMALL;
     const uint32_t C = (uint32_t)U + (uint32_t)pc * (uint32_t)Z;
     const uint32_t P = min(grid, max(1u, C / (PIECE_COST_SMALL + 1)));
+    // the CTA's share of the cost, [x0, x1)
+    uint32_t x0 = C, x1 = C;
+    if (blockIdx.x < P) {
+        if (P == grid) {
+            const uint32_t cq = (uint32_t)a.div_grid.div((int)C), cr = C - cq * grid;        // floor(c C / P): c cr < 2^16
+            x0 = blockIdx.x * cq + (uint32_t)a.div_grid.div((int)(blockIdx.x * cr));
+            x1 = (blockIdx.x + 1) * cq + (uint32_t)a.div_grid.div((int)((blockIdx.x + 1) * cr));
+        } else {
+            const uint32_t cq = C / P, cr = C - cq * P;
+            x0 = blockIdx.x * cq + blockIdx.x * cr / P;
+            x1 = (blockIdx.x + 1) * cq + (blockIdx.x + 1) * cr / P;
+        }
+    }
+    if (one_chunk) {
+        // whose granule holds an end of the share finds the unit it stands for (a position in a row's padding: the row's first)
+        if (tid <= a.n_gran) {
+            const int u = tid < a.n_gran ? (int)(my_before & 0xfffffu) : U, z = tid < a.n_gran ? (int)(my_before >> 20) : Z;
+            before_s[tid] = make_int2(u, z);
+            const uint32_t c = (uint32_t)u + (uint32_t)pc * (uint32_t)z, pad = my_head ? (uint32_t)pc : 0u;
+            if (tid < a.n_gran) {
+                if (x0 >= c && x0 < c + pad + my_n) { s_unit[0] = u + (x0 > c + pad ? (int)(x0 - c - pad) : 0); s_gran = tid; }
+                if (x1 >= c && x1 < c + pad + my_n) s_unit[1] = u + (x1 > c + pad ? (int)(x1 - c - pad) : 0);
+            }
+        }
+        __syncthreads();
+    }
     if (warp == 0) {
         // ---- for the merge kernel and the caller, shared out over the CTAs (all of them find the same layout): the
         // streaming CTAs that hold units of each row, and the number of blocks fetched per row.  CTA c has the cost
@@ -255,8 +314,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 int u = bu + pre_u, z = bz + pre_z;
 #pragma unroll
                 for (int m = 0; m < LGRAN; ++m) {
-                    const int q = ch * CHUNK + lane * a.lane_gran + m;
-                    if (m < a.lane_gran && q < a.n_gran) {
+                    const int q = ch * CHUNK + lane * LGRAN + m;
+                    if (q < a.n_gran) {
                         int r, pos;
                         a.div_gpr.divmod(q, r, pos);
                         if (pos == 0 && r >= r_lo && r <= r_hi) span[r - r_lo] = make_int2(u, z);
@@ -264,15 +323,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                     }
                 }
             };
-            if (one_chunk) {
-                store_rows(0, 0, 0);
-            } else {
+            if (!one_chunk) {
                 const int ch0 = (r_lo * a.gpr) / CHUNK, ch1 = min(a.n_chunks - 1, (r_hi * a.gpr) / CHUNK);
                 int bu = 0, bz = 0, ch = 0;
                 for (; ch + a.super <= ch0; ch += a.super) { bu += super_s[ch / a.super].x; bz += super_s[ch / a.super].y; }
                 for (; ch <= ch1; ++ch) {
                     lane_flags(ch);
-                    load_chunk(ch, false);
+                    load_chunk(ch);
                     scan_chunk();
                     if (ch >= ch0) store_rows(ch, bu, bz);
                     bu += tot_u; bz += tot_z;
@@ -280,10 +337,12 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             }
             __syncwarp();
             for (int k = lane; k < r_hi - r_lo; k += 32) {
-                const int rr = r_lo + k, units = span[k + 1].x - span[k].x;
+                const int rr = r_lo + k;
+                const int2 from = one_chunk ? before_s[rr * a.gpr] : span[k], to = one_chunk ? before_s[(rr + 1) * a.gpr] : span[k + 1];
+                const int units = to.x - from.x;
                 int c_lo = 0, n_span = 0;
                 if (units > 0) {
-                    const int64_t cs = (int64_t)span[k].x + (int64_t)pc * span[k].y, ce = cs + pc + units;
+                    const int64_t cs = (int64_t)from.x + (int64_t)pc * from.y, ce = cs + pc + units;
                     const int c_hi = (int)((ce * P - 1) / C);
                     c_lo = (int)(((cs + pc + 1) * P + C - 1) / C) - 1;
                     n_span = c_hi - c_lo + 1;
@@ -298,36 +357,21 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
 
     if (warp == PRODUCER_WARP) {
         // ------------------------------------------------------------ producer
-        // the CTA's share of the cost, [x0, x1), and the units it stands for
-        uint32_t x0 = C, x1 = C;
-        if (blockIdx.x < P) {
-            if (P == grid) {
-                const uint32_t cq = (uint32_t)a.div_grid.div((int)C), cr = C - cq * grid;        // floor(c C / P): c cr < 2^16
-                x0 = blockIdx.x * cq + (uint32_t)a.div_grid.div((int)(blockIdx.x * cr));
-                x1 = (blockIdx.x + 1) * cq + (uint32_t)a.div_grid.div((int)((blockIdx.x + 1) * cr));
-            } else {
-                const uint32_t cq = C / P, cr = C - cq * P;
-                x0 = blockIdx.x * cq + blockIdx.x * cr / P;
-                x1 = (blockIdx.x + 1) * cq + (blockIdx.x + 1) * cr / P;
-            }
-        }
         // cost position x < C -> unit, a granule at or before the one that holds it, units before that granule.  A position in a
         // row's padding stands for the row's first unit.
         auto locate = [&](uint32_t x, int& unit, int& gq, int& gu) {
             int bu = 0, bz = 0, ch = 0;
-            if (!one_chunk) {
-                for (int sc = 0; sc + 1 < n_super; ++sc) {
-                    const int2 t = super_s[sc];
-                    if (x < (uint32_t)(bu + t.x) + (uint32_t)pc * (uint32_t)(bz + t.y)) break;
-                    bu += t.x; bz += t.y; ch += a.super;
-                }
-                while (true) {
-                    lane_flags(ch);
-                    load_chunk(ch, false);
-                    scan_chunk();
-                    if (ch + 1 >= a.n_chunks || x < (uint32_t)(bu + tot_u) + (uint32_t)pc * (uint32_t)(bz + tot_z)) break;
-                    bu += tot_u; bz += tot_z; ++ch;
-                }
+            for (int sc = 0; sc + 1 < n_super; ++sc) {
+                const int2 t = super_s[sc];
+                if (x < (uint32_t)(bu + t.x) + (uint32_t)pc * (uint32_t)(bz + t.y)) break;
+                bu += t.x; bz += t.y; ch += a.super;
+            }
+            while (true) {
+                lane_flags(ch);
+                load_chunk(ch);
+                scan_chunk();
+                if (ch + 1 >= a.n_chunks || x < (uint32_t)(bu + tot_u) + (uint32_t)pc * (uint32_t)(bz + tot_z)) break;
+                bu += tot_u; bz += tot_z; ++ch;
             }
             int u = bu + pre_u, fu = 0, fq = 0, fgu = 0;
             uint32_t c = (uint32_t)u + (uint32_t)pc * (uint32_t)(bz + pre_z);
@@ -335,15 +379,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             bool found = false;
 #pragma unroll
             for (int m = 0; m < LGRAN; ++m) {
-                if (m < a.lane_gran) {
-                    const uint32_t pad = ((headm >> m) & 1) ? (uint32_t)pc : 0u;
-                    if (!found && x < c + pad + (uint32_t)us[m]) {
-                        found = true;
-                        fu = u + (x > c + pad ? (int)(x - c - pad) : 0);
-                        fq = ch * CHUNK + lane * a.lane_gran + m; fgu = u;
-                    }
-                    c += pad + (uint32_t)us[m]; u += us[m];
+                const uint32_t pad = ((headm >> m) & 1) ? (uint32_t)pc : 0u;
+                if (!found && x < c + pad + (uint32_t)us[m]) {
+                    found = true;
+                    fu = u + (x > c + pad ? (int)(x - c - pad) : 0);
+                    fq = ch * CHUNK + lane * LGRAN + m; fgu = u;
                 }
+                c += pad + (uint32_t)us[m]; u += us[m];
             }
             unit = __shfl_sync(0xffffffffu, fu, src);
             gq = __shfl_sync(0xffffffffu, fq, src);
@@ -351,23 +393,33 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         };
         int u0 = U, u1 = U, wq = 0, wu = 0;          // the CTA's units; the window's first granule, units before it
         if (x0 < C) {
-            int nq, nu;
-            if (x1 < C) locate(x1, u1, nq, nu);
-            locate(x0, u0, wq, wu);
+            if (one_chunk) {
+                u0 = s_unit[0];
+                wq = s_gran;
+                if (x1 < C) u1 = s_unit[1];
+            } else {
+                int nq, nu;
+                if (x1 < C) locate(x1, u1, nq, nu);
+                locate(x0, u0, wq, wu);
+            }
         }
         if (tl2 && lane == 0) tl2[3] = (unsigned long long)clock64() - clk0;
-        const int tpu = a.b > TS ? a.b / TS : 1;          // tiles of a full unit
+        const int tpu_shift = a.b > TS ? 1 : 0, tpu = 1 << tpu_shift;          // tiles of a full unit: two for 128 tokens, else one
         // Window: granule wq + l in lane l, its counts in shared memory, the units before it in pre_w.
         uint4* const win = reinterpret_cast<uint4*>(smem + L::WIN_OFF);
         int pre_w = 0, wend = 0;
-        bool first_window = one_chunk;
         auto load_window = [&]() {
+            if (one_chunk) {
+                pre_w = before_s[min(wq + lane, a.n_gran)].x;
+                wend = before_s[min(wq + 32, a.n_gran)].x;
+                return;
+            }
             __syncwarp();
             const int q = wq + lane;
             uint4 v = make_uint4(0, 0, 0, 0);
             int tail = 0;
             if (q < a.n_gran) {
-                v = first_window ? gran_s[q] : __ldcg(gran + q);
+                v = __ldcg(gran + q);
                 int r, pos;
                 a.div_gpr.divmod(q, r, pos);
                 tail = (pos == a.gpr - 1) ? (rowinfo[r] >> 1) & 1 : 0;
@@ -396,7 +448,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         // make the window hold the granule of unit ub; -> number of units of the batch starting at ub
         auto batch_size = [&](int ub) {
             while (true) {
-                const int want = min(32 / tpu, u1 - ub);
+                const int want = min((32 >> tpu_shift), u1 - ub);
                 if (wq + 32 >= a.n_gran || wend >= ub + want) return want;
                 if (wend <= ub) { wq += 32; wu = wend; load_window(); continue; }
                 const int k0 = search(ub);
@@ -406,33 +458,40 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
                 load_window();
             }
         };
-        // per-lane description of unit ub + lane / tpu (row < 0: no such unit in this batch)
+        // per-lane description of unit ub + (lane >> tpu_shift) (row < 0: no such unit in this batch)
         auto fetch = [&](int ub, int nb, int& row, int& ent, int& nrows, int& page) {
-            const int uu = ub + min(lane / tpu, nb - 1);
+            const int uu = ub + min((lane >> tpu_shift), nb - 1);
             const int k = search(uu);
             int off = uu - __shfl_sync(0xffffffffu, pre_w, k);
             row = -1; ent = 0; nrows = 0; page = 0;
-            if (lane / tpu < nb) {
-                const uint4 v = win[k];
+            if ((lane >> tpu_shift) < nb) {
+                const uint4 v = one_chunk ? gran_s[wq + k] : win[k];
                 int r, pos;
                 a.div_gpr.divmod(wq + k, r, pos);
                 // the segment whose units include number `off` of the granule: first the word, then the byte
                 const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-                int sg = 0;
-                uint32_t w = 0;
-                bool in = false;
+                int n4[4], sg = 0, first = 0;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int n = (int)__dp4a(w4[j], 0x01010101u, 0u);
-                    if (!in) {
-                        if (off < n) { in = true; w = w4[j]; sg = 4 * j; } else off -= n;
-                    }
+                for (int j = 0; j < 4; ++j) n4[j] = (int)__dp4a(w4[j], 0x01010101u, 0u);
+                uint32_t w = w4[0];
+                int upto = n4[0];
+#pragma unroll
+                for (int j = 1; j < 4; ++j) {
+                    if (off >= upto) { sg = 4 * j; w = w4[j]; first = upto; }
+                    upto += n4[j];
                 }
+                const bool in = off < upto;
+                off -= first;
+                upto = 0;
+                first = 0;
+                int sub = 0;
 #pragma unroll
                 for (int j = 0; j < 3; ++j) {
-                    const int n = (int)(w & 0xffu);
-                    if (in && off >= n) { off -= n; w >>= 8; ++sg; } else if (in) { w = 0x7fu; }
+                    upto += (int)((w >> (8 * j)) & 0xffu);
+                    if (off >= upto) { sub = j + 1; first = upto; }
                 }
+                off -= first;
+                sg += sub;
                 row = r;
                 int T = 0;
                 if (!in || a.ungate_last) {
@@ -460,7 +519,6 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             return;
         }
         load_window();
-        first_window = false;
         int u = u0;
         int nb = batch_size(u);
         if (tl2 && lane == 0) tl2[6] = (unsigned long long)clock64() - clk0;
@@ -472,7 +530,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
         // together, so a tile costs the warp a fraction of a pass through this loop; with one tile per pass (its
         // description broadcast by shuffles) the producer took 550 ns a tile, which held every tile of less than 32 KB (64
         // columns or 32 tokens) below half of the copy rate.
-        const int usub = lane % tpu;
+        const int usub = (lane & (tpu - 1));
         const uint64_t once = l2_policy(a.read_once != 0);
         uint32_t fill = 0;
         int piece = -1, prev_row = -1;
@@ -500,13 +558,6 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             unsigned starts = __ballot_sync(0xffffffffu, c_row >= 0 && c_row != (lane == 0 ? prev_row : left));
             const int my_piece = piece + __popc(starts & (0xffffffffu >> (31 - lane)));
             piece += __popc(starts);
-            for (; starts; starts &= starts - 1) {
-                const int sl = __ffs(starts) - 1;
-                const uint32_t f = __shfl_sync(0xffffffffu, my_fill, sl);
-                close_piece(f);
-                prev_row = __shfl_sync(0xffffffffu, c_row, sl);
-                piece_f0 = f;
-            }
             const int stage = (int)(my_fill % NSTAGE);
             const uint32_t parity = ((my_fill / NSTAGE) & 1) ^ 1;
             bool done = !valid;
@@ -546,6 +597,13 @@ decode_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ C
             };
             if (tl2 && lane == 0 && fill == 0) tl2[1] = (unsigned long long)clock64() - clk0;
             bool more = issue_pass();
+            for (; starts; starts &= starts - 1) {
+                const int sl = __ffs(starts) - 1;
+                const uint32_t f = __shfl_sync(0xffffffffu, my_fill, sl);
+                close_piece(f);
+                prev_row = __shfl_sync(0xffffffffu, c_row, sl);
+                piece_f0 = f;
+            }
             // the next batch is fetched once what fits of this one is on its way
             int nbn = 0, n_row = -1, n_ent = 0, n_nrows = 0, n_page = 0;
             if (un < u1) {
@@ -1019,7 +1077,6 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     da.gpr = L.gpr; da.n_gran = L.rows * L.gpr;
     da.n_chunks = (da.n_gran + CHUNK - 1) / CHUNK;
     da.super = (da.n_chunks + MAX_SUPER - 1) / MAX_SUPER;
-    da.lane_gran = da.n_chunks == 1 ? (da.n_gran + 31) / 32 : LGRAN;
     da.ungate_last = (!dense && (params->flags & ETA_FLAG_UNGATE_LAST)) ? 1 : 0;
     da.block_table = pages ? pages->block_table : nullptr;
     da.table_stride = pages ? pages->table_stride : 0;

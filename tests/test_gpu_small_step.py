@@ -114,3 +114,25 @@ def test_small_step_equals_the_general_path(B, Hkv, G, d, b, NB, tail, kw):
         again = small.decode(params, q, tau, const)
         assert all(torch.equal(x, y) for x, y in zip(got[:3], again[:3]))
 
+
+@pytest.mark.parametrize("B,Hkv,b,NB", [(255, 1, 32, 20), (256, 1, 32, 17), (257, 1, 32, 16), (32, 8, 32, 19), (129, 2, 64, 17)])
+def test_a_batch_equals_its_sequences_alone(B, Hkv, b, NB):
+    """Batches that the general path splits over its CTAs by up to 256 or more granules of segments, in one or more warps, against each
+    sequence by itself, which goes the other way."""
+    eb = _eb()
+    G, d, T = 2, 64, NB * b + 9
+    gen = torch.Generator().manual_seed(B)
+    K = (torch.randn((B, Hkv, NB + 1, 1, d), generator=gen) + 0.6 * torch.randn((B, Hkv, NB + 1, b, d), generator=gen))
+    K = K.reshape(B, Hkv, -1, d)[:, :, :T].bfloat16().to(DEV)
+    V = torch.randn((B, Hkv, T, d), generator=gen).bfloat16().to(DEV)
+    q = torch.randn((B, G * Hkv, d), generator=gen).bfloat16().to(DEV)
+    lens = torch.randint(0, T + 1, (B,), generator=gen, dtype=torch.int32)
+    lens[:4 if B > 4 else 1] = torch.tensor([T, 0, b, b - 1][:4 if B > 4 else 1], dtype=torch.int32)
+    tau = (0.8 + 0.3 * torch.randn((B, G * Hkv), generator=gen)).to(DEV)
+    side = _Side(eb, K, V, lens.to(DEV), G * Hkv, b, NB + 1, False, False)
+    out, sel, stats, _ = side.decode(eb.DecodeParams(), q, tau, None)
+    for i in range(B):
+        one = _Side(eb, K[i:i + 1], V[i:i + 1], lens[i:i + 1].to(DEV), G * Hkv, b, NB + 1, False, False)
+        o, m, n, _ = one.decode(eb.DecodeParams(), q[i:i + 1], tau[i:i + 1], None)
+        assert torch.equal(m[0], sel[i]) and torch.equal(n[0], stats[i])
+        assert float((o[0] - out[i]).abs().max()) <= 1.4e-5
