@@ -83,6 +83,17 @@ __device__ __forceinline__ void umma_bf16(uint32_t acc, uint32_t a, uint64_t b, 
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(acc), "r"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// mbar_wait for a warp that others wait for: no sleep between two polls
+__device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity) {
+    for (uint32_t it = 0; it < WAIT_LIMIT; ++it)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
 // arrives on the barrier when every MMA issued so far has completed
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -114,7 +125,8 @@ __device__ __forceinline__ void tmem_store16(uint32_t addr, const uint4 (&q)[4])
 template <int D>
 struct CalSmem {
     static constexpr int K_BYTES = CAL_KEYS * D * 2;
-    static constexpr size_t bytes(int n_bins) { return 1024 + 2 * K_BYTES + 8 * (size_t)n_bins; }
+    static constexpr int copies(int n_bins) { return n_bins <= 2048 ? 2 : 1; }
+    static constexpr size_t bytes(int n_bins) { return 1024 + 2 * K_BYTES + 8 * (size_t)n_bins * copies(n_bins); }
 };
 
 // Clears the histogram (512 KB at 32 heads x 2048 bins: latency).  A kernel of its own, not a memset: the next one is launched
@@ -140,9 +152,14 @@ __global__ void __launch_bounds__(256) calib_clear_kernel(uint4* __restrict__ p,
 // tensor memory, and the queries sit there too (as an operand in shared memory they were read again for every tile: 14
 // million passes, 4.7 are left).  One accumulator of 64 keys: the MMA of a tile runs while the second half of the tile before
 // it is counted.  Two of 32 keys with a barrier each (347 us a calibration, against 313) cost more than they hide, two of 64
-// do not fit the tensor memory of three CTAs beside the queries.  Four CTAs at 56 registers: 321.  With 2048 bins: 515 -> 333 (queries in shared memory) ->
-// 313 us, of which the histogram 435 -> 290; with the launches and the root of today 305.
-template <int D>
+// do not fit the tensor memory of three CTAs beside the queries.  Four CTAs at 56 registers: 321.  Up to 2048 bins the planes have two
+// copies, on even and on odd banks, for even and for odd lanes: 3.46 passes an atomic instead of 3.56 for scores spread over a
+// hundred bins and more, and half as many where they crowd (all scores in one bin, 4 x 1024 tokens: 546 -> 288 us).  The MMAs are issued from
+// a warp that walks along as a whole, their descriptors in uniform registers: 100 cycles a tile, not 600.  With 2048 bins: 515 -> 333
+// (queries in shared memory) -> 313 us, of which the histogram 435 -> 290; with the launches and the root of today 305, with both of
+// these 302.5.  Within 1 % of that: gates in fours over one reciprocal; two CTAs of three groups of warps that count tiles of their
+// own.  What would count for more is fewer passes, but a byte per row and bin takes the shared memory of a whole SM.
+template <int D, int COPIES>
 __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
     const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const float* __restrict__ tau,
     int Hq, int Hkv, int T, float c2, float scale, int n_bins, float s_min, float inv_w,
@@ -151,7 +168,7 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
     extern __shared__ unsigned char cal_raw[];
     unsigned char* sK = cal_raw + ((1024 - (smem_u32(cal_raw) & 1023)) & 1023);       // two key tiles, first of all the queries
     uint32_t* lo = reinterpret_cast<uint32_t*>(sK + 2 * L::K_BYTES);   // histogram: sums of w mod 2^16
-    uint32_t* hi = lo + n_bins;                                        // sums of w / 2^16
+    uint32_t* hi = lo + COPIES * n_bins;                                        // sums of w / 2^16
     __shared__ double s_red[CAL_WARPS];
     __shared__ __align__(8) uint64_t bar_q, bar_in[2], bar_acc, bar_free;      // queries, keys arrived; scores complete; ... read by all
     __shared__ uint32_t s_tmem;
@@ -174,7 +191,7 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
                      ::"r"(smem_u32(&s_tmem)), "r"(CAL_TMEM) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    for (int b = tid; b < 2 * n_bins; b += CAL_THREADS) lo[b] = 0u;
+    for (int b = tid; b < 2 * COPIES * n_bins; b += CAL_THREADS) lo[b] = 0u;
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
@@ -202,42 +219,52 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
     auto flush = [&]() {
         pdl_wait();          // the histogram in memory has been cleared
         for (int b = tid; b < n_bins; b += 32 * CAL_WARPS) {
-            const unsigned long long v = ((unsigned long long)hi[b] << CAL_SPLIT) + lo[b];
+            unsigned long long v;
+            if constexpr (COPIES == 2) {
+                const uint2 l = reinterpret_cast<const uint2*>(lo)[b], u = reinterpret_cast<const uint2*>(hi)[b];
+                v = (((unsigned long long)u.x + u.y) << CAL_SPLIT) + l.x + l.y;
+            } else {
+                v = ((unsigned long long)hi[b] << CAL_SPLIT) + lo[b];
+            }
             if (v) {
                 atomicAdd(&hist[(int64_t)h * n_bins + b], v);
-                lo[b] = 0u; hi[b] = 0u;
+                if constexpr (COPIES == 2) reinterpret_cast<uint2*>(lo)[b] = reinterpret_cast<uint2*>(hi)[b] = make_uint2(0u, 0u);
+                else lo[b] = hi[b] = 0u;
             }
         }
     };
     auto meet = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(32 * CAL_WARPS) : "memory"); };
 
     if (warp == CAL_WARPS) {
-        if (lane == 0) {
-            const int hk = x * Hkv + h / (Hq / Hkv);
-            auto load = [&](int i) {
-                mbar_arrive_expect_tx(&bar_in[i & 1], L::K_BYTES);
-                tma_load_4d(sK + (i & 1) * L::K_BYTES, &tmK, 0, i * CAL_KEYS, 0, hk, &bar_in[i & 1]);
-            };
-            load(0);
-            int issued = 0;                                // tiles whose MMAs are under way or complete
-            for (int i = 0; i < n_tiles; ++i) {
-                // a wait that runs out: nothing more is issued; what is still on its way gets as long again
-                if (!mbar_wait(&bar_in[i & 1], (i >> 1) & 1)) { mbar_wait(&bar_in[i & 1], (i >> 1) & 1); break; }
-                if (i > 0 && !mbar_wait(&bar_free, (i - 1) & 1)) break;
-                if (i + 1 < n_tiles) load(i + 1);          // the scores of the tile before are complete: its keys have been read
-                tmem_fence_after();
-                const uint32_t keys = smem_u32(sK) + (i & 1) * L::K_BYTES;
+        // The whole warp walks along and one lane issues: what an MMA takes (its descriptors) is then computed by the uniform
+        // datapath.
+        const int hk = x * Hkv + h / (Hq / Hkv);
+        const uint64_t keys_0 = umma_operand(smem_u32(sK));
+        auto load = [&](int i) {
+            mbar_arrive_expect_tx(&bar_in[i & 1], L::K_BYTES);
+            tma_load_4d(sK + (i & 1) * L::K_BYTES, &tmK, 0, i * CAL_KEYS, 0, hk, &bar_in[i & 1]);
+        };
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_spin(bar, parity)) != 0; };
+        if (elect_one()) load(0);
+        int issued = 0;                                // tiles whose MMAs are under way or complete
+        for (int i = 0; i < n_tiles; ++i) {
+            // a wait that runs out: nothing more is issued; what is still on its way gets as long again
+            if (!wait(&bar_in[i & 1], (i >> 1) & 1)) { wait(&bar_in[i & 1], (i >> 1) & 1); break; }
+            if (i > 0 && !wait(&bar_free, (i - 1) & 1)) break;
+            tmem_fence_after();
+            const uint64_t keys = keys_0 + (uint32_t)((i & 1) * (L::K_BYTES >> 4));
+            if (elect_one()) {
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k)       // 16 columns: 32 bytes along the swizzled row of a 64-column half
-                    umma_bf16(tmem_acc, tmem + 8 * k, umma_operand(keys + (k / 4) * (CAL_KEYS * 128) + (k % 4) * 32),
-                              CAL_IDESC, k > 0);
+                    umma_bf16(tmem_acc, tmem + 8 * k, keys + (k / 4) * (CAL_KEYS * 128 >> 4) + (k % 4) * 2, CAL_IDESC, k > 0);
                 umma_commit(&bar_acc);
-                ++issued;
+                if (i + 1 < n_tiles) load(i + 1);      // the scores of the tile before are complete: its keys have been read
             }
-            // the counting warps have waited for the last tile already, unless their wait ran out: the MMAs get as long again
-            // before the tensor memory is given back
-            if (issued) mbar_wait(&bar_acc, (issued - 1) & 1);
+            ++issued;
         }
+        // the counting warps have waited for the last tile already, unless their wait ran out: the MMAs get as long again
+        // before the tensor memory is given back
+        if (issued) mbar_wait(&bar_acc, (issued - 1) & 1);
         __syncwarp();
     } else {
         const int l16 = (warp & 3) * 32 + (warp >> 2) * 16;      // the warp's 16 lanes of tensor memory
@@ -255,12 +282,13 @@ __global__ void __launch_bounds__(CAL_THREADS, 3) calib_hist_kernel(
         const uint64_t one2 = pack2(1.f, 1.f);
         uint64_t gs[2] = {one2, one2}, ge[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
         const float b_max = (float)n_bins - 0.5f;
-        const uint32_t lo_addr = smem_u32(lo) - (0x4B000000u << 2), hi_off = (uint32_t)n_bins * 4;
+        constexpr int SHIFT = COPIES == 2 ? 3 : 2;
+        const uint32_t lo_addr = smem_u32(lo) + (COPIES == 2 ? 4 * (lane & 1) : 0) - (0x4B000000u << SHIFT), hi_off = (uint32_t)n_bins * 4 * COPIES;
 
         auto add = [&](float y, int row) {
             // floor(y) sits in the low bits of 2^23 + y rounded down; the exponent bits are folded into lo_addr
             const float f = __fadd_rd(fminf(fmaxf(y, 0.f), b_max), 8388608.f);
-            const uint32_t addr = lo_addr + (__float_as_uint(f) << 2);
+            const uint32_t addr = lo_addr + (__float_as_uint(f) << SHIFT);
             red_shared(addr, wl[row]);
             red_shared(addr + hi_off, wh[row]);
         };
@@ -449,10 +477,11 @@ template <int D>
 static int launch_hist(const CUtensorMap& tmQ, const CUtensorMap& tmK, const float* tau, int Hq, int Hkv, int T, int n_seq,
                        float c2, float scale, int n_bins, float s_min, float inv_w, unsigned long long* hist, double* dpart,
                        cudaStream_t s) {
-    const int rc = configure_kernel(reinterpret_cast<const void*>(calib_hist_kernel<D>), CalSmem<D>::bytes(4096));
+    auto kernel = CalSmem<D>::copies(n_bins) == 2 ? calib_hist_kernel<D, 2> : calib_hist_kernel<D, 1>;
+    const int rc = configure_kernel(reinterpret_cast<const void*>(kernel), CalSmem<D>::bytes(4096));
     if (rc != ETA_OK) return rc;
     const dim3 grid((unsigned)Hq, (unsigned)n_seq, (unsigned)((T + CAL_ROWS - 1) / CAL_ROWS));
-    return launch_pdl("calibration histogram", calib_hist_kernel<D>, grid, dim3(CAL_THREADS), CalSmem<D>::bytes(n_bins), s, tmQ, tmK,
+    return launch_pdl("calibration histogram", kernel, grid, dim3(CAL_THREADS), CalSmem<D>::bytes(n_bins), s, tmQ, tmK,
                       tau, Hq, Hkv, T, c2, scale, n_bins, s_min, inv_w, hist, dpart);
 }
 
