@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4
         a.div_hkv.divmod(rr, i, hk);
         Traw = __ldg(a.seq_lens + i);
     }
+    const uint4 q_piece = dense ? make_uint4(0, 0, 0, 0) : load_qtab<D, G>(a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
     const int r = i * a.Hkv + hk, head = max(tp, a.need);
     const int p_first = c == 0 ? 0 : head + (c - 1) * tp, p_last = min(P, head + c * tp);
     const int T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4
     __syncwarp();
     TileStream<D, G, PACKED> ts{sm + L::TILE_OFF + warp * a.nbuf * TL::BYTES, bars, rec_row, mn_row, dense ? 0 : NB, a.nbuf, 0, 0, 0u, true};
     for (int p = p_first; p < min(p_last, p_first + a.nbuf); ++p) ts.issue(p * TL::PASS + warp * TL::RECS);
-    if (!dense) build_qtab<D, G>(tab, a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
+    if (!dense) build_qtab<D, G>(tab, q_piece, tid);
 
     // an ungated newest token must be attended: when it closes a full block, that block counts as pinned
     const int lwb = ((a.flags & ETA_FLAG_UNGATE_LAST) && T > 0 && (T & (a.b - 1)) == 0 && a.lwb < 1) ? 1 : a.lwb;
@@ -388,6 +389,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     // for 1.07 GB, three inputs in turn.)
     pdl_wait();
     int T = __ldcg(seq_lens + i);
+    const uint4 q_piece = load_qtab<D, G>(q + ((int64_t)i * Hq + hk * G) * D, tid);
     T = T < 0 ? 0 : (T > t_cap ? t_cap : T);
     const int NB = min(T / b, nb_cap);
     const int first = (blockIdx.x % chunks) * per * TL::PASS;
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
                                 mnorm + (int64_t)r * nb_cap, NB, 1, 0, 0, 0u, true};
     const int last = min(NB, first + per * TL::PASS);
     ts.issue(first + warp * TL::RECS);
-    build_qtab<D, G>(tab, q + ((int64_t)i * Hq + hk * G) * D, tid);
+    build_qtab<D, G>(tab, q_piece, tid);
     for (int j0 = first + warp * TL::RECS; j0 < last; j0 += TL::PASS) {
         const int n = min(TL::RECS, NB - j0);
         ts.bounds(tab, j0, z, scale, sb);

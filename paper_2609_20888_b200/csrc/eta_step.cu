@@ -25,7 +25,7 @@ template <int D, int TS, int G>
 struct StepSmem {
     static constexpr int STAGE_BYTES = 4 * D * TS, NSTAGE = STEP_RING / STAGE_BYTES;
     static_assert(NSTAGE % 3 == 0, "a stage serves the same group in every round");
-    static_assert(STEP_WARPS * TileOf<D>::BYTES <= STEP_RING && STEP_WARPS * G * D * 4 <= STEP_RING, "what shares the ring fits it");
+    static_assert(2 * STEP_WARPS * TileOf<D>::BYTES <= STEP_RING && STEP_WARPS * G * D * 4 <= STEP_RING, "what shares the ring fits it");
     static constexpr int BAR_OFF = STEP_RING;           // full[NSTAGE], empty[NSTAGE], two per warp for its records
     static constexpr int TAB_OFF = (BAR_OFF + 8 * (2 * NSTAGE + 2 * STEP_WARPS) + 15) / 16 * 16;
     static constexpr int BOUND_OFF = TAB_OFF + (int)((sizeof(QTab<D, G>) + 15) / 16 * 16);
@@ -40,10 +40,12 @@ struct StepSmem {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-// What bounds it: latency, of a chain that starts when the thresholds are there: the newest bound and admission (1 us), the list (0.5),
-// the first tiles (1.5 from the L2, more from memory), a tile every 0.6 us of a CTA, the parts of the warps and of the CTAs (1.5).
+// What bounds it: latency, of a chain of short parts: us from the entry, 8 rows of 16K tokens: query table 1.5, bounds 3.1, those of
+// the other CTAs 5.2, thresholds 5.5 (they have been there), list 7.0, first tile 8.2, last 10.6, the parts of the warps and of the CTAs 3.4.
+// What it took out of the chain to load q beside the length (it sets the entry's time), to read a record's bounds in one piece and a
+// head's rescue once, and to load the CTAs' parts eight at a time: 17.7 -> 17.2 us a step there, 12.9 -> 12.3 for 2 rows of 2K.
 // Bounds of the row in each CTA where they are one round of its warps, else in shares, which the cluster exchanges: 1.2 us slower
-// for 32 blocks, 1.2 faster for 257 and 4 for 511.  Six 32 KB tiles in flight: with three, rows of 256 blocks, half of them
+// for 32 blocks, 1.1 faster for 256 and 4 for 511.  Two tiles of records in flight per warp where a share is more than one.  Six 32 KB tiles in flight: with three, rows of 256 blocks, half of them
 // attended, took 29.5 us instead of 25.5.  Parts are stored to the CTA that adds them up, not fetched by it: one barrier of the
 // cluster instead of two, 0.6 to 0.8 us.
 template <int D, int TS, int G, bool PACKED>
@@ -69,7 +71,9 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
     const int r = blockIdx.x / n_ranks;
     int i, hk;
     a.div_hkv.divmod(r, i, hk);
-    const int Traw = __ldcg(a.seq_lens + i), T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
+    const int Traw = __ldcg(a.seq_lens + i);
+    const uint4 q_piece = load_qtab<D, G>(a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
+    const int T = Traw < 0 ? 0 : (Traw > a.t_cap ? a.t_cap : Traw);
     const int NB = min(T >> a.b_shift, a.nb_cap), b = 1 << a.b_shift;
     const unsigned char* const rec_row = reinterpret_cast<const unsigned char*>(a.musig) + (int64_t)r * a.nb_cap * REC_BYTES;
     const float* const mn_row = a.mnorm + (int64_t)r * a.nb_cap;
@@ -77,7 +81,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
     // ------------------------------------------------------------ bounds of the row's blocks, a share per CTA: needs neither the
     // thresholds nor the newest record (see below), so it does not wait for the kernels that make them
     if (a.shared) cluster_arrive();       // (all CTAs of the cluster run when all have come by here)
-    const int of = a.shared ? n_ranks : 1, mine = a.shared ? rank : 0;
+    const int of = a.shared ? n_ranks : 1, first = (warp * of + (a.shared ? rank : 0)) * TL::RECS, stride = STEP_WARPS * of * TL::RECS;
     if (tid == 0) {
         for (int s = 0; s < L::NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], WARPS_PER_GROUP); }
         fence_barrier_init();
@@ -85,19 +89,19 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
         prefetch_tmap(&tmV);
     }
     uint64_t* const bars = empty + L::NSTAGE + 2 * warp;
-    TileStream<D, G, PACKED> ts{sm + warp * TL::BYTES, bars, rec_row, mn_row, NB, 1, 0, 0, 0u, true};
+    TileStream<D, G, PACKED> ts{sm + warp * 2 * TL::BYTES, bars, rec_row, mn_row, NB, 2, 0, 0, 0u, true};
     if (warp < STEP_WARPS) {
         if (lane == 0) { mbar_init(&bars[0], 1); mbar_init(&bars[1], 1); fence_barrier_init(); }
         __syncwarp();
-        ts.issue((warp * of + mine) * TL::RECS);
+        ts.issue(first);
+        ts.issue(first + stride);
     }
-    build_qtab<D, G>(tab, a.q + ((int64_t)i * a.Hq + hk * G) * D, tid);
+    build_qtab<D, G>(tab, q_piece, tid);
     bool ok = true;
-    const int first = (warp * of + mine) * TL::RECS, stride = STEP_WARPS * of * TL::RECS;
     if (warp < STEP_WARPS) {
         for (int j = first; j < NB; j += stride) {
             ok = ts.bounds(tab, j, a.z, a.scale, sbound + j * G) && ok;
-            if (j + stride < NB) ts.issue(j + stride);
+            if (j + 2 * stride < NB) ts.issue(j + 2 * stride);
         }
     }
     Attend<D, TS> at(lane, warp % WARPS_PER_GROUP, G);
@@ -160,19 +164,30 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
     unsigned m[SEG / 32] = {};
     int carry = 0;
     if (warp < STEP_SEGS && j0 < a.nb_cap) {
+        float te_g[G];
+        int best[G];
 #pragma unroll
         for (int gq = 0; gq < G; ++gq) {
-            const float te_g = __shfl_sync(0xffffffffu, te_l, gq);
-            const int best = rescues && key_bound(s_bkey[gq]) < te_g ? s_best[gq] : -1;
-#pragma unroll
-            for (int half = 0; half < SEG / 32; ++half) {
-                const int j = j0 + half * 32 + lane;
-                if (j < NB && (j >= NB - lwb || j == best || !(sbound[j * G + gq] < te_g))) m[half] |= 1u << gq;
-            }
+            te_g[gq] = __shfl_sync(0xffffffffu, te_l, gq);
+            best[gq] = rescues && key_bound(s_bkey[gq]) < te_g[gq] ? s_best[gq] : -1;
         }
 #pragma unroll
         for (int half = 0; half < SEG / 32; ++half) {
             const int j = j0 + half * 32 + lane;
+            if (j < NB) {
+                const bool pinned = j >= NB - lwb;
+                float bd[G];
+                constexpr int V = G < 4 ? G : 4;              // a record's bounds in pieces of up to 16 bytes
+#pragma unroll
+                for (int g0 = 0; g0 < G; g0 += V) {
+                    if constexpr (V == 4) *reinterpret_cast<float4*>(bd + g0) = *reinterpret_cast<const float4*>(sbound + j * G + g0);
+                    else if constexpr (V == 2) *reinterpret_cast<float2*>(bd) = *reinterpret_cast<const float2*>(sbound + j * 2);
+                    else bd[0] = sbound[j];
+                }
+#pragma unroll
+                for (int gq = 0; gq < G; ++gq)
+                    if (pinned || j == best[gq] || !(bd[gq] < te_g[gq])) m[half] |= 1u << gq;
+            }
             if (rank == 0 && j < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j] = (uint8_t)m[half];
             carry += __popc(__ballot_sync(0xffffffffu, m[half] != 0));
         }
@@ -303,16 +318,30 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
     if (tid < per && idx < G * D / 4) {
         const int h = idx / (D / 4);
         float M = -INFINITY, l = 0.f;
-        for (int c = 0; c < n_ranks; ++c) M = fmaxf(M, in_ml[c * G + h].x);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (M != -INFINITY) {
-            for (int c = 0; c < n_ranks; ++c) {
-                const float2 p = in_ml[c * G + h];
-                const float4 x = in_o[c * per + tid];
-                const float sc = exp2f((p.x - M) * LOG2E);            // a CTA without tiles: 0
-                acc.x = fmaf(x.x, sc, acc.x); acc.y = fmaf(x.y, sc, acc.y);
-                acc.z = fmaf(x.z, sc, acc.z); acc.w = fmaf(x.w, sc, acc.w);
-                l = fmaf(p.y, sc, l);
+#pragma unroll 1
+        for (int c0 = 0; c0 < n_ranks; c0 += 8) {               // eight parts at a time
+            float2 p[8];
+            float4 x[8];
+            float top = M;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const bool in = c0 + c < n_ranks;
+                p[c] = in ? in_ml[(c0 + c) * G + h] : make_float2(-INFINITY, 0.f);
+                x[c] = in ? in_o[(c0 + c) * per + tid] : make_float4(0.f, 0.f, 0.f, 0.f);
+                top = fmaxf(top, p[c].x);
+            }
+            if (top == -INFINITY) continue;
+            const float keep = exp2f((M - top) * LOG2E);
+            acc.x *= keep; acc.y *= keep; acc.z *= keep; acc.w *= keep;
+            l *= keep;
+            M = top;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const float sc = exp2f((p[c].x - M) * LOG2E);            // a CTA without tiles: 0
+                acc.x = fmaf(x[c].x, sc, acc.x); acc.y = fmaf(x[c].y, sc, acc.y);
+                acc.z = fmaf(x[c].z, sc, acc.z); acc.w = fmaf(x[c].w, sc, acc.w);
+                l = fmaf(p[c].y, sc, l);
             }
         }
         if (l > 0.f) { acc.x /= l; acc.y /= l; acc.z /= l; acc.w /= l; }
