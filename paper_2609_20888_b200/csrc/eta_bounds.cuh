@@ -22,11 +22,11 @@ __device__ __forceinline__ float key_bound(uint32_t k) { return __uint_as_float(
 
 constexpr int SCR_WARPS = 4;
 
-// A warp's tile: 8 KB of unpacked records, NT 8-column MMA tiles
+// A warp's tile: 8 KB of unpacked records, MT MMA tiles of 16 rows
 template <int D>
 struct TileOf {
-    static constexpr int NT = 256 / D;                        // 2 at head_dim 128, 4 at 64
-    static constexpr int RECS = 8 * NT;
+    static constexpr int MT = 128 / D;                        // 1 at head_dim 128, 2 at 64
+    static constexpr int RECS = 16 * MT;
     static constexpr int PASS = SCR_WARPS * RECS;             // records a CTA bounds at a time: 64 or 128
     static constexpr int BYTES = RECS * 4 * D;
     static_assert(PASS % SEG == 0, "a pass covers whole segments");
@@ -43,16 +43,16 @@ __device__ __forceinline__ void mma_tf32_1688(float (&c)[4], float a0, float a1,
 // the rest of a 22-bit product fits tf32 too
 __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
-// The query side of a row's bounds, in the order the MMAs want it.  Lane (hd = lane / 4, t = lane % 4) feeds row hd (and
-// hd + 8) of A; in k-group j (32 coordinates) it holds coordinates 8 (4 j + t) .. + 7, the ones its 16-byte piece of a
-// record covers on the B side (a dot product does not care about the order of k).
+// The query side of a row's bounds, in the order the MMAs want it.  Lane (hd = lane / 4, t = lane % 4) feeds column hd of B; in
+// k-group j (32 coordinates) it holds coordinates 8 (4 j + t) .. + 7, the ones its 16-byte pieces of two records cover on the A
+// side (a dot product does not care about the order of k).
 template <int D, int G>
 struct QTab {
     static constexpr int J = D / 32;
-    static constexpr int NLO = (G == 8) ? 1 : 0;      // eight heads fill rows 0-7 of A: the second parts go to rows 8-15
+    static constexpr int NLO = (G == 8) ? 1 : 0;      // eight heads fill the columns of B: the second parts are another B
     uint4 f16[J][32];                                 // scaled q as fp16
-    float4 sq[J][32][2];                              // q^2: rows 0-3 leading parts of heads 0-3, rows 4-7 the rest (G <= 4);
-                                                      //      rows 0-7 leading parts (G = 8)
+    float4 sq[J][32][2];                              // q^2: columns 0-3 leading parts of heads 0-3, columns 4-7 the rest (G <= 4);
+                                                      //      columns 0-7 leading parts (G = 8)
     float4 sq_lo[NLO ? J : 1][NLO ? 32 : 1][2];       // G = 8: the rest
     uint4 raw[G * D / 8];                             // the queries as they are (bf16)
     float n2[J][8];                                   // partial squared norms
@@ -77,7 +77,7 @@ __device__ __forceinline__ float qtab_unscale(float qn) {
 // step; 512K: 42.9 -> 42.5).
 template <int D, int G>
 __device__ __forceinline__ uint4 load_qtab(const __nv_bfloat16* q, int tid) {
-    const int head = ((tid & 31) >> 2) & (G == 8 ? 7 : 3);         // rows 4-7 hold the second parts of heads 0-3
+    const int head = ((tid & 31) >> 2) & (G == 8 ? 7 : 3);         // columns 4-7 hold the second parts of heads 0-3
     uint4 v = make_uint4(0, 0, 0, 0);
     if (tid < D && head < G) v = __ldcg(reinterpret_cast<const uint4*>(q + head * D + 8 * (4 * (tid >> 5) + (tid & 3))));
     return v;
@@ -166,64 +166,88 @@ __device__ __forceinline__ void sigma_f32(const SigmaPiece<PACKED>& s, float (&o
 // `lane`.  sigma^2 has at most 22 significant bits (sigma is fp16) and q^2 sixteen: each is the sum of two tf32 values, every
 // product of parts is exact and the accumulation is fp32, so the variance term is as good as one computed on the fp32
 // pipe, without a shuffle tree and with a quarter of the fp32 instructions.
-// -> whether some lane saw a NaN among the bounds of the first n records.  Two accumulators for the variance term: a tile
-// is a chain of dependent MMAs, and its latency is what a CTA of one or two tiles per warp takes (unrolling k gained nothing).
+// -> whether some lane saw a NaN among the bounds of the first n records.
+// What bounds it: an MMA of this kind takes a scheduler 8 cycles whatever its k, 21 in a chain.  So the records are the rows of A (16)
+// and the queries the columns of B (eight heads, or four and their second parts): 40 MMAs for 8 KB of records at d = 128 and G <= 4
+// where queries as rows, half of them empty, took 80, and the same sums in the same order.  us a step before and after: 16 rows of up
+// to 64K tokens 131.8 -> 129.1, 512K x 1 43.0 -> 42.2, 128K x 4 58.9 -> 58.1, 16K x 1 17.4 -> 17.0.  Two accumulators for the variance
+// term: a tile is a chain of dependent MMAs.  Unrolling the loop over j by two (129.8) or pairs in the packed fp32 instructions (130.0)
+// gained nothing.
 template <int D, int G, bool PACKED>
 __device__ __forceinline__ bool bound_tile(const QTab<D, G>& tab, uint32_t recs, int n, float mn, float z, float scale,
                                            float* __restrict__ sb) {
-    constexpr int J = D / 32, NT = TileOf<D>::NT, REC = PACKED ? 3 * D : 4 * D;
+    constexpr int J = D / 32, MT = TileOf<D>::MT, REC = PACKED ? 3 * D : 4 * D, NQ = G == 8 ? 2 : 1;
     const int lane = threadIdx.x & 31, n8 = lane >> 2, t = lane & 3;
     const uint32_t rp = recs + n8 * REC;
-    float dot[NT][4], vhi[NT][4], vlo[NT][4];
+    float dot[MT][4], vhi[MT][NQ][4], vlo[MT][NQ][4];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { dot[nt][c] = 0.f; vhi[nt][c] = 0.f; vlo[nt][c] = 0.f; }
+        for (int c = 0; c < 4; ++c) {
+            dot[mt][c] = 0.f;
+#pragma unroll
+            for (int p = 0; p < NQ; ++p) { vhi[mt][p][c] = 0.f; vlo[mt][p][c] = 0.f; }
+        }
 #pragma unroll 1
     for (int j = 0; j < J; ++j) {
         const uint4 qa = tab.f16[j][lane];
-        const float4 sa = tab.sq[j][lane][0], sb4 = tab.sq[j][lane][1];
-        float4 la = make_float4(0.f, 0.f, 0.f, 0.f), lb = la;
-        if constexpr (G == 8) { la = tab.sq_lo[j][lane][0]; lb = tab.sq_lo[j][lane][1]; }
-        uint4 mu[NT];
-        SigmaPiece<PACKED> sg[NT];
+        float4 q2[NQ][2] = {{tab.sq[j][lane][0], tab.sq[j][lane][1]}};
+        if constexpr (G == 8) { q2[1][0] = tab.sq_lo[j][lane][0]; q2[1][1] = tab.sq_lo[j][lane][1]; }
+        uint4 mu[MT][2];
+        SigmaPiece<PACKED> sg[MT][2];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            mu[nt] = lds128(rp + nt * 8 * REC + (4 * j + t) * 16);
-            load_sigma_shared<D, PACKED>(sg[nt], rp + nt * 8 * REC, 4 * j + t);
-        }
+        for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            mma_f16_16816(dot[nt], qa.x, 0u, qa.y, 0u, mu[nt].x, mu[nt].y);
-            mma_f16_16816(dot[nt], qa.z, 0u, qa.w, 0u, mu[nt].z, mu[nt].w);
-            float s[8], hi[8];
-            sigma_f32<PACKED>(sg[nt], s);
+            for (int e = 0; e < 2; ++e) {             // records n8 and n8 + 8
+                mu[mt][e] = lds128(rp + (mt * 16 + e * 8) * REC + (4 * j + t) * 16);
+                load_sigma_shared<D, PACKED>(sg[mt][e], rp + (mt * 16 + e * 8) * REC, 4 * j + t);
+            }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) { s[k] *= s[k]; hi[k] = tf32_hi(s[k]); s[k] -= hi[k]; }
-            mma_tf32_1688(vhi[nt], sa.x, la.x, sa.y, la.y, hi[0], hi[1]);
-            mma_tf32_1688(vlo[nt], sa.x, la.x, sa.y, la.y, s[0], s[1]);
-            mma_tf32_1688(vhi[nt], sa.z, la.z, sa.w, la.w, hi[2], hi[3]);
-            mma_tf32_1688(vlo[nt], sa.z, la.z, sa.w, la.w, s[2], s[3]);
-            mma_tf32_1688(vhi[nt], sb4.x, lb.x, sb4.y, lb.y, hi[4], hi[5]);
-            mma_tf32_1688(vlo[nt], sb4.x, lb.x, sb4.y, lb.y, s[4], s[5]);
-            mma_tf32_1688(vhi[nt], sb4.z, lb.z, sb4.w, lb.w, hi[6], hi[7]);
-            mma_tf32_1688(vlo[nt], sb4.z, lb.z, sb4.w, lb.w, s[6], s[7]);
+        for (int mt = 0; mt < MT; ++mt) {
+            mma_f16_16816(dot[mt], mu[mt][0].x, mu[mt][1].x, mu[mt][0].y, mu[mt][1].y, qa.x, qa.y);
+            mma_f16_16816(dot[mt], mu[mt][0].z, mu[mt][1].z, mu[mt][0].w, mu[mt][1].w, qa.z, qa.w);
+            float hi[2][8], lo[2][8];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                sigma_f32<PACKED>(sg[mt][e], lo[e]);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) { lo[e][k] *= lo[e][k]; hi[e][k] = tf32_hi(lo[e][k]); lo[e][k] -= hi[e][k]; }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; k += 2)
+#pragma unroll
+                for (int p = 0; p < NQ; ++p) {
+                    const float4 b = q2[p][k / 4];
+                    const float b0 = k % 4 ? b.z : b.x, b1 = k % 4 ? b.w : b.y;
+                    mma_tf32_1688(vhi[mt][p], hi[0][k], hi[1][k], hi[0][k + 1], hi[1][k + 1], b0, b1);
+                    mma_tf32_1688(vlo[mt][p], lo[0][k], lo[1][k], lo[0][k + 1], lo[1][k + 1], b0, b1);
+                }
         }
     }
-    // lane (head n8, t) holds records 8 nt + 2 t and + 1
-    const float qn = tab.norm[n8 < G ? n8 : 0], un = qtab_unscale(qn);
+    // lane (n8, t) holds records n8 and n8 + 8 of columns 2 t and 2 t + 1
+    const bool mine = 2 * t < G;
+    float qn[2], un[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) { qn[c] = tab.norm[2 * t + c < G ? 2 * t + c : 0]; un[c] = qtab_unscale(qn[c]); }
     bool bad = false;
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const float v = vhi[nt][c] + vlo[nt][c];
-            const float v2 = v + (G == 8 ? vhi[nt][c + 2] + vlo[nt][c + 2] : __shfl_xor_sync(0xffffffffu, v, 16));
-            const int rec = nt * 8 + 2 * t + c;
+        for (int e = 0; e < 2; ++e) {
+            const int rec = mt * 16 + e * 8 + n8;
             const float m = __shfl_sync(0xffffffffu, mn, rec);
-            const float bound = scale * min_keep_nan((dot[nt][c] + z * sqrtf(v2)) * un, qn * m);
-            if (n8 < G) sb[rec * G + n8] = bound;
-            bad = bad || (n8 < G && rec < n && bound != bound);
+            float bound[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float v = vhi[mt][0][2 * e + c] + vlo[mt][0][2 * e + c];
+                const float v2 = v + (G == 8 ? vhi[mt][NQ - 1][2 * e + c] + vlo[mt][NQ - 1][2 * e + c] : __shfl_xor_sync(0xffffffffu, v, 2));
+                bound[c] = scale * min_keep_nan((dot[mt][2 * e + c] + z * sqrtf(v2)) * un[c], qn[c] * m);
+                bad = bad || (2 * t + c < G && rec < n && bound[c] != bound[c]);
+            }
+            if (mine) {
+                if constexpr (G == 1) sb[rec] = bound[0];
+                else *reinterpret_cast<float2*>(sb + rec * G + 2 * t) = make_float2(bound[0], bound[1]);
+            }
         }
     __syncwarp();
     return __any_sync(0xffffffffu, bad);
