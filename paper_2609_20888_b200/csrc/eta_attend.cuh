@@ -27,8 +27,10 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 // One warp's part.  Lane (g, t) = (lane / 4, lane % 4) holds head g's scores and statistics (its share of the sum l_run: tokens are
-// spread over t), and heads 2 t and 2 t + 1 of the accumulators.
-template <int D, int TS>
+// spread over t), and heads 2 t and 2 t + 1 of the accumulators.  CHAINS = 2: a score is summed in two halves, so that a tile waits for
+// half as many dependent MMAs (21 cycles each); for a kernel that is bound by a tile's latency (8 rows of 16K tokens 16.7 -> 16.2 us
+// a step), not for one that streams (128K x 4 57.7 -> 58.0: registers).
+template <int D, int TS, int CHAINS = 1>
 struct Attend {
     static constexpr int HALVES = D / 64;
     static constexpr int WT = TS / WARPS_PER_GROUP;    // tokens per warp per tile (8 or 16)
@@ -91,11 +93,13 @@ struct Attend {
         constexpr float LOG2E = 1.4426950408889634f;
         const uint32_t vbase = kbase + HALVES * TILE_BYTES;
         // ---- S = q K^T for this warp's WT tokens: heads on M (rows 8..15 are padding), tokens on N
-        float sacc[NT][4];
+        float sacc[CHAINS][NT][4];
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) sacc[nt][c] = 0.f;
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int h = 0; h < CHAINS; ++h) sacc[h][nt][c] = 0.f;
         {
             uint4 kv[HALVES][2][NT];
 #pragma unroll
@@ -110,8 +114,8 @@ struct Attend {
                 for (int m = 0; m < 2; ++m)
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
-                        mma_bf16_16816(sacc[nt], qa[hf][m][0], 0u, qa[hf][m][1], 0u, kv[hf][m][nt].x, kv[hf][m][nt].y);
-                        mma_bf16_16816(sacc[nt], qa[hf][m][2], 0u, qa[hf][m][3], 0u, kv[hf][m][nt].z, kv[hf][m][nt].w);
+                        mma_bf16_16816(sacc[0][nt], qa[hf][m][0], 0u, qa[hf][m][1], 0u, kv[hf][m][nt].x, kv[hf][m][nt].y);
+                        mma_bf16_16816(sacc[CHAINS - 1][nt], qa[hf][m][2], 0u, qa[hf][m][3], 0u, kv[hf][m][nt].z, kv[hf][m][nt].w);
                     }
         }
         // V pieces are requested now so that their latency hides behind the softmax arithmetic
@@ -133,7 +137,7 @@ struct Attend {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int trow = rb + nt * 8 + (c ? r1 : r0);
-                const float S = sacc[nt][c] * scale;
+                const float S = (CHAINS == 2 ? sacc[0][nt][c] + sacc[CHAINS - 1][nt][c] : sacc[0][nt][c]) * scale;
                 float gated = S;
                 if (gate_on) {
                     const float x = (beta == 0.f) ? 0.f : beta * (S - te);

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
             if (j + 2 * stride < NB) ts.issue(j + 2 * stride);
         }
     }
-    Attend<D, TS> at(lane, warp % WARPS_PER_GROUP, G);
+    Attend<D, TS, 2> at(lane, warp % WARPS_PER_GROUP, G);
     at.load_q(a.q + ((int64_t)i * a.Hq + hk * G + (at.head ? at.g : 0)) * D);
     if (a.shared) {                       // every CTA gets all of them
         cluster_wait();
