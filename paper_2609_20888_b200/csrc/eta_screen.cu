@@ -56,9 +56,10 @@ __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
 // resident at once, because none can finish before the thresholds are there.  A step of 65536 blocks at d = 128, G = 4 took
 // 68.8 us instead of 71.1 with it (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
 // barrier per segment); 65536 blocks at d = 64, G = 8, where both terms were on that pipe, 116.3 instead of 126.9.
-// 80 registers at d = 128, 96 at 64: CTAs start beside those of the append and the predictor, and with 88 fewer of them fit
-// there (32K x 8 48.8 -> 49.5 us, 128K x 4 55.5 -> 57.2, graph replay).  The bound of six CTAs holds the instances to 80 that would
-// take more by themselves; the others take 78 to 80 at five and lose by it (512K x 1 43.4 -> 44.4 with the 73 that six give).
+// Registers: CTAs start beside those of the append and the predictor, and with more registers fewer of them fit there.  The bound of
+// six CTAs holds the instances to 80 that would take many more by themselves.  The others take 78 to 86 at five (96 at d = 64, G = 8):
+// six gives d = 128, G = 4 48.5 instead of 49.1 us at 32K x 8, but 57.9 instead of 57.6 at 128K x 4 and 41.9 instead of 41.5 at 512K x 1,
+// and d = 64 32.8 instead of 31.8 at 64K x 4 (G = 1).
 template <int D, int G, bool PACKED>
 __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4 && PACKED)) ? 6 : 5) screen_kernel(
     const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const ScreenArgs a) {

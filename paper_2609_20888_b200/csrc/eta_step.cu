@@ -44,6 +44,8 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // the other CTAs 5.2, thresholds 5.5 (they have been there), list 7.0, first tile 8.2, last 10.6, the parts of the warps and of the CTAs 3.4.
 // What it took out of the chain to load q beside the length (it sets the entry's time), to read a record's bounds in one piece and a
 // head's rescue once, and to load the CTAs' parts eight at a time: 17.7 -> 17.2 us a step there, 12.9 -> 12.3 for 2 rows of 2K.
+// Code that runs once is fetched as it runs: admission as a loop over a segment's halves, not unrolled, 4 rows of 32K 18.9 -> 18.6, 8
+// rows 19.7 -> 19.1.
 // Bounds of the row in each CTA where they are one round of its warps, else in shares, which the cluster exchanges: 1.2 us slower
 // for 32 blocks, 1.1 faster for 256 and 4 for 511.  Two tiles of records in flight per warp where a share is more than one.  Six 32 KB tiles in flight: with three, rows of 256 blocks, half of them
 // attended, took 29.5 us instead of 25.5.  Parts are stored to the CTA that adds them up, not fetched by it: one barrier of the
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
 
     // ------------------------------------------------------------ admission, a warp per segment
     const int j0 = warp * SEG;
-    unsigned m[SEG / 32] = {};
+    unsigned admitted = 0;                // a byte per half: heads that attend record j0 + 32 half + lane
     int carry = 0;
     if (warp < STEP_SEGS && j0 < a.nb_cap) {
         float te_g[G];
@@ -171,9 +173,10 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
             te_g[gq] = __shfl_sync(0xffffffffu, te_l, gq);
             best[gq] = rescues && key_bound(s_bkey[gq]) < te_g[gq] ? s_best[gq] : -1;
         }
-#pragma unroll
+#pragma unroll 1
         for (int half = 0; half < SEG / 32; ++half) {
             const int j = j0 + half * 32 + lane;
+            unsigned m = 0;
             if (j < NB) {
                 const bool pinned = j >= NB - lwb;
                 float bd[G];
@@ -186,25 +189,23 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
                 }
 #pragma unroll
                 for (int gq = 0; gq < G; ++gq)
-                    if (pinned || j == best[gq] || !(bd[gq] < te_g[gq])) m[half] |= 1u << gq;
+                    if (pinned || j == best[gq] || !(bd[gq] < te_g[gq])) m |= 1u << gq;
             }
-            if (rank == 0 && j < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j] = (uint8_t)m[half];
-            carry += __popc(__ballot_sync(0xffffffffu, m[half] != 0));
+            if (rank == 0 && j < a.nb_cap) a.sel_mask[(int64_t)r * a.nb_cap + j] = (uint8_t)m;
+            admitted |= m << (8 * half);
+            carry += __popc(__ballot_sync(0xffffffffu, m != 0));
         }
     }
     if (warp < STEP_SEGS && lane == 0) s_cnt[warp] = carry;
     __syncthreads();
-    int n_blocks = 0, at_list = 0;
-#pragma unroll
-    for (int s = 0; s < STEP_SEGS; ++s) {
-        if (s < warp) at_list += s_cnt[s];
-        n_blocks += s_cnt[s];
-    }
+    const int cnt = lane < STEP_SEGS ? s_cnt[lane] : 0;
+    const int n_blocks = __reduce_add_sync(0xffffffffu, cnt);
+    int at_list = __reduce_add_sync(0xffffffffu, lane < warp ? cnt : 0);
     if (warp < STEP_SEGS) {
-#pragma unroll
+#pragma unroll 1
         for (int half = 0; half < SEG / 32; ++half) {
-            const unsigned nz = __ballot_sync(0xffffffffu, m[half] != 0);
-            if (m[half]) list[at_list + __popc(nz & ((1u << lane) - 1u))] = (j0 + half * 32 + lane) | (int)(m[half] << 24);
+            const unsigned m = (admitted >> (8 * half)) & 0xff, nz = __ballot_sync(0xffffffffu, m != 0);
+            if (m) list[at_list + __popc(nz & ((1u << lane) - 1u))] = (j0 + half * 32 + lane) | (int)(m << 24);
             at_list += __popc(nz);
         }
     }
@@ -376,11 +377,12 @@ static int launch_step_t(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& 
 }
 
 // Which problems, by what the host knows: the capacity.  A row's cluster has to do alone what the general path spreads over the GPU,
-// so a step is bound by the fullest row; what it saves is two kernels, 6 to 7 us.  us a step, general and this, half / a tenth of
-// the blocks attended (d = 128, blocks of 64, queued calls): 8 rows of 2K 20.7, 14.2 / 19.8, 13.7; 16K 29.2, 24.2 / 22.7, 17.7; 32K
-// 35.3, 32.5 / 23.7, 20.0; 16 rows of 16K 34.5, 30.5 / 23.2, 18.4; 64 rows of 2K 29.1, 23.2 / 21.6, 16.4; 128 rows of 2K 38.7, 31.2 /
-// 28.1, 21.9.  Beyond the line rows of unequal lengths and survivors lose: 24 rows of up to 32K 46.0, 60.7 / 29.5, 27.4, 64 of up to
-// 16K 50.0, 70.6 / 30.7, 35.4.  One or two rows of more than 128 or 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
+// so a step is bound by the fullest row; what it saves is two kernels, 2 to 6 us.  us a step, general and this, half / a tenth of
+// the blocks attended (d = 128, blocks of 64, graph replay): 8 rows of 2K 20.0, 14.4 / 18.5, 14.4; 16K 28.3, 26.0 / 20.5, 18.5; 32K
+// 34.9, 33.8 / 22.5, 19.1; 16 rows of 16K 34.6, 31.6 / 22.6, 20.5; 64 rows of 2K 28.7, 25.2 / 20.5, 18.5; 128 rows of 2K 36.3, 32.8 /
+// 24.7, 22.6.  Beyond the line rows of unequal lengths and survivors lose (queued calls, before bounds took half as many MMAs on both
+// sides): 24 rows of up to 32K 46.0, 60.7 / 29.5, 27.4, 64 of up to 16K 50.0, 70.6 / 30.7, 35.4.  One or two rows of more than 128 or
+// 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
 // How many CTAs: clusters that fit the GPU at once, 18 SMs to a group, with some to spare for the predictor's: 16 rows in clusters of
 // 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
 int step_cluster(int rows, int nb_cap, int b, int n_sm) {
