@@ -5,6 +5,8 @@ import glob
 import os
 import subprocess
 import sys
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -35,14 +37,14 @@ def build(force: bool = False, verbose: bool = False, lib: str = LIB, extra_flag
         build_torch_module(force)
     if not force and not needs_build(lib):
         return lib
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC", "-shared", "-o", lib] + list(extra_flags) + sources()
-    cmd[1:1] = os.environ.get("ETA_NVCC_FLAGS", "").split()     # e.g. -DETA_WAIT_LIMIT=65536 while debugging
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-    subprocess.run(cmd, check=True)
+    cmd = [os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), *os.environ.get("ETA_NVCC_FLAGS", "").split(),
+           "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
+    cmd += (["-Xptxas", "-v"] if verbose else []) + list(extra_flags)
+    # a compiler per source file, side by side: two files with instances by the dozen take most of the time
+    with tempfile.TemporaryDirectory() as tmp, ThreadPoolExecutor(os.cpu_count() or 1) as pool:
+        objects = [os.path.join(tmp, os.path.basename(src) + ".o") for src in sources()]
+        list(pool.map(lambda so: subprocess.run([*cmd, "-c", so[0], "-o", so[1]], check=True), zip(sources(), objects)))
+        subprocess.run([*cmd, "-shared", "-o", lib, *objects], check=True)
     return lib
 
 
