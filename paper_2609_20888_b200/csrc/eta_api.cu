@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "eta_common.cuh"
+#include "eta_step.h"
 #include "eta_timeline.h"
 
 namespace eta {
@@ -103,12 +104,13 @@ int KernelAttrTable::configure(int dev, const void* kernel, size_t dyn_smem, Set
 static KernelAttrTable g_attr_table;
 
 static int cuda_setter(void*, const void* kernel, int attr, size_t value) {
-    cudaError_t e = (attr == KernelAttrTable::ATTR_CARVEOUT)
+    const cudaError_t e = (attr == KernelAttrTable::ATTR_CARVEOUT)
         ? cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)
         : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)value);
-    // (a permission only: clusters of more than eight CTAs, for the kernel that is launched in them)
-    if (e == cudaSuccess && attr == KernelAttrTable::ATTR_CARVEOUT)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // (a permission only: clusters of more than eight CTAs, for the kernel that is launched in them; without it they do not fit)
+    if (e == cudaSuccess && attr == KernelAttrTable::ATTR_CARVEOUT &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();
     if (e != cudaSuccess) { set_cuda_error(e, "kernel attribute"); return ETA_ERR_CUDA; }
     return 0;
 }
@@ -118,6 +120,50 @@ int configure_kernel(const void* kernel, size_t dyn_smem) {
     const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaGetDevice"); return ETA_ERR_CUDA; }
     return g_attr_table.configure(dev, kernel, dyn_smem, cuda_setter, nullptr);
+}
+
+// ---- clusters that fit
+void ClusterTable::get(int dev, const void* kernel, int (&fit)[MAX_CLUSTER + 1], Query query, void* ctx) {
+    std::lock_guard<std::mutex> lock(mu_);
+    const bool known_dev = dev >= 0 && dev < MAX_DEVICES;
+    if (known_dev)
+        for (int k = 0; k < n_[dev]; ++k)
+            if (tab_[dev][k].kernel == kernel) {
+                for (int c = 0; c <= MAX_CLUSTER; ++c) fit[c] = tab_[dev][k].fit[c];
+                return;
+            }
+    bool failed = false;
+    fit[0] = 0;
+    for (int c = 1; c <= MAX_CLUSTER; ++c) {
+        const int n = query(ctx, kernel, c);
+        failed = failed || n < 0;
+        fit[c] = n < 0 ? 0 : (n > INT16_MAX ? INT16_MAX : n);
+    }
+    // a device or kernel beyond the table's capacity is asked on every call, and so is one that could not answer
+    if (failed || !known_dev || n_[dev] == MAX_KERNELS) return;
+    Entry& e = tab_[dev][n_[dev]++];
+    e.kernel = kernel;
+    for (int c = 0; c <= MAX_CLUSTER; ++c) e.fit[c] = (int16_t)fit[c];
+}
+
+static ClusterTable g_cluster_table;
+
+struct ClusterQuery { int threads; size_t smem; };
+static int query_clusters(void* ctx, const void* kernel, int size) {
+    const ClusterQuery* q = static_cast<const ClusterQuery*>(ctx);
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(size, 1, q->threads, q->smem, attr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+    cudaGetLastError();                  // answered with "none": not an error of the call that asks
+    return -1;
+}
+
+void clusters_that_fit(const void* kernel, int threads, size_t smem, int (&fit)[MAX_CLUSTER + 1]) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    ClusterQuery q{threads, smem};
+    g_cluster_table.get(dev, kernel, fit, query_clusters, &q);
 }
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -192,6 +238,50 @@ int eta_selftest_kernel_attr_table(void) {
     int kc = 0;
     if (t.configure(2, &kc, 200 * 1024, fail, nullptr) != -4) return 9;
     if (t.configure(2, &kc, 200 * 1024, rec, &log) != 0 || log.carve != 6 || log.smem != 6) return 10;  // a failure is not remembered
+    return 0;
+}
+
+// Host-only check of the bookkeeping of clusters that fit and of the rule that goes by it, with made-up answers.  Not part of
+// the public interface; called by the CPU test-suite.  -> 0, or the number of the first expectation that failed.
+int eta_selftest_cluster_table(void) {
+    using T = eta::ClusterTable;
+    struct Gpu { int asked = 0, largest = 0, sms = 0; bool broken = false; } gpu;
+    auto query = [](void* ctx, const void*, int size) {
+        Gpu* g = static_cast<Gpu*>(ctx);
+        ++g->asked;
+        return g->broken ? -1 : (size > g->largest ? 0 : g->sms / size);
+    };
+    static T t;                        // own instance: the library's table is left alone
+    int ka = 0, kb = 0, fit[eta::MAX_CLUSTER + 1];
+    gpu.largest = 16; gpu.sms = 148;
+    t.get(0, &ka, fit, query, &gpu);
+    if (gpu.asked != eta::MAX_CLUSTER || fit[1] != 148 || fit[16] != 9) return 1;
+    t.get(0, &ka, fit, query, &gpu);
+    if (gpu.asked != eta::MAX_CLUSTER || fit[4] != 37) return 2;                         // remembered
+    gpu.largest = 4; gpu.sms = 20;
+    t.get(1, &ka, fit, query, &gpu);
+    if (gpu.asked != 2 * eta::MAX_CLUSTER || fit[4] != 5 || fit[5] != 0) return 3;       // another device: again
+    gpu.broken = true;
+    t.get(0, &kb, fit, query, &gpu);
+    if (fit[1] != 0 || fit[16] != 0) return 4;                                           // no answer: nothing fits
+    gpu.broken = false;
+    t.get(0, &kb, fit, query, &gpu);
+    if (fit[4] != 5) return 5;                                                           // a failure is not remembered
+    const int asked = gpu.asked;
+    t.get(T::MAX_DEVICES, &ka, fit, query, &gpu);
+    t.get(T::MAX_DEVICES, &ka, fit, query, &gpu);
+    if (gpu.asked != asked + 2 * eta::MAX_CLUSTER) return 6;                             // untracked: every call
+    // the rule never asks for clusters that do not fit, whatever the device
+    for (int largest = 0; largest <= eta::MAX_CLUSTER; ++largest)
+        for (int sms : {0, 1, 7, 18, 74, 148}) {
+            for (int c = 0; c <= eta::MAX_CLUSTER; ++c) fit[c] = c && c <= largest ? sms / c : 0;
+            for (int rows = 1; rows <= 256; ++rows)
+                for (int nb : {1, 31, 64, 65, 128, 263, 511, 512, 513})
+                    for (int b : {32, 64, 128}) {
+                        const int c = eta::step_cluster_rule(rows, nb, b, fit);
+                        if (c < 0 || c > eta::MAX_CLUSTER || (c && fit[c] < rows) || (c && nb > 512)) return 7;
+                    }
+        }
     return 0;
 }
 

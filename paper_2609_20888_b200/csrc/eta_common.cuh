@@ -151,6 +151,36 @@ private:
     int n_[MAX_DEVICES] = {};
 };
 
+// Clusters of each size that the current device holds at once of a kernel, asked for once per (device, kernel).  A launch in
+// clusters is refused where not even one fits (a part of a GPU, fewer SMs to a group), so whoever has another way asks first.
+constexpr int MAX_CLUSTER = 16;
+class ClusterTable {
+public:
+    static constexpr int MAX_DEVICES = 64, MAX_KERNELS = 32;
+    typedef int (*Query)(void* ctx, const void* kernel, int size);       // clusters of `size` CTAs; negative: the query failed
+    void get(int dev, const void* kernel, int (&fit)[MAX_CLUSTER + 1], Query query, void* ctx);
+private:
+    struct Entry { const void* kernel; int16_t fit[MAX_CLUSTER + 1]; };
+    std::mutex mu_;
+    Entry tab_[MAX_DEVICES][MAX_KERNELS] = {};
+    int n_[MAX_DEVICES] = {};
+};
+// fit[c]: clusters of c CTAs (1 .. MAX_CLUSTER); 0 where the query failed
+void clusters_that_fit(const void* kernel, int threads, size_t smem, int (&fit)[MAX_CLUSTER + 1]);
+// Launch configuration of `clusters` clusters of `size` CTAs; attr[0] holds the size, attr[1] is free
+inline cudaLaunchConfig_t cluster_config(int size, int clusters, int threads, size_t smem, cudaLaunchAttribute (&attr)[2]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * clusters));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 template <typename... KArgs, typename... Args>
 inline int launch_pdl(const char* what, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                       Args&&... args) {

@@ -1021,7 +1021,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     rc = make_tmap(&tmV, V, desc, desc->v_stride_b, desc->v_stride_h, desc->v_stride_t, TS, n_pages);
     if (rc != ETA_OK) return rc;
 
-    int step_ctas = dense ? 0 : step_cluster(L.rows, desc->nb_cap, b, n_sm);
+    int step_ctas = dense ? 0 : step_cluster(L.rows, desc->nb_cap, b, D, TS, G, (params->flags & ETA_FLAG_PACKED_SIGMA) != 0);
 #ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
     step_ctas = 0;                      // the test is of the streaming kernel
 #endif

@@ -351,29 +351,20 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
     }
 }
 
-template <int D, int TS, int G, bool PACKED>
-static int launch_step_t(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int n_ranks, cudaStream_t s) {
-    using L = StepSmem<D, TS, G>;
-    a.shared = n_ranks > 1 && a.nb_cap > STEP_WARPS * TileOf<D>::RECS;
-    const int rc = configure_kernel(reinterpret_cast<const void*>(step_kernel<D, TS, G, PACKED>), L::BYTES);
-    if (rc != ETA_OK) return rc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(rows * n_ranks));
-    cfg.blockDim = dim3(STEP_THREADS);
-    cfg.dynamicSmemBytes = L::BYTES;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)n_ranks;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, step_kernel<D, TS, G, PACKED>, tmK, tmV, a);
-    if (e != cudaSuccess) { set_cuda_error(e, "step launch"); return ETA_ERR_CUDA; }
-    return check_launch("step launch");
+// One instance of the kernel
+struct StepVariant {
+    void (*kernel)(CUtensorMap, CUtensorMap, StepArgs);
+    size_t smem;
+    int recs;                            // records that a warp bounds at a time
+};
+static bool step_variant(int D, int TS, int G, bool packed, StepVariant& v) {
+#define ETA_CASE(DD, TT, GG) if (D == DD && TS == TT && G == GG) { \
+        v = {packed ? step_kernel<DD, TT, GG, true> : step_kernel<DD, TT, GG, false>, StepSmem<DD, TT, GG>::BYTES, TileOf<DD>::RECS}; return true; }
+#define ETA_CASES(GG) ETA_CASE(128, 64, GG) ETA_CASE(128, 32, GG) ETA_CASE(64, 64, GG) ETA_CASE(64, 32, GG)
+    ETA_CASES(1) ETA_CASES(2) ETA_CASES(4) ETA_CASES(8)
+#undef ETA_CASES
+#undef ETA_CASE
+    return false;
 }
 
 // Which problems, by what the host knows: the capacity.  A row's cluster has to do alone what the general path spreads over the GPU,
@@ -383,27 +374,44 @@ static int launch_step_t(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& 
 // 24.7, 22.6.  Beyond the line rows of unequal lengths and survivors lose (queued calls, before bounds took half as many MMAs on both
 // sides): 24 rows of up to 32K 46.0, 60.7 / 29.5, 27.4, 64 of up to 16K 50.0, 70.6 / 30.7, 35.4.  One or two rows of more than 128 or
 // 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
-// How many CTAs: clusters that fit the GPU at once, 18 SMs to a group, with some to spare for the predictor's: 16 rows in clusters of
-// 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
-int step_cluster(int rows, int nb_cap, int b, int n_sm) {
+// How many CTAs: clusters that all fit the GPU at once, by its own answer (a B200 holds 45 of three CTAs, 33 of four, 22 of six, 15 of
+// eight, 7 of sixteen; a launch in clusters of which not one fits would be refused), with some to spare for the predictor's: 16 rows in
+// clusters of 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
+// fit[c]: clusters of c CTAs that the GPU holds at once.  -> 0: not a problem for this kernel, or not a GPU for it
+int step_cluster_rule(int rows, int nb_cap, int b, const int* fit) {
     const int tiles = b > 64 ? 2 * nb_cap : nb_cap;
     if (nb_cap > STEP_MAX_BLOCKS || (int64_t)rows * tiles > STEP_MAX_TILES || tiles > 128 * rows) return 0;
-    if (rows <= 4 && tiles > 64) return STEP_MAX_CLUSTER;
-    const int group = n_sm / 8;
+    if (rows <= 4 && tiles > 64 && fit[STEP_MAX_CLUSTER] >= rows) return STEP_MAX_CLUSTER;
     for (int c = 8; c >= 1; --c)
-        if (80 * (group / c) >= rows * (c > 4 ? 11 : 10)) return c;
+        if (10 * fit[c] >= rows * (c > 4 ? 11 : 10)) return c;
     return 0;
 }
 
-int launch_step(const StepArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int TS, int G, int n_ranks, cudaStream_t s) {
-    const bool packed = (a.flags & ETA_FLAG_PACKED_SIGMA) != 0;
-#define ETA_CASE(DD, TT, GG) if (D == DD && TS == TT && G == GG) return packed ? launch_step_t<DD, TT, GG, true>(a, tmK, tmV, rows, n_ranks, s) \
-                                                                               : launch_step_t<DD, TT, GG, false>(a, tmK, tmV, rows, n_ranks, s);
-#define ETA_CASES(GG) ETA_CASE(128, 64, GG) ETA_CASE(128, 32, GG) ETA_CASE(64, 64, GG) ETA_CASE(64, 32, GG)
-    ETA_CASES(1) ETA_CASES(2) ETA_CASES(4) ETA_CASES(8)
-#undef ETA_CASES
-#undef ETA_CASE
-    return ETA_ERR_UNSUPPORTED;
+int step_cluster(int rows, int nb_cap, int b, int D, int TS, int G, bool packed) {
+    StepVariant v;
+    if (nb_cap > STEP_MAX_BLOCKS || !step_variant(D, TS, G, packed, v)) return 0;
+    const void* const kernel = reinterpret_cast<const void*>(v.kernel);
+    if (configure_kernel(kernel, v.smem) != ETA_OK) return 0;
+    int fit[STEP_MAX_CLUSTER + 1];
+    clusters_that_fit(kernel, STEP_THREADS, v.smem, fit);
+    return step_cluster_rule(rows, nb_cap, b, fit);
+}
+
+int launch_step(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int TS, int G, int n_ranks, cudaStream_t s) {
+    StepVariant v;
+    if (!step_variant(D, TS, G, (a.flags & ETA_FLAG_PACKED_SIGMA) != 0, v)) return ETA_ERR_UNSUPPORTED;
+    a.shared = n_ranks > 1 && a.nb_cap > STEP_WARPS * v.recs;
+    const int rc = configure_kernel(reinterpret_cast<const void*>(v.kernel), v.smem);
+    if (rc != ETA_OK) return rc;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(n_ranks, rows, STEP_THREADS, v.smem, attr);
+    cfg.stream = s;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, v.kernel, tmK, tmV, a);
+    if (e != cudaSuccess) { set_cuda_error(e, "step launch"); return ETA_ERR_CUDA; }
+    return check_launch("step launch");
 }
 
 }  // namespace eta

@@ -7,7 +7,7 @@ namespace eta {
 
 constexpr int STEP_MAX_BLOCKS = 512;     // of a row: their bounds and the list of survivors stay in shared memory
 constexpr int STEP_MAX_TILES = 4096;     // of 64 (or 32) tokens, of all rows
-constexpr int STEP_MAX_CLUSTER = 16;     // CTAs of a row
+constexpr int STEP_MAX_CLUSTER = MAX_CLUSTER;     // CTAs of a row
 
 struct StepArgs {
     const __nv_bfloat16* q;
@@ -29,8 +29,9 @@ struct StepArgs {
     int32_t* stats;
     uint32_t* status;
 };
-// CTAs that a row gets in the one-kernel step; 0: the problem is not one for it
-int step_cluster(int rows, int nb_cap, int b, int n_sm);
-int launch_step(const StepArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int TS, int G, int n_ranks, cudaStream_t s);
+// CTAs that a row gets in the one-kernel step; 0: the problem is not one for it, or the GPU does not hold such clusters
+int step_cluster_rule(int rows, int nb_cap, int b, const int* fit);
+int step_cluster(int rows, int nb_cap, int b, int D, int TS, int G, bool packed);
+int launch_step(StepArgs a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int TS, int G, int n_ranks, cudaStream_t s);
 
 }  // namespace eta
