@@ -282,6 +282,15 @@ int eta_selftest_cluster_table(void) {
                         if (c < 0 || c > eta::MAX_CLUSTER || (c && fit[c] < rows) || (c && nb > 512)) return 7;
                     }
         }
+    // on a B200: neither clusters that do not all fit beside their predecessor's, nor more work than a row's CTAs do in the time
+    // that the general path takes
+    const int b200[eta::MAX_CLUSTER + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+    struct { int rows, nb, b, c; } want[] = {{8, 263, 64, 8}, {2, 64, 32, 8}, {1, 128, 64, 16}, {4, 512, 64, 16}, {16, 200, 64, 6},
+                                             {24, 128, 64, 4}, {64, 32, 64, 2}, {128, 24, 64, 1}, {48, 32, 64, 2}, {48, 64, 64, 0},
+                                             {5, 263, 64, 0}, {6, 512, 64, 0}, {8, 380, 64, 0}, {96, 32, 64, 0}, {1, 129, 64, 0},
+                                             {8, 131, 128, 8}, {8, 137, 128, 0}, {8, 513, 64, 0}};
+    for (const auto& w : want)
+        if (eta::step_cluster_rule(w.rows, w.nb, w.b, b200) != w.c) return 8;
     return 0;
 }
 

@@ -368,22 +368,29 @@ static bool step_variant(int D, int TS, int G, bool packed, StepVariant& v) {
 }
 
 // Which problems, by what the host knows: the capacity.  A row's cluster has to do alone what the general path spreads over the GPU,
-// so a step is bound by the fullest row; what it saves is two kernels, 2 to 6 us.  us a step, general and this, half / a tenth of
-// the blocks attended (d = 128, blocks of 64, graph replay): 8 rows of 2K 20.0, 14.4 / 18.5, 14.4; 16K 28.3, 26.0 / 20.5, 18.5; 32K
-// 34.9, 33.8 / 22.5, 19.1; 16 rows of 16K 34.6, 31.6 / 22.6, 20.5; 64 rows of 2K 28.7, 25.2 / 20.5, 18.5; 128 rows of 2K 36.3, 32.8 /
-// 24.7, 22.6.  Beyond the line rows of unequal lengths and survivors lose (queued calls, before bounds took half as many MMAs on both
-// sides): 24 rows of up to 32K 46.0, 60.7 / 29.5, 27.4, 64 of up to 16K 50.0, 70.6 / 30.7, 35.4.  One or two rows of more than 128 or
-// 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
+// so a step is bound by the fullest row's tiles per CTA (0.6 us a tile of 32 KB that is attended); what it saves is two kernels.  Beside
+// it, us a step by the general path and by this one, half / a twentieth of the blocks attended (d = 128, blocks of 64, G = 4, one
+// step a graph): 8 rows of 2K tokens 19.5, 14.4 / 18.4, 14.4; of 8K 22.6, 18.4 / 20.5, 14.4; of 16K (33 tiles a CTA) 24.6, 24.6 / 18.5,
+// 16.4; 16 rows of 12K (33) 25.3, 24.6 / 20.5, 16.7; 24 rows of 8K (32) 26.5, 24.6 / 20.5, 16.4; 4 rows of 32K (32) 22.8, 24.6 / 18.5,
+// 16.8; 64 rows of 2K (16) 24.5, 22.6 / 19.9, 16.6.  Not taken, because what half the blocks lose is more than what few of them gain:
+// 6 rows of 16K (33, in 48 CTAs) 22.6, 26.7 / 18.5, 16.4, of 32K (64) 24.6, 41.3 / 20.2, 18.5; 14 rows of 12K (33) 24.6, 30.7 / 20.5,
+// 20.5; 48 rows of 4K in clusters of two (32) 25.0, 28.7 / 19.2, 17.6; 96 rows of 2K, one CTA each (32) 27.2, 28.8 / 20.5, 19.4.  So: up
+// to 24 tiles a CTA, and up to 34 where the problem is large enough to leave the general path something to do and clusters of
+// four or more take the difference between rows.  Of 900 problems of 1 to 256 rows at 0.1 to 0.95 sparsity 17 lose more than 3 % this
+// way (12 % at most, with half or more of the blocks attended); by the number of tiles in all alone it was 90 (39 %).  One or two
+// rows of more than 128 or 256 tiles leave most of the GPU idle: 2 rows of 510 21.2, 23.7.
 // How many CTAs: clusters that all fit the GPU at once, by its own answer (a B200 holds 45 of three CTAs, 33 of four, 22 of six, 15 of
 // eight, 7 of sixteen; a launch in clusters of which not one fits would be refused), with some to spare for the predictor's: 16 rows in
-// clusters of 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
+// clusters of 6 15.5 us, of 3 16.6, of 8, which do not all fit beside it, 24.1; 48 rows of 2K in clusters of three, which do not fit
+// either, 24.6, of two 16.4; four rows of many tiles in clusters of 16 24.1, of 8 28.1.
 // fit[c]: clusters of c CTAs that the GPU holds at once.  -> 0: not a problem for this kernel, or not a GPU for it
 int step_cluster_rule(int rows, int nb_cap, int b, const int* fit) {
-    const int tiles = b > 64 ? 2 * nb_cap : nb_cap;
-    if (nb_cap > STEP_MAX_BLOCKS || (int64_t)rows * tiles > STEP_MAX_TILES || tiles > 128 * rows) return 0;
+    const int tiles = b > 64 ? 2 * nb_cap : nb_cap, all = rows * tiles;
+    if (nb_cap > STEP_MAX_BLOCKS || rows > STEP_MAX_TILES || all > STEP_MAX_TILES || tiles > 128 * rows) return 0;
     if (rows <= 4 && tiles > 64 && fit[STEP_MAX_CLUSTER] >= rows) return STEP_MAX_CLUSTER;
     for (int c = 8; c >= 1; --c)
-        if (10 * fit[c] >= rows * (c > 4 ? 11 : 10)) return c;
+        if (c > 4 ? 10 * fit[c] >= 11 * rows : fit[c] > rows)
+            return tiles <= 24 * c || (tiles <= 34 * c && c >= 4 && all >= 2000) ? c : 0;
     return 0;
 }
 

@@ -8,8 +8,8 @@ from paper_2609_20888_b200 import build as ebuild
 
 def test_clusters_that_do_not_fit_are_not_launched():
     """A self-check of the library with made-up devices: the answer is asked for once per (device, kernel), a query that fails
-    counts as "none" and is not remembered, and the rule falls back to smaller clusters or to the general path.  0 = every
-    expectation held."""
+    counts as "none" and is not remembered, and the rule falls back to smaller clusters or to the general path; with a B200's
+    answers, problems on either side of the line.  0 = every expectation held."""
     ebuild.build()
     lib = eb.load()
     lib.eta_selftest_cluster_table.restype = ctypes.c_int
