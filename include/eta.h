@@ -144,7 +144,7 @@ int eta_append_summary(const eta_cache_desc* desc, const void* K, const int32_t*
  * Both 16-byte aligned, the size a multiple of 16 bytes (else ETA_ERR_UNSUPPORTED).  Ordered like any kernel on
  * `stream`; the calls that follow on the stream see the complete copy.  Launched with programmatic dependent launch: the
  * kernel waits for everything before it in the stream before it reads or writes, and releases its successors only as it
- * ends.  The host buffer must stay unchanged until the kernel has run.  In the same way `out` of eta_decode may be page-locked host memory: the merge kernel's
+ * ends.  The host buffer must stay unchanged until the kernel has run.  In the same way `out` of eta_decode may be page-locked host memory: the last kernel's
  * stores then go straight to the host and are visible once the stream has been synchronised.
  */
 int eta_stage_query(int32_t batch, int32_t n_q_heads, int32_t head_dim, const void* q_host, void* q_dev,
@@ -288,7 +288,8 @@ int eta_decode_static(const eta_cache_desc* desc, const eta_params* params, cons
  * of the sequence; entries for j up to floor((T_i - 1) / block_size) must be valid page numbers in [0, n_pages)
  * (the last of them is the partly filled tail page), the others are never read.  The summaries (musig, mnorm) and
  * sel_mask stay indexed by (sequence, KV head, block) as in the contiguous case: they are the held-out table.
- * The three calls compute exactly what their contiguous counterparts compute on the gathered cache, bit for bit.
+ * The three calls compute exactly what their contiguous counterparts compute on the gathered cache with the same nb_cap, bit for bit
+ * (another nb_cap may select another of eta_decode's paths: the same blocks, outputs that differ by rounding).
  * Ownership, alignment, error behaviour: as for the contiguous calls; a NULL table, table_stride too small or
  * n_pages <= 0 return ETA_ERR_INVALID_ARG.  Page numbers are not range-checked on the device.
  */
@@ -312,10 +313,18 @@ int eta_decode_paged(const eta_cache_desc* desc, const eta_page_table* pages, co
 /* Size of the built-in scratch of eta_decode_static, in bytes. */
 size_t eta_static_scratch_bytes(void);
 
-/* Number of kernels one eta_decode call launches (for launch accounting); a rescue window that spans more blocks than one
- * CTA screens (by default more than 128, head_dim 128, or 256, head_dim 64) takes one more, and a small problem (by
- * the capacity of the cache: up to 512 blocks a sequence) only one in all, which leaves the workspace alone. */
+/* Number of kernels an eta_decode call launches where nothing makes it more or fewer: see eta_decode_launches. */
 int eta_decode_kernel_count(void);
+
+/*
+ * Number of kernels that an eta_decode (or eta_decode_paged, eta_decode_static) call with this descriptor and these parameters
+ * launches on the current device, for launch accounting; or a negative status.  It is 3 (screen, decode, merge) as a rule; 4
+ * where the rescue window spans more blocks than one CTA screens (by default more than 128, head_dim 128, or 256, head_dim 64);
+ * and 1 for a small problem, which leaves the workspace alone.  What counts as small goes by the descriptor: at most 512 blocks a
+ * sequence (nb_cap), and few enough for the CTAs that a (sequence, KV head) row gets.  So a cache that is described with the
+ * capacity it needs for now gets the faster path of the two, one that is described with room for much more does not.
+ */
+int eta_decode_launches(const eta_cache_desc* desc, const eta_params* params);
 
 /*
  * Per-kernel timing of a decode step (measurement aid; the paper has no counterpart).  While enabled,
@@ -324,7 +333,8 @@ int eta_decode_kernel_count(void);
  * eta_profile_read waits for the most recent eta_decode to finish and writes the time from each launch to the
  * next, in milliseconds, to ms[0 .. count-1] (n >= 5), in the order append, predict, screen, decode, merge,
  * returning the count, or a negative status when no profiled eta_decode has run.  The first two are 0
- * unless those calls were made, in that order, right before the eta_decode.  Process-wide state (one set of
+ * unless those calls were made, in that order, right before the eta_decode.  Where eta_decode_launches is 1 the one kernel's time is
+ * reported as decode, and screen and merge are next to nothing.  Process-wide state (one set of
  * events, created on the device that is current at the first mark; calls are serialised by a lock): for one
  * measuring thread on one device; leave disabled in production.
  */

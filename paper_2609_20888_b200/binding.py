@@ -27,7 +27,7 @@ ETA_DEV_TIMEOUT, ETA_DEV_LEN_CLAMPED, ETA_DEV_EMPTY_ROW = 1, 2, 4
 
 EXPORTS = ("eta_workspace_bytes", "eta_build_block_summaries", "eta_append_summary", "eta_build_block_summaries_paged",
            "eta_append_summary_paged", "eta_decode_paged", "eta_stage_query", "eta_predict_threshold",
-           "eta_score_dual", "eta_calibration_workspace_bytes", "eta_calibrate_head_const", "eta_decode", "eta_decode_static", "eta_static_scratch_bytes", "eta_decode_kernel_count", "eta_profile_enable", "eta_profile_read",
+           "eta_score_dual", "eta_calibration_workspace_bytes", "eta_calibrate_head_const", "eta_decode", "eta_decode_static", "eta_static_scratch_bytes", "eta_decode_kernel_count", "eta_decode_launches", "eta_profile_enable", "eta_profile_read",
            "eta_profile_kernel_name", "eta_set_pdl", "eta_strerror", "eta_last_cuda_error")
 
 
@@ -111,6 +111,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         lib.eta_decode_static.argtypes = [D, P, vp, vp, vp, i32p, vp, f32p, f32p, f32p, f32p, vp, i32p, vp, vp]
         lib.eta_static_scratch_bytes.restype = ctypes.c_size_t
         lib.eta_decode_kernel_count.restype = ctypes.c_int
+        lib.eta_decode_launches.argtypes = [D, P]
         lib.eta_strerror.restype = ctypes.c_char_p
         lib.eta_strerror.argtypes = [ctypes.c_int]
         lib.eta_last_cuda_error.restype = ctypes.c_char_p
@@ -331,6 +332,14 @@ def eta_static_scratch_bytes() -> int:
 
 def eta_decode_kernel_count() -> int:
     return load().eta_decode_kernel_count()
+
+
+def eta_decode_launches(desc: CacheDesc, params: DecodeParams) -> int:
+    """Kernels that eta_decode launches for this cache and these parameters on the current device."""
+    n = load().eta_decode_launches(ctypes.byref(desc), ctypes.byref(params.c()))
+    if n < 0:
+        _check(n, "eta_decode_launches")
+    return n
 
 
 def eta_set_pdl(on: bool) -> None:

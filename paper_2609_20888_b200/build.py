@@ -17,7 +17,7 @@ HEADER = os.path.join(os.path.dirname(HERE), "include", "eta.h")
 # A second copy of the library for one test: a consumer warp of the streaming kernel skips a barrier arrival, and the
 # bounded waits are short (2^16 polls, a few milliseconds), so that a give-up path runs and can be checked.
 GIVEUP_LIB = os.path.join(HERE, "libeta_b200_test_giveup.so")
-GIVEUP_FLAGS = ["-DETA_TEST_SKIP_FLUSH_ARRIVE", "-DETA_WAIT_LIMIT=65536"]
+GIVEUP_FLAGS = ["-DETA_TEST_SKIP_FLUSH_ARRIVE", "-DETA_TEST_GENERAL_PATH", "-DETA_WAIT_LIMIT=65536"]
 
 
 def sources() -> list[str]:

@@ -115,6 +115,7 @@ struct ScreenArgs {
 };
 int encode_tiles(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
                  const cuuint32_t* box);
+int screen_launches(int rows, int nseg, int nb_cap, int D, int window, bool dense, int n_sm);       // kernels that launch_screen launches
 int launch_screen(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int D, int G, int n_sm, cudaStream_t s);
 
 // Launch with programmatic dependent launch allowed: the grid may start while its predecessor in the stream is

@@ -956,6 +956,26 @@ static int launch_decode_t(const CUtensorMap& tmK, const CUtensorMap& tmV, const
                       dim3(32 * (WARPS_PER_GROUP * NGROUPS + 1)), smem, s, tmK, tmV, a);
 }
 
+// Streaming multiprocessors of the current device; negative: an eta_status
+static int sm_count() {
+    int dev = 0, n_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) { set_cuda_error(e, "device query"); return ETA_ERR_CUDA; }
+    return n_sm;
+}
+
+// CTAs that a row gets in the one-kernel step; 0: the general path
+static int step_ctas(const eta_cache_desc* desc, const eta_params* params) {
+#ifdef ETA_TEST_GENERAL_PATH
+    return 0;                           // test builds of the general path
+#endif
+    const int b = desc->block_size;
+    if (params->flags & ETA_FLAG_DENSE) return 0;
+    return step_cluster(desc->batch * desc->n_kv_heads, desc->nb_cap, b, desc->head_dim, b < 64 ? b : 64,
+                        desc->n_q_heads / desc->n_kv_heads, (params->flags & ETA_FLAG_PACKED_SIGMA) != 0);
+}
+
 // eta_decode and eta_decode_paged: `pages` null selects the contiguous cache
 static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, const eta_params* params, const void* q,
                        const void* K, const void* V, const int32_t* seq_lens, const void* musig, const float* mnorm,
@@ -982,10 +1002,8 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     const int G = desc->n_q_heads / desc->n_kv_heads;
     const float scale = params->scale > 0.f ? params->scale : 1.0f / sqrtf((float)D);
 
-    int dev = 0, n_sm = 0;
-    cudaError_t ce = cudaGetDevice(&dev);
-    if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (ce != cudaSuccess) { set_cuda_error(ce, "device query"); return ETA_ERR_CUDA; }
+    const int n_sm = sm_count();
+    if (n_sm < 0) return n_sm;
     const int TS = b < 64 ? b : 64;
     int n_ctas = n_sm;                  // one persistent CTA per SM; the shared-memory ring fills the SM
     if (n_ctas > MAX_CTAS) n_ctas = MAX_CTAS;
@@ -1021,11 +1039,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
     rc = make_tmap(&tmV, V, desc, desc->v_stride_b, desc->v_stride_h, desc->v_stride_t, TS, n_pages);
     if (rc != ETA_OK) return rc;
 
-    int step_ctas = dense ? 0 : step_cluster(L.rows, desc->nb_cap, b, D, TS, G, (params->flags & ETA_FLAG_PACKED_SIGMA) != 0);
-#ifdef ETA_TEST_SKIP_FLUSH_ARRIVE
-    step_ctas = 0;                      // the test is of the streaming kernel
-#endif
-    if (step_ctas) {
+    if (const int ctas = step_ctas(desc, params)) {
         StepArgs st;
         st.q = sa.q; st.musig = sa.musig; st.mnorm = mnorm; st.seq_lens = seq_lens; st.tau = tau; st.head_const = head_const;
         st.z = params->z; st.a = params->a; st.scale = scale; st.beta = params->beta;
@@ -1037,7 +1051,7 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
         st.out = out; st.sel_mask = sel_mask; st.stats = stats; st.status = status_dev;
         profile_mark(2, s);
         profile_mark(3, s);
-        rc = launch_step(st, tmK, tmV, L.rows, D, TS, G, step_ctas, s);
+        rc = launch_step(st, tmK, tmV, L.rows, D, TS, G, ctas, s);
         profile_mark(4, s);
         profile_mark(5, s);
         return rc;
@@ -1115,6 +1129,18 @@ static int decode_impl(const eta_cache_desc* desc, const eta_page_table* pages, 
 extern "C" {
 
 int eta_decode_kernel_count(void) { return 3; }
+
+int eta_decode_launches(const eta_cache_desc* desc, const eta_params* params) {
+    using namespace eta;
+    const int rc = validate_desc(desc);
+    if (rc != ETA_OK) return rc;
+    if (!params || params->rescue_window < 1 || params->lwb < 0) return ETA_ERR_INVALID_ARG;
+    const int n_sm = sm_count();
+    if (n_sm < 0) return n_sm;
+    if (step_ctas(desc, params)) return 1;
+    const WsLayout L = ws_layout(desc);
+    return 2 + screen_launches(L.rows, L.nseg, desc->nb_cap, desc->head_dim, params->rescue_window, (params->flags & ETA_FLAG_DENSE) != 0, n_sm);
+}
 
 int eta_decode(const eta_cache_desc* desc, const eta_params* params, const void* q, const void* K, const void* V,
                const int32_t* seq_lens, const void* musig, const float* mnorm, const float* tau,

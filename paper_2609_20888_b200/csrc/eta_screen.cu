@@ -458,6 +458,24 @@ __global__ void __launch_bounds__(128) score_dual_warp_kernel(
 
 // ------------------------------------------------------------------ launchers (host)
 
+// Passes that all CTAs but a row's first take at full length, passes that the rescue window spans, and whether rescue_kernel settles
+// rescue.  A window of more passes than a row's other CTAs take would be its first CTA's work alone, one pass after another: a kernel
+// of its own settles rescue then, for 1 to 3 us a step.  128K x 4 (d = 128, two passes per CTA), windows of 128 blocks 58 us;
+// 256 63.8 in the first CTA, 60.2 this way; 1024 90.9 and 60.5; all blocks 117.6 and 61.0 (512K x 1: 192 and 38.7; 64K, d = 64,
+// G = 8: 76.0 and 32.6).
+struct ScreenSplit { int tp, need; bool late; };
+static ScreenSplit screen_split(int rows, int nseg, int nb_cap, int pass, int window, bool dense, int n_sm) {
+    const int passes = (nseg + pass / SEG - 1) / (pass / SEG), slots = SCR_SLOTS * n_sm;
+    ScreenSplit p;
+    p.tp = (int)(((int64_t)rows * passes + slots - 1) / slots);
+    p.need = ((window < nb_cap ? window : nb_cap) + pass - 1) / pass;
+    p.late = !dense && p.need > (p.tp > SCR_WINDOW ? p.tp : SCR_WINDOW);
+    return p;
+}
+int screen_launches(int rows, int nseg, int nb_cap, int D, int window, bool dense, int n_sm) {
+    return screen_split(rows, nseg, nb_cap, D == 128 ? TileOf<128>::PASS : TileOf<64>::PASS, window, dense, n_sm).late ? 2 : 1;
+}
+
 template <int D, int G, bool PACKED>
 static int launch_screen_t(const ScreenArgs& a, const CUtensorMap& tmK, const CUtensorMap& tmV, int rows, int n_sm, cudaStream_t s) {
     constexpr int SPP = TileOf<D>::PASS / SEG;
@@ -465,18 +483,13 @@ static int launch_screen_t(const ScreenArgs& a, const CUtensorMap& tmK, const CU
     b2.passes = (a.nseg + SPP - 1) / SPP;
     b2.batch = rows / a.Hkv;
     b2.slots = SCR_SLOTS * n_sm;
-    const int window = a.rescue_window < a.nb_cap ? a.rescue_window : a.nb_cap;
-    b2.need = (window + TileOf<D>::PASS - 1) / TileOf<D>::PASS;
     // the split at full length: what rows of any length stay below, and what is used where there are too many to look at
     const int64_t all = (int64_t)rows * b2.passes;
-    b2.tp = (int)((all + b2.slots - 1) / b2.slots);
-    // A window of more passes than a row's other CTAs take would be its first CTA's work alone, one pass after another: a kernel
-    // of its own settles rescue then, for 1 to 3 us a step.  128K x 4 (d = 128, two passes per CTA), windows of 128 blocks 58 us;
-    // 256 63.8 in the first CTA, 60.2 this way; 1024 90.9 and 60.5; all blocks 117.6 and 61.0 (512K x 1: 192 and 38.7; 64K, d = 64,
-    // G = 8: 76.0 and 32.6).
-    const bool late = !(a.flags & ETA_FLAG_DENSE) && b2.need > (b2.tp > SCR_WINDOW ? b2.tp : SCR_WINDOW);
-    if (late) b2.need = 0;
-    else b2.resc = nullptr;
+    const ScreenSplit split = screen_split(rows, a.nseg, a.nb_cap, TileOf<D>::PASS, a.rescue_window, (a.flags & ETA_FLAG_DENSE) != 0, n_sm);
+    const bool late = split.late;
+    b2.tp = split.tp;
+    b2.need = late ? 0 : split.need;
+    if (!late) b2.resc = nullptr;
     const int head = b2.tp > b2.need ? b2.tp : b2.need;
     b2.ctas_row = b2.passes <= head ? 1 : 1 + (b2.passes - head + b2.tp - 1) / b2.tp;
     b2.div_ctas = FastDiv(b2.ctas_row);
