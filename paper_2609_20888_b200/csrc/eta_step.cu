@@ -301,8 +301,9 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
         if (M != -INFINITY) {
 #pragma unroll
             for (int w = 0; w < STEP_WARPS; ++w) {
-                const float sc = exp2f((warp_m[w * 8 + h] - M) * LOG2E);
-                const float4 x = *reinterpret_cast<const float4*>(parts + (w * G + h) * D + 4 * dq);
+                // (a warp whose tiles the head did not attend: its part may be 0 * infinity)
+                const float m = warp_m[w * 8 + h], sc = exp2f((m - M) * LOG2E);
+                const float4 x = m == -INFINITY ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(parts + (w * G + h) * D + 4 * dq);
                 acc.x = fmaf(x.x, sc, acc.x); acc.y = fmaf(x.y, sc, acc.y);
                 acc.z = fmaf(x.z, sc, acc.z); acc.w = fmaf(x.w, sc, acc.w);
                 lacc = fmaf(warp_l[w * 8 + h], sc, lacc);
