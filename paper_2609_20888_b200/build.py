@@ -14,10 +14,12 @@ LIB = os.path.join(HERE, "libeta_b200.so")
 HEADER = os.path.join(os.path.dirname(HERE), "include", "eta.h")
 
 
-# A second copy of the library for one test: a consumer warp of the streaming kernel skips a barrier arrival, and the
-# bounded waits are short (2^16 polls, a few milliseconds), so that a give-up path runs and can be checked.
+# Copies of the library for tests.  Two in which a consumer warp, of the streaming kernel or of the one-kernel step, skips a
+# barrier arrival and the bounded waits are short (2^16 polls, a few milliseconds), so that a give-up path runs and can be checked.
 GIVEUP_LIB = os.path.join(HERE, "libeta_b200_test_giveup.so")
 GIVEUP_FLAGS = ["-DETA_TEST_SKIP_FLUSH_ARRIVE", "-DETA_TEST_GENERAL_PATH", "-DETA_WAIT_LIMIT=65536"]
+GIVEUP_STEP_LIB = os.path.join(HERE, "libeta_b200_test_giveup_step.so")
+GIVEUP_STEP_FLAGS = ["-DETA_TEST_SKIP_STAGE_ARRIVE", "-DETA_WAIT_LIMIT=65536"]
 
 
 def sources() -> list[str]:
@@ -96,6 +98,10 @@ def build_torch_module(force: bool = False) -> str:
 
 def build_giveup_variant(force: bool = False) -> str:
     return build(force=force, lib=GIVEUP_LIB, extra_flags=tuple(GIVEUP_FLAGS))
+
+
+def build_giveup_step_variant(force: bool = False) -> str:
+    return build(force=force, lib=GIVEUP_STEP_LIB, extra_flags=tuple(GIVEUP_STEP_FLAGS))
 
 
 if __name__ == "__main__":

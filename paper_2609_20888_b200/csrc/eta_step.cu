@@ -36,7 +36,9 @@ struct StepSmem {
     static constexpr size_t BYTES = 1024 + WARP_ML_OFF + 8 * STEP_WARPS * 8;
 };
 
-// A barrier of the cluster in two halves; what was stored before the first is there after the second
+// A barrier of the cluster in two halves; what was stored before the first is there after the second.  The hardware has no bounded
+// form of it.  Every thread reaches every one: what stands between two barriers are bounded waits, after which a warp goes on to the
+// next barrier with whatever it has (no early return in the kernel).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
@@ -261,8 +263,14 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_cons
             locate(k, ent, sub, rows);
             const int nvalid = min(TS, rows), last = T - 1 - ((ent & 0xffffff) * b + sub * TS);      // the newest token's row of the tile
             const int urow = (a.flags & ETA_FLAG_UNGATE_LAST) && last < TS ? last : 0xff;
-            at.tile(smem_u32(sm + stage * L::STAGE_BYTES), (ent >> 24) & 0xff, urow, nvalid, a.scale, a.beta,
-                    [&]() { if (lane == 0) mbar_arrive(&empty[stage]); });
+            at.tile(smem_u32(sm + stage * L::STAGE_BYTES), (ent >> 24) & 0xff, urow, nvalid, a.scale, a.beta, [&]() {
+#ifdef ETA_TEST_SKIP_STAGE_ARRIVE
+                // test build only: one warp of the first CTA never releases its stages, so that the waits of the warp that issues the
+                // copies, and then of the warps that wait for them, run out
+                if (blockIdx.x == 0 && warp == 1) return;
+#endif
+                if (lane == 0) mbar_arrive(&empty[stage]);
+            });
         }
     }
     if (!ok && lane == 0 && a.status) atomicOr(a.status, ETA_DEV_TIMEOUT);
