@@ -20,6 +20,9 @@ GIVEUP_LIB = os.path.join(HERE, "libeta_b200_test_giveup.so")
 GIVEUP_FLAGS = ["-DETA_TEST_SKIP_FLUSH_ARRIVE", "-DETA_TEST_GENERAL_PATH", "-DETA_WAIT_LIMIT=65536"]
 GIVEUP_STEP_LIB = os.path.join(HERE, "libeta_b200_test_giveup_step.so")
 GIVEUP_STEP_FLAGS = ["-DETA_TEST_SKIP_STAGE_ARRIVE", "-DETA_WAIT_LIMIT=65536"]
+# And one that takes the general path whatever the size: small problems reach its edges too.
+GENERAL_LIB = os.path.join(HERE, "libeta_b200_test_general.so")
+GENERAL_FLAGS = ["-DETA_TEST_GENERAL_PATH"]
 
 
 def sources() -> list[str]:
@@ -102,6 +105,10 @@ def build_giveup_variant(force: bool = False) -> str:
 
 def build_giveup_step_variant(force: bool = False) -> str:
     return build(force=force, lib=GIVEUP_STEP_LIB, extra_flags=tuple(GIVEUP_STEP_FLAGS))
+
+
+def build_general_variant(force: bool = False) -> str:
+    return build(force=force, lib=GENERAL_LIB, extra_flags=tuple(GENERAL_FLAGS))
 
 
 if __name__ == "__main__":
