@@ -57,8 +57,8 @@ __device__ __forceinline__ void zero_bytes(uint8_t* p, int n, int tid) {
 // 68.8 us instead of 71.1 with it (two persistent CTAs per SM, the variance term on the fp32 pipe behind a shuffle tree and a CTA
 // barrier per segment); 65536 blocks at d = 64, G = 8, where both terms were on that pipe, 116.3 instead of 126.9.
 // Registers: CTAs start beside those of the append and the predictor, and with more registers fewer of them fit there.  The bound of
-// six CTAs holds the instances to 80 that would take many more by themselves.  The others take 78 to 86 at five (96 at d = 64, G = 8):
-// six gives d = 128, G = 4 48.5 instead of 49.1 us at 32K x 8, but 57.9 instead of 57.6 at 128K x 4 and 41.9 instead of 41.5 at 512K x 1,
+// six CTAs holds the instances to 80 that would take many more by themselves.  The others take 77 to 88 at five, at d = 64, G = 8
+// 95 (packed 96 and 32 bytes spilled): six gives d = 128, G = 4 48.5 instead of 49.1 us at 32K x 8, but 57.9 instead of 57.6 at 128K x 4 and 41.9 instead of 41.5 at 512K x 1,
 // and d = 64 32.8 instead of 31.8 at 64K x 4 (G = 1).
 template <int D, int G, bool PACKED>
 __global__ void __launch_bounds__(32 * SCR_WARPS, D == 128 && (G == 8 || (G == 4 && PACKED)) ? 6 : 5) screen_kernel(
@@ -367,9 +367,11 @@ __global__ void __launch_bounds__(256) rescue_kernel(const int2* span, const int
 }
 
 // Eq. dual_bound_eq for every block, for its own sake: the tiles of the screening kernel, stored instead of compared.
-// Bound by HBM (33.8 MB of records in, 8.4 MB of bounds out at 65536 blocks, d = 128, G = 4: 6.4 us at the copy rate); a
-// record is read once for all heads of its group.  12.2 us there for the kernel alone, against 108 us with a warp per (head,
-// block) that read every record G times in 2-byte pieces and reduced three sums over 32 lanes for each.
+// Bound by HBM (33.8 MB of records in, 1.05 MB of bounds out at 65536 blocks, d = 128, G = 4: 5.3 us at the copy rate) and by the two
+// round trips of a CTA's two passes; a record is read once for all heads of its group.  8.2 us a call there as one of four nodes of a
+// graph (9.2 before the records were the rows of the MMAs; of 65536 blocks at d = 64, 7.3 -> 5.5 for G = 1, 6.7 -> 5.6 for G = 4), some
+// 10 queued eagerly, which is what the host takes for a call; 108 us with a warp per (head, block) that read every record G times in
+// 2-byte pieces and reduced three sums over 32 lanes for each.
 template <int D, int G, bool PACKED>
 __global__ void __launch_bounds__(32 * SCR_WARPS, 5) score_dual_kernel(
     const __nv_bfloat16* q, const unsigned char* musig, const float* mnorm, const int32_t* seq_lens, int Hq, int Hkv, int b,

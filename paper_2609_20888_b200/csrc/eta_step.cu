@@ -52,6 +52,8 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 // for 32 blocks, 1.1 faster for 256 and 4 for 511.  Two tiles of records in flight per warp where a share is more than one.  Six 32 KB tiles in flight: with three, rows of 256 blocks, half of them
 // attended, took 29.5 us instead of 25.5.  Parts are stored to the CTA that adds them up, not fetched by it: one barrier of the
 // cluster instead of two, 0.6 to 0.8 us.
+// Registers: the 13th warp, which issues the copies, makes four warps on one scheduler and so 128 registers the most.  At head_dim 128 the
+// instances want a few more (28 to 64 bytes spilled), at 64 they take 98 to 115.
 template <int D, int TS, int G, bool PACKED>
 __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                const __grid_constant__ CUtensorMap tmV, const StepArgs a) {
