@@ -334,7 +334,7 @@ int eta_decode_launches(const eta_cache_desc* desc, const eta_params* params);
  * next, in milliseconds, to ms[0 .. count-1] (n >= 5), in the order append, predict, screen, decode, merge,
  * returning the count, or a negative status when no profiled eta_decode has run.  The first two are 0
  * unless those calls were made, in that order, right before the eta_decode.  Where eta_decode_launches is 1 the one kernel's time is
- * reported as decode, and screen and merge are next to nothing.  Process-wide state (one set of
+ * reported as decode, and screen and merge hold what two events in a row take.  Process-wide state (one set of
  * events, created on the device that is current at the first mark; calls are serialised by a lock): for one
  * measuring thread on one device; leave disabled in production.
  */
